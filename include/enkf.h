@@ -107,7 +107,9 @@ typedef struct enkf_config {
                              max_iter bounds them                                         */
   double inner_tol;       /* FP32, BF16 and FP16 modes: relative tolerance of each inner
                              solve (default 1e-5); the tensor-core modes raise it to the
-                             floor their operator allows (see refresh_every)              */
+                             floor their operator allows (see refresh_every). Solves in
+                             Krylov coordinates (see precondition) do not use it: their
+                             inner solve reaches tol itself                               */
   int32_t refresh_every;  /* BF16/FP16 modes: cap on CG steps between double-float residual
                              refreshes; 0 (default): each inner solve runs until its
                              residual fell by inner_tol, but not below what the operator
@@ -121,7 +123,15 @@ typedef struct enkf_config {
   int32_t grid_blocks;    /* 0: automatic persistent-grid size; > 0: use this many CTAs  */
   int32_t precondition;   /* ENKF_CGD: 0 plain CG (the paper's method); 1 CG preconditioned
                              by R (Jacobi), which ends within about N steps because
-                             R^-1/2 S R^-1/2 is the identity plus a rank < N term        */
+                             R^-1/2 S R^-1/2 is the identity plus a rank < N term. With 1,
+                             fixed_iters = 0 and (BF16/FP16) lowprec_terms != 1 and
+                             refresh_every <= 0, the FP32, BF16 and FP16 modes all carry
+                             the recurrences in the coordinates of their Krylov space:
+                             z = R^-1 (d - HA w) with an N-vector w per column, started at
+                             w = 0 (z = R^-1 d). The products with HA that remain run on the
+                             tensor cores with operands of five 9-bit FP16 slices (44 bits,
+                             exact FP32 sums), the N x N recurrences in FP32 pairs, and the
+                             result is certified by the true residual as in every mode    */
   int32_t lowprec_terms;  /* BF16/FP16 modes: 3 (or 0, the default) splits every operand
                              into hi + lo parts and forms hi*hi + hi*lo + lo*hi (about 16
                              significant bits); 1 uses single BF16/FP16 operands, whose
@@ -173,6 +183,7 @@ enkf_status enkf_config_default(enkf_config* cfg, int64_t n, int64_t m, int32_t 
    and are copied to the device. cuda_stream is a cudaStream_t (NULL: the legacy default
    stream); every later call on the handle is ordered on it. Allocates all workspace
    (about 56 m N + 4 n N bytes in ENKF_FP32 mode, 4 m N more in the tensor-core modes,
+   28 m N + 4 n N in either when the solve runs in Krylov coordinates (see precondition),
    48 m N + 8 n N in ENKF_FP64 mode, plus O(grid N^2); ENKF_CGD_REDUCED and ENKF_SENKF keep
    no m x N arrays: 4 or 8 n N bytes plus O(grid N^2)). Errors: ENKF_ERR_INVALID_ARG (bad
    shape, column index outside [0, n), decreasing rowptr, r <= 0), ENKF_ERR_UNSUPPORTED
@@ -272,9 +283,11 @@ enkf_status enkf_set_phase_timing(enkf_handle h, int32_t enable);
 enkf_status enkf_get_phase_times(enkf_handle h, float* ms);
 
 /* Synchronise and return the in-kernel phase timers of the last timed solve, measured by
-   CTA 0 with the global nanosecond timer, in microseconds: us[0] set-up reductions,
-   us[1] fused CG passes, us[2] first grid barrier, us[3] cross-CTA reduction, us[4] second
-   grid barrier, us[5] scalar recurrences and staging, us[6] FP64 refreshes, us[7] unused.
+   CTA 0 with the global nanosecond timer, in microseconds (in brackets: a solve in Krylov
+   coordinates): us[0] set-up reductions [products K and F], us[1] fused CG passes [the N x N
+   recurrences], us[2] first grid barrier, us[3] cross-CTA reduction, us[4] second
+   grid barrier, us[5] scalar recurrences and staging, us[6] FP64 refreshes [forming Z and
+   its true residual], us[7] unused.
    ENKF_ERR_INVALID_ARG unless enkf_set_phase_timing(h, 2) preceded a timed analysis. */
 enkf_status enkf_get_solve_phases(enkf_handle h, double* us);
 
@@ -315,7 +328,7 @@ enkf_status enkf_analyze_noalloc(const enkf_config* cfg, const int32_t* d_rowptr
 /* Create a batched handle for `count` problems. cfgs[count] are HOST configs, each checked
    as by enkf_create; h_rowptr, h_col, h_w and r_diag are HOST arrays of `count` HOST
    pointers to each problem's CSR operator and R diagonal (copied to the device). cfgs[0]
-   .grid_blocks > 0 caps the persistent grid. Allocates one device arena (about 56 m N bytes
+   .grid_blocks > 0 caps the persistent grid. Allocates one device arena (about 28 m N bytes
    per problem, plus O(grid N_max^2)) and plans the launch as enkf_batch_plan does with
    alpha = 1 (large problems get teams of CTAs, the rest are queued for single CTAs). If the
    environment variable ENKF_TUNE_CACHE names a file holding a tuning result for this batch

@@ -32,7 +32,7 @@ void free_workspace(Workspace& ws) {
                   ws.Res, ws.P, ws.Sv, ws.prof, ws.Tpart, ws.Tred, ws.rrpart, ws.Wacc, ws.W, ws.col_iters,
                   ws.col_relres, ws.col_true, ws.col_warm, ws.status, ws.bar, ws.stage_Xf, ws.stage_y,
                   ws.Hrowptr, ws.Hcol, ws.Hw, ws.wa, ws.wb, ws.wcp, ws.wmu, ws.wU, ws.wV, ws.wcarry,
-                  ws.wcarryV, ws.Xw, ws.yw, ws.Tk, ws.Tacc, ws.hamax};
+                  ws.wcarryV, ws.Xw, ws.yw, ws.Tk, ws.Tacc, ws.hamax, ws.rdf, ws.rinv, ws.rsq, ws.kpart, ws.ksmall};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   ws = Workspace{};
@@ -174,6 +174,7 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
   h->stream = static_cast<cudaStream_t>(cuda_stream);
   h->nnz = nnz;
   h->tri = tri;
+  h->krylov = enkf::krylov_config(c);
   if (!tri && c.m > 0) {
     double sl = 0.0;
     for (int64_t i = 0; i < c.m; ++i) sl += std::log2(r_diag[i]);
@@ -182,7 +183,8 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
   }
   cudaError_t e = cudaGetDevice(&h->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
-  if (e == cudaSuccess) e = mixed ? enkf::plan_solve_mixed(h) : enkf::plan_solve(h);
+  if (e == cudaSuccess)
+    e = h->krylov ? enkf::plan_krylov(h) : mixed ? enkf::plan_solve_mixed(h) : enkf::plan_solve(h);
   if (e != cudaSuccess) {
     enkf_status s = cuda_fail(nullptr, e, "enkf_create: device query / planning");
     delete h;
@@ -196,7 +198,8 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
   struct Alloc { void** p; size_t bytes; };
   // the Reduced variant and the sEnKF comparator work from one Gram pass and keep no m x N arrays
   const bool gram = c.variant != ENKF_CGD;
-  const int64_t tpart = gram ? (int64_t)enkf::reduced_grid(h) * 2 * c.N * c.N : (int64_t)G * NE;
+  const bool krylov = h->krylov;
+  const int64_t tpart = gram ? (int64_t)enkf::reduced_grid(h) * 2 * c.N * c.N : krylov ? 1 : (int64_t)G * NE;
   std::vector<Alloc> allocs = {
       {(void**)&ws.rowptr, sizeof(int32_t) * (c.m + 1)},
       {(void**)&ws.col, sizeof(int32_t) * (size_t)std::max<int64_t>(nnz, 1)},
@@ -217,7 +220,15 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
       {(void**)&ws.stage_y, sizeof(double) * c.m},
       {(void**)&ws.prof, sizeof(unsigned long long) * 8},
   };
-  if (!gram) {
+  if (krylov) {   // HA, D and Z in double-float and the residual: no CG vectors
+    allocs.push_back({(void**)&ws.r32, sizeof(float) * c.m});
+    allocs.push_back({(void**)&ws.B, vs * mN});
+    for (void** q : {&ws.HAdf, &ws.Ddf, &ws.Zdf}) allocs.push_back({q, 8 * (size_t)mN});
+    for (void** q : {&ws.rdf, &ws.rinv, &ws.rsq}) allocs.push_back({q, 8 * (size_t)c.m});
+    allocs.push_back({&ws.kpart, enkf::krylov_part_bytes(h)});
+    allocs.push_back({&ws.ksmall, 8 * ((size_t)4 * c.N * c.N + 2 * c.N)});
+  }
+  if (!gram && !krylov) {
     allocs.push_back({(void**)&ws.Sv, vs * mN});
     allocs.push_back({(void**)&ws.D, sizeof(double) * mN});
     allocs.push_back({(void**)&ws.Res, vs * mN});
@@ -227,7 +238,7 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
       allocs.push_back({(void**)&ws.Z, sizeof(double) * mN});
     }
   }
-  if (!gram && c.precision != ENKF_FP64) {
+  if (!gram && !krylov && c.precision != ENKF_FP64) {
     allocs.push_back({(void**)&ws.HA32, sizeof(float) * mN});
     allocs.push_back({(void**)&ws.r32, sizeof(float) * c.m});
     allocs.push_back({(void**)&ws.B, vs * mN});
@@ -236,12 +247,12 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
     allocs.push_back({(void**)&ws.Ddf, 8 * (size_t)mN});
     allocs.push_back({(void**)&ws.Zdf, 8 * (size_t)mN});
   }
-  if (mixed) {
+  if (mixed && !krylov) {
     allocs.push_back({(void**)&ws.HA16, enkf::mixed_image_bytes(h)});
     allocs.push_back({(void**)&ws.Tk, sizeof(float) * 2 * c.N * c.N});
     allocs.push_back({(void**)&ws.hamax, sizeof(unsigned) * 4});
   }
-  if (c.precision != ENKF_FP64 && c.variant == ENKF_CGD)
+  if (c.precision != ENKF_FP64 && c.variant == ENKF_CGD && !krylov)
     allocs.push_back({(void**)&ws.Tacc, sizeof(double) * 3 * ((size_t)c.N * c.N + 4 * c.N)});
   const int64_t hnnz = h_rowptr[c.m];
   const int64_t nblk = enkf::whiten_blocks(c.m);
@@ -294,6 +305,7 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
   if (e == cudaSuccess && ws.HA16) e = cudaMemset(ws.HA16, 0, enkf::mixed_image_bytes(h));
   if (e == cudaSuccess) e = cudaMemset(ws.bar, 0, sizeof(unsigned) * 4);
   if (e == cudaSuccess) e = enkf::launch_convert_r(h);
+  if (e == cudaSuccess && krylov) e = enkf::launch_krylov_rows(h);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) {
     free_workspace(ws);
@@ -378,6 +390,7 @@ static enkf_status analyze_impl(enkf_handle h, const void* d_Xf, const double* d
   if (h->timing) e = cudaEventRecord(h->ev[1], h->stream);
   if (e == cudaSuccess)
     e = gram ? enkf::launch_nxn_stage(h)
+             : h->krylov ? (c.warm_start ? enkf::warm_solve(h) : enkf::launch_krylov(h))
              : (h->cfg.precision >= ENKF_BF16_REFINE ? enkf::launch_solve_mixed(h) : enkf::launch_solve(h));
   if (e != cudaSuccess) return cuda_fail(h, e, "analyze: CG launch");
   if (h->timing) e = cudaEventRecord(h->ev[2], h->stream);
@@ -556,7 +569,9 @@ enkf_status enkf_copy_intermediates(enkf_handle h, double* d_HA, double* d_D, do
     if (d_HA) e = enkf::launch_df32_to_f64(h->ws.HAdf, d_HA, cnt, h->stream);
     if (e == cudaSuccess && d_Z) e = enkf::launch_df32_to_f64(h->ws.Zdf, d_Z, cnt, h->stream);
   }
-  if (e == cudaSuccess && d_D) e = cudaMemcpyAsync(d_D, h->ws.D, mN, cudaMemcpyDeviceToDevice, h->stream);
+  if (e == cudaSuccess && d_D)   // D = hi + lo rounded once, as the innovations kernel's FP64 copy
+    e = h->krylov ? enkf::launch_df32_to_f64(h->ws.Ddf, d_D, c.m * c.N, h->stream)
+                  : cudaMemcpyAsync(d_D, h->ws.D, mN, cudaMemcpyDeviceToDevice, h->stream);
   if (e == cudaSuccess && d_W)
     e = cudaMemcpyAsync(d_W, h->ws.W, sizeof(double) * c.N * c.N, cudaMemcpyDeviceToDevice, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "copy_intermediates");

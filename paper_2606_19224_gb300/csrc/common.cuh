@@ -152,6 +152,12 @@ struct Workspace {
   float* Tk = nullptr;          // [2][N][N] T of the tensor-core step, carried between steps
   double* Tacc = nullptr;       // [3][N N + 4 N] step sums of the tensor-core solve (atomic adds)
   unsigned* hamax = nullptr;    // tensor-core modes: largest |HA| of the analysis (float bits)
+  // the preconditioned solve in Krylov coordinates (krylov.cuh)
+  void* rdf = nullptr;          // [m] R, 1/R and 1/sqrt(R) in double-float
+  void* rinv = nullptr;
+  void* rsq = nullptr;
+  void* kpart = nullptr;        // [G][2 N JC + 128] double-float partial products
+  void* ksmall = nullptr;       // four N x N matrices, two N-vectors (double-float)
   // tridiagonal R (kernels_whiten.cu): the caller's H, the whitening scan's coefficients and
   // buffers; rowptr / col / w / r above then hold H' = I and r' = 1 of the whitened problem
   int32_t* Hrowptr = nullptr;   // [m+1]
@@ -200,6 +206,7 @@ struct enkf_handle_s {
   cudaEvent_t host_ev[2] = {nullptr, nullptr};
   enkf::BatchState* batch = nullptr;   // non-NULL for a handle made by enkf_batch_create
   enkf::WarmState* warm = nullptr;     // learned warm start (enkf_set_warm_model / enkf_warm_features)
+  bool krylov = false;                 // the solve runs in Krylov coordinates (kernels_krylov.cu)
   bool tri = false;                    // tridiagonal R: analyses run on the whitened problem
   float r_pow2 = 1.f;                  // power of two nearest the geometric mean of R's diagonal
                                        // (1 for the whitened problem)
@@ -216,6 +223,13 @@ cudaError_t launch_convert_r(enkf_handle_s* h);
 cudaError_t plan_solve_mixed(enkf_handle_s* h);
 cudaError_t launch_solve_mixed(enkf_handle_s* h);
 size_t mixed_image_bytes(const enkf_handle_s* h);   // tile images of HA (zeroed at create)
+// kernels_krylov.cu: CG preconditioned by R in the coordinates of its Krylov space
+bool krylov_config(const enkf_config& c);
+cudaError_t plan_krylov(enkf_handle_s* h);
+size_t krylov_part_bytes(const enkf_handle_s* h);
+cudaError_t launch_krylov_rows(enkf_handle_s* h);
+// phase 0: the whole solve; 1: the products K and F only; 2: the rest, from a learned start
+cudaError_t launch_krylov(enkf_handle_s* h, int phase = 0, const float* w0 = nullptr, const double* wnorm = nullptr);
 cudaError_t launch_update(enkf_handle_s* h, const void* Xf, void* Xa);
 // kernels_update_tc.cu: X_a = X_f + A W on the tensor cores (FP32 ensembles)
 cudaError_t launch_update_tc(enkf_handle_s* h, const void* Xf, void* Xa);
@@ -259,6 +273,7 @@ cudaError_t warm_features(enkf_handle_s* h, int K, float* F, float* T);
 cudaError_t warm_set_model(enkf_handle_s* h, const enkf_mlp_shape* shape, const float* params, std::string& err);
 bool warm_ready(const enkf_handle_s* h);
 cudaError_t warm_prepare(enkf_handle_s* h);
+cudaError_t warm_solve(enkf_handle_s* h);   // the rest of a solve in Krylov coordinates from the learned start
 void warm_free(enkf_handle_s* h);
 int64_t mlp_param_count(const enkf_mlp_shape* s);
 int64_t mlp_work_bytes(const enkf_mlp_shape* s, int B);

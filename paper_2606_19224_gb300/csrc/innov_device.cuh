@@ -276,7 +276,7 @@ __device__ __forceinline__ void innov_rows_df(
         }
         if ((N & 1) == 0) {
           // both members present and e0 even: one 8- or 16-byte store per array per lane
-          *reinterpret_cast<double2*>(D + e0) = make_double2(df_to_double(dv[0]), df_to_double(dv[1]));
+          if (D) *reinterpret_cast<double2*>(D + e0) = make_double2(df_to_double(dv[0]), df_to_double(dv[1]));
           if (HA32) *reinterpret_cast<float2*>(HA32 + e0) = make_float2(hv[0].hi, hv[1].hi);
           if (B32) *reinterpret_cast<float2*>(B32 + e0) = make_float2(dv[0].hi, dv[1].hi);
           if (HAdf) *reinterpret_cast<float4*>(HAdf + e0) = make_float4(hv[0].hi, hv[0].lo, hv[1].hi, hv[1].lo);
@@ -286,7 +286,7 @@ __device__ __forceinline__ void innov_rows_df(
           for (int b = 0; b < 2; ++b) {
             if (jp + b >= N) continue;
             const int64_t e = e0 + b;
-            D[e] = df_to_double(dv[b]);
+            if (D) D[e] = df_to_double(dv[b]);
             if (HA32) HA32[e] = hv[b].hi;
             if (B32) B32[e] = dv[b].hi;
             if (HAdf) HAdf[e] = hv[b];

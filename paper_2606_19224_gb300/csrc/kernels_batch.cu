@@ -28,14 +28,16 @@
 #include <vector>
 
 #include "innov_device.cuh"
+#include "krylov.cuh"
 #include "solve_body.cuh"
 
 namespace enkf {
 
 struct BatchProblem {
-  SolveParams sp;
+  KrylovParams sp;   // part, the N x N matrices, sums and rrpart belong to the team
   int64_t n;
   int NT;
+  const double* r;
   const int32_t* rowptr;
   const int32_t* col;
   const double* w;
@@ -47,12 +49,17 @@ struct BatchIO {
   uint64_t seed, counter;
 };
 
+// Double-float entries a CTA contributes to its team's buffers: two partials (a CTA alone takes both
+// column groups), two rows of column sums, four N x N matrices and two N-vectors.
+__host__ __device__ constexpr int64_t team_stride(int64_t part_max, int n_max) {
+  return 2 * part_max + 256 + 4 * (int64_t)n_max * n_max + 2 * n_max;
+}
+
 // The per-problem phases as separate (not inlined) device functions, so that each gets the
 // register allocation of its own loop nest instead of the union of all of them.
 template <int NT>
-__device__ __noinline__ void batch_solve(const SolveParams& sp, int G, int rank, GridBarrier& bar,
-                                         unsigned char* smem) {
-  solve_body<float, NT, true>(sp, G, rank, bar, smem);
+__device__ __noinline__ void batch_solve(const KrylovParams& sp, int G, int rank, GridBarrier& bar, KCta& cta) {
+  krylov_body<NT>(sp, G, rank, bar, cta);
 }
 template <int NT>
 __device__ __noinline__ void batch_update(const BatchIO& io, const double* W, int64_t n, int N,
@@ -60,9 +67,8 @@ __device__ __noinline__ void batch_update(const BatchIO& io, const double* W, in
   update_rows<float, NT, 0>(io.Xf, io.Xa, W, n, N, rank, G, smem);
 }
 
-// NTMAX bounds the column tile of every problem in the batch. One CTA per SM (the
-// double-buffered fused pass takes most of the shared memory). The solve is the
-// Jacobi-preconditioned (M = R) form. A CTA first works through its team's list of problems
+// NTMAX bounds the column tile of every problem in the batch. One CTA per SM (it holds the
+// SM's tensor memory). The solve is the one preconditioned by R, in Krylov coordinates (krylov.cuh). A CTA first works through its team's list of problems
 // (order[team_first[team] .. team_first[team + 1])), then takes problems one at a time from
 // the shared queue order[queue_first .. count) (longest first) and solves each alone.
 template <int NTMAX>
@@ -71,16 +77,21 @@ __global__ void __launch_bounds__(kThreads, 1) batch_kernel(
     const int* __restrict__ cta_team, const int* __restrict__ cta_rank,
     const int* __restrict__ team_size, const int* __restrict__ team_first,
     const int* __restrict__ order, int queue_first, int count, unsigned* __restrict__ queue_head,
-    double* __restrict__ team_buf, int max_grid, int ne_max, int perturb,
+    df32* __restrict__ team_buf, int64_t part_max, int n_max, int perturb,
     unsigned long long* __restrict__ times) {
   constexpr int NT2 = NTMAX >= 64 ? 64 : 32;
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ SolveParams s_sp;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t mbar;
+  __shared__ uint32_t tmem_slot;
+  __shared__ KrylovParams s_sp;
   __shared__ BatchIO s_io;
   __shared__ int64_t s_n;
   __shared__ int s_nt;
   __shared__ int s_q;
   const int warp = threadIdx.x >> 5;
+  KCta cta;
+  krylov_begin(cta, smem, &mbar, &tmem_slot, nullptr);
+  const int64_t buf = team_stride(part_max, n_max);
   // problem pi on a team of G CTAs in which this CTA has `rank` (the team's CTAs are
   // contiguous, so its reduction slices start at CTA blockIdx.x - rank); false if a barrier
   // of the problem gave up
@@ -88,32 +99,41 @@ __global__ void __launch_bounds__(kThreads, 1) batch_kernel(
     __syncthreads();
     if (threadIdx.x == 0) {
       s_sp = probs[pi].sp;
-      const int64_t c0 = (int64_t)blockIdx.x - rank;
-      s_sp.Tpart = team_buf + c0 * ne_max;                                      // [G][NE]
-      s_sp.Tred = team_buf + (int64_t)max_grid * ne_max + c0 * ne_max;          // [NE]
-      s_sp.rrpart = team_buf + (int64_t)2 * max_grid * ne_max + c0 * 256;       // [2][G][NT]
+      // the team's buffers start at those of its first CTA: partials, column sums of the residuals
+      // and, at that CTA alone, the N x N matrices
+      const int64_t c0 = (int64_t)blockIdx.x - rank, NN = (int64_t)s_sp.N * s_sp.N;
+      df32* own = team_buf + c0 * buf;
+      df32* small = own + G * (2 * part_max + 256);
+      s_sp.part = own;
+      s_sp.rrpart = reinterpret_cast<double*>(own + (int64_t)G * 2 * part_max);   // [2][G][NT]
+      s_sp.Kred = small;
+      s_sp.Fred = small + NN;
+      s_sp.wred = small + 2 * NN;
+      s_sp.Tred = small + 3 * NN;
+      s_sp.sums = small + 4 * NN;
       s_io = io[pi];
       s_n = probs[pi].n;
       s_nt = probs[pi].NT;
       if (rank == 0) times[2 * pi] = global_ns();
     }
     __syncthreads();
-    const SolveParams& sp = s_sp;
+    const KrylovParams& sp = s_sp;
+    cta.status = sp.status;
+    cta.ok = true;
     const int NT = s_nt;
     GridBarrier bar{sp.bar, reinterpret_cast<int*>(sp.bar + 1), sp.status, (unsigned)G, 0u};
-    // innovations over this CTA's block of observation rows (the solve uses the same blocks)
+    // innovations over this CTA's share of the observation rows
     const int64_t rows_per = (sp.m + G - 1) / G;
     const int64_t r0 = imin64(sp.m, (int64_t)rank * rows_per), r1 = imin64(sp.m, r0 + rows_per);
-    innov_rows<float>(s_io.Xf, probs[pi].rowptr, probs[pi].col, probs[pi].w, s_io.y, sp.r, nullptr,
-                      perturb ? 2 : 0, s_io.seed, s_io.counter, sp.m, sp.N, nullptr,
-                      static_cast<float*>(const_cast<void*>(sp.HA)), const_cast<double*>(sp.D),
-                      static_cast<float*>(sp.B), nullptr, nullptr, 0, const_cast<df32*>(sp.HAdf),
+    innov_rows<float>(s_io.Xf, probs[pi].rowptr, probs[pi].col, probs[pi].w, s_io.y, probs[pi].r, nullptr,
+                      perturb ? 2 : 0, s_io.seed, s_io.counter, sp.m, sp.N, nullptr, nullptr, nullptr, nullptr,
+                      nullptr, nullptr, 0, const_cast<df32*>(sp.HAdf),
                       const_cast<df32*>(sp.Ddf), r0, r1, warp, kThreads / 32);
     bool ok = bar.sync();
     if (ok) {
-      if (NT == 32) batch_solve<32>(sp, G, rank, bar, smem);
-      else if (NT == 64) batch_solve<NT2>(sp, G, rank, bar, smem);
-      else batch_solve<NTMAX>(sp, G, rank, bar, smem);
+      if (NT == 32) batch_solve<32>(sp, G, rank, bar, cta);
+      else if (NT == 64) batch_solve<NT2>(sp, G, rank, bar, cta);
+      else batch_solve<NTMAX>(sp, G, rank, bar, cta);
       ok = bar.sync();   // W of this problem complete and visible to the team
     }
     if (!ok) return false;
@@ -143,6 +163,7 @@ __global__ void __launch_bounds__(kThreads, 1) batch_kernel(
     if (q >= count) break;
     run(order[q], 1, 0);   // one CTA: its barriers never wait
   }
+  krylov_end(cta);
 }
 
 // ------------------------------------------------------------------ host side
@@ -168,7 +189,7 @@ struct BatchState {
   int count = 0;
   int perturb = 1;
   int ntmax = 32;
-  int ne_max = 0;
+  int n_max = 0;
   size_t smem = 0;
   int max_grid = 0;
   std::vector<enkf_config> cfg;
@@ -183,7 +204,7 @@ struct BatchState {
                                        // (grid, grid, teams, teams + 1, count entries)
   int* d_status = nullptr;             // [count][4]: status bits, refinements
   unsigned* d_bar = nullptr;           // [count][4]: barrier counter, abort flag; then the queue head
-  double* d_team = nullptr;            // Tpart [max_grid][NE], Tred [max_grid][NE], rrpart [max_grid][256]
+  df32* d_team = nullptr;              // [max_grid][team_stride]
   unsigned long long* d_time = nullptr;   // [count][2]: start, end (global ns, by each team's rank 0)
   unsigned long long* d_phase = nullptr;  // [count][PH_COUNT] solve phase timers, or nullptr when off
   BatchPlan plan;
@@ -351,11 +372,10 @@ bool batch_plan_host(int count, const enkf_config* cfgs, int max_grid, double al
 }
 
 // Dynamic shared memory of a batch whose tiles go up to NTMAX: the largest need of any
-// column tile it may run (the NT = 32 and 64 solves use the double-buffered fused pass and
-// need more than the NT = 128 one).
+// column tile it may run.
 template <int NT>
 static size_t tile_smem() {
-  return std::max<size_t>(solve_smem_bytes<float, NT>(), update_smem_bytes<float, NT>());
+  return std::max<size_t>(KLayout<NT>::bytes, update_smem_bytes<float, NT>());
 }
 template <int NTMAX>
 static size_t batch_smem_nt() {
@@ -406,11 +426,12 @@ static cudaError_t enqueue_batch(BatchState& B, cudaStream_t s) {
   const BatchIO* io = B.d_io;
   int perturb = B.perturb;
   unsigned long long* times = B.d_time;
-  int queue_first = P.queue_first, count = B.count, max_grid = B.max_grid, ne_max = B.ne_max;
+  int queue_first = P.queue_first, count = B.count, n_max = B.n_max;
+  int64_t part_max = krylov_part(B.n_max);
   unsigned* queue_head = B.d_bar + 4 * (size_t)B.count;
-  double* team_buf = B.d_team;
+  df32* team_buf = B.d_team;
   void* args[] = {&probs, &io, &cta_team, &cta_rank, &team_size, &team_first, &order, &queue_first, &count,
-                  &queue_head, &team_buf, &max_grid, &ne_max, &perturb, &times};
+                  &queue_head, &team_buf, &part_max, &n_max, &perturb, &times};
   return cudaLaunchCooperativeKernel(batch_fn(B.ntmax), dim3(P.grid), dim3(kThreads), args,
                                      B.smem, s);
 }
@@ -478,7 +499,7 @@ cudaError_t batch_build(enkf_handle_s* h, int count, const enkf_config* cfgs,
     nmax = std::max(nmax, (int)cfgs[i].N);
   }
   B.ntmax = nt_of(nmax);
-  B.ne_max = nmax * nmax + 4 * nmax;
+  B.n_max = nmax;
   B.smem = B.ntmax == 32 ? batch_smem_nt<32>() : B.ntmax == 64 ? batch_smem_nt<64>() : batch_smem_nt<128>();
   void* fn = batch_fn(B.ntmax);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B.smem);
@@ -488,8 +509,8 @@ cudaError_t batch_build(enkf_handle_s* h, int count, const enkf_config* cfgs,
   if (occ < 1) { err = "enkf_batch_create: kernel does not fit on an SM"; return cudaErrorInvalidConfiguration; }
   B.max_grid = occ * h->sms;
   if (h->cfg.grid_blocks > 0) B.max_grid = std::min(B.max_grid, h->cfg.grid_blocks);
-  // one arena: per problem HA, HAdf, D, Ddf, Zdf, B, X, Res, P, Sv, r, r32, rowptr, col, w,
-  // W, column iterations / residuals
+  // one arena: per problem HA, D and Z in double-float, B, R (FP64), R, 1/R and 1/sqrt(R) in
+  // double-float, rowptr, col, w, W, column iterations / residuals
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   std::vector<std::vector<size_t>> parts(count);
   std::vector<size_t> off(count + 1, 0);
@@ -497,13 +518,12 @@ cudaError_t batch_build(enkf_handle_s* h, int count, const enkf_config* cfgs,
     const auto& c = cfgs[i];
     const size_t mN = (size_t)c.m * c.N, m = (size_t)c.m, N = (size_t)c.N;
     const size_t nnz = (size_t)std::max(1, rowptr[i][c.m]);
-    parts[i] = {4 * mN, 8 * mN, 8 * mN, 8 * mN, 8 * mN, 4 * mN, 4 * mN, 4 * mN, 4 * mN, 4 * mN,
-                8 * m, 4 * m, 4 * (m + 1), 4 * nnz, 8 * nnz, 8 * N * N, 4 * N, 8 * N, 8 * N};
+    parts[i] = {8 * mN, 8 * mN, 8 * mN, 4 * mN, 8 * m, 8 * m, 8 * m, 8 * m,
+                4 * (m + 1), 4 * nnz, 8 * nnz, 8 * N * N, 4 * N, 8 * N, 8 * N};
     size_t sz = 0;
     for (size_t b : parts[i]) sz += al(b);
     off[i + 1] = off[i] + sz;
   }
-  const size_t NE = (size_t)B.ne_max;
   e = cudaMalloc(&B.arena, off[count]);
   if (e == cudaSuccess) e = cudaMalloc((void**)&B.d_probs, sizeof(BatchProblem) * count);
   if (e == cudaSuccess) e = cudaMalloc((void**)&B.d_io, sizeof(BatchIO) * count);
@@ -515,7 +535,7 @@ cudaError_t batch_build(enkf_handle_s* h, int count, const enkf_config* cfgs,
   if (e == cudaSuccess) e = cudaMalloc((void**)&B.d_time, sizeof(unsigned long long) * 2 * count);
   if (e == cudaSuccess) e = cudaMemset(B.d_time, 0, sizeof(unsigned long long) * 2 * count);
   if (e == cudaSuccess)
-    e = cudaMalloc((void**)&B.d_team, sizeof(double) * (2 * (size_t)B.max_grid * NE + (size_t)B.max_grid * 256));
+    e = cudaMalloc((void**)&B.d_team, sizeof(df32) * (size_t)team_stride(krylov_part(nmax), nmax) * B.max_grid);
   if (e != cudaSuccess) { err = "enkf_batch_create: device allocation"; return e; }
   unsigned char* base = static_cast<unsigned char*>(B.arena);
   for (int i = 0; i < count && e == cudaSuccess; ++i) {
@@ -524,52 +544,40 @@ cudaError_t batch_build(enkf_handle_s* h, int count, const enkf_config* cfgs,
     std::vector<void*> ptr;
     for (size_t b : parts[i]) { ptr.push_back(q); q += al(b); }
     BatchProblem bp{};
-    SolveParams& sp = bp.sp;
+    KrylovParams& sp = bp.sp;
     sp.m = c.m;
     sp.N = c.N;
-    sp.mode = 1;
-    sp.HA = ptr[0];
-    sp.HA64 = nullptr;
-    sp.HAdf = static_cast<const df32*>(ptr[1]);
-    sp.D = static_cast<const double*>(ptr[2]);
-    sp.Ddf = static_cast<const df32*>(ptr[3]);
-    sp.Zdf = static_cast<df32*>(ptr[4]);
-    sp.B = ptr[5];
-    sp.X = ptr[6];
-    sp.Res = ptr[7];
-    sp.P = ptr[8];
-    sp.Sv = ptr[9];
-    sp.Z = nullptr;
-    sp.r = static_cast<const double*>(ptr[10]);
-    sp.rv = ptr[11];
-    sp.W = static_cast<double*>(ptr[15]);
-    sp.col_iters = static_cast<int*>(ptr[16]);
-    sp.col_relres = static_cast<double*>(ptr[17]);
-    sp.col_true = static_cast<double*>(ptr[18]);
+    sp.HAdf = static_cast<const df32*>(ptr[0]);
+    sp.Ddf = static_cast<const df32*>(ptr[1]);
+    sp.Zdf = static_cast<df32*>(ptr[2]);
+    sp.B = static_cast<float*>(ptr[3]);
+    bp.r = static_cast<const double*>(ptr[4]);
+    sp.rdf = static_cast<const df32*>(ptr[5]);
+    sp.rinv = static_cast<const df32*>(ptr[6]);
+    sp.rsq = static_cast<const df32*>(ptr[7]);
+    sp.W = static_cast<double*>(ptr[11]);
+    sp.col_iters = static_cast<int*>(ptr[12]);
+    sp.col_relres = static_cast<double*>(ptr[13]);
+    sp.col_true = static_cast<double*>(ptr[14]);
     sp.tol = c.tol;
-    sp.inner_tol = c.inner_tol;
     sp.max_iter = c.max_iter;
-    sp.fixed_iters = 0;
     sp.max_refine = c.max_refine;
-    sp.true_residual = c.true_residual;
     sp.status = B.d_status + 4 * i;
     sp.bar = B.d_bar + 4 * i;
     sp.prof = nullptr;
     bp.n = c.n;
     bp.NT = nt_of(c.N);
-    bp.rowptr = static_cast<const int32_t*>(ptr[12]);
-    bp.col = static_cast<const int32_t*>(ptr[13]);
-    bp.w = static_cast<const double*>(ptr[14]);
+    bp.rowptr = static_cast<const int32_t*>(ptr[8]);
+    bp.col = static_cast<const int32_t*>(ptr[9]);
+    bp.w = static_cast<const double*>(ptr[10]);
     const int64_t nnz = rowptr[i][c.m];
-    e = cudaMemcpy(ptr[12], rowptr[i], 4 * ((size_t)c.m + 1), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && nnz > 0) e = cudaMemcpy(ptr[13], col[i], 4 * (size_t)nnz, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && nnz > 0) e = cudaMemcpy(ptr[14], w[i], 8 * (size_t)nnz, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(ptr[10], r[i], 8 * (size_t)c.m, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) {
-      std::vector<float> r32(c.m);
-      for (int64_t k = 0; k < c.m; ++k) r32[k] = (float)r[i][k];
-      e = cudaMemcpy(ptr[11], r32.data(), 4 * (size_t)c.m, cudaMemcpyHostToDevice);
-    }
+    e = cudaMemcpy(ptr[8], rowptr[i], 4 * ((size_t)c.m + 1), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && nnz > 0) e = cudaMemcpy(ptr[9], col[i], 4 * (size_t)nnz, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && nnz > 0) e = cudaMemcpy(ptr[10], w[i], 8 * (size_t)nnz, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(ptr[4], r[i], 8 * (size_t)c.m, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+      e = launch_krylov_rows(bp.r, c.m, static_cast<df32*>(ptr[5]), static_cast<df32*>(ptr[6]),
+                             static_cast<df32*>(ptr[7]), h->stream);
     B.probs.push_back(bp);
   }
   if (e != cudaSuccess) { err = "enkf_batch_create: upload of the observation operators"; return e; }
@@ -793,7 +801,7 @@ cudaError_t batch_stats(enkf_handle_s* h, int32_t* status, int32_t* iters_max, d
   std::vector<int> st(4 * (size_t)B.count);
   if (e == cudaSuccess) e = cudaMemcpy(st.data(), B.d_status, sizeof(int) * 4 * B.count, cudaMemcpyDeviceToHost);
   for (int i = 0; i < B.count && e == cudaSuccess; ++i) {
-    const SolveParams& sp = B.probs[i].sp;
+    const KrylovParams& sp = B.probs[i].sp;
     const int N = B.cfg[i].N;
     std::vector<int> it(N);
     std::vector<double> rel(N);

@@ -135,7 +135,7 @@ cudaError_t launch_innovations(enkf_handle_s* h, const void* Xf, const double* y
   else
     innov_kernel<float><<<blocks, kThreads, 0, h->stream>>>(
         static_cast<const float*>(Xf), ws.rowptr, ws.col, ws.w, y, ws.r, E, emode, seed, counter,
-        c.m, c.N, ws.HA64, ws.HA32, ws.D, static_cast<float*>(ws.B),
+        c.m, c.N, ws.HA64, ws.HA32, ws.D, h->krylov ? nullptr : static_cast<float*>(ws.B),
         nullptr, nullptr, 0, static_cast<df32*>(ws.HAdf), static_cast<df32*>(ws.Ddf), ws.hamax);
   return cudaGetLastError();
 }

@@ -382,8 +382,8 @@ static cudaError_t mlp_loss_grad_impl(const MlpLayout& L, const float* P, const 
 constexpr int kWarmRows = 32;
 
 template <int AM>
-__global__ void __launch_bounds__(kThreads) warm_gram_kernel(const float* __restrict__ HA,
-                                                             const double* __restrict__ D,
+__global__ void __launch_bounds__(kThreads) warm_gram_kernel(const df32* __restrict__ HA,
+                                                             const df32* __restrict__ D,
                                                              const float* __restrict__ r32, int64_t m, int N,
                                                              int64_t rows_per, double* __restrict__ part) {
   constexpr int NT = 16 * AM, LD = NT + 4, RW = AM == 8 ? kWarmRows / 2 : kWarmRows;   // static smem < 48 KB
@@ -408,10 +408,10 @@ __global__ void __launch_bounds__(kThreads) warm_gram_kernel(const float* __rest
       const int64_t i = ib + ii;
       const bool in = i < i1 && k < N;
       const float rinv = sRi[ii];
-      const float h = in ? HA[i * N + k] : 0.f;
+      const float h = in ? HA[i * N + k].hi : 0.f;
       sH[ii][k] = h;
       sHr[ii][k] = h * rinv;
-      sD[ii][k] = in ? (float)D[i * N + k] * rinv : 0.f;
+      sD[ii][k] = in ? D[i * N + k].hi * rinv : 0.f;
     }
     __syncthreads();
 #pragma unroll 4
@@ -461,8 +461,18 @@ __global__ void warm_reduce_kernel(const double* __restrict__ part, int nparts, 
   g[e] = s;
 }
 
+// The same sums from the products of a solve in Krylov coordinates: K = HA^T R^-1 HA/(N-1) and
+// F^T = (HA^T R^-1 D)^T in double-float.
+__global__ void warm_sums_kernel(const df32* __restrict__ K, const df32* __restrict__ F, int N, double* __restrict__ g) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= N * N) return;
+  const int k = e / N, j = e % N;
+  g[e] = (double)F[(int64_t)j * N + k];
+  g[N * N + e] = (double)K[e] * (double)(N - 1);
+}
+
 // Features of column j (one CTA per column): sketch values, their RMS s_j, and g_j/s_j.
-__global__ void __launch_bounds__(kThreads) warm_features_kernel(const double* __restrict__ D, int64_t m, int N,
+__global__ void __launch_bounds__(kThreads) warm_features_kernel(const df32* __restrict__ D, int64_t m, int N,
                                                                  int K, const double* __restrict__ gsum,
                                                                  float* __restrict__ F,
                                                                  float* __restrict__ s_out) {
@@ -472,7 +482,7 @@ __global__ void __launch_bounds__(kThreads) warm_features_kernel(const double* _
   double q = 0.0;
   for (int k = t; k < K; k += kThreads) {
     const int64_t i = ((int64_t)k * m) / K;
-    const double v = D[i * N + j];
+    const double v = (double)D[i * N + j];
     q += v * v;
   }
   red[t] = q;
@@ -486,7 +496,7 @@ __global__ void __launch_bounds__(kThreads) warm_features_kernel(const double* _
   const int in = K + N;
   for (int k = t; k < K; k += kThreads) {
     const int64_t i = ((int64_t)k * m) / K;
-    F[(int64_t)j * in + k] = (float)(D[i * N + j] / sj);
+    F[(int64_t)j * in + k] = (float)((double)D[i * N + j] / sj);
   }
   for (int k = t; k < N; k += kThreads) F[(int64_t)j * in + K + k] = (float)(gsum[k * N + j] * inv_nm1 / sj);
   if (t == 0) s_out[j] = (float)sj;
@@ -527,8 +537,8 @@ __global__ void __launch_bounds__(128) warm_coef_kernel(const float* __restrict_
 // of the FP32 solve, and its residual B[i][j] = sum_k HA[i][k] E[k][j] as the first inner
 // right-hand side (FP32; the refreshes recompute the true residual in double-float).
 template <int RB>
-__global__ void __launch_bounds__(kThreads) warm_decode_kernel(const float* __restrict__ HA,
-                                                               const double* __restrict__ D,
+__global__ void __launch_bounds__(kThreads) warm_decode_kernel(const df32* __restrict__ HA,
+                                                               const df32* __restrict__ D,
                                                                const float* __restrict__ r32, int64_t m, int N,
                                                                const float* __restrict__ C,
                                                                const float* __restrict__ Ecoef,
@@ -551,7 +561,7 @@ __global__ void __launch_bounds__(kThreads) warm_decode_kernel(const float* __re
     for (int e = t; e < 16 * N; e += kThreads) {
       const int ii = e / N, k = e % N;
       const int64_t i = ib + ii;
-      sHt[ii * LD + k] = i < m ? HA[i * N + k] : 0.f;
+      sHt[ii * LD + k] = i < m ? HA[i * N + k].hi : 0.f;
     }
     __syncthreads();
     constexpr int NGR = 16 / RB;   // row groups covering the 16 rows
@@ -574,12 +584,61 @@ __global__ void __launch_bounds__(kThreads) warm_decode_kernel(const float* __re
       for (int x = 0; x < RB; ++x) {
         const int64_t i = ib + g * RB + x;
         if (i < m) {
-          const float z = ((float)D[i * N + j] - a1[x]) / r32[i];
+          const float z = (D[i * N + j].hi - a1[x]) / r32[i];
           Z0[i * N + j] = df32(z, 0.f);
           B[i * N + j] = a2[x];
         }
       }
     }
+  }
+}
+
+// ||B_j||^2 of the start's residual B = HA E alone (a solve in Krylov coordinates starts from C
+// itself): 16-row tiles as in the decoder, column sums in FP64 per CTA, then over the CTAs in order.
+template <int RB>
+__global__ void __launch_bounds__(kThreads) warm_resid_kernel(const df32* __restrict__ HA, int64_t m, int N,
+                                                              const float* __restrict__ Ecoef,
+                                                              double* __restrict__ part) {
+  extern __shared__ float wsm[];   // E [N][N + 1], a 16-row tile of HA [16][N + 1], then column sums
+  const int LD = N + 1;
+  float* sE = wsm;
+  float* sHt = wsm + N * LD;
+  const int t = threadIdx.x;
+  constexpr int NGR = 16 / RB;
+  for (int e = t; e < N * N; e += kThreads) sE[(e / N) * LD + e % N] = Ecoef[e];
+  double sum = 0.0;   // N NGR <= kThreads: one (column, row group) per thread
+  for (int64_t ib = (int64_t)blockIdx.x * 16; ib < m; ib += (int64_t)gridDim.x * 16) {
+    __syncthreads();
+    for (int e = t; e < 16 * N; e += kThreads) {
+      const int ii = e / N, k = e % N;
+      sHt[ii * LD + k] = ib + ii < m ? HA[(ib + ii) * N + k].hi : 0.f;
+    }
+    __syncthreads();
+    if (t < N * NGR) {
+      const int j = t % N, g = t / N;
+      float a[RB];
+#pragma unroll
+      for (int x = 0; x < RB; ++x) a[x] = 0.f;
+#pragma unroll 4
+      for (int k = 0; k < N; ++k) {
+        const float ev = sE[k * LD + j];
+#pragma unroll
+        for (int x = 0; x < RB; ++x) a[x] = fmaf(sHt[(g * RB + x) * LD + k], ev, a[x]);
+      }
+      float q = 0.f;
+#pragma unroll
+      for (int x = 0; x < RB; ++x) q = fmaf(a[x], a[x], q);
+      sum += (double)q;
+    }
+  }
+  __syncthreads();
+  double* red = reinterpret_cast<double*>(wsm);
+  if (t < N * NGR) red[t] = sum;
+  __syncthreads();
+  if (t < N) {
+    double s = 0.0;
+    for (int g = 0; g < NGR; ++g) s += red[g * N + t];
+    part[(int64_t)blockIdx.x * N + t] = s;
   }
 }
 
@@ -601,6 +660,7 @@ struct WarmState {
   float* s = nullptr;              // [N] column scales
   float* Y = nullptr;              // [N][N] raw predictions
   float* work = nullptr;           // MLP activations for a batch of N rows
+  double* rpart = nullptr;         // [2 SMs + 1][N] residual norms of the start per CTA, then their sum
   int K_alloc = 0;
 };
 
@@ -617,6 +677,7 @@ static cudaError_t warm_alloc(enkf_handle_s* h, int K) {
     if (e == cudaSuccess) e = cudaMalloc((void**)&w.E, sizeof(float) * N * N);
     if (e == cudaSuccess) e = cudaMalloc((void**)&w.s, sizeof(float) * N);
     if (e == cudaSuccess) e = cudaMalloc((void**)&w.Y, sizeof(float) * N * N);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&w.rpart, sizeof(double) * (2 * (size_t)h->sms + 1) * N);
   }
   if (e == cudaSuccess && K > w.K_alloc) {
     if (w.F) cudaFree(w.F);
@@ -627,27 +688,34 @@ static cudaError_t warm_alloc(enkf_handle_s* h, int K) {
   return e;
 }
 
-static cudaError_t warm_features_into(enkf_handle_s* h, int K, float* F) {
+// HA^T R^-1 D and HA^T R^-1 HA of the last analysis's innovations into w.gsum
+static cudaError_t warm_sums(enkf_handle_s* h) {
   WarmState& w = *h->warm;
   const auto& c = h->cfg;
   const int64_t rows_per = (c.m + w.nparts - 1) / w.nparts;
+  const df32* HAdf = static_cast<const df32*>(h->ws.HAdf);
+  const df32* Ddf = static_cast<const df32*>(h->ws.Ddf);
   if (c.N <= 32)
-    warm_gram_kernel<2><<<w.nparts, kThreads, 0, h->stream>>>(h->ws.HA32, h->ws.D, h->ws.r32, c.m, c.N, rows_per, w.part);
+    warm_gram_kernel<2><<<w.nparts, kThreads, 0, h->stream>>>(HAdf, Ddf, h->ws.r32, c.m, c.N, rows_per, w.part);
   else if (c.N <= 64)
-    warm_gram_kernel<4><<<w.nparts, kThreads, 0, h->stream>>>(h->ws.HA32, h->ws.D, h->ws.r32, c.m, c.N, rows_per, w.part);
+    warm_gram_kernel<4><<<w.nparts, kThreads, 0, h->stream>>>(HAdf, Ddf, h->ws.r32, c.m, c.N, rows_per, w.part);
   else
-    warm_gram_kernel<8><<<w.nparts, kThreads, 0, h->stream>>>(h->ws.HA32, h->ws.D, h->ws.r32, c.m, c.N, rows_per, w.part);
+    warm_gram_kernel<8><<<w.nparts, kThreads, 0, h->stream>>>(HAdf, Ddf, h->ws.r32, c.m, c.N, rows_per, w.part);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   warm_reduce_kernel<<<(2 * c.N * c.N + 255) / 256, 256, 0, h->stream>>>(w.part, w.nparts, 2 * c.N * c.N, w.gsum);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  warm_features_kernel<<<c.N, kThreads, 0, h->stream>>>(h->ws.D, c.m, c.N, K, w.gsum, F, w.s);
+  return cudaGetLastError();
+}
+static cudaError_t warm_features_into(enkf_handle_s* h, int K, float* F) {
+  WarmState& w = *h->warm;
+  const auto& c = h->cfg;
+  warm_features_kernel<<<c.N, kThreads, 0, h->stream>>>(static_cast<const df32*>(h->ws.Ddf), c.m, c.N, K, w.gsum, F, w.s);
   return cudaGetLastError();
 }
 
 cudaError_t warm_features(enkf_handle_s* h, int K, float* F, float* T) {
   cudaError_t e = warm_alloc(h, 0);
+  if (e == cudaSuccess) e = warm_sums(h);
   if (e == cudaSuccess) e = warm_features_into(h, K, F);
   if (e == cudaSuccess && T) {
     warm_targets_kernel<<<(h->cfg.N * h->cfg.N + 255) / 256, 256, 0, h->stream>>>(h->ws.W, h->warm->s, h->cfg.N, T);
@@ -672,6 +740,9 @@ cudaError_t warm_set_model(enkf_handle_s* h, const enkf_mlp_shape* shape, const 
   e = cudaFuncSetAttribute(warm_decode_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(warm_decode_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(warm_decode_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const int rsm = (int)(sizeof(float) * (size_t)(N + 16) * (N + 1));   // up to 74 KB
+  if (e == cudaSuccess && rsm > 48 * 1024)
+    e = cudaFuncSetAttribute(warm_resid_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, rsm);
   if (e != cudaSuccess) { err = "decoder shared memory"; return e; }
   w.L = L;
   w.params = params;
@@ -685,7 +756,17 @@ bool warm_ready(const enkf_handle_s* h) { return h->warm && h->warm->params; }
 cudaError_t warm_prepare(enkf_handle_s* h) {
   WarmState& w = *h->warm;
   const auto& c = h->cfg;
-  cudaError_t e = warm_features_into(h, w.K, w.F);
+  cudaError_t e = cudaSuccess;
+  if (h->krylov) {   // the solve's own products, formed ahead of it
+    e = launch_krylov(h, 1);
+    if (e != cudaSuccess) return e;
+    const df32* small = static_cast<const df32*>(h->ws.ksmall);
+    warm_sums_kernel<<<(c.N * c.N + 255) / 256, 256, 0, h->stream>>>(small, small + c.N * c.N, c.N, w.gsum);
+    e = cudaGetLastError();
+  } else {
+    e = warm_sums(h);
+  }
+  if (e == cudaSuccess) e = warm_features_into(h, w.K, w.F);
   if (e != cudaSuccess) return e;
   const MlpWork W = carve(w.L, c.N, w.work);
   e = mlp_forward_impl(w.L, w.params, w.F, nullptr, c.N, W, w.Y, h->stream);
@@ -693,23 +774,44 @@ cudaError_t warm_prepare(enkf_handle_s* h) {
   warm_coef_kernel<<<c.N, 128, 0, h->stream>>>(w.Y, w.s, w.gsum, c.N, w.C, w.E);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const size_t smem = sizeof(float) * (size_t)(2 * c.N + 16) * (c.N + 1);
   const int grid = (int)std::min<int64_t>(2 * (int64_t)h->sms, (c.m + 15) / 16);
+  if (h->krylov) {
+    const size_t rsm = std::max(sizeof(float) * (size_t)(c.N + 16) * (c.N + 1), sizeof(double) * (size_t)kThreads);
+    const df32* HAk = static_cast<const df32*>(h->ws.HAdf);
+    if (c.N <= 32)
+      warm_resid_kernel<2><<<grid, kThreads, rsm, h->stream>>>(HAk, c.m, c.N, w.E, w.rpart);
+    else if (c.N <= 64)
+      warm_resid_kernel<4><<<grid, kThreads, rsm, h->stream>>>(HAk, c.m, c.N, w.E, w.rpart);
+    else
+      warm_resid_kernel<8><<<grid, kThreads, rsm, h->stream>>>(HAk, c.m, c.N, w.E, w.rpart);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    warm_reduce_kernel<<<(c.N + 255) / 256, 256, 0, h->stream>>>(w.rpart, grid, c.N, w.rpart + (size_t)2 * h->sms * c.N);
+    return cudaGetLastError();
+  }
+  const size_t smem = sizeof(float) * (size_t)(2 * c.N + 16) * (c.N + 1);
+  const df32* HAdf = static_cast<const df32*>(h->ws.HAdf);
+  const df32* Ddf = static_cast<const df32*>(h->ws.Ddf);
   df32* Z0 = static_cast<df32*>(h->ws.Zdf);
   float* B0 = static_cast<float*>(h->ws.B);
   if (c.N <= 32)
-    warm_decode_kernel<2><<<grid, kThreads, smem, h->stream>>>(h->ws.HA32, h->ws.D, h->ws.r32, c.m, c.N, w.C, w.E, Z0, B0);
+    warm_decode_kernel<2><<<grid, kThreads, smem, h->stream>>>(HAdf, Ddf, h->ws.r32, c.m, c.N, w.C, w.E, Z0, B0);
   else if (c.N <= 64)
-    warm_decode_kernel<4><<<grid, kThreads, smem, h->stream>>>(h->ws.HA32, h->ws.D, h->ws.r32, c.m, c.N, w.C, w.E, Z0, B0);
+    warm_decode_kernel<4><<<grid, kThreads, smem, h->stream>>>(HAdf, Ddf, h->ws.r32, c.m, c.N, w.C, w.E, Z0, B0);
   else
-    warm_decode_kernel<8><<<grid, kThreads, smem, h->stream>>>(h->ws.HA32, h->ws.D, h->ws.r32, c.m, c.N, w.C, w.E, Z0, B0);
+    warm_decode_kernel<8><<<grid, kThreads, smem, h->stream>>>(HAdf, Ddf, h->ws.r32, c.m, c.N, w.C, w.E, Z0, B0);
   return cudaGetLastError();
+}
+
+cudaError_t warm_solve(enkf_handle_s* h) {
+  const WarmState& w = *h->warm;
+  return launch_krylov(h, 2, w.C, w.rpart + (size_t)2 * h->sms * h->cfg.N);
 }
 
 void warm_free(enkf_handle_s* h) {
   WarmState* w = h->warm;
   if (!w) return;
-  void* ptrs[] = {w->part, w->gsum, w->C, w->E, w->F, w->s, w->Y, w->work};
+  void* ptrs[] = {w->part, w->gsum, w->C, w->E, w->F, w->s, w->Y, w->work, w->rpart};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete w;

@@ -1,0 +1,1060 @@
+// CG preconditioned by R on S Z = D, carried in the coordinates of its Krylov space.
+//
+// With the preconditioner M = R, z0 = R^{-1} b has the residual b - S z0 = -HA (HA^T R^{-1} b)/(N-1),
+// and every later iterate, direction and residual of the CG recurrences is R^{-1} or S times a
+// combination of the columns of HA: z_k = R^{-1} (b - HA w_k) with an N-vector w_k per column.
+// In these coordinates, with K = HA^T R^{-1} HA / (N-1) and g = HA^T R^{-1} b / (N-1), the residual
+// is r_k = -HA rho_k, rho_k = g - (I + K) w_k, its preconditioned norm is (r_k, R^{-1} r_k) =
+// (N-1) rho_k^T K rho_k, and a direction p = R^{-1} HA f has (p, S p) = (N-1) (K f)^T (f + K f): the
+// same alpha, beta and iterates as the recurrences on m-vectors (Sec. 3.1-3.3 of the paper, Eq.
+// matvec_decomp for S p), with one N x N product per step in place of two passes over HA.
+// What remains of a solve is three passes over the observation rows:
+//
+//   pass G   K and F = HA^T R^{-1} b                           (two products m N^2)
+//   CG       N independent recurrences, one CTA per column, vectors of length N
+//   pass Z   Z += R^{-1} (b - HA w), T = HA^T Z                 (two products)
+//   pass R   the true residual D - R Z - HA T/(N-1)            (one product)
+//
+// and a column whose true residual misses the tolerance gets another cycle with that residual
+// as b (iterative refinement). Z is formed entry by entry and certified by its own true
+// residual, as before; nothing in the certificate uses K or F.
+//
+// The products need more than FP32 (the residual's terms cancel to 1e-8 and below), and double-
+// float products on the CUDA cores cost 12 FP32 operations per term: 0.16 ms per product pair at
+// m = 65,536, N = 64, measured 0.33 ms per refresh, with the tensor cores idle. Here every operand
+// is a fixed-point number of five signed 9-bit slices (44 bits below a power of two at least the
+// largest entry of its row or column), each slice an integer of at most 256 in FP16. A product
+// of two slices is at most 2^16 and a sum of 64 of them (one tile) at most 2^22, so that the sums
+// that belong to one power of two (slices i and j with i + j = g, g = 0..4: 15 MMAs of kind::f16)
+// accumulate in FP32 in tensor memory without rounding (integers below 2^24 are exact there;
+// measured with constant, alternating and random operands). The five sums of an entry are then
+// combined into a double-float number with error-free additions. The dropped slice products and
+// the rounding of the operands are 2^-44 of the largest product, which is where the double-float
+// sums of the CUDA cores were.
+#pragma once
+
+#include "tc_mixed.cuh"
+
+namespace enkf {
+
+constexpr int kSl = 5;       // slices per operand
+constexpr int kKR = 64;      // observation rows per tile
+
+struct KrylovParams {
+  int64_t m;
+  int N;
+  const df32* HAdf;     // [m][N]
+  const df32* Ddf;      // [m][N]
+  df32* Zdf;            // [m][N]
+  float* B;             // [m][N] residual of the current Z, the next cycle's right-hand side
+  const df32* rdf;      // [m] R, 1/R and 1/sqrt(R) in double-float
+  const df32* rinv;
+  const df32* rsq;
+  df32* part;           // [G][krylov_part(N)] partial products and column sums of the CTAs
+  df32* Kred;           // [N][N]
+  df32* Fred;           // [N][N] F^T: row j is column j of F
+  df32* wred;           // [N][N] row j holds w_j
+  df32* Tred;           // [N][N] T^T
+  df32* sums;           // [2][N] ||d_j||^2 and (b_j, R^{-1} b_j)
+  double* rrpart;       // [2][G][NT]
+  double* W;            // [N][N]
+  double tol;
+  int max_iter, max_refine;
+  int* col_iters;
+  double* col_relres;
+  double* col_true;
+  int* status;
+  unsigned* bar;
+  unsigned long long* prof;
+  int phase;               // 0: the whole solve; 1: pass G only; 2: what follows pass G
+  // learned start (phase 2): w0 [N][N] (column j starts at w = w0_j), ||d_j - S z0_j||^2 per column
+  const float* w0;
+  const double* wnorm;
+  int warm_accept;
+  double* col_warm;
+};
+
+// kernels_krylov.cu: R, 1/R and 1/sqrt(R) in double-float from R in FP64
+cudaError_t launch_krylov_rows(const double* r, int64_t m, df32* rdf, df32* rinv, df32* rsq, cudaStream_t s);
+
+// entries of one CTA's partial: K and F columns of its column group, then two column sums
+__host__ __device__ constexpr int krylov_part(int N) { return 2 * N * (N < 64 ? N : 64) + 2 * 64; }
+
+template <int NT> struct KLayout {
+  static constexpr int JC = NT < 64 ? NT : 64;       // columns j of one CTA
+  static constexpr int CW = NT == 128 ? 192 : 128;    // pass G image: [U | V] columns
+  static constexpr int TROWS = NT == 128 ? 64 : 128;  // rows of the T operand (copies of its JC columns for NT <= 64)
+  static constexpr int HP = kKR * NT * 2;             // bytes per slice of the HA tile
+  static constexpr int CP = kKR * CW * 2;             // ... of the pass G image
+  static constexpr int TP = TROWS * NT * 2;           // ... of the T operand
+  static constexpr int VP = JC * kKR * 2;             // ... of the Z tile (rows j, K-major over i)
+  static constexpr int off_t = 0;
+  static constexpr int off_h = kSl * TP;
+  static constexpr int off_v = off_h + kSl * HP;
+  // (an M = 128 operand of fewer rows or columns reads on into the next region: rows that no
+  // result uses)
+  static constexpr int end_z = off_v + kSl * VP;
+  static constexpr int end_g = kSl * CP;
+  static constexpr int uni = end_z > end_g ? end_z : end_g;
+  // scalars: six FP64 and two int arrays of NT, row and column scales, column maxima, scratch
+  static constexpr int off_scal = uni;
+  static constexpr int off_row = off_scal + NT * (6 * 8 + 2 * 4);
+  static constexpr int off_col = off_row + 2 * 4 * kKR;
+  static constexpr int off_max = off_col + 4 * 256;
+  static constexpr int off_scr = off_max + 4 * 8 * 192;
+  static constexpr int need = off_scr + kThreads * 8;
+  // one CTA per SM whatever NT: each holds all of its SM's tensor memory
+  static constexpr int bytes = need < 120 * 1024 ? 120 * 1024 : need;
+  static_assert(bytes <= 226 * 1024, "shared memory");
+};
+
+// The power of two above |mx| (inv) and its inverse (scale). Entries below 2^-86 count as that size,
+// which keeps scale 2^26 finite (a row or column of zeros has scale 2^86).
+__device__ __forceinline__ void pow2_of(float mx, float& scale, float& inv) {
+  int E = (int)((__float_as_uint(mx) >> 23) & 0xFFu);
+  E = max(40, min(252, E));
+  scale = __uint_as_float((uint32_t)(253 - E) << 23);
+  inv = __uint_as_float((uint32_t)(E + 1) << 23);
+}
+
+__device__ __forceinline__ float rint_magic(float x) {   // |x| < 2^22
+  return __fsub_rn(__fadd_rn(x, 12582912.f), 12582912.f);
+}
+// the five slices of (h + l) scale, |h scale| <= 1: integers in FP32, weights 2^-8, 2^-17, ...
+__device__ __forceinline__ void slice5(float h, float l, float scale, float (&v)[kSl]) {
+  float x = __fmul_rn(h, scale * 256.f);
+  v[0] = rint_magic(x);
+  x = __fmul_rn(__fsub_rn(x, v[0]), 512.f);
+  v[1] = rint_magic(x);
+  x = __fmul_rn(__fsub_rn(x, v[1]), 512.f);
+  float s, e;
+  df_two_sum(x, __fmul_rn(l, scale * 67108864.f), s, e);   // l in units of the third slice (2^26)
+  v[2] = rint_magic(s);
+  x = __fmul_rn(__fadd_rn(__fsub_rn(s, v[2]), e), 512.f);
+  v[3] = rint_magic(x);
+  x = __fmul_rn(__fsub_rn(x, v[3]), 512.f);
+  v[4] = rint_magic(x);
+}
+__device__ __forceinline__ uint32_t pack_half2(float a, float b) {
+  const __half2 h = __floats2half2_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+// eight consecutive elements along the 16-byte direction of a core row, each slice one store
+__device__ __forceinline__ void store_slices8(unsigned char* base, int part_bytes, int off, const df32 (&x)[8],
+                                              const float (&scale)[8]) {
+  uint32_t w[kSl][4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    float a[kSl], b[kSl];
+    slice5(x[2 * q].hi, x[2 * q].lo, scale[2 * q], a);
+    slice5(x[2 * q + 1].hi, x[2 * q + 1].lo, scale[2 * q + 1], b);
+#pragma unroll
+    for (int s = 0; s < kSl; ++s) w[s][q] = pack_half2(a[s], b[s]);
+  }
+#pragma unroll
+  for (int s = 0; s < kSl; ++s)
+    *reinterpret_cast<uint4*>(base + s * part_bytes + off) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+}
+__device__ __forceinline__ void load_df8(df32 (&x)[8], const df32* row, int c0, int N, bool ok) {
+  if (ok && (N & 1) == 0 && c0 + 8 <= N) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float4 v = *reinterpret_cast<const float4*>(row + c0 + 2 * q);
+      x[2 * q] = df32(v.x, v.y);
+      x[2 * q + 1] = df32(v.z, v.w);
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] = (ok && c0 + q < N) ? row[c0 + q] : df32(0.f, 0.f);
+  }
+}
+// the same from data other CTAs of this launch wrote (read through L2)
+__device__ __forceinline__ void load_df8_cg(df32 (&x)[8], const df32* row, int c0, int N) {
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    x[q] = df32(0.f, 0.f);
+    if (c0 + q < N) {
+      const float2 v = __ldcg(reinterpret_cast<const float2*>(row + c0 + q));
+      x[q] = df32(v.x, v.y);
+    }
+  }
+}
+
+// tcgen05.ld of eight columns of the five level sums (levels `stride` columns apart)
+__device__ __forceinline__ void tmem_ld_levels(uint32_t taddr, uint32_t stride, float (&a)[kSl][8]) {
+  uint32_t r[kSl][8];
+#pragma unroll
+  for (int g = 0; g < kSl; ++g)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[g][0]), "=r"(r[g][1]), "=r"(r[g][2]), "=r"(r[g][3]), "=r"(r[g][4]), "=r"(r[g][5]),
+                   "=r"(r[g][6]), "=r"(r[g][7])
+                 : "r"(taddr + g * stride));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int g = 0; g < kSl; ++g)
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      // keep every use of the loaded registers behind the wait
+      asm volatile("" : "+r"(r[g][q]));
+      a[g][q] = __uint_as_float(r[g][q]);
+    }
+}
+// sum_g a_g 2^(-9 g) as an unevaluated pair (s, l): a_0..a_2 enter exactly, the two last levels are
+// 2^-27 of a_0's unit and below
+__device__ __forceinline__ void join_levels(float a0, float a1, float a2, float a3, float a4, float& s, float& l) {
+  float t, e, e2;
+  df_two_sum(a0, __fmul_rn(a1, 0x1p-9f), t, e);
+  df_two_sum(t, __fmul_rn(a2, 0x1p-18f), s, e2);
+  l = __fadd_rn(__fadd_rn(e, e2), __fmaf_rn(a4, 0x1p-36f, __fmul_rn(a3, 0x1p-27f)));
+}
+
+// The 15 slice products of D_g = sum_{i + j = g} A_i B_j over KS blocks of 16 along K: level g in
+// the `cols` tensor-memory columns at d + g cols. One thread.
+template <int KS>
+__device__ __forceinline__ void issue_levels(uint32_t d, int cols, uint64_t a, uint32_t a_part, uint32_t a_step,
+                                             uint64_t b, uint32_t b_part, uint32_t b_step, uint32_t idesc) {
+#pragma unroll 1
+  for (int g = 0; g < kSl; ++g)
+#pragma unroll 1
+    for (int i = 0; i <= g; ++i) {
+      const uint64_t ai = a + (uint64_t)((i * a_part) >> 4), bj = b + (uint64_t)(((g - i) * b_part) >> 4);
+#pragma unroll
+      for (int kb = 0; kb < KS; ++kb)
+        umma_f16(d + (uint32_t)(g * cols), ai + (uint64_t)((kb * a_step) >> 4), bj + (uint64_t)((kb * b_step) >> 4),
+                 idesc, (i > 0 || kb > 0) ? 1u : 0u);
+    }
+}
+// kind::f16 descriptor of FP16 operands with M = 128 and each operand K-major or MN-major
+__host__ __device__ constexpr uint32_t sl_idesc(int N, bool a_mn, bool b_mn) {
+  return umma_idesc(0, N, b_mn) | ((a_mn ? 1u : 0u) << 15);
+}
+
+// what the passes of one CTA share
+struct KCta {
+  unsigned char* smem;
+  uint32_t tmem;
+  uint64_t* mbar;
+  uint32_t phase;
+  int* status;
+  bool ok;
+};
+__device__ __forceinline__ void k_wait(KCta& c) {
+  if (!mbar_wait(c.mbar, c.phase, c.status)) c.ok = false;
+  c.phase ^= 1u;
+  tc_fence_after();
+}
+
+// A 64-row tile of a [rows][N] matrix into the K-major image of width W, each row scaled by a
+// power of two above its largest entry (inverse scales into s_inv[64]). COPIES: image row q holds
+// source row q % COPIES (the T operand); L2: read through L2.
+template <int W, int ROWS, int SRC, bool L2>
+__device__ __forceinline__ void slice_rows(const df32* __restrict__ src, int64_t row0, int64_t row1, int N,
+                                           unsigned char* img, float* s_inv) {
+  constexpr int G8 = W / 8, RPS = kThreads / G8, PART = ROWS * W * 2;
+  const int t = threadIdx.x, g = t % G8, c0 = 8 * g;
+#pragma unroll
+  for (int it = 0; it < ROWS / RPS; ++it) {
+    const int q = t / G8 + it * RPS;
+    const int64_t i = row0 + q % SRC;
+    df32 x[8];
+    if (L2) {
+      if (i < row1) load_df8_cg(x, src + i * N, c0, N);
+      else
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[e] = df32(0.f, 0.f);
+    } else {
+      load_df8(x, src + i * N, c0, N, i < row1);
+    }
+    float mx = 0.f;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) mx = fmaxf(mx, fabsf(x[e].hi));
+#pragma unroll
+    for (int o = G8 / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    float sc, inv;
+    pow2_of(mx, sc, inv);
+    const float scale[8] = {sc, sc, sc, sc, sc, sc, sc, sc};
+    store_slices8(img, PART, core_idx(q, c0, W) * 2, x, scale);
+    if (g == 0) s_inv[q] = inv;
+  }
+}
+
+// ------------------------------------------------------------------ pass G
+// The CTA's rows of U = R^{-1/2} HA and V = R^{-1/2} b (b = D, or the FP32 residual B) as one sliced
+// image [U | V] per tile, each column scaled by the power of two above its largest entry in the
+// tile, and K = U^T U, F = U^T V accumulated over the tiles in double-float registers. Column
+// group c takes the columns [64 c, 64 c + JC) of K and F. NT <= 64: one product [U | V]^T U
+// (M = 128: rows k of K, then rows j of F^T); NT = 128: U^T U_c, then U^T V.
+template <int NT>
+__device__ __noinline__ void pass_gram(const KrylovParams& p, bool from_b, int c, int64_t row0, int64_t row1,
+                                       KCta& cta, df32* __restrict__ out) {
+  using L = KLayout<NT>;
+  constexpr int JC = L::JC, CW = L::CW;
+  constexpr int UI = kKR * (NT / 8) / kThreads > 0 ? kKR * (NT / 8) / kThreads : 1;   // items of U per thread
+  constexpr int VI = kKR * (JC / 8) / kThreads > 0 ? kKR * (JC / 8) / kThreads : 1;
+  unsigned char* img = cta.smem;
+  float* s_max = reinterpret_cast<float*>(cta.smem + L::off_max);     // [8 warps][CW]
+  float* s_sc = reinterpret_cast<float*>(cta.smem + L::off_col);      // [CW] inverse column scales
+  const int N = p.N, t = threadIdx.x, warp = t >> 5, lane = t & 31, qd = warp & 3, half = warp >> 2;
+  const int gu = t % (NT / 8), ru = t / (NT / 8), gv = t % (JC / 8), rv = t / (JC / 8);
+  constexpr int RU = kThreads / (NT / 8), RV = kThreads / (JC / 8);   // rows per sweep
+  const int cv0 = c * 64 + 8 * gv;   // this thread's columns of b
+  const int L_ = 32 * qd + lane;
+  constexpr int NC = JC / 2;         // columns of a product per thread
+  DFAcc acc[NC], accF[NT == 128 ? NC : 1];
+  SqAcc s1[8], s2[8];
+  const uint32_t base = smem_addr(img);
+  constexpr uint32_t rg = (CW / 8) * 128;   // row-group stride
+  for (int64_t i0 = row0; i0 < row1 && cta.ok; i0 += kKR) {
+    df32 u[UI][8], v[VI][8];
+#pragma unroll
+    for (int it = 0; it < UI; ++it) {
+      const int r = ru + it * RU;
+      const int64_t i = i0 + r;
+      const bool in = r < kKR && i < row1;
+      load_df8(u[it], p.HAdf + i * N, 8 * gu, N, in);
+      if (in) {
+        const df32 q = p.rsq[i];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) u[it][e] = u[it][e] * q;
+      }
+    }
+#pragma unroll
+    for (int it = 0; it < VI; ++it) {
+      const int r = rv + it * RV;
+      const int64_t i = i0 + r;
+      const bool in = r < kKR && i < row1;
+      if (from_b) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[it][e] = df32((in && cv0 + e < N) ? p.B[i * N + cv0 + e] : 0.f, 0.f);
+      } else {
+        load_df8(v[it], p.Ddf + i * N, cv0, N, in);
+      }
+      if (in) {
+        const df32 q = p.rsq[i];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          s1[e].add(v[it][e].hi);
+          v[it][e] = v[it][e] * q;
+          s2[e].add(v[it][e].hi);
+        }
+      }
+    }
+    // column maxima of the tile: over the thread's items, the warp's lanes of the same columns,
+    // then the warps
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      float mu = 0.f, mv = 0.f;
+#pragma unroll
+      for (int it = 0; it < UI; ++it) mu = fmaxf(mu, fabsf(u[it][e].hi));
+#pragma unroll
+      for (int it = 0; it < VI; ++it) mv = fmaxf(mv, fabsf(v[it][e].hi));
+#pragma unroll
+      for (int o = 16; o >= NT / 8; o >>= 1) mu = fmaxf(mu, __shfl_xor_sync(0xffffffffu, mu, o));
+#pragma unroll
+      for (int o = 16; o >= JC / 8; o >>= 1) mv = fmaxf(mv, __shfl_xor_sync(0xffffffffu, mv, o));
+      if (lane < NT / 8) s_max[warp * CW + 8 * gu + e] = mu;
+      if (lane < JC / 8) s_max[warp * CW + NT + 8 * gv + e] = mv;
+    }
+    tc_fence_before();
+    __syncthreads();   // also: the previous tile's sums have left tensor memory
+    float su[8], sv[8];
+    {
+      float dummy;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        float mu = 0.f, mv = 0.f;
+#pragma unroll
+        for (int w = 0; w < kThreads / 32; ++w) {
+          mu = fmaxf(mu, s_max[w * CW + 8 * gu + e]);
+          mv = fmaxf(mv, s_max[w * CW + NT + 8 * gv + e]);
+        }
+        pow2_of(mu, su[e], dummy);
+        if (ru == 0) s_sc[8 * gu + e] = dummy;
+        pow2_of(mv, sv[e], dummy);
+        if (rv == 0) s_sc[NT + 8 * gv + e] = dummy;
+      }
+    }
+#pragma unroll
+    for (int it = 0; it < UI; ++it) {
+      const int r = ru + it * RU;
+      if (r < kKR) store_slices8(img, L::CP, core_idx(r, 8 * gu, CW) * 2, u[it], su);
+    }
+#pragma unroll
+    for (int it = 0; it < VI; ++it) {
+      const int r = rv + it * RV;
+      if (r < kKR) store_slices8(img, L::CP, core_idx(r, NT + 8 * gv, CW) * 2, v[it], sv);
+    }
+    fence_async_smem();
+    __syncthreads();
+    // K = rows of the tile, both operands MN-major (columns contiguous)
+    const uint64_t A = umma_desc(base, rg, 128);
+    if (t == 0) {
+      tc_fence_after();
+      issue_levels<kKR / 16>(cta.tmem, JC, A, L::CP, 2 * rg, umma_desc(base + (NT == 128 ? c * 1024 : 0), rg, 128),
+                             L::CP, 2 * rg, sl_idesc(JC, true, true));
+      umma_commit(cta.mbar);
+    }
+    k_wait(cta);
+    auto flush = [&](DFAcc* a, float rs, const float* cs) {
+#pragma unroll
+      for (int q0 = 0; q0 < NC; q0 += 8) {
+        float lv[kSl][8];
+        tmem_ld_levels(cta.tmem + ((uint32_t)(32 * qd) << 16) + half * NC + q0, JC, lv);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          float s, l, tt, e;
+          join_levels(lv[0][q], lv[1][q], lv[2][q], lv[3][q], lv[4][q], s, l);
+          const float f = rs * cs[q0 + q];
+          df_two_sum(a[q0 + q].s, s * f, tt, e);
+          a[q0 + q].s = tt;
+          a[q0 + q].c = __fadd_rn(a[q0 + q].c, __fmaf_rn(l, f, e));
+          a[q0 + q].renorm();
+        }
+      }
+    };
+    const float rs = s_sc[min(L_, CW - 1)] * 0x1p-16f;
+    flush(acc, rs, s_sc + (NT == 128 ? 64 * c : 0) + half * NC);
+    if constexpr (NT == 128) {
+      tc_fence_before();
+      __syncthreads();
+      if (t == 0) {
+        tc_fence_after();
+        issue_levels<kKR / 16>(cta.tmem, JC, A, L::CP, 2 * rg, umma_desc(base + (NT / 8) * 128, rg, 128), L::CP,
+                               2 * rg, sl_idesc(JC, true, true));
+        umma_commit(cta.mbar);
+      }
+      k_wait(cta);
+      flush(accF, rs, s_sc + NT + half * NC);
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  // the CTA's partial: K[k][jl] at k JC + jl, F[k][jl] behind it, then the column sums
+  const int NJ = min(JC, N);
+  if constexpr (NT == 128) {
+    if (L_ < N)
+#pragma unroll
+      for (int q = 0; q < NC; ++q) {
+        const int jl = half * NC + q;
+        out[L_ * NJ + jl] = acc[q].value();
+        out[N * NJ + L_ * NJ + jl] = accF[q].value();
+      }
+  } else {
+    // lanes [0, NT): K[k = lane][col]; lanes [NT, 2 NT): F^T[j = lane - NT][k = col]
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+      const int col = half * NC + q;
+      if (col < N) {
+        if (L_ < N) out[L_ * NJ + col] = acc[q].value();
+        else if (L_ >= NT && L_ - NT < N) out[N * NJ + col * NJ + (L_ - NT)] = acc[q].value();
+      }
+    }
+  }
+  // column sums over the threads of each column, fixed order
+  double* red = reinterpret_cast<double*>(cta.smem);   // [RV][JC] twice
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    red[rv * JC + 8 * gv + e] = s1[e].value();
+    red[(RV + rv) * JC + 8 * gv + e] = s2[e].value();
+  }
+  __syncthreads();
+  if (t < 2 * JC) {
+    const int which = t / JC, j = t % JC;
+    double s = 0.0;
+    for (int q = 0; q < RV; ++q) s += red[(which * RV + q) * JC + j];
+    out[2 * N * NJ + which * 64 + j] = df32(s);
+  }
+  __syncthreads();
+}
+
+// Entries [0, ngr cnt) of the partials (entry e of column group c: part[c cstride + q stride + e],
+// q < RB), summed over q in a fixed order: this CTA (b of G) takes a contiguous chunk, several
+// threads per entry where the chunk is shorter than the CTA, and hands (c, e, total) to store.
+template <class Store>
+__device__ __forceinline__ void reduce_parts(const df32* __restrict__ part, int64_t cstride, int64_t stride, int RB,
+                                             int ngr, int cnt, int G, int b, df32* scratch, Store&& store) {
+  const int t = threadIdx.x, total = ngr * cnt;
+  const int chunk = (total + G - 1) / G;
+  const int e0 = min(total, b * chunk), n = min(total, e0 + chunk) - e0;
+  auto add_range = [&](int e, int q0, int q1) {
+    const df32* src = part + (int64_t)(e / cnt) * cstride + e % cnt;
+    DFAcc a;
+#pragma unroll 8
+    for (int q = q0; q < q1; ++q) {
+      const float2 v = __ldcg(reinterpret_cast<const float2*>(src + q * stride));
+      float s, r;
+      df_two_sum(a.s, v.x, s, r);
+      a.s = s;
+      a.c = __fadd_rn(a.c, __fadd_rn(r, v.y));
+    }
+    return a.value();
+  };
+  if (n <= 0) return;
+  if (n >= kThreads) {
+    for (int e = e0 + t; e < e0 + n; e += kThreads) store(e / cnt, e % cnt, add_range(e, 0, RB));
+    return;
+  }
+  const int parts = kThreads / n, el = t % n, w = t / n;
+  scratch[t] = w < parts ? add_range(e0 + el, (int)((int64_t)w * RB / parts), (int)((int64_t)(w + 1) * RB / parts))
+                         : df32(0.f, 0.f);
+  __syncthreads();
+  if (t < n) {
+    df32 v = scratch[t];
+    for (int q = 1; q < parts; ++q) v = v + scratch[q * n + t];
+    const int e = e0 + t;
+    store(e / cnt, e % cnt, v);
+  }
+  __syncthreads();
+}
+
+// ------------------------------------------------------------------ CG in the coordinates
+__device__ __forceinline__ df32 df_div(const df32& a, const df32& b) {   // two corrections: about 46 bits
+  const float r = __frcp_rn(b.hi);
+  const float q0 = __fmul_rn(a.hi, r);
+  df32 e = a - b * df32(q0, 0.f);
+  const float q1 = __fmul_rn(e.hi, r);
+  e = e - b * df32(q1, 0.f);
+  const df32 q = df_fast2sum(q0, q1);
+  return q + df32(__fmul_rn(e.hi, r), 0.f);
+}
+__device__ __forceinline__ df32 df_shfl_xor(const df32& v, int o) {
+  return df32(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
+}
+__device__ __forceinline__ df32 ld_df(const df32* p) {
+  const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
+  return df32(v.x, v.y);
+}
+
+// Columns j0, j0 + step, ... (nc <= 8, one per warp) of this cycle: (I + K) w = g from w = 0 (or the
+// learned start) by the recurrences at the head of this file until (r, R^{-1} r) <= itol^2
+// (b, R^{-1} b) or the column's step limit; w into row j of wred, the steps taken added to
+// col_iters[j]. Everything is double-float: on this part an FP64 instruction holds a scheduler's
+// FP64 unit for about 64 cycles, and the first form of this loop, with the vectors and scalars of
+// a step in FP64 (some 60 such instructions in one warp's serial chain), took 2.9 us per step at
+// N = 64 and 5.3 at N = 128. A step is one product (each thread keeps its block of K in
+// registers, shared by the CTA's columns) and one round of sums: with kr = K rho, (p, S p)
+// is (rho, kr) + (kr, kr) - beta^2 (p, S p)_old.
+template <int NT>
+struct KMat {
+  static constexpr int TPR = kThreads / NT, KPT = NT / TPR;   // threads per row, entries per thread
+  df32 k[KPT];
+};
+struct KColumns {
+  const df32* F;         // [N][N]
+  df32* w;               // [N][N]
+  const double* bb;      // shared: (b_j, R^{-1} b_j), tolerance, done and rejected starts per column
+  const double* itol;
+  const int* done;
+  const int* bad;
+  const float* w0;       // learned start or nullptr
+  int* iters;            // [N] steps so far (global)
+  bool first;            // first cycle: iters is not read
+  int max_iter;
+  int* status;
+};
+template <int NT>
+__device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 inv_nm1, int j0, int step, int nc,
+                                          const KColumns& C, unsigned char* sm) {
+  constexpr int TPR = KMat<NT>::TPR, KPT = KMat<NT>::KPT, EPL = NT / 32;
+  df32* s_rho = reinterpret_cast<df32*>(sm);                  // [8][NT]
+  df32* s_part = s_rho + 8 * NT;                              // [8][TPR][NT]
+  int* s_act = reinterpret_cast<int*>(s_part + 8 * kThreads); // [8]
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, r = t % NT, g = t / NT;
+  const bool mine = warp < nc;
+  const int j = j0 + warp * step;
+  df32 rho[EPL], f[EPL], h[EPL], w[EPL], rr, pq;
+  float stop = 0.f;
+  int it = 0, limit = 0, used = 0, act = 0;
+  bool start = false;
+  if (mine) {
+    used = C.first ? 0 : *(volatile int*)&C.iters[j];
+    limit = C.done[j] ? 0 : max(0, C.max_iter - used);
+    stop = (float)(C.itol[j] * C.itol[j] * C.bb[j] * (double)inv_nm1.hi);   // of rho^T K rho
+    start = C.w0 && !C.bad[j] && !C.done[j];
+    act = 1;
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) {
+      const int k = lane + 32 * e;
+      rho[e] = k < N ? ld_df(C.F + (int64_t)j * N + k) * inv_nm1 : df32(0.f, 0.f);
+      if (start && k < N) w[e] = df32(C.w0[(int64_t)k * N + j], 0.f);
+      s_rho[warp * NT + k] = start ? w[e] : rho[e];
+    }
+  }
+  if (t < 8) s_act[t] = t < nc;
+  // K times the vectors in s_rho of the active columns: thread (g, r) its entries of row r
+  auto product = [&]() {
+#pragma unroll 1
+    for (int c = 0; c < nc; ++c) {
+      if (!s_act[c]) continue;
+      const df32* v = s_rho + c * NT + g * KPT;
+      DFAcc a0, a1;
+#pragma unroll
+      for (int q = 0; q < KPT; q += 2) {
+        const float4 x = *reinterpret_cast<const float4*>(v + q);
+        a0.add(M.k[q], df32(x.x, x.y));
+        a1.add(M.k[q + 1], df32(x.z, x.w));
+        if ((q & 7) == 6) { a0.renorm(); a1.renorm(); }
+      }
+      s_part[c * kThreads + g * NT + r] = a0.value() + a1.value();
+    }
+    __syncthreads();
+  };
+  auto row = [&](int k) {
+    df32 s = s_part[warp * kThreads + k];
+#pragma unroll
+    for (int q = 1; q < TPR; ++q) s = s + s_part[warp * kThreads + q * NT + k];
+    return s;
+  };
+  if (C.w0) {   // rho = g - (I + K) w0 (the same for every column; without a start w = 0)
+    __syncthreads();
+    product();
+    if (mine)
+#pragma unroll
+      for (int e = 0; e < EPL; ++e) {
+        if (start) rho[e] = rho[e] - (w[e] + row(lane + 32 * e));
+        s_rho[warp * NT + lane + 32 * e] = rho[e];
+      }
+  }
+  while (__syncthreads_or(act)) {
+    product();
+    if (act) {
+      df32 kr[EPL], d1, d2;
+#pragma unroll
+      for (int e = 0; e < EPL; ++e) {
+        kr[e] = row(lane + 32 * e);
+        d1 = fma(rho[e], kr[e], d1);
+        d2 = fma(kr[e], kr[e], d2);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        d1 = d1 + df_shfl_xor(d1, o);
+        d2 = d2 + df_shfl_xor(d2, o);
+      }
+      // a non-finite value ends the column (the true residual reports it); so does a (p, S p) that
+      // is not positive: rounding has used up this cycle
+      if (!isfinite(d1.hi)) {
+        if (lane == 0) atomicOr(C.status, DS_NONFINITE);
+        act = 0;
+      } else if (d1.hi <= stop || it >= limit) {
+        act = 0;
+      } else {
+        df32 beta;
+        if (it > 0) beta = df_div(d1, rr);
+        pq = (d1 + d2) - (it > 0 ? beta * beta * pq : df32(0.f, 0.f));
+        rr = d1;
+        if (!(pq.hi > 0.f) || !isfinite(pq.hi)) {
+          act = 0;
+        } else {
+          const df32 alpha = df_div(rr, pq);
+#pragma unroll
+          for (int e = 0; e < EPL; ++e) {
+            f[e] = it > 0 ? fma(beta, f[e], rho[e]) : rho[e];
+            h[e] = it > 0 ? fma(beta, h[e], kr[e]) : kr[e];
+            w[e] = fma(alpha, f[e], w[e]);
+            rho[e] = rho[e] - alpha * (f[e] + h[e]);
+            s_rho[warp * NT + lane + 32 * e] = rho[e];
+          }
+          ++it;
+        }
+      }
+      if (!act && lane == 0) s_act[warp] = 0;
+    }
+  }
+  if (mine) {
+#pragma unroll
+    for (int e = 0; e < EPL; ++e)
+      if (lane + 32 * e < N) C.w[(int64_t)j * N + lane + 32 * e] = w[e];
+    if (lane == 0) C.iters[j] = used + it;
+  }
+  __syncthreads();
+}
+
+// ------------------------------------------------------------------ passes Z and R
+// The T operand of u = HA T: the CTA's JC columns of a reduced N x N matrix (row j of `src` is
+// column j), sliced with a power of two per column; inverse scales into s_inv[128].
+template <int NT>
+__device__ __forceinline__ void stage_columns(const df32* __restrict__ src, int c, int N, unsigned char* img,
+                                              float* s_inv) {
+  using L = KLayout<NT>;
+  slice_rows<NT, L::TROWS, L::JC, true>(src, (int64_t)c * 64, N, N, img, s_inv);
+}
+
+// Both passes: u = HA T for a tile arrives as D[j][i] (lane j, tensor-memory column i), so that a
+// thread owns one column j and RPT consecutive rows, its accesses to D and Z are contiguous
+// across the warp, and column sums and maxima stay in the thread. For NT <= 64 the T operand holds
+// 128 / NT copies of its columns, so that all 128 lanes carry work (copy d takes the rows
+// [16 d, ...) of a tile); at NT = 128 two such copies do not fit and half of the lanes idle.
+// RESID = false: Z (+)= R^{-1} (b - u), then T += HA^T Z (out: T[k][jl]).
+// RESID = true: B = D - R Z - u/(N-1) and rr[j] = ||B_j||^2 over the CTA's rows.
+template <int NT, bool RESID>
+__device__ __noinline__ void pass_rows(const KrylovParams& p, bool from_b, int c, int64_t row0, int64_t row1,
+                                       KCta& cta, const int* s_done, df32* __restrict__ out, double* rr_out) {
+  using L = KLayout<NT>;
+  constexpr int JC = L::JC;
+  constexpr int CP = NT == 128 ? 1 : 128 / NT;    // copies
+  constexpr int RPT = kKR / (2 * CP);             // rows per thread: 8, 16, 32
+  unsigned char* sT = cta.smem + L::off_t;
+  unsigned char* sH = cta.smem + L::off_h;
+  unsigned char* sV = cta.smem + L::off_v;
+  float* s_row = reinterpret_cast<float*>(cta.smem + L::off_row);   // [64] inverse row scales
+  float* s_col = reinterpret_cast<float*>(cta.smem + L::off_col);   // [128] inverse scales of T
+  float* s_max = reinterpret_cast<float*>(cta.smem + L::off_max);   // [2 CP][64] column maxima
+  const int N = p.N, t = threadIdx.x, warp = t >> 5, lane = t & 31, qd = warp & 3, half = warp >> 2;
+  const int ln = 32 * qd + lane, jl = ln % JC, j = 64 * c + jl;
+  const int copy = ln / JC;                       // NT = 128: lanes 64.. hold no column
+  const bool live = copy < CP && j < N;
+  // a column that is done keeps its Z: its right-hand side is zero in the cycles of the others
+  const bool frozen = !RESID && from_b && live && s_done[j];
+  const int rg = copy * 2 + half, r0 = rg * RPT;  // this thread's rows of the tile
+  const uint32_t aT = smem_addr(sT), aH = smem_addr(sH), aV = smem_addr(sV);
+  constexpr uint32_t hst = (NT / 8) * 128;
+  const float tsc = s_col[min(ln, L::TROWS - 1)] * 0x1p-16f;
+  const df32 inv_nm1(1.0 / (double)(N - 1));
+  DFAcc acc[RESID ? 1 : JC / 2];
+  float rr = 0.f;
+  double rr64 = 0.0;
+  for (int64_t i0 = row0; i0 < row1 && cta.ok; i0 += kKR) {
+    slice_rows<NT, kKR, kKR, false>(p.HAdf, i0, row1, N, sH, s_row);
+    fence_async_smem();
+    tc_fence_before();
+    __syncthreads();
+    if (t == 0) {
+      tc_fence_after();
+      issue_levels<NT / 16>(cta.tmem, kKR, umma_desc(aT, 128, hst), L::TP, 256, umma_desc(aH, 128, hst), L::HP, 256,
+                            sl_idesc(kKR, false, false));
+      umma_commit(cta.mbar);
+    }
+    // this thread's entries, in flight behind the products
+    df32 d[RPT], z[RPT];
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+      const int64_t i = i0 + r0 + q;
+      const bool in = live && i < row1;
+      d[q] = df32(0.f, 0.f);
+      z[q] = df32(0.f, 0.f);
+      if (in) {
+        if (!RESID && from_b) d[q] = df32(frozen ? 0.f : p.B[i * N + j], 0.f);
+        else d[q] = p.Ddf[i * N + j];
+        if (RESID || from_b) z[q] = p.Zdf[i * N + j];
+      }
+    }
+    k_wait(cta);
+    float mx = 0.f;
+#pragma unroll
+    for (int q0 = 0; q0 < RPT; q0 += 8) {
+      float lv[kSl][8];
+      tmem_ld_levels(cta.tmem + ((uint32_t)(32 * qd) << 16) + (r0 & (kKR - 1)) + q0, kKR, lv);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int rq = r0 + q0 + q;
+        const int64_t i = i0 + rq;
+        if (!(live && i < row1)) continue;
+        float s, l;
+        join_levels(lv[0][q], lv[1][q], lv[2][q], lv[3][q], lv[4][q], s, l);
+        const float f = tsc * s_row[rq];
+        const df32 u = df_fast2sum(s * f, l * f);
+        if (RESID) {
+          const df32 res = d[q0 + q] - fma(p.rdf[i], z[q0 + q], u * inv_nm1);
+          rr = __fmaf_rn(res.hi, res.hi, rr);
+          p.B[i * N + j] = res.hi;
+        } else {
+          const df32 zn = z[q0 + q] + (d[q0 + q] - u) * p.rinv[i];
+          p.Zdf[i * N + j] = zn;
+          // times the inverse of the HA row's scale: HA_ik z_ij = (HA_ik s_i) (z_ij / s_i)
+          z[q0 + q] = df32(zn.hi * s_row[rq], zn.lo * s_row[rq]);
+          mx = fmaxf(mx, fabsf(z[q0 + q].hi));
+        }
+      }
+    }
+    if constexpr (RESID) {
+      rr64 += (double)rr;
+      rr = 0.f;
+      tc_fence_before();
+      __syncthreads();   // the tile image and tensor memory are rewritten by the next tile
+    } else {
+      if (copy < CP) s_max[rg * 64 + jl] = mx;
+      __syncthreads();
+      float m2 = mx;
+#pragma unroll
+      for (int q = 0; q < 2 * CP; ++q) m2 = fmaxf(m2, s_max[q * 64 + jl]);
+      float sc, inv;
+      pow2_of(m2, sc, inv);
+      const float scale[8] = {sc, sc, sc, sc, sc, sc, sc, sc};
+      if (copy < CP)
+#pragma unroll
+        for (int q0 = 0; q0 < RPT; q0 += 8) {
+          const df32 x[8] = {z[q0], z[q0 + 1], z[q0 + 2], z[q0 + 3], z[q0 + 4], z[q0 + 5], z[q0 + 6], z[q0 + 7]};
+          store_slices8(sV, L::VP, core_idx(jl, r0 + q0, kKR) * 2, x, scale);
+        }
+      if (rg == 0) s_max[2 * CP * 64 + jl] = inv;
+      fence_async_smem();
+      tc_fence_before();
+      __syncthreads();
+      if (t == 0) {
+        tc_fence_after();
+        // T[k][jl]: A = the HA tile MN-major (M = k), B = the Z tile K-major
+        issue_levels<kKR / 16>(cta.tmem, JC, umma_desc(aH, hst, 128), L::HP, 2 * hst, umma_desc(aV, 128, 1024),
+                               L::VP, 256, sl_idesc(JC, true, false));
+        umma_commit(cta.mbar);
+      }
+      k_wait(cta);
+      if (32 * qd < N) {   // uniform in the warp
+        constexpr int NC = JC / 2;
+#pragma unroll
+        for (int q0 = 0; q0 < NC; q0 += 8) {
+          float lv[kSl][8];
+          tmem_ld_levels(cta.tmem + ((uint32_t)(32 * qd) << 16) + half * NC + q0, JC, lv);
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            float s, l, tt, e;
+            join_levels(lv[0][q], lv[1][q], lv[2][q], lv[3][q], lv[4][q], s, l);
+            const float f = s_max[2 * CP * 64 + half * NC + q0 + q] * 0x1p-16f;
+            df_two_sum(acc[q0 + q].s, s * f, tt, e);
+            acc[q0 + q].s = tt;
+            acc[q0 + q].c = __fadd_rn(acc[q0 + q].c, __fmaf_rn(l, f, e));
+            acc[q0 + q].renorm();
+          }
+        }
+      }
+      tc_fence_before();
+      __syncthreads();
+    }
+  }
+  if constexpr (RESID) {
+    double* red = reinterpret_cast<double*>(cta.smem + L::off_h);   // [2 CP][64]
+    __syncthreads();
+    if (copy < CP) red[rg * 64 + jl] = rr64;
+    __syncthreads();
+    if (t < JC) {
+      double s = 0.0;
+      for (int q = 0; q < 2 * CP; ++q) s += red[q * 64 + t];
+      rr_out[64 * c + t] = s;
+    }
+    __syncthreads();
+  } else {
+    const int NJ = min(JC, N);
+#pragma unroll
+    for (int q = 0; q < JC / 2; ++q) {
+      const int col = half * (JC / 2) + q;
+      if (ln < N && col < NJ) out[ln * NJ + col] = acc[q].value();
+    }
+  }
+}
+
+// ------------------------------------------------------------------ the solve
+// CTA b of the G co-resident CTAs of one problem (the grid, or a team of a batched launch). The
+// rows are split over G / CG row blocks; at NT = 128 two CTAs share a row block, one per column
+// group (a single CTA takes both groups in turn). Partial sums are reduced in a fixed order.
+template <int NT>
+__device__ void krylov_body(const KrylovParams& p, const int G, const int b, GridBarrier& bar, KCta& cta) {
+  using L = KLayout<NT>;
+  constexpr int JC = L::JC;
+  double* s_dn2 = reinterpret_cast<double*>(cta.smem + L::off_scal);
+  double* s_true = s_dn2 + NT;
+  double* s_prev = s_true + NT;
+  double* s_itol = s_prev + NT;
+  double* s_tmp = s_itol + NT;
+  double* s_bb = s_tmp + NT;
+  int* s_done = reinterpret_cast<int*>(s_bb + NT);
+  int* s_bad = s_done + NT;
+  double* scratch = reinterpret_cast<double*>(cta.smem + L::off_scr);
+  const int N = p.N, t = threadIdx.x, NJ = min(JC, N);
+  if (dynamic_smem_bytes() < (unsigned)L::bytes) {
+    if (t == 0) atomicOr(p.status, DS_SMEM);
+    return;
+  }
+  const int ngr = (N + JC - 1) / JC;              // column groups in use
+  const int RB = max(1, G / ngr);                 // row blocks
+  const int rb = G >= ngr ? b / ngr : 0;
+  const int c0 = G >= ngr ? b % ngr : 0, c1 = G >= ngr ? c0 + 1 : ngr;
+  const bool has_rows = rb < RB;
+  const int64_t rows_per = (p.m + RB - 1) / RB;
+  const int64_t row0 = has_rows ? imin64(p.m, (int64_t)rb * rows_per) : p.m;
+  const int64_t row1 = imin64(p.m, row0 + rows_per);
+  const int64_t PS = krylov_part(N);
+  auto part_of = [&](int q, int c) { return p.part + ((int64_t)q * ngr + c) * PS; };
+  const double inv_nm1 = 1.0 / (double)(N - 1);
+  const bool prof = p.prof != nullptr && b == 0 && t == 0;
+  unsigned long long ph[PH_COUNT] = {0, 0, 0, 0, 0, 0, 0, 0};
+  unsigned long long tp = prof ? global_ns() : 0ull;
+  auto tick = [&](int slot) {
+    if (prof) {
+      const unsigned long long now = global_ns();
+      ph[slot] += now - tp;
+      tp = now;
+    }
+  };
+  int par = 0;
+  bool ok = true;
+  if (t < NT) {
+    s_done[t] = t >= N;
+    s_true[t] = -1.0;
+    s_prev[t] = 0.0;
+    s_dn2[t] = 0.0;
+    s_itol[t] = fmin(0.5, fmax(0.02 * p.tol, 1e-14));
+  }
+  __syncthreads();
+  // a reduction over the G CTAs' per-column sums (s_tmp in, s_tmp out)
+  auto column_totals = [&]() -> bool {
+    if (t < NT) p.rrpart[((int64_t)par * G + b) * NT + t] = s_tmp[t];
+    if (!bar.sync()) return false;
+    reduce_all<NT>(p.rrpart + (int64_t)par * G * NT, G, N, s_tmp, scratch);
+    par ^= 1;
+    return true;
+  };
+  tick(PH_SETUP);
+
+  int cycles = 0;
+  for (;;) {
+    const bool from_b = cycles > 0;
+    if (from_b || p.phase != 2) {
+    // ---- pass G and its reduction
+    for (int c = c0; c < c1; ++c)
+      if (has_rows) pass_gram<NT>(p, from_b, c, row0, row1, cta, part_of(rb, c));
+    tick(PH_SETUP);
+    if (!(ok = bar.sync() && cta.ok)) break;
+    tick(PH_BAR1);
+    reduce_parts(p.part, PS, ngr * PS, RB, ngr, 2 * N * NJ + 128, G, b,
+                 reinterpret_cast<df32*>(scratch), [&](int c, int e, df32 v) {
+      const int nj = min(JC, N - 64 * c);
+      if (e < N * NJ) {
+        const int k = e / NJ, jl = e % NJ;
+        if (jl < nj) p.Kred[k * N + 64 * c + jl] = df32((double)v * inv_nm1);
+      } else if (e < 2 * N * NJ) {
+        const int k = (e - N * NJ) / NJ, jl = (e - N * NJ) % NJ;
+        if (jl < nj) p.Fred[(int64_t)(64 * c + jl) * N + k] = v;
+      } else {
+        const int which = (e - 2 * N * NJ) / 64, jl = (e - 2 * N * NJ) % 64;
+        if (jl < nj) p.sums[which * N + 64 * c + jl] = v;
+      }
+    });
+    tick(PH_RED);
+    if (!from_b && p.phase == 1) return;
+    if (!(ok = bar.sync())) break;
+    tick(PH_BAR2);
+    }
+    if (t < N) {
+      const float2 a = __ldcg(reinterpret_cast<const float2*>(p.sums + t));
+      const float2 q = __ldcg(reinterpret_cast<const float2*>(p.sums + N + t));
+      if (!from_b) {
+        s_dn2[t] = (double)a.x + (double)a.y;
+        if (s_dn2[t] == 0.0) { s_done[t] = 1; s_true[t] = 0.0; }
+      }
+      s_bb[t] = (double)q.x + (double)q.y;
+    }
+    __syncthreads();
+    if (!from_b && p.w0) {
+      // the learned start's true residual judges it: a column whose start is non-finite or (unless
+      // warm_accept) whose residual is larger than the zero start's (d_j) starts from w = 0
+      if (t < NT) {
+        const double v = t < N ? p.wnorm[t] : 0.0;
+        const bool zero = t >= N || s_dn2[t] == 0.0;
+        s_bad[t] = !zero && (p.warm_accept ? !isfinite(v) : !(v <= s_dn2[t])) ? 1 : 0;
+        if (b == 0 && t < N) p.col_warm[t] = zero ? 0.0 : sqrt(v / s_dn2[t]);
+      }
+      const int nbad = __syncthreads_count(t < NT && s_bad[t]);
+      if (b == 0 && t == 0) p.status[2] = nbad;
+    }
+    // ---- the recurrences, column j on CTA j mod G
+    if (b < N) {
+      KMat<NT> M;
+      const int r = t % NT, g = t / NT;
+#pragma unroll
+      for (int q = 0; q < KMat<NT>::KPT; ++q) {
+        const int k = g * KMat<NT>::KPT + q;
+        M.k[q] = df32(0.f, 0.f);
+        if (k < N && r < N) {
+          const float2 v = __ldcg(reinterpret_cast<const float2*>(p.Kred + k * N + r));
+          M.k[q] = df32(v.x, v.y);
+        }
+      }
+      const KColumns C{p.Fred, p.wred, s_bb, s_itol, s_done, s_bad, from_b ? nullptr : p.w0,
+                       p.col_iters, !from_b, p.max_iter, p.status};
+      for (int j = b; j < N; j += 8 * G)
+        krylov_cg<NT>(M, N, df32(inv_nm1), j, G, min(8, (N - j + G - 1) / G), C, cta.smem);
+    }
+    tick(PH_PASS);
+    if (!(ok = bar.sync())) break;
+    tick(PH_BAR1);
+    // ---- pass Z and the reduction of T (W = T/(N-1))
+    for (int c = c0; c < c1; ++c)
+      if (has_rows) {
+        stage_columns<NT>(p.wred, c, N, cta.smem + L::off_t, reinterpret_cast<float*>(cta.smem + L::off_col));
+        __syncthreads();
+        pass_rows<NT, false>(p, from_b, c, row0, row1, cta, s_done, part_of(rb, c), nullptr);
+      }
+    tick(PH_REFRESH);
+    if (!(ok = bar.sync() && cta.ok)) break;
+    tick(PH_BAR1);
+    reduce_parts(p.part, PS, ngr * PS, RB, ngr, N * NJ, G, b, reinterpret_cast<df32*>(scratch),
+                 [&](int c, int e, df32 v) {
+      const int k = e / NJ, jl = e % NJ;
+      if (jl < min(JC, N - 64 * c)) {
+        p.Tred[(int64_t)(64 * c + jl) * N + k] = v;
+        p.W[k * N + 64 * c + jl] = (double)v * inv_nm1;
+      }
+    });
+    tick(PH_RED);
+    if (!(ok = bar.sync())) break;
+    tick(PH_BAR2);
+    // ---- pass R: the true residual
+    if (t < NT) s_tmp[t] = 0.0;
+    __syncthreads();
+    for (int c = c0; c < c1; ++c)
+      if (has_rows) {
+        stage_columns<NT>(p.Tred, c, N, cta.smem + L::off_t, reinterpret_cast<float*>(cta.smem + L::off_col));
+        __syncthreads();
+        pass_rows<NT, true>(p, from_b, c, row0, row1, cta, s_done, nullptr, s_tmp);
+      }
+    if (!(ok = column_totals() && cta.ok)) break;
+    ++cycles;
+    if (t < N) {
+      // a non-finite residual or ||d_j|| (NaN or Inf in the inputs) ends the column with the
+      // non-finite status
+      const bool fin = isfinite(s_dn2[t]) && isfinite(s_tmp[t]);
+      if (!fin) atomicOr(p.status, DS_NONFINITE);
+      const double tr = !fin ? (double)NAN : (s_dn2[t] > 0.0 ? sqrt(s_tmp[t] / s_dn2[t]) : 0.0);
+      s_true[t] = tr;
+      const int used = *(volatile int*)&p.col_iters[t];
+      // done: converged, non-finite, stalled (no halving over a cycle) or out of steps
+      if (!fin || tr <= p.tol || (cycles >= 2 && tr > 0.5 * s_prev[t]) || used >= p.max_iter) s_done[t] = 1;
+      s_prev[t] = tr;
+      s_itol[t] = fmin(0.5, fmax(tr > 0.0 ? 0.02 * p.tol / tr : 0.5, 1e-14));
+    }
+    const int all_done = __syncthreads_and(t >= N || s_done[t]);
+    tick(PH_REFRESH);
+    if (all_done || cycles > p.max_refine) break;
+  }
+  if (b == 0) {
+    if (t < N) {
+      p.col_relres[t] = s_true[t];
+      p.col_true[t] = s_true[t];
+      if (ok && !(s_true[t] >= 0.0 && s_true[t] <= p.tol)) atomicOr(p.status, DS_NOT_CONVERGED);
+    }
+    if (t == 0) p.status[1] = cycles;
+    if (prof)
+      for (int q = 0; q < PH_COUNT; ++q) p.prof[q] = ph[q];
+  }
+}
+
+// tensor memory and the completion barrier of a CTA (all 512 columns: one CTA per SM)
+__device__ __forceinline__ void krylov_begin(KCta& cta, unsigned char* smem, uint64_t* mbar, uint32_t* tmem_slot,
+                                             int* status) {
+  if (threadIdx.x == 0) mbar_init(mbar);
+  if (threadIdx.x < 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)), "r"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  cta = KCta{smem, *tmem_slot, mbar, 0u, status, true};
+}
+__device__ __forceinline__ void krylov_end(const KCta& cta) {
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(cta.tmem), "r"(512));
+}
+
+}  // namespace enkf

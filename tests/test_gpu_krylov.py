@@ -1,0 +1,69 @@
+"""The preconditioned solve in Krylov coordinates (csrc/krylov.cuh) at the sizes where its tiling
+can go wrong: N around the column tiles (32, 64, 128) and odd, m around the 64-row tile and
+the row blocks of several grids, one CTA for two column groups, variances spread over four
+decades, and members of very different spread. Against the exact FP64 analysis; the bar is the
+FP32 path's (1e-6 relative Frobenius error: X_a is stored in FP32) and the certificate the true
+residual within tol."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def _problem(N, m, seed, r_decades=0.0, outlier=1.0):
+    rng = np.random.default_rng(seed)
+    n = max(2 * m, 8)
+    side = int(np.ceil(np.sqrt(n)))
+    p = synth.grf_problem(side, max(1.0, side / 12), N, m, 0.5, 1.5, seed, dtype=np.float32)
+    p.r = p.r * 10.0 ** rng.uniform(-r_decades / 2, r_decades / 2, m)
+    p.Xf[:, 0] *= np.float32(outlier)
+    return p
+
+
+def _check(lib, p, prec="fp32", tol=1e-8, **cfg):
+    an = lib.Analysis(p.n, p.m, p.N, p.rowptr, p.col, p.w, p.r, precision=prec, precondition=1, tol=tol, **cfg)
+    Xa = an.analyze(torch.from_numpy(p.Xf).cuda(), torch.from_numpy(p.y).cuda(), seed=4, counter=9)
+    st = an.stats()
+    E = oracle.obs_perturbations(4, 9, p.r, p.N)
+    ref = oracle.enkf_exact(p.Xf.astype(np.float64), p.rowptr, p.col, p.w, p.r, p.y, E)
+    err = oracle.rel_frobenius(Xa.double().cpu().numpy(), ref)
+    assert st["status"] == "ok" and 0 <= st["true_relres_max"] <= tol, st
+    assert err <= 1e-6, (err, st)
+    an.close()
+
+
+@pytest.mark.parametrize("N", [2, 3, 31, 32, 33, 63, 64, 65, 96, 127, 128])
+@pytest.mark.parametrize("m,G", [(1, 0), (63, 0), (64, 1), (65, 2), (450, 3), (700, 5)])
+def test_tile_edges(lib, N, m, G):
+    _check(lib, _problem(N, m, 1000 * N + m), grid_blocks=G)
+
+
+@pytest.mark.parametrize("N", [20, 64, 100])
+def test_spread_variances_and_members(lib, N):
+    _check(lib, _problem(N, 900, 7 + N, r_decades=4.0))
+    _check(lib, _problem(N, 900, 9 + N, outlier=300.0))
+
+
+def test_tight_tolerance_takes_another_cycle(lib):
+    _check(lib, _problem(64, 4000, 3), tol=1e-12)
+
+
+@pytest.mark.parametrize("cfg", [dict(prec="fp16", refresh_every=6), dict(prec="fp32", fixed_iters=70)])
+def test_configurations_about_the_m_vectors_keep_their_recurrences(lib, cfg):
+    # a cap on the steps between refreshes, and a step count fixed by the caller
+    p = _problem(32, 500, 21)
+    c = dict(cfg)
+    an = lib.Analysis(p.n, p.m, p.N, p.rowptr, p.col, p.w, p.r, precision=c.pop("prec"), precondition=1, tol=1e-6, **c)
+    Xa = an.analyze(torch.from_numpy(p.Xf).cuda(), torch.from_numpy(p.y).cuda(), seed=4, counter=9)
+    st = an.stats()
+    E = oracle.obs_perturbations(4, 9, p.r, p.N)
+    ref = oracle.enkf_exact(p.Xf.astype(np.float64), p.rowptr, p.col, p.w, p.r, p.y, E)
+    assert st["status"] == "ok", st
+    assert oracle.rel_frobenius(Xa.double().cpu().numpy(), ref) <= 1e-4
+    if "fixed_iters" in cfg:
+        it, _, _ = an.column_stats()
+        assert np.all(it <= 70) and it.max() > 32   # m-vector steps past N: not the N-space count
