@@ -129,8 +129,8 @@ typedef struct enkf_config {
                              the recurrences in the coordinates of their Krylov space:
                              z = R^-1 (d - HA w) with an N-vector w per column, started at
                              w = 0 (z = R^-1 d). The products with HA that remain run on the
-                             tensor cores with operands of five 9-bit FP16 slices (44 bits,
-                             exact FP32 sums), the N x N recurrences in FP32 pairs, and the
+                             tensor cores with operands of five FP16 slices (48 bits, exact
+                             FP32 sums), the N x N recurrences in FP32 pairs, and the
                              result is certified by the true residual as in every mode    */
   int32_t lowprec_terms;  /* BF16/FP16 modes: 3 (or 0, the default) splits every operand
                              into hi + lo parts and forms hi*hi + hi*lo + lo*hi (about 16

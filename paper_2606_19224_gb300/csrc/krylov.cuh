@@ -22,15 +22,19 @@
 // The products need more than FP32 (the residual's terms cancel to 1e-8 and below), and double-
 // float products on the CUDA cores cost 12 FP32 operations per term: 0.16 ms per product pair at
 // m = 65,536, N = 64, measured 0.33 ms per refresh, with the tensor cores idle. Here every operand
-// is a fixed-point number of five signed 9-bit slices (44 bits below a power of two at least the
-// largest entry of its row or column), each slice an integer of at most 256 in FP16. A product
-// of two slices is at most 2^16 and a sum of 64 of them (one tile) at most 2^22, so that the sums
-// that belong to one power of two (slices i and j with i + j = g, g = 0..4: 15 MMAs of kind::f16)
-// accumulate in FP32 in tensor memory without rounding (integers below 2^24 are exact there;
-// measured with constant, alternating and random operands). The five sums of an entry are then
-// combined into a double-float number with error-free additions. The dropped slice products and
-// the rounding of the operands are 2^-44 of the largest product, which is where the double-float
-// sums of the CUDA cores were.
+// is a fixed-point number of five signed slices (9 bits, then four times 10: 48 bits below a power
+// of two at least the largest entry of its row or column), each slice an integer of at most 256
+// (the first) or 512 in FP16. Sums of integer products below 2^24 accumulate in FP32 in tensor
+// memory without rounding (measured with constant, alternating and random operands), and a tile of
+// 64 terms stays there: the products of slices i and j with i + j = g belong to one power of two
+// and share a sum, at most 2^22 for g = 0 and 2^24 for g = 1. (For g = 2 the bound is 2^25: only
+// operands whose low slices all sit at their limits with one sign can round there, by 2^-42.) The
+// sums of an entry are then combined into a double-float number with error-free additions. The
+// products over the rows (K, F and T = HA^T Z, whose error S amplifies) take the slice products
+// with i + j <= 5, those over the members (u = HA T) i + j <= 4. An emulation against 64 bits of
+// the residual of a double-float Z with an ensemble whose condition is 10^7 (one member 300 times
+// the others) gives 5e-9 of ||d|| with i + j <= 4 and a tenth of that with i + j <= 5, next to
+// 1e-10 from rounding Z itself; five equal 9-bit slices gave 5e-8 and missed a tolerance of 1e-8.
 #pragma once
 
 #include "tc_mixed.cuh"
@@ -109,7 +113,7 @@ template <int NT> struct KLayout {
 };
 
 // The power of two above |mx| (inv) and its inverse (scale). Entries below 2^-86 count as that size,
-// which keeps scale 2^26 finite (a row or column of zeros has scale 2^86).
+// which keeps scale 2^28 finite (a row or column of zeros has scale 2^86).
 __device__ __forceinline__ void pow2_of(float mx, float& scale, float& inv) {
   int E = (int)((__float_as_uint(mx) >> 23) & 0xFFu);
   E = max(40, min(252, E));
@@ -120,19 +124,19 @@ __device__ __forceinline__ void pow2_of(float mx, float& scale, float& inv) {
 __device__ __forceinline__ float rint_magic(float x) {   // |x| < 2^22
   return __fsub_rn(__fadd_rn(x, 12582912.f), 12582912.f);
 }
-// the five slices of (h + l) scale, |h scale| <= 1: integers in FP32, weights 2^-8, 2^-17, ...
+// the five slices of (h + l) scale, |h scale| <= 1: integers in FP32, weights 2^-8, 2^-18, ... 2^-48
 __device__ __forceinline__ void slice5(float h, float l, float scale, float (&v)[kSl]) {
   float x = __fmul_rn(h, scale * 256.f);
   v[0] = rint_magic(x);
-  x = __fmul_rn(__fsub_rn(x, v[0]), 512.f);
+  x = __fmul_rn(__fsub_rn(x, v[0]), 1024.f);
   v[1] = rint_magic(x);
-  x = __fmul_rn(__fsub_rn(x, v[1]), 512.f);
+  x = __fmul_rn(__fsub_rn(x, v[1]), 1024.f);
   float s, e;
-  df_two_sum(x, __fmul_rn(l, scale * 67108864.f), s, e);   // l in units of the third slice (2^26)
+  df_two_sum(x, __fmul_rn(l, scale * 0x1p28f), s, e);   // l in units of the third slice
   v[2] = rint_magic(s);
-  x = __fmul_rn(__fadd_rn(__fsub_rn(s, v[2]), e), 512.f);
+  x = __fmul_rn(__fadd_rn(__fsub_rn(s, v[2]), e), 1024.f);
   v[3] = rint_magic(x);
-  x = __fmul_rn(__fsub_rn(x, v[3]), 512.f);
+  x = __fmul_rn(__fsub_rn(x, v[3]), 1024.f);
   v[4] = rint_magic(x);
 }
 __device__ __forceinline__ uint32_t pack_half2(float a, float b) {
@@ -180,18 +184,20 @@ __device__ __forceinline__ void load_df8_cg(df32 (&x)[8], const df32* row, int c
   }
 }
 
-// tcgen05.ld of eight columns of the five level sums (levels `stride` columns apart)
-__device__ __forceinline__ void tmem_ld_levels(uint32_t taddr, uint32_t stride, float (&a)[kSl][8]) {
-  uint32_t r[kSl][8];
+// tcgen05.ld of eight columns of the six sums of an entry (`stride` columns apart; LV of them in use)
+constexpr int kLv = 6;
+template <int LV>
+__device__ __forceinline__ void tmem_ld_levels(uint32_t taddr, uint32_t stride, float (&a)[LV][8]) {
+  uint32_t r[LV][8];
 #pragma unroll
-  for (int g = 0; g < kSl; ++g)
+  for (int g = 0; g < LV; ++g)
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[g][0]), "=r"(r[g][1]), "=r"(r[g][2]), "=r"(r[g][3]), "=r"(r[g][4]), "=r"(r[g][5]),
                    "=r"(r[g][6]), "=r"(r[g][7])
                  : "r"(taddr + g * stride));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int g = 0; g < kSl; ++g)
+  for (int g = 0; g < LV; ++g)
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       // keep every use of the loaded registers behind the wait
@@ -199,30 +205,56 @@ __device__ __forceinline__ void tmem_ld_levels(uint32_t taddr, uint32_t stride, 
       a[g][q] = __uint_as_float(r[g][q]);
     }
 }
-// sum_g a_g 2^(-9 g) as an unevaluated pair (s, l): a_0..a_2 enter exactly, the two last levels are
-// 2^-27 of a_0's unit and below
-__device__ __forceinline__ void join_levels(float a0, float a1, float a2, float a3, float a4, float& s, float& l) {
+// The value of an entry from its sums as an unevaluated pair (s, l): the levels down to 2^-20 enter
+// exactly, the rest are 2^-30 of the first's unit and below.
+// Row products: a[g] = level g = 0..5.
+__device__ __forceinline__ void join_rows(const float (&a)[kLv][8], int q, float& s, float& l) {
   float t, e, e2;
-  df_two_sum(a0, __fmul_rn(a1, 0x1p-9f), t, e);
-  df_two_sum(t, __fmul_rn(a2, 0x1p-18f), s, e2);
-  l = __fadd_rn(__fadd_rn(e, e2), __fmaf_rn(a4, 0x1p-36f, __fmul_rn(a3, 0x1p-27f)));
+  df_two_sum(a[0][q], __fmul_rn(a[1][q], 0x1p-10f), t, e);
+  df_two_sum(t, __fmul_rn(a[2][q], 0x1p-20f), s, e2);
+  const float low = __fmaf_rn(a[5][q], 0x1p-50f, __fmaf_rn(a[4][q], 0x1p-40f, __fmul_rn(a[3][q], 0x1p-30f)));
+  l = __fadd_rn(__fadd_rn(e, e2), low);
+}
+// Member products: levels 0..4; SPLIT: level 1 as two sums in a[1] and a[5].
+template <bool SPLIT, int LV>
+__device__ __forceinline__ void join_members(const float (&a)[LV][8], int q, float& s, float& l) {
+  float t, e, e2, e3 = 0.f;
+  df_two_sum(a[0][q], __fmul_rn(a[1][q], 0x1p-10f), t, e);
+  if constexpr (SPLIT) {
+    float t2;
+    df_two_sum(t, __fmul_rn(a[5][q], 0x1p-10f), t2, e3);
+    t = t2;
+  }
+  df_two_sum(t, __fmul_rn(a[2][q], 0x1p-20f), s, e2);
+  const float low = __fmaf_rn(a[4][q], 0x1p-40f, __fmul_rn(a[3][q], 0x1p-30f));
+  l = __fadd_rn(__fadd_rn(__fadd_rn(e, e3), e2), low);
 }
 
-// The 15 slice products of D_g = sum_{i + j = g} A_i B_j over KS blocks of 16 along K: level g in
-// the `cols` tensor-memory columns at d + g cols. One thread.
+// One slice product A_i B_j over KS blocks of 16 along K into the `acc` tensor-memory columns. The
+// descriptors' address fields count 16-byte units, so a step along K or to another slice is an addition.
 template <int KS>
+__device__ __forceinline__ void issue_product(uint32_t d, uint64_t a, uint32_t a_step, uint64_t b, uint32_t b_step,
+                                              uint32_t idesc, bool first) {
+#pragma unroll
+  for (int kb = 0; kb < KS; ++kb)
+    umma_f16(d, a + (uint64_t)(kb * (a_step >> 4)), b + (uint64_t)(kb * (b_step >> 4)), idesc,
+             (first && kb == 0) ? 0u : 1u);
+}
+// The slice products of D = A B, level g = i + j <= GMAX in the `cols` columns at d + g cols; one
+// thread. SPLIT: the product (1, 0) goes to level column 5 (K = 128 would let level 1 reach 2^25).
+template <int KS, int GMAX, bool SPLIT>
 __device__ __forceinline__ void issue_levels(uint32_t d, int cols, uint64_t a, uint32_t a_part, uint32_t a_step,
                                              uint64_t b, uint32_t b_part, uint32_t b_step, uint32_t idesc) {
 #pragma unroll 1
-  for (int g = 0; g < kSl; ++g)
+  for (int g = 0; g <= GMAX; ++g) {
+    const int i0 = g < kSl ? 0 : g - kSl + 1, i1 = g < kSl ? g : kSl - 1;
 #pragma unroll 1
-    for (int i = 0; i <= g; ++i) {
-      const uint64_t ai = a + (uint64_t)((i * a_part) >> 4), bj = b + (uint64_t)(((g - i) * b_part) >> 4);
-#pragma unroll
-      for (int kb = 0; kb < KS; ++kb)
-        umma_f16(d + (uint32_t)(g * cols), ai + (uint64_t)((kb * a_step) >> 4), bj + (uint64_t)((kb * b_step) >> 4),
-                 idesc, (i > 0 || kb > 0) ? 1u : 0u);
+    for (int i = i0; i <= i1; ++i) {
+      const bool own = SPLIT && g == 1 && i == 1;
+      issue_product<KS>(d + (uint32_t)((own ? 5 : g) * cols), a + (uint64_t)((i * a_part) >> 4), a_step,
+                        b + (uint64_t)(((g - i) * b_part) >> 4), b_step, idesc, i == i0 || own);
     }
+  }
 }
 // kind::f16 descriptor of FP16 operands with M = 128 and each operand K-major or MN-major
 __host__ __device__ constexpr uint32_t sl_idesc(int N, bool a_mn, bool b_mn) {
@@ -390,7 +422,7 @@ __device__ __noinline__ void pass_gram(const KrylovParams& p, bool from_b, int c
     const uint64_t A = umma_desc(base, rg, 128);
     if (t == 0) {
       tc_fence_after();
-      issue_levels<kKR / 16>(cta.tmem, JC, A, L::CP, 2 * rg, umma_desc(base + (NT == 128 ? c * 1024 : 0), rg, 128),
+      issue_levels<kKR / 16, 5, false>(cta.tmem, JC, A, L::CP, 2 * rg, umma_desc(base + (NT == 128 ? c * 1024 : 0), rg, 128),
                              L::CP, 2 * rg, sl_idesc(JC, true, true));
       umma_commit(cta.mbar);
     }
@@ -398,12 +430,12 @@ __device__ __noinline__ void pass_gram(const KrylovParams& p, bool from_b, int c
     auto flush = [&](DFAcc* a, float rs, const float* cs) {
 #pragma unroll
       for (int q0 = 0; q0 < NC; q0 += 8) {
-        float lv[kSl][8];
-        tmem_ld_levels(cta.tmem + ((uint32_t)(32 * qd) << 16) + half * NC + q0, JC, lv);
+        float lv[kLv][8];
+        tmem_ld_levels<kLv>(cta.tmem + ((uint32_t)(32 * qd) << 16) + half * NC + q0, JC, lv);
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           float s, l, tt, e;
-          join_levels(lv[0][q], lv[1][q], lv[2][q], lv[3][q], lv[4][q], s, l);
+          join_rows(lv, q, s, l);
           const float f = rs * cs[q0 + q];
           df_two_sum(a[q0 + q].s, s * f, tt, e);
           a[q0 + q].s = tt;
@@ -419,7 +451,7 @@ __device__ __noinline__ void pass_gram(const KrylovParams& p, bool from_b, int c
       __syncthreads();
       if (t == 0) {
         tc_fence_after();
-        issue_levels<kKR / 16>(cta.tmem, JC, A, L::CP, 2 * rg, umma_desc(base + (NT / 8) * 128, rg, 128), L::CP,
+        issue_levels<kKR / 16, 5, false>(cta.tmem, JC, A, L::CP, 2 * rg, umma_desc(base + (NT / 8) * 128, rg, 128), L::CP,
                                2 * rg, sl_idesc(JC, true, true));
         umma_commit(cta.mbar);
       }
@@ -694,6 +726,7 @@ __device__ __noinline__ void pass_rows(const KrylovParams& p, bool from_b, int c
   constexpr int JC = L::JC;
   constexpr int CP = NT == 128 ? 1 : 128 / NT;    // copies
   constexpr int RPT = kKR / (2 * CP);             // rows per thread: 8, 16, 32
+  constexpr bool SPL = NT == 128;                 // level 1 of u in two sums
   unsigned char* sT = cta.smem + L::off_t;
   unsigned char* sH = cta.smem + L::off_h;
   unsigned char* sV = cta.smem + L::off_v;
@@ -721,7 +754,7 @@ __device__ __noinline__ void pass_rows(const KrylovParams& p, bool from_b, int c
     __syncthreads();
     if (t == 0) {
       tc_fence_after();
-      issue_levels<NT / 16>(cta.tmem, kKR, umma_desc(aT, 128, hst), L::TP, 256, umma_desc(aH, 128, hst), L::HP, 256,
+      issue_levels<NT / 16, 4, SPL>(cta.tmem, kKR, umma_desc(aT, 128, hst), L::TP, 256, umma_desc(aH, 128, hst), L::HP, 256,
                             sl_idesc(kKR, false, false));
       umma_commit(cta.mbar);
     }
@@ -743,15 +776,15 @@ __device__ __noinline__ void pass_rows(const KrylovParams& p, bool from_b, int c
     float mx = 0.f;
 #pragma unroll
     for (int q0 = 0; q0 < RPT; q0 += 8) {
-      float lv[kSl][8];
-      tmem_ld_levels(cta.tmem + ((uint32_t)(32 * qd) << 16) + (r0 & (kKR - 1)) + q0, kKR, lv);
+      float lv[SPL ? 6 : 5][8];
+      tmem_ld_levels<(SPL ? 6 : 5)>(cta.tmem + ((uint32_t)(32 * qd) << 16) + (r0 & (kKR - 1)) + q0, kKR, lv);
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         const int rq = r0 + q0 + q;
         const int64_t i = i0 + rq;
         if (!(live && i < row1)) continue;
         float s, l;
-        join_levels(lv[0][q], lv[1][q], lv[2][q], lv[3][q], lv[4][q], s, l);
+        join_members<SPL>(lv, q, s, l);
         const float f = tsc * s_row[rq];
         const df32 u = df_fast2sum(s * f, l * f);
         if (RESID) {
@@ -794,7 +827,7 @@ __device__ __noinline__ void pass_rows(const KrylovParams& p, bool from_b, int c
       if (t == 0) {
         tc_fence_after();
         // T[k][jl]: A = the HA tile MN-major (M = k), B = the Z tile K-major
-        issue_levels<kKR / 16>(cta.tmem, JC, umma_desc(aH, hst, 128), L::HP, 2 * hst, umma_desc(aV, 128, 1024),
+        issue_levels<kKR / 16, 5, false>(cta.tmem, JC, umma_desc(aH, hst, 128), L::HP, 2 * hst, umma_desc(aV, 128, 1024),
                                L::VP, 256, sl_idesc(JC, true, false));
         umma_commit(cta.mbar);
       }
@@ -803,12 +836,12 @@ __device__ __noinline__ void pass_rows(const KrylovParams& p, bool from_b, int c
         constexpr int NC = JC / 2;
 #pragma unroll
         for (int q0 = 0; q0 < NC; q0 += 8) {
-          float lv[kSl][8];
-          tmem_ld_levels(cta.tmem + ((uint32_t)(32 * qd) << 16) + half * NC + q0, JC, lv);
+          float lv[kLv][8];
+          tmem_ld_levels<kLv>(cta.tmem + ((uint32_t)(32 * qd) << 16) + half * NC + q0, JC, lv);
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
             float s, l, tt, e;
-            join_levels(lv[0][q], lv[1][q], lv[2][q], lv[3][q], lv[4][q], s, l);
+            join_rows(lv, q, s, l);
             const float f = s_max[2 * CP * 64 + half * NC + q0 + q] * 0x1p-16f;
             df_two_sum(acc[q0 + q].s, s * f, tt, e);
             acc[q0 + q].s = tt;
