@@ -32,7 +32,7 @@ void free_workspace(Workspace& ws) {
                   ws.Res, ws.P, ws.Sv, ws.prof, ws.Tpart, ws.Tred, ws.rrpart, ws.Wacc, ws.W, ws.col_iters,
                   ws.col_relres, ws.col_true, ws.col_warm, ws.status, ws.bar, ws.stage_Xf, ws.stage_y,
                   ws.Hrowptr, ws.Hcol, ws.Hw, ws.wa, ws.wb, ws.wcp, ws.wmu, ws.wU, ws.wV, ws.wcarry,
-                  ws.wcarryV, ws.Xw, ws.yw, ws.Tk, ws.Tacc, ws.hamax, ws.rdf, ws.rinv, ws.rsq, ws.kpart, ws.ksmall};
+                  ws.wcarryV, ws.Xw, ws.yw, ws.Tk, ws.Tacc, ws.hamax, ws.rdf, ws.rinv, ws.rsq, ws.hs, ws.kpart, ws.ksmall};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   ws = Workspace{};
@@ -225,6 +225,8 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
     allocs.push_back({(void**)&ws.B, vs * mN});
     for (void** q : {&ws.HAdf, &ws.Ddf, &ws.Zdf}) allocs.push_back({q, 8 * (size_t)mN});
     for (void** q : {&ws.rdf, &ws.rinv, &ws.rsq}) allocs.push_back({q, 8 * (size_t)c.m});
+    allocs.push_back({(void**)&ws.hs, sizeof(float) * c.m});
+    allocs.push_back({(void**)&ws.hamax, sizeof(unsigned) * 4});
     allocs.push_back({&ws.kpart, enkf::krylov_part_bytes(h)});
     allocs.push_back({&ws.ksmall, 8 * ((size_t)4 * c.N * c.N + 2 * c.N)});
   }
@@ -525,7 +527,7 @@ enkf_status enkf_get_stats(enkf_handle h, enkf_stats* out) {
     for (int j = 0; j < N; ++j) out->warm_relres_max = std::max(out->warm_relres_max, wr[j]);
     out->warm_fallbacks = st[2];
   }
-  out->grid_blocks = h->launch.G;
+  out->grid_blocks = h->small_c ? h->cfg.N * h->small_c : h->launch.G;
   enkf_status status = ENKF_OK;
   if (bits & enkf::DS_SMEM) status = ENKF_ERR_CUDA;
   else if (bits & enkf::DS_TIMEOUT) status = ENKF_ERR_TIMEOUT;

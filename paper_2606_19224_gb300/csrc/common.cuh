@@ -151,11 +151,13 @@ struct Workspace {
   unsigned long long* prof = nullptr;  // [8] in-kernel phase timers of the solve (ns)
   float* Tk = nullptr;          // [2][N][N] T of the tensor-core step, carried between steps
   double* Tacc = nullptr;       // [3][N N + 4 N] step sums of the tensor-core solve (atomic adds)
-  unsigned* hamax = nullptr;    // tensor-core modes: largest |HA| of the analysis (float bits)
+  unsigned* hamax = nullptr;    // tensor-core modes: largest |HA| of the analysis (float bits);
+                                // in Krylov coordinates: largest |HA_ik| / sqrt(r_i)
   // the preconditioned solve in Krylov coordinates (krylov.cuh)
   void* rdf = nullptr;          // [m] R, 1/R and 1/sqrt(R) in double-float
   void* rinv = nullptr;
   void* rsq = nullptr;
+  float* hs = nullptr;          // [m] a power of two above each row's largest |HA|
   void* kpart = nullptr;        // [G][2 N JC + 128] double-float partial products
   void* ksmall = nullptr;       // four N x N matrices, two N-vectors (double-float)
   // tridiagonal R (kernels_whiten.cu): the caller's H, the whitening scan's coefficients and
@@ -207,6 +209,7 @@ struct enkf_handle_s {
   enkf::BatchState* batch = nullptr;   // non-NULL for a handle made by enkf_batch_create
   enkf::WarmState* warm = nullptr;     // learned warm start (enkf_set_warm_model / enkf_warm_features)
   bool krylov = false;                 // the solve runs in Krylov coordinates (kernels_krylov.cu)
+  int small_c = 0;                     // > 0: CTAs per column of the small-problem solve (kernels_small.cu)
   bool tri = false;                    // tridiagonal R: analyses run on the whitened problem
   float r_pow2 = 1.f;                  // power of two nearest the geometric mean of R's diagonal
                                        // (1 for the whitened problem)
@@ -223,6 +226,10 @@ cudaError_t launch_convert_r(enkf_handle_s* h);
 cudaError_t plan_solve_mixed(enkf_handle_s* h);
 cudaError_t launch_solve_mixed(enkf_handle_s* h);
 size_t mixed_image_bytes(const enkf_handle_s* h);   // tile images of HA (zeroed at create)
+// kernels_small.cu: one cluster of CTAs per column (0: not for this problem)
+int small_cluster(const enkf_config& c, int sms);
+cudaError_t plan_small(enkf_handle_s* h);
+cudaError_t launch_small(enkf_handle_s* h);
 // kernels_krylov.cu: CG preconditioned by R in the coordinates of its Krylov space
 bool krylov_config(const enkf_config& c);
 cudaError_t plan_krylov(enkf_handle_s* h);

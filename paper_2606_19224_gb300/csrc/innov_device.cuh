@@ -196,6 +196,15 @@ __device__ __forceinline__ void innov_rows_f64(
   }
 }
 
+// What a solve in Krylov coordinates takes from the innovations besides HA and D (FP32 modes): a power
+// of two above the largest |HA| of each row, and the largest |HA_ik| / sqrt(r_i) of the problem
+// (atomic maximum of the float bits).
+struct InnovRows {
+  float* scale = nullptr;
+  const df32* rsq = nullptr;
+  unsigned* umax = nullptr;
+};
+
 // The same rows for FP32 ensembles (the FP32 and tensor-core modes), in double-float (FP32
 // pair) arithmetic: this part issues FP32 at 64x its FP64 rate, and the FP64 version spends
 // its time in FP64 adds and FP32<->FP64 conversions. z = sum w_k x_k accumulates exact
@@ -213,10 +222,11 @@ __device__ __forceinline__ void innov_rows_df(
     double* __restrict__ HA64, float* __restrict__ HA32, double* __restrict__ D,
     float* __restrict__ B32, __nv_bfloat16* __restrict__ HAb, __half* __restrict__ HAh,
     int split_lo, df32* __restrict__ HAdf, df32* __restrict__ Ddf, int64_t i_begin, int64_t i_end,
-    int64_t warp, int64_t nwarps, unsigned* hamax = nullptr) {
+    int64_t warp, int64_t nwarps, unsigned* hamax = nullptr, const InnovRows kr = InnovRows{}) {
   static_assert(sizeof(VT) == 4, "double-float innovations take an FP32 ensemble");
   const int lane = threadIdx.x & 31;
   float hmax = 0.f;   // largest |HA| of the warp's rows (hamax: atomic maximum of the float bits)
+  float umax = 0.f;   // largest |HA| / sqrt(r) of the warp's rows
   const df32 inv_n(1.0 / (double)N);
   const bool wide = N > 64;   // members 64..127 present (warp-uniform)
   // The warp's rows are i0 + q nwarps, q = 0, 1, ...; the per-row values that come from FP64
@@ -255,6 +265,17 @@ __device__ __forceinline__ void innov_rows_df(
       for (int o = 16; o > 0; o >>= 1)
         s = s + df32(__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o));
       const df32 zbar = s * inv_n;
+      if (kr.scale) {
+        float rm = 0.f;
+  #pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (2 * lane + (q & 1) + 64 * (q >> 1) < N) rm = fmaxf(rm, fabsf((z[q] - zbar).hi));
+        rm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(rm)));
+        umax = fmaxf(umax, rm * kr.rsq[i].hi);
+        // the exponent field of the power of two above rm (bounded away from both ends of the range)
+        const int E = max(40, min(252, (int)(__float_as_uint(rm) >> 23)));
+        if (lane == 0) kr.scale[i] = __uint_as_float((uint32_t)(E + 1) << 23);
+      }
   #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int jp = 2 * lane + 64 * h;   // even member of the pair
@@ -313,6 +334,7 @@ __device__ __forceinline__ void innov_rows_df(
       }
     }
   }
+  if (kr.umax && lane == 0 && umax > 0.f) atomicMax(kr.umax, __float_as_uint(umax));
   if (hamax) {
     // non-negative floats order as their bit patterns
     const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(hmax));
@@ -330,10 +352,10 @@ __device__ __forceinline__ void innov_rows(
     double* __restrict__ HA64, float* __restrict__ HA32, double* __restrict__ D,
     float* __restrict__ B32, __nv_bfloat16* __restrict__ HAb, __half* __restrict__ HAh,
     int split_lo, df32* __restrict__ HAdf, df32* __restrict__ Ddf, int64_t i_begin, int64_t i_end,
-    int64_t warp, int64_t nwarps, unsigned* hamax = nullptr) {
+    int64_t warp, int64_t nwarps, unsigned* hamax = nullptr, const InnovRows kr = InnovRows{}) {
   if constexpr (sizeof(VT) == 4)
     innov_rows_df<VT>(Xf, rowptr, col, w, y, r, E, emode, seed, counter, m, N, HA64, HA32, D, B32,
-                      HAb, HAh, split_lo, HAdf, Ddf, i_begin, i_end, warp, nwarps, hamax);
+                      HAb, HAh, split_lo, HAdf, Ddf, i_begin, i_end, warp, nwarps, hamax, kr);
   else
     innov_rows_f64<VT>(Xf, rowptr, col, w, y, r, E, emode, seed, counter, m, N, HA64, HA32, D, B32,
                        HAb, HAh, split_lo, HAdf, Ddf, i_begin, i_end, warp, nwarps);

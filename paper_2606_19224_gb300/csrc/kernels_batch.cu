@@ -64,7 +64,7 @@ __device__ __noinline__ void batch_solve(const KrylovParams& sp, int G, int rank
 template <int NT>
 __device__ __noinline__ void batch_update(const BatchIO& io, const double* W, int64_t n, int N,
                                           int rank, int G, unsigned char* smem) {
-  update_rows<float, NT, 0>(io.Xf, io.Xa, W, n, N, rank, G, smem);
+  update_rows<float, NT, 0, kKT>(io.Xf, io.Xa, W, n, N, rank, G, smem);
 }
 
 // NTMAX bounds the column tile of every problem in the batch. One CTA per SM (it holds the
@@ -72,7 +72,7 @@ __device__ __noinline__ void batch_update(const BatchIO& io, const double* W, in
 // (order[team_first[team] .. team_first[team + 1])), then takes problems one at a time from
 // the shared queue order[queue_first .. count) (longest first) and solves each alone.
 template <int NTMAX>
-__global__ void __launch_bounds__(kThreads, 1) batch_kernel(
+__global__ void __launch_bounds__(kKT, 1) batch_kernel(
     const BatchProblem* __restrict__ probs, const BatchIO* __restrict__ io,
     const int* __restrict__ cta_team, const int* __restrict__ cta_rank,
     const int* __restrict__ team_size, const int* __restrict__ team_first,
@@ -128,7 +128,8 @@ __global__ void __launch_bounds__(kThreads, 1) batch_kernel(
     innov_rows<float>(s_io.Xf, probs[pi].rowptr, probs[pi].col, probs[pi].w, s_io.y, probs[pi].r, nullptr,
                       perturb ? 2 : 0, s_io.seed, s_io.counter, sp.m, sp.N, nullptr, nullptr, nullptr, nullptr,
                       nullptr, nullptr, 0, const_cast<df32*>(sp.HAdf),
-                      const_cast<df32*>(sp.Ddf), r0, r1, warp, kThreads / 32);
+                      const_cast<df32*>(sp.Ddf), r0, r1, warp, kKT / 32, nullptr,
+                      InnovRows{const_cast<float*>(sp.hs), sp.rsq, const_cast<unsigned*>(sp.umax)});
     bool ok = bar.sync();
     if (ok) {
       if (NT == 32) batch_solve<32>(sp, G, rank, bar, cta);
@@ -375,7 +376,7 @@ bool batch_plan_host(int count, const enkf_config* cfgs, int max_grid, double al
 // column tile it may run.
 template <int NT>
 static size_t tile_smem() {
-  return std::max<size_t>(KLayout<NT>::bytes, update_smem_bytes<float, NT>());
+  return std::max<size_t>(KLayout<NT>::bytes, update_smem_bytes<float, NT, kKT>());
 }
 template <int NTMAX>
 static size_t batch_smem_nt() {
@@ -432,7 +433,7 @@ static cudaError_t enqueue_batch(BatchState& B, cudaStream_t s) {
   df32* team_buf = B.d_team;
   void* args[] = {&probs, &io, &cta_team, &cta_rank, &team_size, &team_first, &order, &queue_first, &count,
                   &queue_head, &team_buf, &part_max, &n_max, &perturb, &times};
-  return cudaLaunchCooperativeKernel(batch_fn(B.ntmax), dim3(P.grid), dim3(kThreads), args,
+  return cudaLaunchCooperativeKernel(batch_fn(B.ntmax), dim3(P.grid), dim3(kKT), args,
                                      B.smem, s);
 }
 
@@ -504,13 +505,13 @@ cudaError_t batch_build(enkf_handle_s* h, int count, const enkf_config* cfgs,
   void* fn = batch_fn(B.ntmax);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B.smem);
   int occ = 0;
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kThreads, B.smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kKT, B.smem);
   if (e != cudaSuccess) { err = "enkf_batch_create: occupancy query"; return e; }
   if (occ < 1) { err = "enkf_batch_create: kernel does not fit on an SM"; return cudaErrorInvalidConfiguration; }
   B.max_grid = occ * h->sms;
   if (h->cfg.grid_blocks > 0) B.max_grid = std::min(B.max_grid, h->cfg.grid_blocks);
   // one arena: per problem HA, D and Z in double-float, B, R (FP64), R, 1/R and 1/sqrt(R) in
-  // double-float, rowptr, col, w, W, column iterations / residuals
+  // double-float, rowptr, col, w, W, column iterations / residuals, row scales of HA
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   std::vector<std::vector<size_t>> parts(count);
   std::vector<size_t> off(count + 1, 0);
@@ -519,7 +520,7 @@ cudaError_t batch_build(enkf_handle_s* h, int count, const enkf_config* cfgs,
     const size_t mN = (size_t)c.m * c.N, m = (size_t)c.m, N = (size_t)c.N;
     const size_t nnz = (size_t)std::max(1, rowptr[i][c.m]);
     parts[i] = {8 * mN, 8 * mN, 8 * mN, 4 * mN, 8 * m, 8 * m, 8 * m, 8 * m,
-                4 * (m + 1), 4 * nnz, 8 * nnz, 8 * N * N, 4 * N, 8 * N, 8 * N};
+                4 * (m + 1), 4 * nnz, 8 * nnz, 8 * N * N, 4 * N, 8 * N, 8 * N, 4 * m};
     size_t sz = 0;
     for (size_t b : parts[i]) sz += al(b);
     off[i + 1] = off[i] + sz;
@@ -555,6 +556,8 @@ cudaError_t batch_build(enkf_handle_s* h, int count, const enkf_config* cfgs,
     sp.rdf = static_cast<const df32*>(ptr[5]);
     sp.rinv = static_cast<const df32*>(ptr[6]);
     sp.rsq = static_cast<const df32*>(ptr[7]);
+    sp.hs = static_cast<const float*>(ptr[15]);
+    sp.umax = B.d_bar + 4 * i + 2;   // zeroed with the barrier words before each launch
     sp.W = static_cast<double*>(ptr[11]);
     sp.col_iters = static_cast<int*>(ptr[12]);
     sp.col_relres = static_cast<double*>(ptr[13]);

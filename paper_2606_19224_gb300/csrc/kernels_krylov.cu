@@ -7,7 +7,7 @@
 namespace enkf {
 
 template <int NT>
-__global__ void __launch_bounds__(kThreads, 1) krylov_kernel(KrylovParams p) {
+__global__ void __launch_bounds__(kKT, 1) krylov_kernel(KrylovParams p) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tmem_slot;
@@ -56,7 +56,7 @@ cudaError_t plan_krylov(enkf_handle_s* h) {
   cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   int occ = 0;
-  err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kThreads, smem);
+  err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kKT, smem);
   if (err != cudaSuccess) return err;
   if (occ < 1) return cudaErrorInvalidConfiguration;
   // one CTA per SM (it holds the SM's tensor memory), and no more than have a tile of rows (times
@@ -94,6 +94,8 @@ cudaError_t launch_krylov(enkf_handle_s* h, int phase, const float* w0, const do
   p.rdf = static_cast<const df32*>(ws.rdf);
   p.rinv = static_cast<const df32*>(ws.rinv);
   p.rsq = static_cast<const df32*>(ws.rsq);
+  p.hs = ws.hs;
+  p.umax = ws.hamax;
   df32* q = static_cast<df32*>(ws.kpart);
   p.part = q;
   q = static_cast<df32*>(ws.ksmall);   // four N x N matrices and two N-vectors
@@ -124,7 +126,7 @@ cudaError_t launch_krylov(enkf_handle_s* h, int phase, const float* w0, const do
   if (err == cudaSuccess && phase != 2) err = cudaMemsetAsync(ws.status, 0, 4 * sizeof(int32_t), h->stream);
   if (err != cudaSuccess) return err;
   void* args[] = {&p};
-  return cudaLaunchCooperativeKernel(krylov_fn(h->launch.NT), dim3(h->launch.G), dim3(kThreads), args,
+  return cudaLaunchCooperativeKernel(krylov_fn(h->launch.NT), dim3(h->launch.G), dim3(kKT), args,
                                      h->launch.smem, h->stream);
 }
 

@@ -43,6 +43,8 @@ namespace enkf {
 
 constexpr int kSl = 5;       // slices per operand
 constexpr int kKR = 64;      // observation rows per tile
+constexpr int kKT = 512;     // threads per CTA: four warps per scheduler hide the latency of the slicing
+                             // and joining chains (256 threads spent 5 of 8 cycles waiting)
 
 struct KrylovParams {
   int64_t m;
@@ -54,6 +56,8 @@ struct KrylovParams {
   const df32* rdf;      // [m] R, 1/R and 1/sqrt(R) in double-float
   const df32* rinv;
   const df32* rsq;
+  const float* hs;      // [m] a power of two above the largest |HA| of each row
+  const unsigned* umax; // largest |HA_ik| / sqrt(r_i) (float bits)
   df32* part;           // [G][krylov_part(N)] partial products and column sums of the CTAs
   df32* Kred;           // [N][N]
   df32* Fred;           // [N][N] F^T: row j is column j of F
@@ -86,27 +90,35 @@ __host__ __device__ constexpr int krylov_part(int N) { return 2 * N * (N < 64 ? 
 
 template <int NT> struct KLayout {
   static constexpr int JC = NT < 64 ? NT : 64;       // columns j of one CTA
-  static constexpr int CW = NT == 128 ? 192 : 128;    // pass G image: [U | V] columns
+  static constexpr int BR = kSl * JC * 16;            // pass G, operand B: bytes per row group (all slices)
   static constexpr int TROWS = NT == 128 ? 64 : 128;  // rows of the T operand (copies of its JC columns for NT <= 64)
+  static constexpr int NB = NT == 128 ? 1 : 2;        // HA images: the next tile is sliced behind the products
   static constexpr int HP = kKR * NT * 2;             // bytes per slice of the HA tile
-  static constexpr int CP = kKR * CW * 2;             // ... of the pass G image
+  static constexpr int CP = kKR * 128 * 2;            // ... of the pass G operand A
   static constexpr int TP = TROWS * NT * 2;           // ... of the T operand
   static constexpr int VP = JC * kKR * 2;             // ... of the Z tile (rows j, K-major over i)
   static constexpr int off_t = 0;
   static constexpr int off_h = kSl * TP;
-  static constexpr int off_v = off_h + kSl * HP;
+  static constexpr int off_v = off_h + NB * kSl * HP;
   // (an M = 128 operand of fewer rows or columns reads on into the next region: rows that no
   // result uses)
   static constexpr int end_z = off_v + kSl * VP;
-  static constexpr int end_g = kSl * CP;
-  static constexpr int uni = end_z > end_g ? end_z : end_g;
-  // scalars: six FP64 and two int arrays of NT, row and column scales, column maxima, scratch
+  static constexpr int off_gu = kSl * CP;             // pass G operands B: slices of U, then (NT = 128) of V
+  static constexpr int off_gv = off_gu + 8 * BR;
+  static constexpr int SQ = 24;                       // column sums of squares, floats per thread
+  static constexpr int off_sq = off_gv + (NT == 128 ? 8 * BR : 0);
+  static constexpr int end_g = off_sq + SQ * 4 * kKT;
+  static constexpr int end_cg = 16 * NT * 8 + 16 * kKT * 8 + 64;   // the recurrences of 16 columns
+  static constexpr int uni0 = end_z > end_g ? end_z : end_g;
+  static constexpr int uni = uni0 > end_cg ? uni0 : end_cg;
+  // scalars: six FP64 and two int arrays of NT; per tile buffer the rows' scales and r (or 1/r); the
+  // T operand's column scales; column maxima and scales of a tile; scratch
   static constexpr int off_scal = uni;
   static constexpr int off_row = off_scal + NT * (6 * 8 + 2 * 4);
-  static constexpr int off_col = off_row + 2 * 4 * kKR;
-  static constexpr int off_max = off_col + 4 * 256;
-  static constexpr int off_scr = off_max + 4 * 8 * 192;
-  static constexpr int need = off_scr + kThreads * 8;
+  static constexpr int off_col = off_row + 2 * 12 * kKR;
+  static constexpr int off_max = off_col + 4 * 128;
+  static constexpr int off_scr = off_max + 4 * (8 * 64 + 64);
+  static constexpr int need = off_scr + kKT * 8;
   // one CTA per SM whatever NT: each holds all of its SM's tensor memory
   static constexpr int bytes = need < 120 * 1024 ? 120 * 1024 : need;
   static_assert(bytes <= 226 * 1024, "shared memory");
@@ -121,85 +133,78 @@ __device__ __forceinline__ void pow2_of(float mx, float& scale, float& inv) {
   inv = __uint_as_float((uint32_t)(E + 1) << 23);
 }
 
-__device__ __forceinline__ float rint_magic(float x) {   // |x| < 2^22
-  return __fsub_rn(__fadd_rn(x, 12582912.f), 12582912.f);
-}
 // the five slices of (h + l) scale, |h scale| <= 1: integers in FP32, weights 2^-8, 2^-18, ... 2^-48
 __device__ __forceinline__ void slice5(float h, float l, float scale, float (&v)[kSl]) {
-  float x = __fmul_rn(h, scale * 256.f);
-  v[0] = rint_magic(x);
-  x = __fmul_rn(__fsub_rn(x, v[0]), 1024.f);
-  v[1] = rint_magic(x);
-  x = __fmul_rn(__fsub_rn(x, v[1]), 1024.f);
+  constexpr float M = 12582912.f;   // adding and subtracting it rounds to an integer (|x| < 2^22)
+  const float x = __fmul_rn(h, scale * 256.f);
+  v[0] = __fsub_rn(__fadd_rn(x, M), M);
+  const float d0 = __fsub_rn(x, v[0]);
+  v[1] = __fsub_rn(__fmaf_rn(d0, 1024.f, M), M);
+  const float d1 = __fmaf_rn(d0, 1024.f, -v[1]);
   float s, e;
-  df_two_sum(x, __fmul_rn(l, scale * 0x1p28f), s, e);   // l in units of the third slice
-  v[2] = rint_magic(s);
-  x = __fmul_rn(__fadd_rn(__fsub_rn(s, v[2]), e), 1024.f);
-  v[3] = rint_magic(x);
-  x = __fmul_rn(__fsub_rn(x, v[3]), 1024.f);
-  v[4] = rint_magic(x);
+  df_two_sum(__fmul_rn(d1, 1024.f), __fmul_rn(l, scale * 0x1p28f), s, e);   // l in units of the third slice
+  v[2] = __fsub_rn(__fadd_rn(s, M), M);
+  const float d2 = __fadd_rn(__fsub_rn(s, v[2]), e);
+  v[3] = __fsub_rn(__fmaf_rn(d2, 1024.f, M), M);
+  const float d3 = __fmaf_rn(d2, 1024.f, -v[3]);
+  v[4] = __fsub_rn(__fmaf_rn(d3, 1024.f, M), M);
 }
 __device__ __forceinline__ uint32_t pack_half2(float a, float b) {
   const __half2 h = __floats2half2_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 // eight consecutive elements along the 16-byte direction of a core row, each slice one store
-__device__ __forceinline__ void store_slices8(unsigned char* base, int part_bytes, int off, const df32 (&x)[8],
-                                              const float (&scale)[8]) {
-  uint32_t w[kSl][4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    float a[kSl], b[kSl];
-    slice5(x[2 * q].hi, x[2 * q].lo, scale[2 * q], a);
-    slice5(x[2 * q + 1].hi, x[2 * q + 1].lo, scale[2 * q + 1], b);
-#pragma unroll
-    for (int s = 0; s < kSl; ++s) w[s][q] = pack_half2(a[s], b[s]);
-  }
-#pragma unroll
-  for (int s = 0; s < kSl; ++s)
-    *reinterpret_cast<uint4*>(base + s * part_bytes + off) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
-}
-__device__ __forceinline__ void load_df8(df32 (&x)[8], const df32* row, int c0, int N, bool ok) {
-  if (ok && (N & 1) == 0 && c0 + 8 <= N) {
+struct Slices8 {
+  uint4 w[kSl];
+  __device__ __forceinline__ void make(const df32 (&x)[8], const float (&scale)[8]) {
+    uint32_t u[kSl][4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const float4 v = *reinterpret_cast<const float4*>(row + c0 + 2 * q);
-      x[2 * q] = df32(v.x, v.y);
-      x[2 * q + 1] = df32(v.z, v.w);
-    }
-  } else {
+      float a[kSl], b[kSl];
+      slice5(x[2 * q].hi, x[2 * q].lo, scale[2 * q], a);
+      slice5(x[2 * q + 1].hi, x[2 * q + 1].lo, scale[2 * q + 1], b);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) x[q] = (ok && c0 + q < N) ? row[c0 + q] : df32(0.f, 0.f);
-  }
-}
-// the same from data other CTAs of this launch wrote (read through L2)
-__device__ __forceinline__ void load_df8_cg(df32 (&x)[8], const df32* row, int c0, int N) {
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    x[q] = df32(0.f, 0.f);
-    if (c0 + q < N) {
-      const float2 v = __ldcg(reinterpret_cast<const float2*>(row + c0 + q));
-      x[q] = df32(v.x, v.y);
+      for (int s = 0; s < kSl; ++s) u[s][q] = pack_half2(a[s], b[s]);
     }
+#pragma unroll
+    for (int s = 0; s < kSl; ++s) w[s] = make_uint4(u[s][0], u[s][1], u[s][2], u[s][3]);
   }
+  __device__ __forceinline__ void make(const df32 (&x)[8], float scale) {
+    const float sc[8] = {scale, scale, scale, scale, scale, scale, scale, scale};
+    make(x, sc);
+  }
+  __device__ __forceinline__ void store(unsigned char* at, int slice_bytes) const {
+#pragma unroll
+    for (int s = 0; s < kSl; ++s) *reinterpret_cast<uint4*>(at + s * slice_bytes) = w[s];
+  }
+};
+
+__device__ __forceinline__ df32 ld_df(const df32* p) {   // through L2: other CTAs of this launch wrote it
+  const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
+  return df32(v.x, v.y);
 }
 
-// tcgen05.ld of eight columns of the six sums of an entry (`stride` columns apart; LV of them in use)
+// tcgen05.ld of LC columns of the six sums of an entry (`stride` columns apart; LV of them in use)
 constexpr int kLv = 6;
-template <int LV>
-__device__ __forceinline__ void tmem_ld_levels(uint32_t taddr, uint32_t stride, float (&a)[LV][8]) {
-  uint32_t r[LV][8];
+template <int LV, int LC>   // LC: 8 or 4 columns
+__device__ __forceinline__ void tmem_ld_levels(uint32_t taddr, uint32_t stride, float (&a)[LV][LC]) {
+  uint32_t r[LV][LC];
 #pragma unroll
-  for (int g = 0; g < LV; ++g)
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[g][0]), "=r"(r[g][1]), "=r"(r[g][2]), "=r"(r[g][3]), "=r"(r[g][4]), "=r"(r[g][5]),
-                   "=r"(r[g][6]), "=r"(r[g][7])
-                 : "r"(taddr + g * stride));
+  for (int g = 0; g < LV; ++g) {
+    if constexpr (LC == 8)
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                   : "=r"(r[g][0]), "=r"(r[g][1]), "=r"(r[g][2]), "=r"(r[g][3]), "=r"(r[g][4]), "=r"(r[g][5]),
+                     "=r"(r[g][6]), "=r"(r[g][7])
+                   : "r"(taddr + g * stride));
+    else
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                   : "=r"(r[g][0]), "=r"(r[g][1]), "=r"(r[g][2]), "=r"(r[g][3]) : "r"(taddr + g * stride));
+  }
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int g = 0; g < LV; ++g)
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < LC; ++q) {
       // keep every use of the loaded registers behind the wait
       asm volatile("" : "+r"(r[g][q]));
       a[g][q] = __uint_as_float(r[g][q]);
@@ -208,7 +213,8 @@ __device__ __forceinline__ void tmem_ld_levels(uint32_t taddr, uint32_t stride, 
 // The value of an entry from its sums as an unevaluated pair (s, l): the levels down to 2^-20 enter
 // exactly, the rest are 2^-30 of the first's unit and below.
 // Row products: a[g] = level g = 0..5.
-__device__ __forceinline__ void join_rows(const float (&a)[kLv][8], int q, float& s, float& l) {
+template <int LC>
+__device__ __forceinline__ void join_rows(const float (&a)[kLv][LC], int q, float& s, float& l) {
   float t, e, e2;
   df_two_sum(a[0][q], __fmul_rn(a[1][q], 0x1p-10f), t, e);
   df_two_sum(t, __fmul_rn(a[2][q], 0x1p-20f), s, e2);
@@ -216,8 +222,8 @@ __device__ __forceinline__ void join_rows(const float (&a)[kLv][8], int q, float
   l = __fadd_rn(__fadd_rn(e, e2), low);
 }
 // Member products: levels 0..4; SPLIT: level 1 as two sums in a[1] and a[5].
-template <bool SPLIT, int LV>
-__device__ __forceinline__ void join_members(const float (&a)[LV][8], int q, float& s, float& l) {
+template <bool SPLIT, int LV, int LC>
+__device__ __forceinline__ void join_members(const float (&a)[LV][LC], int q, float& s, float& l) {
   float t, e, e2, e3 = 0.f;
   df_two_sum(a[0][q], __fmul_rn(a[1][q], 0x1p-10f), t, e);
   if constexpr (SPLIT) {
@@ -230,37 +236,60 @@ __device__ __forceinline__ void join_members(const float (&a)[LV][8], int q, flo
   l = __fadd_rn(__fadd_rn(__fadd_rn(e, e3), e2), low);
 }
 
-// One slice product A_i B_j over KS blocks of 16 along K into the `acc` tensor-memory columns. The
-// descriptors' address fields count 16-byte units, so a step along K or to another slice is an addition.
-template <int KS>
-__device__ __forceinline__ void issue_product(uint32_t d, uint64_t a, uint32_t a_step, uint64_t b, uint32_t b_step,
-                                              uint32_t idesc, bool first) {
-#pragma unroll
-  for (int kb = 0; kb < KS; ++kb)
-    umma_f16(d, a + (uint64_t)(kb * (a_step >> 4)), b + (uint64_t)(kb * (b_step >> 4)), idesc,
-             (first && kb == 0) ? 0u : 1u);
-}
-// The slice products of D = A B, level g = i + j <= GMAX in the `cols` columns at d + g cols; one
-// thread. SPLIT: the product (1, 0) goes to level column 5 (K = 128 would let level 1 reach 2^25).
-template <int KS, int GMAX, bool SPLIT>
-__device__ __forceinline__ void issue_levels(uint32_t d, int cols, uint64_t a, uint32_t a_part, uint32_t a_step,
-                                             uint64_t b, uint32_t b_part, uint32_t b_step, uint32_t idesc) {
-#pragma unroll 1
-  for (int g = 0; g <= GMAX; ++g) {
-    const int i0 = g < kSl ? 0 : g - kSl + 1, i1 = g < kSl ? g : kSl - 1;
-#pragma unroll 1
-    for (int i = i0; i <= i1; ++i) {
-      const bool own = SPLIT && g == 1 && i == 1;
-      issue_product<KS>(d + (uint32_t)((own ? 5 : g) * cols), a + (uint64_t)((i * a_part) >> 4), a_step,
-                        b + (uint64_t)(((g - i) * b_part) >> 4), b_step, idesc, i == i0 || own);
-    }
-  }
+__device__ __forceinline__ void umma_lead(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc,
+                                          uint32_t lead) {
+  asm volatile("{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+               " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+               ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(lead));
 }
 // kind::f16 descriptor of FP16 operands with M = 128 and each operand K-major or MN-major
 __host__ __device__ constexpr uint32_t sl_idesc(int N, bool a_mn, bool b_mn) {
   return umma_idesc(0, N, b_mn) | ((a_mn ? 1u : 0u) << 15);
 }
-
+// The slice products of D = A B, level g = i + j <= GMAX in the JC columns at d + g JC, over KS blocks of
+// 16 along K. The slices of B lie one behind the other along N (B_SL bytes apart), so that
+// A_i [B_j0 .. B_j1] is one MMA into the consecutive levels i + j0 .. i + j1: with M = 128 an MMA takes
+// 64 cycles for any N <= 64, 75 for 128 and 135 for 256 (the reads of A bound the narrow ones), and
+// the 19 products of 64 columns 2,700 cycles per 64 terms instead of 4,900. SPLIT: the product (1, 0)
+// goes to level column 5 (K = 128 would let level 1 reach 2^25). Called by one whole warp with `lead`
+// on one lane, so that addresses stay warp-uniform.
+template <int KS, int GMAX, bool SPLIT, int JC, bool AMN, bool BMN, int A_PART, int A_STEP, int B_SL, int B_STEP>
+__device__ __forceinline__ void issue_levels(uint32_t d, uint64_t a, uint64_t b, uint64_t* mbar, uint32_t lead) {
+  // recomputed here for each tile: hoisted out of the tile loop the descriptors would be spilled
+  asm volatile("" : "+l"(a), "+l"(b), "+r"(d));
+  constexpr int NMAX = 256 / JC < kSl ? 256 / JC : kSl;   // slices of B per MMA at most
+  auto mma = [&](int i, int j0, int nj, int kb, int col, bool acc) {
+    umma_lead(d + (uint32_t)(col * JC), a + (uint64_t)((i * A_PART + kb * A_STEP) >> 4),
+              b + (uint64_t)((j0 * B_SL + kb * B_STEP) >> 4), sl_idesc(nj * JC, AMN, BMN), acc ? 1u : 0u, lead);
+  };
+#pragma unroll
+  for (int kb = 0; kb < KS; ++kb)
+#pragma unroll
+    for (int i = 0; i < kSl; ++i) {
+      const int nj = GMAX - i + 1 < kSl ? GMAX - i + 1 : kSl;   // j = 0 .. nj - 1
+      int j = 0;
+      if (SPLIT && i == 1) {
+        mma(1, 0, 1, kb, 5, kb > 0);
+        j = 1;
+      }
+      // the level GMAX of GMAX = kSl begins at (1, kSl - 1): on its own in the first block along K
+      const int end = (GMAX == kSl && i == 1 && kb == 0) ? nj - 1 : nj;
+#pragma unroll
+      for (int q = 0; q < kSl; ++q)   // in pieces of even size, at most NMAX slices each
+        if (j < end) {
+          const int left = end - j, pieces = (left + NMAX - 1) / NMAX, n = (left + pieces - 1) / pieces;
+          mma(i, j, n, kb, i + j, i > 0 || kb > 0);
+          j += n;
+        }
+      if (end < nj) mma(i, end, 1, kb, i + end, false);
+    }
+  if (lead) umma_commit(mbar);
+}
+__device__ __forceinline__ uint32_t elect_lane() {
+  uint32_t v;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(v));
+  return v;
+}
 // what the passes of one CTA share
 struct KCta {
   unsigned char* smem;
@@ -271,230 +300,290 @@ struct KCta {
   bool ok;
 };
 __device__ __forceinline__ void k_wait(KCta& c) {
-  if (!mbar_wait(c.mbar, c.phase, c.status)) c.ok = false;
+  // a few hardware waits before the bounded one, which reads the global timer
+  uint32_t done = 0;
+#pragma unroll 1
+  for (int q = 0; q < 4 && !done; ++q)
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(done) : "r"(smem_addr(c.mbar)), "r"(c.phase) : "memory");
+  if (!done && !mbar_wait(c.mbar, c.phase, c.status)) c.ok = false;
   c.phase ^= 1u;
   tc_fence_after();
 }
 
-// A 64-row tile of a [rows][N] matrix into the K-major image of width W, each row scaled by a
-// power of two above its largest entry (inverse scales into s_inv[64]). COPIES: image row q holds
-// source row q % COPIES (the T operand); L2: read through L2.
-template <int W, int ROWS, int SRC, bool L2>
-__device__ __forceinline__ void slice_rows(const df32* __restrict__ src, int64_t row0, int64_t row1, int N,
-                                           unsigned char* img, float* s_inv) {
-  constexpr int G8 = W / 8, RPS = kThreads / G8, PART = ROWS * W * 2;
-  const int t = threadIdx.x, g = t % G8, c0 = 8 * g;
+// Eight consecutive df32 of a row of N, zeros past N or when !ok. N % 8 == 0: unconditional 16-byte
+// loads (from row 0 of the array when !ok), so that several rows' loads are in flight together.
+__device__ __forceinline__ void load_row8(df32 (&x)[8], const df32* base, int64_t i, int c0, int N, bool ok) {
+  if ((N & 7) == 0) {
+    const bool in = ok && c0 < N;
+    const df32* row = base + (in ? i * N + c0 : 0);
 #pragma unroll
-  for (int it = 0; it < ROWS / RPS; ++it) {
-    const int q = t / G8 + it * RPS;
-    const int64_t i = row0 + q % SRC;
-    df32 x[8];
-    if (L2) {
-      if (i < row1) load_df8_cg(x, src + i * N, c0, N);
-      else
-#pragma unroll
-        for (int e = 0; e < 8; ++e) x[e] = df32(0.f, 0.f);
-    } else {
-      load_df8(x, src + i * N, c0, N, i < row1);
+    for (int q = 0; q < 4; ++q) {
+      const float4 v = *reinterpret_cast<const float4*>(row + 2 * q);
+      x[2 * q] = in ? df32(v.x, v.y) : df32(0.f, 0.f);
+      x[2 * q + 1] = in ? df32(v.z, v.w) : df32(0.f, 0.f);
     }
-    float mx = 0.f;
+  } else {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) mx = fmaxf(mx, fabsf(x[e].hi));
-#pragma unroll
-    for (int o = G8 / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    float sc, inv;
-    pow2_of(mx, sc, inv);
-    const float scale[8] = {sc, sc, sc, sc, sc, sc, sc, sc};
-    store_slices8(img, PART, core_idx(q, c0, W) * 2, x, scale);
-    if (g == 0) s_inv[q] = inv;
+    for (int q = 0; q < 8; ++q) {
+      const bool in = ok && c0 + q < N;
+      const float2 v = *reinterpret_cast<const float2*>(base + (in ? i * N + c0 + q : 0));
+      x[q] = in ? df32(v.x, v.y) : df32(0.f, 0.f);
+    }
   }
 }
 
+// Who slices what: an item is eight columns of one row, a warp takes eight rows (lane & 7: their
+// 16-byte pieces of a core matrix are one 128-byte line, so the stores are free of bank conflicts)
+// of four column groups (lane >> 3). W columns: 2 W / 8 warp items per tile of 64 rows.
+template <int W> struct KItems {
+  static constexpr int G4 = W / 32;                       // warp items per eight rows
+  static constexpr int N = (8 * G4 + 15) / 16;            // items per thread (W = 32: half the warps)
+  __device__ static bool live(int warp, int it) { return warp + 16 * it < 8 * G4; }
+  __device__ static int row(int warp, int lane, int it) { return (warp + 16 * it) / G4 * 8 + (lane & 7); }
+  __device__ static int col(int warp, int lane, int it) { return (warp + 16 * it) % G4 * 32 + (lane >> 3) * 8; }
+};
+
+// The T operand of u = HA T: JC columns of a reduced N x N matrix (row j of `src` is column j; other
+// CTAs wrote it) as ROWS rows of W, row q holding column q % JC, each scaled by a power of two above
+// its largest entry (s_inv: the scale's inverse).
+template <int W, int ROWS, int JC>
+__device__ __forceinline__ void stage_columns(const df32* __restrict__ src, int j0, int N, unsigned char* img,
+                                              float* s_inv) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int q = 8 * warp + (lane & 7), j = j0 + q % JC;
+  if (8 * warp >= ROWS) return;   // uniform in the warp
+  df32 x[W / 32][8];
+  float mx = 0.f;
+#pragma unroll
+  for (int g = 0; g < W / 32; ++g)
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int k = 32 * g + (lane >> 3) * 8 + e;
+      x[g][e] = (j < N && k < N) ? ld_df(src + (int64_t)j * N + k) : df32(0.f, 0.f);
+      mx = fmaxf(mx, fabsf(x[g][e].hi));
+    }
+  mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+  mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+  float sc, inv;
+  pow2_of(mx, sc, inv);
+#pragma unroll
+  for (int g = 0; g < W / 32; ++g) {
+    Slices8 sl;
+    sl.make(x[g], sc);
+    sl.store(img + core_idx(q, 32 * g + (lane >> 3) * 8, W) * 2, ROWS * W * 2);
+  }
+  if (lane < 8) s_inv[q] = inv;
+}
+
 // ------------------------------------------------------------------ pass G
-// The CTA's rows of U = R^{-1/2} HA and V = R^{-1/2} b (b = D, or the FP32 residual B) as one sliced
-// image [U | V] per tile, each column scaled by the power of two above its largest entry in the
-// tile, and K = U^T U, F = U^T V accumulated over the tiles in double-float registers. Column
-// group c takes the columns [64 c, 64 c + JC) of K and F. NT <= 64: one product [U | V]^T U
-// (M = 128: rows k of K, then rows j of F^T); NT = 128: U^T U_c, then U^T V.
+// The CTA's rows of U = R^{-1/2} HA and V = R^{-1/2} b (b = D, or the FP32 residual B), sliced per tile:
+// U scaled by the power of two above its largest entry in the problem (the innovations record it),
+// each column of V by that of its largest entry in the tile; K = U^T U and F = U^T V accumulate over
+// the tiles in double-float registers. Column group c takes the columns [64 c, 64 c + JC) of K and F.
+// NT <= 64: one product [U | V]^T U (M = 128: rows k of K, then rows j of F^T); NT = 128: U^T U_c, then
+// U^T V. Operand A holds [U | V] (U) slice by slice, operand B the slices of U_c (and V) side by side;
+// the loads of the next tile are in flight behind the products.
 template <int NT>
 __device__ __noinline__ void pass_gram(const KrylovParams& p, bool from_b, int c, int64_t row0, int64_t row1,
                                        KCta& cta, df32* __restrict__ out) {
   using L = KLayout<NT>;
-  constexpr int JC = L::JC, CW = L::CW;
-  constexpr int UI = kKR * (NT / 8) / kThreads > 0 ? kKR * (NT / 8) / kThreads : 1;   // items of U per thread
-  constexpr int VI = kKR * (JC / 8) / kThreads > 0 ? kKR * (JC / 8) / kThreads : 1;
-  unsigned char* img = cta.smem;
-  float* s_max = reinterpret_cast<float*>(cta.smem + L::off_max);     // [8 warps][CW]
-  float* s_sc = reinterpret_cast<float*>(cta.smem + L::off_col);      // [CW] inverse column scales
-  const int N = p.N, t = threadIdx.x, warp = t >> 5, lane = t & 31, qd = warp & 3, half = warp >> 2;
-  const int gu = t % (NT / 8), ru = t / (NT / 8), gv = t % (JC / 8), rv = t / (JC / 8);
-  constexpr int RU = kThreads / (NT / 8), RV = kThreads / (JC / 8);   // rows per sweep
-  const int cv0 = c * 64 + 8 * gv;   // this thread's columns of b
-  const int L_ = 32 * qd + lane;
-  constexpr int NC = JC / 2;         // columns of a product per thread
+  using UI = KItems<NT>;
+  using VI = KItems<L::JC>;
+  constexpr int JC = L::JC;
+  constexpr bool PRE = NT <= 64;     // the next tile's U is held in registers behind the products
+  constexpr int LC = PRE ? 8 : 4;
+  float* s_max = reinterpret_cast<float*>(cta.smem + L::off_max);     // [8 row blocks][64]
+  float* s_sc = reinterpret_cast<float*>(cta.smem + L::off_col);      // [64] inverse scales of V
+  const int N = p.N, t = threadIdx.x, lane = t & 31, qd = (t >> 5) & 3, sub = t >> 7;
+  const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);               // warp-uniform
+  const int ln = 32 * qd + lane;
+  constexpr int NC = JC / 4;         // columns of a product per thread
   DFAcc acc[NC], accF[NT == 128 ? NC : 1];
-  SqAcc s1[8], s2[8];
-  const uint32_t base = smem_addr(img);
-  constexpr uint32_t rg = (CW / 8) * 128;   // row-group stride
-  for (int64_t i0 = row0; i0 < row1 && cta.ok; i0 += kKR) {
-    df32 u[UI][8], v[VI][8];
+  // ||b_j||^2 over the thread's rows as compensated pairs and (b_j, R^{-1} b_j): in shared memory,
+  // [24][threads] (in registers they spilled the accumulators)
+  float* s_sq = reinterpret_cast<float*>(cta.smem + L::off_sq) + t;
 #pragma unroll
-    for (int it = 0; it < UI; ++it) {
-      const int r = ru + it * RU;
-      const int64_t i = i0 + r;
-      const bool in = r < kKR && i < row1;
-      load_df8(u[it], p.HAdf + i * N, 8 * gu, N, in);
-      if (in) {
-        const df32 q = p.rsq[i];
+  for (int e = 0; e < L::SQ; ++e) s_sq[e * kKT] = 0.f;
+  float su, uinv;
+  pow2_of(__uint_as_float(*(volatile const unsigned*)p.umax), su, uinv);
+  const uint32_t base = smem_addr(cta.smem), lead = warp == 0 ? elect_lane() : 0u;
+  const bool vlive = VI::live(warp, 0);
+  const int vr = VI::row(warp, lane, 0), vc = VI::col(warp, lane, 0), cv0 = c * 64 + vc;
+  df32 u[PRE ? UI::N : 1][8], v[8], uq[PRE ? UI::N : 1], vq;
+  auto load_u = [&](int64_t i0, int it, int slot) {
+    const int64_t i = i0 + UI::row(warp, lane, it);
+    const bool in = UI::live(warp, it) && i < row1;
+    load_row8(u[slot], p.HAdf, i, UI::col(warp, lane, it), N, in);
+    uq[slot] = p.rsq[in ? i : 0];
+  };
+  auto load = [&](int64_t i0) {
+    if (PRE)
 #pragma unroll
-        for (int e = 0; e < 8; ++e) u[it][e] = u[it][e] * q;
+      for (int it = 0; it < UI::N; ++it) load_u(i0, it, it);
+    const int64_t i = i0 + vr;
+    const bool in = vlive && i < row1;
+    if (from_b) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = df32((in && cv0 + e < N) ? p.B[i * N + cv0 + e] : 0.f, 0.f);
+    } else {
+      load_row8(v, p.Ddf, i, cv0, N, in);
+    }
+    vq = p.rsq[in ? i : 0];
+  };
+  // address of core row (r, column cc of slice 0) of an operand B
+  auto b_at = [&](int off, int r, int cc) {
+    return cta.smem + off + (r >> 3) * L::BR + (cc >> 3) * 128 + (r & 7) * 16;
+  };
+  // the tile from i0 on into the operands: U at once, V after its column maxima
+  auto slice = [&](int64_t i0) {
+#pragma unroll(PRE ? UI::N : 1)
+    for (int it = 0; it < UI::N; ++it) {
+      const int q = PRE ? it : 0;
+      if (!PRE) load_u(i0, it, 0);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) u[q][e] = u[q][e] * uq[q];
+      if (UI::live(warp, it)) {
+        const int r = UI::row(warp, lane, it), cc = UI::col(warp, lane, it);
+        Slices8 sl;
+        sl.make(u[q], su);
+        sl.store(cta.smem + core_idx(r, cc, 128) * 2, L::CP);
+        if (NT < 128 || (cc >> 6) == c) sl.store(b_at(L::off_gu, r, cc & (JC - 1)), JC * 16);
       }
     }
-#pragma unroll
-    for (int it = 0; it < VI; ++it) {
-      const int r = rv + it * RV;
-      const int64_t i = i0 + r;
-      const bool in = r < kKR && i < row1;
-      if (from_b) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[it][e] = df32((in && cv0 + e < N) ? p.B[i * N + cv0 + e] : 0.f, 0.f);
-      } else {
-        load_df8(v[it], p.Ddf + i * N, cv0, N, in);
-      }
-      if (in) {
-        const df32 q = p.rsq[i];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          s1[e].add(v[it][e].hi);
-          v[it][e] = v[it][e] * q;
-          s2[e].add(v[it][e].hi);
-        }
-      }
-    }
-    // column maxima of the tile: over the thread's items, the warp's lanes of the same columns,
-    // then the warps
+    float mx[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      float mu = 0.f, mv = 0.f;
+      SqAcc sq;
+      sq.s = s_sq[e * kKT];
+      sq.c = s_sq[(8 + e) * kKT];
+      sq.add(v[e].hi);
+      s_sq[e * kKT] = sq.s;
+      s_sq[(8 + e) * kKT] = sq.c;
+      v[e] = v[e] * vq;
+      s_sq[(16 + e) * kKT] = fmaf(v[e].hi, v[e].hi, s_sq[(16 + e) * kKT]);
+      mx[e] = fabsf(v[e].hi);
 #pragma unroll
-      for (int it = 0; it < UI; ++it) mu = fmaxf(mu, fabsf(u[it][e].hi));
-#pragma unroll
-      for (int it = 0; it < VI; ++it) mv = fmaxf(mv, fabsf(v[it][e].hi));
-#pragma unroll
-      for (int o = 16; o >= NT / 8; o >>= 1) mu = fmaxf(mu, __shfl_xor_sync(0xffffffffu, mu, o));
-#pragma unroll
-      for (int o = 16; o >= JC / 8; o >>= 1) mv = fmaxf(mv, __shfl_xor_sync(0xffffffffu, mv, o));
-      if (lane < NT / 8) s_max[warp * CW + 8 * gu + e] = mu;
-      if (lane < JC / 8) s_max[warp * CW + NT + 8 * gv + e] = mv;
+      for (int o = 4; o > 0; o >>= 1) mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], o));
     }
-    tc_fence_before();
-    __syncthreads();   // also: the previous tile's sums have left tensor memory
-    float su[8], sv[8];
-    {
-      float dummy;
+    if (vlive && (lane & 7) == 0) {
+      *reinterpret_cast<float4*>(s_max + (vr >> 3) * 64 + vc) = make_float4(mx[0], mx[1], mx[2], mx[3]);
+      *reinterpret_cast<float4*>(s_max + (vr >> 3) * 64 + vc + 4) = make_float4(mx[4], mx[5], mx[6], mx[7]);
+    }
+    __syncthreads();
+    if (vlive) {
+      float sv[8];
+#pragma unroll
+      for (int w = 0; w < 8; ++w)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float4 m4 = *reinterpret_cast<const float4*>(s_max + w * 64 + vc + 4 * h);
+          mx[4 * h] = fmaxf(mx[4 * h], m4.x);
+          mx[4 * h + 1] = fmaxf(mx[4 * h + 1], m4.y);
+          mx[4 * h + 2] = fmaxf(mx[4 * h + 2], m4.z);
+          mx[4 * h + 3] = fmaxf(mx[4 * h + 3], m4.w);
+        }
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
-        float mu = 0.f, mv = 0.f;
-#pragma unroll
-        for (int w = 0; w < kThreads / 32; ++w) {
-          mu = fmaxf(mu, s_max[w * CW + 8 * gu + e]);
-          mv = fmaxf(mv, s_max[w * CW + NT + 8 * gv + e]);
-        }
-        pow2_of(mu, su[e], dummy);
-        if (ru == 0) s_sc[8 * gu + e] = dummy;
-        pow2_of(mv, sv[e], dummy);
-        if (rv == 0) s_sc[NT + 8 * gv + e] = dummy;
+        float inv;
+        pow2_of(mx[e], sv[e], inv);
+        if (vr == 0) s_sc[vc + e] = inv;
       }
-    }
-#pragma unroll
-    for (int it = 0; it < UI; ++it) {
-      const int r = ru + it * RU;
-      if (r < kKR) store_slices8(img, L::CP, core_idx(r, 8 * gu, CW) * 2, u[it], su);
-    }
-#pragma unroll
-    for (int it = 0; it < VI; ++it) {
-      const int r = rv + it * RV;
-      if (r < kKR) store_slices8(img, L::CP, core_idx(r, NT + 8 * gv, CW) * 2, v[it], sv);
+      Slices8 sl;
+      sl.make(v, sv);
+      if (NT == 128) sl.store(b_at(L::off_gv, vr, vc), JC * 16);
+      else sl.store(cta.smem + core_idx(vr, NT + vc, 128) * 2, L::CP);
     }
     fence_async_smem();
+    tc_fence_before();
     __syncthreads();
-    // K = rows of the tile, both operands MN-major (columns contiguous)
-    const uint64_t A = umma_desc(base, rg, 128);
-    if (t == 0) {
-      tc_fence_after();
-      issue_levels<kKR / 16, 5, false>(cta.tmem, JC, A, L::CP, 2 * rg, umma_desc(base + (NT == 128 ? c * 1024 : 0), rg, 128),
-                             L::CP, 2 * rg, sl_idesc(JC, true, true));
-      umma_commit(cta.mbar);
-    }
-    k_wait(cta);
-    auto flush = [&](DFAcc* a, float rs, const float* cs) {
+  };
+  auto flush = [&](DFAcc* a, float rs, const float* cs) {   // cs: column scales or nullptr (U's)
 #pragma unroll
-      for (int q0 = 0; q0 < NC; q0 += 8) {
-        float lv[kLv][8];
-        tmem_ld_levels<kLv>(cta.tmem + ((uint32_t)(32 * qd) << 16) + half * NC + q0, JC, lv);
+    for (int q0 = 0; q0 < NC; q0 += LC) {
+      float lv[kLv][LC];
+      tmem_ld_levels<kLv, LC>(cta.tmem + ((uint32_t)(32 * qd) << 16) + sub * NC + q0, JC, lv);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          float s, l, tt, e;
-          join_rows(lv, q, s, l);
-          const float f = rs * cs[q0 + q];
-          df_two_sum(a[q0 + q].s, s * f, tt, e);
-          a[q0 + q].s = tt;
-          a[q0 + q].c = __fadd_rn(a[q0 + q].c, __fmaf_rn(l, f, e));
-          a[q0 + q].renorm();
-        }
+      for (int q = 0; q < LC; ++q) {
+        float s, l, tt, e;
+        join_rows(lv, q, s, l);
+        const float f = rs * (cs ? cs[sub * NC + q0 + q] : uinv);
+        df_two_sum(a[q0 + q].s, s * f, tt, e);
+        a[q0 + q].s = tt;
+        a[q0 + q].c = __fadd_rn(a[q0 + q].c, __fmaf_rn(l, f, e));
+        a[q0 + q].renorm();
       }
-    };
-    const float rs = s_sc[min(L_, CW - 1)] * 0x1p-16f;
-    flush(acc, rs, s_sc + (NT == 128 ? 64 * c : 0) + half * NC);
+    }
+  };
+  // K = rows of the tile, both operands MN-major (columns contiguous)
+  auto issue = [&](int boff) {
+    if (warp == 0) {
+      tc_fence_after();
+      issue_levels<kKR / 16, 5, false, JC, true, true, L::CP, 2 * 2048, JC * 16, 2 * L::BR>(
+          cta.tmem, umma_desc(base, 2048, 128), umma_desc(base + boff, L::BR, 128), cta.mbar, lead);
+    }
+  };
+  if (row0 < row1) {
+    load(row0);
+    slice(row0);
+    issue(L::off_gu);
+  }
+  for (int64_t i0 = row0; i0 < row1 && cta.ok; i0 += kKR) {
+    const bool more = i0 + kKR < row1;
+    if (more) load(i0 + kKR);
+    k_wait(cta);
     if constexpr (NT == 128) {
+      flush(acc, uinv * 0x1p-16f, nullptr);
       tc_fence_before();
       __syncthreads();
-      if (t == 0) {
-        tc_fence_after();
-        issue_levels<kKR / 16, 5, false>(cta.tmem, JC, A, L::CP, 2 * rg, umma_desc(base + (NT / 8) * 128, rg, 128), L::CP,
-                               2 * rg, sl_idesc(JC, true, true));
-        umma_commit(cta.mbar);
-      }
+      issue(L::off_gv);
       k_wait(cta);
-      flush(accF, rs, s_sc + NT + half * NC);
+      flush(accF, uinv * 0x1p-16f, s_sc);
+    } else {
+      // lanes [NT, 2 NT) hold F^T: row scale of V's column
+      flush(acc, (ln < NT ? uinv : s_sc[ln & (NT - 1)]) * 0x1p-16f, nullptr);
+    }
+    if (more) {
+      __syncthreads();   // s_sc is rewritten with the operands
+      slice(i0 + kKR);
+      issue(L::off_gu);
     }
   }
-  tc_fence_before();
-  __syncthreads();
-  // the CTA's partial: K[k][jl] at k JC + jl, F[k][jl] behind it, then the column sums
+  // the CTA's partial: K[k][jl] at k NJ + jl, F[k][jl] behind it, then the column sums
   const int NJ = min(JC, N);
   if constexpr (NT == 128) {
-    if (L_ < N)
+    if (ln < N)
 #pragma unroll
       for (int q = 0; q < NC; ++q) {
-        const int jl = half * NC + q;
-        out[L_ * NJ + jl] = acc[q].value();
-        out[N * NJ + L_ * NJ + jl] = accF[q].value();
+        const int jl = sub * NC + q;
+        out[ln * NJ + jl] = acc[q].value();
+        out[N * NJ + ln * NJ + jl] = accF[q].value();
       }
   } else {
     // lanes [0, NT): K[k = lane][col]; lanes [NT, 2 NT): F^T[j = lane - NT][k = col]
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
-      const int col = half * NC + q;
+      const int col = sub * NC + q;
       if (col < N) {
-        if (L_ < N) out[L_ * NJ + col] = acc[q].value();
-        else if (L_ >= NT && L_ - NT < N) out[N * NJ + col * NJ + (L_ - NT)] = acc[q].value();
+        if (ln < N) out[ln * NJ + col] = acc[q].value();
+        else if (ln >= NT && ln - NT < N) out[N * NJ + col * NJ + (ln - NT)] = acc[q].value();
       }
     }
   }
   // column sums over the threads of each column, fixed order
-  double* red = reinterpret_cast<double*>(cta.smem);   // [RV][JC] twice
+  double* red = reinterpret_cast<double*>(cta.smem);   // [2][64 rows][JC]
   __syncthreads();
+  if (vlive)
 #pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    red[rv * JC + 8 * gv + e] = s1[e].value();
-    red[(RV + rv) * JC + 8 * gv + e] = s2[e].value();
-  }
+    for (int e = 0; e < 8; ++e) {
+      red[vr * JC + vc + e] = (double)s_sq[e * kKT] + (double)s_sq[(8 + e) * kKT];
+      red[(64 + vr) * JC + vc + e] = (double)s_sq[(16 + e) * kKT];
+    }
   __syncthreads();
   if (t < 2 * JC) {
     const int which = t / JC, j = t % JC;
     double s = 0.0;
-    for (int q = 0; q < RV; ++q) s += red[(which * RV + q) * JC + j];
+    for (int q = 0; q < 64; ++q) s += red[(which * 64 + q) * JC + j];
     out[2 * N * NJ + which * 64 + j] = df32(s);
   }
   __syncthreads();
@@ -523,11 +612,11 @@ __device__ __forceinline__ void reduce_parts(const df32* __restrict__ part, int6
     return a.value();
   };
   if (n <= 0) return;
-  if (n >= kThreads) {
-    for (int e = e0 + t; e < e0 + n; e += kThreads) store(e / cnt, e % cnt, add_range(e, 0, RB));
+  if (n >= kKT) {
+    for (int e = e0 + t; e < e0 + n; e += kKT) store(e / cnt, e % cnt, add_range(e, 0, RB));
     return;
   }
-  const int parts = kThreads / n, el = t % n, w = t / n;
+  const int parts = kKT / n, el = t % n, w = t / n;
   scratch[t] = w < parts ? add_range(e0 + el, (int)((int64_t)w * RB / parts), (int)((int64_t)(w + 1) * RB / parts))
                          : df32(0.f, 0.f);
   __syncthreads();
@@ -536,6 +625,28 @@ __device__ __forceinline__ void reduce_parts(const df32* __restrict__ part, int6
     for (int q = 1; q < parts; ++q) v = v + scratch[q * n + t];
     const int e = e0 + t;
     store(e / cnt, e % cnt, v);
+  }
+  __syncthreads();
+}
+
+// Every CTA sums the G CTAs' column sums part[q NT + j] in the same fixed order.
+template <int NT>
+__device__ __forceinline__ void total_columns(const double* __restrict__ part, int G, int N, double* out,
+                                              double* scratch) {
+  constexpr int Q = kKT / NT;
+  const int t = threadIdx.x, j = t % NT, q = t / NT;
+  double s = 0.0;
+  if (j < N) {
+    const int b0 = (int)((int64_t)q * G / Q), b1 = (int)((int64_t)(q + 1) * G / Q);
+#pragma unroll 8
+    for (int b = b0; b < b1; ++b) s += __ldcg(part + (int64_t)b * NT + j);
+  }
+  scratch[t] = s;
+  __syncthreads();
+  if (t < NT) {
+    double v = 0.0;
+    for (int qq = 0; qq < Q; ++qq) v += scratch[qq * NT + t];
+    out[t] = v;
   }
   __syncthreads();
 }
@@ -553,12 +664,7 @@ __device__ __forceinline__ df32 df_div(const df32& a, const df32& b) {   // two 
 __device__ __forceinline__ df32 df_shfl_xor(const df32& v, int o) {
   return df32(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
 }
-__device__ __forceinline__ df32 ld_df(const df32* p) {
-  const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
-  return df32(v.x, v.y);
-}
-
-// Columns j0, j0 + step, ... (nc <= 8, one per warp) of this cycle: (I + K) w = g from w = 0 (or the
+// Columns j0, j0 + step, ... (nc <= 16, one per warp) of this cycle: (I + K) w = g from w = 0 (or the
 // learned start) by the recurrences at the head of this file until (r, R^{-1} r) <= itol^2
 // (b, R^{-1} b) or the column's step limit; w into row j of wred, the steps taken added to
 // col_iters[j]. Everything is double-float: on this part an FP64 instruction holds a scheduler's
@@ -569,7 +675,7 @@ __device__ __forceinline__ df32 ld_df(const df32* p) {
 // is (rho, kr) + (kr, kr) - beta^2 (p, S p)_old.
 template <int NT>
 struct KMat {
-  static constexpr int TPR = kThreads / NT, KPT = NT / TPR;   // threads per row, entries per thread
+  static constexpr int TPR = kKT / NT, KPT = NT / TPR;   // threads per row, entries per thread
   df32 k[KPT];
 };
 struct KColumns {
@@ -589,9 +695,9 @@ template <int NT>
 __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 inv_nm1, int j0, int step, int nc,
                                           const KColumns& C, unsigned char* sm) {
   constexpr int TPR = KMat<NT>::TPR, KPT = KMat<NT>::KPT, EPL = NT / 32;
-  df32* s_rho = reinterpret_cast<df32*>(sm);                  // [8][NT]
-  df32* s_part = s_rho + 8 * NT;                              // [8][TPR][NT]
-  int* s_act = reinterpret_cast<int*>(s_part + 8 * kThreads); // [8]
+  df32* s_rho = reinterpret_cast<df32*>(sm);                  // [16][NT]
+  df32* s_part = s_rho + 16 * NT;                             // [16][TPR][NT]
+  int* s_act = reinterpret_cast<int*>(s_part + 16 * kKT); // [16]
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5, r = t % NT, g = t / NT;
   const bool mine = warp < nc;
   const int j = j0 + warp * step;
@@ -613,7 +719,7 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
       s_rho[warp * NT + k] = start ? w[e] : rho[e];
     }
   }
-  if (t < 8) s_act[t] = t < nc;
+  if (t < 16) s_act[t] = t < nc;
   // K times the vectors in s_rho of the active columns: thread (g, r) its entries of row r
   auto product = [&]() {
 #pragma unroll 1
@@ -622,21 +728,25 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
       const df32* v = s_rho + c * NT + g * KPT;
       DFAcc a0, a1;
 #pragma unroll
-      for (int q = 0; q < KPT; q += 2) {
+      for (int q = 0; q < KPT; q += 2) {   // KPT = 2, 8 or 32
         const float4 x = *reinterpret_cast<const float4*>(v + q);
         a0.add(M.k[q], df32(x.x, x.y));
         a1.add(M.k[q + 1], df32(x.z, x.w));
         if ((q & 7) == 6) { a0.renorm(); a1.renorm(); }
       }
-      s_part[c * kThreads + g * NT + r] = a0.value() + a1.value();
+      s_part[c * kKT + g * NT + r] = a0.value() + a1.value();
     }
     __syncthreads();
   };
   auto row = [&](int k) {
-    df32 s = s_part[warp * kThreads + k];
+    df32 s[TPR];
 #pragma unroll
-    for (int q = 1; q < TPR; ++q) s = s + s_part[warp * kThreads + q * NT + k];
-    return s;
+    for (int q = 0; q < TPR; ++q) s[q] = s_part[warp * kKT + q * NT + k];
+#pragma unroll
+    for (int o = TPR / 2; o > 0; o >>= 1)
+#pragma unroll
+      for (int q = 0; q < o; ++q) s[q] = s[q] + s[q + o];
+    return s[0];
   };
   if (C.w0) {   // rho = g - (I + K) w0 (the same for every column; without a start w = 0)
     __syncthreads();
@@ -703,146 +813,201 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
 }
 
 // ------------------------------------------------------------------ passes Z and R
-// The T operand of u = HA T: the CTA's JC columns of a reduced N x N matrix (row j of `src` is
-// column j), sliced with a power of two per column; inverse scales into s_inv[128].
-template <int NT>
-__device__ __forceinline__ void stage_columns(const df32* __restrict__ src, int c, int N, unsigned char* img,
-                                              float* s_inv) {
-  using L = KLayout<NT>;
-  slice_rows<NT, L::TROWS, L::JC, true>(src, (int64_t)c * 64, N, N, img, s_inv);
-}
-
 // Both passes: u = HA T for a tile arrives as D[j][i] (lane j, tensor-memory column i), so that a
 // thread owns one column j and RPT consecutive rows, its accesses to D and Z are contiguous
 // across the warp, and column sums and maxima stay in the thread. For NT <= 64 the T operand holds
 // 128 / NT copies of its columns, so that all 128 lanes carry work (copy d takes the rows
-// [16 d, ...) of a tile); at NT = 128 two such copies do not fit and half of the lanes idle.
+// [64 d / copies, ...) of a tile); at NT = 128 two such copies do not fit and half of the lanes idle.
 // RESID = false: Z (+)= R^{-1} (b - u), then T += HA^T Z (out: T[k][jl]).
 // RESID = true: B = D - R Z - u/(N-1) and rr[j] = ||B_j||^2 over the CTA's rows.
+// NT <= 64: the next tile is loaded and sliced behind the products of the current one.
 template <int NT, bool RESID>
 __device__ __noinline__ void pass_rows(const KrylovParams& p, bool from_b, int c, int64_t row0, int64_t row1,
                                        KCta& cta, const int* s_done, df32* __restrict__ out, double* rr_out) {
   using L = KLayout<NT>;
-  constexpr int JC = L::JC;
+  using HI = KItems<NT>;
+  constexpr int JC = L::JC, NB = L::NB;
+  constexpr bool PRE = NT <= 64;                  // the next tile's loads are held in registers
+  constexpr int LC = PRE ? 8 : 4;
   constexpr int CP = NT == 128 ? 1 : 128 / NT;    // copies
-  constexpr int RPT = kKR / (2 * CP);             // rows per thread: 8, 16, 32
+  constexpr int NSUB = NT == 32 ? 2 : 4;          // warps per copy and 32 lanes
+  constexpr int GRP = CP * NSUB;                  // row groups of a tile: 8, 8, 4
+  constexpr int RPT = kKR / GRP;                  // rows per thread: 8, 8, 16
   constexpr bool SPL = NT == 128;                 // level 1 of u in two sums
-  unsigned char* sT = cta.smem + L::off_t;
-  unsigned char* sH = cta.smem + L::off_h;
   unsigned char* sV = cta.smem + L::off_v;
-  float* s_row = reinterpret_cast<float*>(cta.smem + L::off_row);   // [64] inverse row scales
-  float* s_col = reinterpret_cast<float*>(cta.smem + L::off_col);   // [128] inverse scales of T
-  float* s_max = reinterpret_cast<float*>(cta.smem + L::off_max);   // [2 CP][64] column maxima
-  const int N = p.N, t = threadIdx.x, warp = t >> 5, lane = t & 31, qd = warp & 3, half = warp >> 2;
+  float* s_row = reinterpret_cast<float*>(cta.smem + L::off_row);         // [2][64] row scales of HA
+  df32* s_r = reinterpret_cast<df32*>(cta.smem + L::off_row + 2 * 4 * kKR);   // [2][64] 1/r or r
+  const float* s_col = reinterpret_cast<const float*>(cta.smem + L::off_col);   // [128] scales of T
+  float* s_max = reinterpret_cast<float*>(cta.smem + L::off_max);         // [GRP][64], then [64] scales of V
+  const int N = p.N, t = threadIdx.x, lane = t & 31, qd = (t >> 5) & 3, sub = t >> 7;
+  const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);
   const int ln = 32 * qd + lane, jl = ln % JC, j = 64 * c + jl;
   const int copy = ln / JC;                       // NT = 128: lanes 64.. hold no column
-  const bool live = copy < CP && j < N;
+  const bool mine = copy < CP && sub < NSUB, live = mine && j < N;
   // a column that is done keeps its Z: its right-hand side is zero in the cycles of the others
   const bool frozen = !RESID && from_b && live && s_done[j];
-  const int rg = copy * 2 + half, r0 = rg * RPT;  // this thread's rows of the tile
-  const uint32_t aT = smem_addr(sT), aH = smem_addr(sH), aV = smem_addr(sV);
+  const int rg = mine ? copy * NSUB + sub : 0, r0 = rg * RPT;   // this thread's rows of the tile
+  const uint32_t lead = warp == 0 ? elect_lane() : 0u;
+  const uint32_t aT = smem_addr(cta.smem + L::off_t), aH = smem_addr(cta.smem + L::off_h), aV = smem_addr(sV);
   constexpr uint32_t hst = (NT / 8) * 128;
   const float tsc = s_col[min(ln, L::TROWS - 1)] * 0x1p-16f;
   const df32 inv_nm1(1.0 / (double)(N - 1));
-  DFAcc acc[RESID ? 1 : JC / 2];
+  constexpr int NC = JC / 4;
+  DFAcc acc[RESID ? 1 : NC];
   float rr = 0.f;
   double rr64 = 0.0;
-  for (int64_t i0 = row0; i0 < row1 && cta.ok; i0 += kKR) {
-    slice_rows<NT, kKR, kKR, false>(p.HAdf, i0, row1, N, sH, s_row);
+  df32 x[PRE ? HI::N : 1][8];
+  float xs[PRE ? HI::N : 1];
+  auto load_x = [&](int64_t i0, int it, int slot) {
+    const int64_t i = i0 + HI::row(warp, lane, it);
+    const bool in = HI::live(warp, it) && i < row1;
+    load_row8(x[slot], p.HAdf, i, HI::col(warp, lane, it), N, in);
+    xs[slot] = p.hs[in ? i : 0];
+  };
+  auto load = [&](int64_t i0) {
+    if (PRE)
+#pragma unroll
+      for (int it = 0; it < HI::N; ++it) load_x(i0, it, it);
+  };
+  auto slice = [&](int b, int64_t i0, int rb) {   // image b, row data rb (two of them at every NT)
+#pragma unroll(PRE ? HI::N : 1)
+    for (int it = 0; it < HI::N; ++it) {
+      const int q = PRE ? it : 0;
+      if (!PRE) load_x(i0, it, 0);
+      // 1/xs: xs is a power of two (2^e -> 2^-e by the exponent field)
+      const float sc = __uint_as_float((254u << 23) - __float_as_uint(xs[q]));
+      if (HI::live(warp, it)) {
+        Slices8 sl;
+        sl.make(x[q], sc);
+        sl.store(cta.smem + L::off_h + b * (kSl * L::HP) + core_idx(HI::row(warp, lane, it), HI::col(warp, lane, it), NT) * 2,
+                 L::HP);
+      }
+    }
+    if (t < kKR) {
+      const int64_t i = i0 + t;
+      s_row[rb * kKR + t] = i < row1 ? p.hs[i] : 1.f;
+      s_r[rb * kKR + t] = i < row1 ? (RESID ? p.rdf[i] : p.rinv[i]) : df32(0.f, 0.f);
+    }
     fence_async_smem();
+  };
+  auto issue_u = [&](int b) {
+    if (warp == 0) {
+      tc_fence_after();
+      issue_levels<NT / 16, 4, SPL, kKR, false, false, L::TP, 256, L::HP, 256>(
+          cta.tmem, umma_desc(aT, 128, hst), umma_desc(aH + b * (kSl * L::HP), 128, hst), cta.mbar, lead);
+    }
+  };
+  int b = 0, rb = 0;
+  if (row0 < row1) {
+    load(row0);
+    slice(0, row0, 0);
     tc_fence_before();
     __syncthreads();
-    if (t == 0) {
-      tc_fence_after();
-      issue_levels<NT / 16, 4, SPL>(cta.tmem, kKR, umma_desc(aT, 128, hst), L::TP, 256, umma_desc(aH, 128, hst), L::HP, 256,
-                            sl_idesc(kKR, false, false));
-      umma_commit(cta.mbar);
-    }
-    // this thread's entries, in flight behind the products
-    df32 d[RPT], z[RPT];
+    issue_u(0);
+  }
+  for (int64_t i0 = row0; i0 < row1 && cta.ok; i0 += kKR, b ^= NB - 1, rb ^= 1) {
+    const bool more = i0 + kKR < row1;
+    // this thread's entries, in flight behind the products (NT = 128: four rows at a time)
+    constexpr int DE = PRE ? RPT : LC;
+    df32 d[DE], z[RESID ? DE : RPT];
+    auto entries = [&](int q0) {
 #pragma unroll
-    for (int q = 0; q < RPT; ++q) {
-      const int64_t i = i0 + r0 + q;
-      const bool in = live && i < row1;
-      d[q] = df32(0.f, 0.f);
-      z[q] = df32(0.f, 0.f);
-      if (in) {
-        if (!RESID && from_b) d[q] = df32(frozen ? 0.f : p.B[i * N + j], 0.f);
-        else d[q] = p.Ddf[i * N + j];
-        if (RESID || from_b) z[q] = p.Zdf[i * N + j];
+      for (int q = 0; q < DE; ++q) {
+        const int64_t i = i0 + r0 + q0 + q;
+        const bool in = live && i < row1;
+        const int64_t e = in ? i * N + j : 0;
+        df32 dv(0.f, 0.f), zv(0.f, 0.f);
+        if (!RESID && from_b) dv.hi = frozen ? 0.f : p.B[e];
+        else dv = p.Ddf[e];
+        if (RESID || from_b) zv = p.Zdf[e];
+        d[q] = in ? dv : df32(0.f, 0.f);
+        z[(RESID ? 0 : q0) + q] = in ? zv : df32(0.f, 0.f);
       }
+    };
+    entries(0);
+    if (RESID && NB == 2 && more) {
+      load(i0 + kKR);
+      slice(b ^ 1, i0 + kKR, rb ^ 1);
     }
     k_wait(cta);
     float mx = 0.f;
+    if (mine || 32 * qd < JC * CP) {   // (the second condition is uniform in the warp)
 #pragma unroll
-    for (int q0 = 0; q0 < RPT; q0 += 8) {
-      float lv[SPL ? 6 : 5][8];
-      tmem_ld_levels<(SPL ? 6 : 5)>(cta.tmem + ((uint32_t)(32 * qd) << 16) + (r0 & (kKR - 1)) + q0, kKR, lv);
+      for (int q0 = 0; q0 < RPT; q0 += LC) {
+        if (!PRE && q0 > 0) entries(q0);
+        float lv[SPL ? 6 : 5][LC];
+        tmem_ld_levels<(SPL ? 6 : 5), LC>(cta.tmem + ((uint32_t)(32 * qd) << 16) + r0 + q0, kKR, lv);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int rq = r0 + q0 + q;
-        const int64_t i = i0 + rq;
-        if (!(live && i < row1)) continue;
-        float s, l;
-        join_members<SPL>(lv, q, s, l);
-        const float f = tsc * s_row[rq];
-        const df32 u = df_fast2sum(s * f, l * f);
-        if (RESID) {
-          const df32 res = d[q0 + q] - fma(p.rdf[i], z[q0 + q], u * inv_nm1);
-          rr = __fmaf_rn(res.hi, res.hi, rr);
-          p.B[i * N + j] = res.hi;
-        } else {
-          const df32 zn = z[q0 + q] + (d[q0 + q] - u) * p.rinv[i];
-          p.Zdf[i * N + j] = zn;
-          // times the inverse of the HA row's scale: HA_ik z_ij = (HA_ik s_i) (z_ij / s_i)
-          z[q0 + q] = df32(zn.hi * s_row[rq], zn.lo * s_row[rq]);
-          mx = fmaxf(mx, fabsf(z[q0 + q].hi));
+        for (int q = 0; q < LC; ++q) {
+          const int rq = r0 + q0 + q;
+          const int64_t i = i0 + rq;
+          if (!(live && i < row1)) continue;
+          float s, l;
+          join_members<SPL>(lv, q, s, l);
+          const float sr = s_row[rb * kKR + rq], f = tsc * sr;
+          const df32 u = df_fast2sum(s * f, l * f);
+          const df32 ri = s_r[rb * kKR + rq];
+          const int qd0 = PRE ? q0 + q : q;
+          if (RESID) {
+            const df32 res = d[qd0] - fma(ri, z[RESID ? qd0 : 0], u * inv_nm1);
+            rr = __fmaf_rn(res.hi, res.hi, rr);
+            p.B[i * N + j] = res.hi;
+          } else {
+            const df32 zn = z[q0 + q] + (d[qd0] - u) * ri;
+            p.Zdf[i * N + j] = zn;
+            // times the HA row's scale: HA_ik z_ij = (HA_ik / s_i) (z_ij s_i)
+            z[q0 + q] = df32(zn.hi * sr, zn.lo * sr);
+            mx = fmaxf(mx, fabsf(z[q0 + q].hi));
+          }
         }
       }
     }
     if constexpr (RESID) {
       rr64 += (double)rr;
       rr = 0.f;
-      tc_fence_before();
-      __syncthreads();   // the tile image and tensor memory are rewritten by the next tile
+      if (NB == 1 && more) slice(0, i0 + kKR, rb ^ 1);
     } else {
-      if (copy < CP) s_max[rg * 64 + jl] = mx;
+      if (mine) s_max[rg * 64 + jl] = mx;
       __syncthreads();
-      float m2 = mx;
+      if (mine) {
+        float m2 = mx;
 #pragma unroll
-      for (int q = 0; q < 2 * CP; ++q) m2 = fmaxf(m2, s_max[q * 64 + jl]);
-      float sc, inv;
-      pow2_of(m2, sc, inv);
-      const float scale[8] = {sc, sc, sc, sc, sc, sc, sc, sc};
-      if (copy < CP)
+        for (int q = 0; q < GRP; ++q) m2 = fmaxf(m2, s_max[q * 64 + jl]);
+        float sc, inv;
+        pow2_of(m2, sc, inv);
 #pragma unroll
         for (int q0 = 0; q0 < RPT; q0 += 8) {
-          const df32 x[8] = {z[q0], z[q0 + 1], z[q0 + 2], z[q0 + 3], z[q0 + 4], z[q0 + 5], z[q0 + 6], z[q0 + 7]};
-          store_slices8(sV, L::VP, core_idx(jl, r0 + q0, kKR) * 2, x, scale);
+          const df32 y[8] = {z[q0], z[q0 + 1], z[q0 + 2], z[q0 + 3], z[q0 + 4], z[q0 + 5], z[q0 + 6], z[q0 + 7]};
+          Slices8 sl;
+          sl.make(y, sc);
+          sl.store(sV + core_idx(jl, r0 + q0, kKR) * 2, L::VP);
         }
-      if (rg == 0) s_max[2 * CP * 64 + jl] = inv;
+        if (rg == 0) s_max[GRP * 64 + jl] = inv;
+      }
       fence_async_smem();
       tc_fence_before();
       __syncthreads();
-      if (t == 0) {
+      if (warp == 0) {
         tc_fence_after();
         // T[k][jl]: A = the HA tile MN-major (M = k), B = the Z tile K-major
-        issue_levels<kKR / 16, 5, false>(cta.tmem, JC, umma_desc(aH, hst, 128), L::HP, 2 * hst, umma_desc(aV, 128, 1024),
-                               L::VP, 256, sl_idesc(JC, true, false));
-        umma_commit(cta.mbar);
+        issue_levels<kKR / 16, 5, false, JC, true, false, L::HP, 2 * hst, L::VP, 256>(
+            cta.tmem, umma_desc(aH + b * (kSl * L::HP), hst, 128), umma_desc(aV, 128, 1024), cta.mbar, lead);
+      }
+      if (NB == 2 && more) {
+        load(i0 + kKR);
+        slice(b ^ 1, i0 + kKR, rb ^ 1);
       }
       k_wait(cta);
       if (32 * qd < N) {   // uniform in the warp
-        constexpr int NC = JC / 2;
 #pragma unroll
-        for (int q0 = 0; q0 < NC; q0 += 8) {
-          float lv[kLv][8];
-          tmem_ld_levels<kLv>(cta.tmem + ((uint32_t)(32 * qd) << 16) + half * NC + q0, JC, lv);
+        for (int q0 = 0; q0 < NC; q0 += LC) {
+          float lv[kLv][LC];
+          tmem_ld_levels<kLv, LC>(cta.tmem + ((uint32_t)(32 * qd) << 16) + sub * NC + q0, JC, lv);
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
+          for (int q = 0; q < LC; ++q) {
             float s, l, tt, e;
             join_rows(lv, q, s, l);
-            const float f = s_max[2 * CP * 64 + half * NC + q0 + q] * 0x1p-16f;
+            const float f = s_max[GRP * 64 + sub * NC + q0 + q] * 0x1p-16f;
             df_two_sum(acc[q0 + q].s, s * f, tt, e);
             acc[q0 + q].s = tt;
             acc[q0 + q].c = __fadd_rn(acc[q0 + q].c, __fmaf_rn(l, f, e));
@@ -850,28 +1015,31 @@ __device__ __noinline__ void pass_rows(const KrylovParams& p, bool from_b, int c
           }
         }
       }
-      tc_fence_before();
-      __syncthreads();
+      if (NB == 1 && more) slice(0, i0 + kKR, rb ^ 1);
     }
+    tc_fence_before();
+    __syncthreads();
+    if (more) issue_u(NB == 2 ? b ^ 1 : 0);
   }
   if constexpr (RESID) {
-    double* red = reinterpret_cast<double*>(cta.smem + L::off_h);   // [2 CP][64]
+    double* red = reinterpret_cast<double*>(cta.smem + L::off_h);   // [GRP][64]
     __syncthreads();
-    if (copy < CP) red[rg * 64 + jl] = rr64;
+    if (mine) red[rg * 64 + jl] = rr64;
     __syncthreads();
     if (t < JC) {
       double s = 0.0;
-      for (int q = 0; q < 2 * CP; ++q) s += red[q * 64 + t];
+      for (int q = 0; q < GRP; ++q) s += red[q * 64 + t];
       rr_out[64 * c + t] = s;
     }
     __syncthreads();
   } else {
     const int NJ = min(JC, N);
 #pragma unroll
-    for (int q = 0; q < JC / 2; ++q) {
-      const int col = half * (JC / 2) + q;
+    for (int q = 0; q < NC; ++q) {
+      const int col = sub * NC + q;
       if (ln < N && col < NJ) out[ln * NJ + col] = acc[q].value();
     }
+    __syncthreads();
   }
 }
 
@@ -932,7 +1100,7 @@ __device__ void krylov_body(const KrylovParams& p, const int G, const int b, Gri
   auto column_totals = [&]() -> bool {
     if (t < NT) p.rrpart[((int64_t)par * G + b) * NT + t] = s_tmp[t];
     if (!bar.sync()) return false;
-    reduce_all<NT>(p.rrpart + (int64_t)par * G * NT, G, N, s_tmp, scratch);
+    total_columns<NT>(p.rrpart + (int64_t)par * G * NT, G, N, s_tmp, scratch);
     par ^= 1;
     return true;
   };
@@ -998,14 +1166,13 @@ __device__ void krylov_body(const KrylovParams& p, const int G, const int b, Gri
         const int k = g * KMat<NT>::KPT + q;
         M.k[q] = df32(0.f, 0.f);
         if (k < N && r < N) {
-          const float2 v = __ldcg(reinterpret_cast<const float2*>(p.Kred + k * N + r));
-          M.k[q] = df32(v.x, v.y);
+          M.k[q] = ld_df(p.Kred + k * N + r);
         }
       }
       const KColumns C{p.Fred, p.wred, s_bb, s_itol, s_done, s_bad, from_b ? nullptr : p.w0,
                        p.col_iters, !from_b, p.max_iter, p.status};
-      for (int j = b; j < N; j += 8 * G)
-        krylov_cg<NT>(M, N, df32(inv_nm1), j, G, min(8, (N - j + G - 1) / G), C, cta.smem);
+      for (int j = b; j < N; j += 16 * G)
+        krylov_cg<NT>(M, N, df32(inv_nm1), j, G, min(16, (N - j + G - 1) / G), C, cta.smem);
     }
     tick(PH_PASS);
     if (!(ok = bar.sync())) break;
@@ -1013,7 +1180,7 @@ __device__ void krylov_body(const KrylovParams& p, const int G, const int b, Gri
     // ---- pass Z and the reduction of T (W = T/(N-1))
     for (int c = c0; c < c1; ++c)
       if (has_rows) {
-        stage_columns<NT>(p.wred, c, N, cta.smem + L::off_t, reinterpret_cast<float*>(cta.smem + L::off_col));
+        stage_columns<NT, L::TROWS, JC>(p.wred, 64 * c, N, cta.smem + L::off_t, reinterpret_cast<float*>(cta.smem + L::off_col));
         __syncthreads();
         pass_rows<NT, false>(p, from_b, c, row0, row1, cta, s_done, part_of(rb, c), nullptr);
       }
@@ -1036,7 +1203,7 @@ __device__ void krylov_body(const KrylovParams& p, const int G, const int b, Gri
     __syncthreads();
     for (int c = c0; c < c1; ++c)
       if (has_rows) {
-        stage_columns<NT>(p.Tred, c, N, cta.smem + L::off_t, reinterpret_cast<float*>(cta.smem + L::off_col));
+        stage_columns<NT, L::TROWS, JC>(p.Tred, 64 * c, N, cta.smem + L::off_t, reinterpret_cast<float*>(cta.smem + L::off_col));
         __syncthreads();
         pass_rows<NT, true>(p, from_b, c, row0, row1, cta, s_done, nullptr, s_tmp);
       }

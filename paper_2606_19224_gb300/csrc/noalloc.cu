@@ -166,7 +166,7 @@ enkf_status enkf_analyze_noalloc(const enkf_config* cfg, const int32_t* d_rowptr
   }
   out_stats->refinements = st[1];
   out_stats->columns_converged = conv;
-  out_stats->grid_blocks = h.launch.G;
+  out_stats->grid_blocks = h.small_c ? c.N * h.small_c : h.launch.G;
   out_stats->warm_relres_max = -1.0;
   out_stats->warm_fallbacks = 0.0;
   enkf_status s = ENKF_OK;

@@ -495,19 +495,19 @@ __device__ void solve_body(const SolveParams& p, const int G, const int b, GridB
 // MODE 0: X_a = X_f + (X_f - xbar 1^T) W (CGD-EnKF, Fig. 2 / Algorithm 1);
 // MODE 1: X_a = X_f W (CGD-EnKF-Reduced, Algorithm 2 with W = V).
 // Row tiles of TRB rows staged in shared memory.
-// Row tiles tile0, tile0 + tstride, ... (TRB rows each) of the update.
-template <typename VT, int NT, int MODE = 0>
+// Row tiles tile0, tile0 + tstride, ... (TRB rows each) of the update by TH threads.
+template <typename VT, int NT, int MODE = 0, int TH = kThreads>
 __device__ __forceinline__ void update_rows(const VT* Xf, VT* Xa, const double* __restrict__ W,
                                             int64_t n, int N, int64_t tile0, int64_t tstride,
                                             unsigned char* smem) {
-  constexpr int LD = NT + 16 / (int)sizeof(VT), TRB = Tile<NT>::TRB, C4 = NT / 4;
+  constexpr int LD = NT + 16 / (int)sizeof(VT), TRB = Tile<NT>::TRB * (TH / kThreads), C4 = NT / 4;
   constexpr int NJ = NT / 4;
   VT* sW = reinterpret_cast<VT*>(smem);
   VT* sXb[2] = {sW + NT * LD, sW + NT * LD + TRB * LD};   // X_f row tiles, double-buffered
   VT* smean = sW + NT * LD + 2 * TRB * LD;
   const int t = threadIdx.x, tj = t % NJ, ti = t / NJ, j0 = tj * 4, r0 = ti * 4;
   const bool vec = (N & 3) == 0;
-  for (int e = t; e < NT * LD; e += kThreads) {
+  for (int e = t; e < NT * LD; e += TH) {
     const int k = e / LD, j = e % LD;
     sW[e] = (k < N && j < N) ? (VT)__ldcg(W + k * N + j) : VT(0);   // W may be written by this launch
   }
@@ -515,7 +515,7 @@ __device__ __forceinline__ void update_rows(const VT* Xf, VT* Xa, const double* 
   // N) when rows are 16-byte aligned (N % 4 == 0), else plain loads
   auto load_tile = [&](int64_t i0, VT* dst) {
 #pragma unroll
-    for (int c = t; c < TRB * C4; c += kThreads) {
+    for (int c = t; c < TRB * C4; c += TH) {
       const int ii = c / C4, c0 = (c % C4) * 4;
       const int64_t i = i0 + ii;
       const bool ok = i < n && c0 < N;
@@ -548,7 +548,7 @@ __device__ __forceinline__ void update_rows(const VT* Xf, VT* Xa, const double* 
     __syncthreads();
     // row means: four threads per row (consecutive rows on consecutive lane groups read
     // distinct banks), partial sums over k = g, g + 4, ..., added by two shuffle steps
-    for (int rr = t / 4; rr < TRB; rr += kThreads / 4) {
+    for (int rr = t / 4; rr < TRB; rr += TH / 4) {
       VT sm = VT(0);
       for (int k = t % 4; k < N; k += 4) sm += sX[rr * LD + k];
       sm += __shfl_xor_sync(0xffffffffu, sm, 1);
@@ -564,7 +564,7 @@ __device__ __forceinline__ void update_rows(const VT* Xf, VT* Xa, const double* 
       for (int y = 0; y < 4; ++y) xf[x][y] = sX[(r0 + x) * LD + j0 + y];
     __syncthreads();
     if (MODE == 0) {
-      for (int e = t; e < TRB * NT; e += kThreads) {
+      for (int e = t; e < TRB * NT; e += TH) {
         const int ii = e / NT, k = e % NT;
         if (k < N) sX[ii * LD + k] -= smean[ii];
       }
@@ -602,9 +602,10 @@ __device__ __forceinline__ void update_rows(const VT* Xf, VT* Xa, const double* 
   cp_async_wait<0>();
 }
 
-template <typename VT, int NT> __host__ __device__ constexpr int update_smem_bytes() {
+template <typename VT, int NT, int TH = kThreads> __host__ __device__ constexpr int update_smem_bytes() {
   constexpr int LD = NT + 16 / (int)sizeof(VT);
-  return (NT * LD + 2 * Tile<NT>::TRB * LD + Tile<NT>::TRB) * (int)sizeof(VT);
+  constexpr int TRB = Tile<NT>::TRB * (TH / kThreads);
+  return (NT * LD + 2 * TRB * LD + TRB) * (int)sizeof(VT);
 }
 
 }  // namespace enkf
