@@ -164,7 +164,7 @@ typedef struct enkf_stats {
   double true_relres_max;    /* max over columns of the FP64 true residual
                                 ||d_j - S z_j|| / ||d_j||; -1 when not computed          */
   int32_t columns_converged; /* columns that met tol                                     */
-  int32_t grid_blocks;       /* persistent-grid size used                                */
+  int32_t grid_blocks;       /* CTAs of the solve (small problems: of all column clusters) */
   double warm_relres_max;    /* learned warm start: max over columns of the start's
                                 relative residual ||d_j - S z0_j|| / ||d_j|| (evaluated in
                                 FP32 through the N x N identity below); -1 if off         */
@@ -185,7 +185,8 @@ enkf_status enkf_config_default(enkf_config* cfg, int64_t n, int64_t m, int32_t 
    (about 56 m N + 4 n N bytes in ENKF_FP32 mode, 4 m N more in the tensor-core modes,
    28 m N + 4 n N in either when the solve runs in Krylov coordinates (see precondition),
    48 m N + 8 n N in ENKF_FP64 mode, plus O(grid N^2); ENKF_CGD_REDUCED and ENKF_SENKF keep
-   no m x N arrays: 4 or 8 n N bytes plus O(grid N^2)). Errors: ENKF_ERR_INVALID_ARG (bad
+   no m x N arrays: 4 or 8 n N bytes plus O(grid N^2), with FP32 also up to 512 rows of HA and D per
+   SM). Errors: ENKF_ERR_INVALID_ARG (bad
    shape, column index outside [0, n), decreasing rowptr, r <= 0), ENKF_ERR_UNSUPPORTED
    (N > 128, unknown precision or variant, a variant other than ENKF_CGD in the BF16/FP16
    modes), ENKF_ERR_OOM, ENKF_ERR_CUDA. *out is NULL on error. */

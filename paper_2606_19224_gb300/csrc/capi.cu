@@ -197,9 +197,11 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
   Workspace& ws = h->ws;
   struct Alloc { void** p; size_t bytes; };
   // the Reduced variant and the sEnKF comparator work from one Gram pass and keep no m x N arrays
+  // (FP32: a chunk of rows per CTA)
   const bool gram = c.variant != ENKF_CGD;
   const bool krylov = h->krylov;
-  const int64_t tpart = gram ? (int64_t)enkf::reduced_grid(h) * 2 * c.N * c.N : krylov ? 1 : (int64_t)G * NE;
+  const bool gram_tc = gram && c.precision == ENKF_FP32;
+  const int64_t tpart = gram_tc || krylov ? 1 : gram ? (int64_t)enkf::reduced_grid(h) * 2 * c.N * c.N : (int64_t)G * NE;
   std::vector<Alloc> allocs = {
       {(void**)&ws.rowptr, sizeof(int32_t) * (c.m + 1)},
       {(void**)&ws.col, sizeof(int32_t) * (size_t)std::max<int64_t>(nnz, 1)},
@@ -220,6 +222,13 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
       {(void**)&ws.stage_y, sizeof(double) * c.m},
       {(void**)&ws.prof, sizeof(unsigned long long) * 8},
   };
+  if (gram_tc) {
+    allocs.push_back({&ws.rdf, 8 * (size_t)c.m});
+    allocs.push_back({&ws.rinv, 8 * (size_t)c.m});
+    allocs.push_back({&ws.rsq, 8 * (size_t)c.m});
+    allocs.push_back({&ws.kpart, enkf::gram_tc_part_bytes(h)});
+    allocs.push_back({&ws.HAdf, enkf::gram_tc_scratch_bytes(h)});
+  }
   if (krylov) {   // HA, D and Z in double-float and the residual: no CG vectors
     allocs.push_back({(void**)&ws.r32, sizeof(float) * c.m});
     allocs.push_back({(void**)&ws.B, vs * mN});
@@ -307,7 +316,7 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
   if (e == cudaSuccess && ws.HA16) e = cudaMemset(ws.HA16, 0, enkf::mixed_image_bytes(h));
   if (e == cudaSuccess) e = cudaMemset(ws.bar, 0, sizeof(unsigned) * 4);
   if (e == cudaSuccess) e = enkf::launch_convert_r(h);
-  if (e == cudaSuccess && krylov) e = enkf::launch_krylov_rows(h);
+  if (e == cudaSuccess && (krylov || gram_tc)) e = enkf::launch_krylov_rows(h);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) {
     free_workspace(ws);

@@ -244,6 +244,8 @@ cudaError_t launch_update_product(enkf_handle_s* h, const void* Xf, void* Xa);
 // kernels_reduced.cu: Gram pass + N x N CG of CGD-EnKF-Reduced; V lands in ws.W,
 // G in ws.Tred, M in ws.Wacc; the CTA partials use ws.Tpart ([reduced_grid][2 N N]).
 int reduced_grid(const enkf_handle_s* h);
+size_t gram_tc_part_bytes(const enkf_handle_s* h);      // FP32 ensembles: ws.kpart and the chunks in ws.HAdf
+size_t gram_tc_scratch_bytes(const enkf_handle_s* h);
 cudaError_t launch_reduced(enkf_handle_s* h, const void* Xf, const double* y, const double* E,
                            int emode, uint64_t seed, uint64_t counter);
 // kernels_batch.cu: batched analyses (planner, arena, persistent kernel, graph, tuner)

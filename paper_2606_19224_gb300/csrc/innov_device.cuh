@@ -196,14 +196,25 @@ __device__ __forceinline__ void innov_rows_f64(
   }
 }
 
-// What a solve in Krylov coordinates takes from the innovations besides HA and D (FP32 modes): a power
-// of two above the largest |HA| of each row, and the largest |HA_ik| / sqrt(r_i) of the problem
-// (atomic maximum of the float bits).
+// What the products on the tensor cores (krylov.cuh) take from the innovations besides HA and D (FP32
+// ensembles): a power of two above the largest |HA| of each row, and the largest |HA_ik| times the row's
+// weight 1/sqrt(r_i) (atomic maximum of the float bits). senkf: the weight is 1/sqrt(s_i) instead,
+// s_i = |HA_i|^2 + (N-1) r_i, and goes to wsq. Outputs are written from row row0 on.
 struct InnovRows {
   float* scale = nullptr;
   const df32* rsq = nullptr;
   unsigned* umax = nullptr;
+  int64_t row0 = 0;
+  bool senkf = false;
+  df32* wsq = nullptr;
 };
+// 1/sqrt(s) in double-float: the FP32 value y and two terms of its correction, e = 1 - s y^2 about 2^-22
+__device__ __forceinline__ df32 df_rsqrt(const df32& s) {
+  const float y = rsqrtf(s.hi);
+  const df32 y2 = df32(y, 0.f) * df32(y, 0.f);
+  const df32 e = df32(1.f, 0.f) - s * y2;
+  return df32(y, 0.f) + df32(y, 0.f) * (e * df32(fmaf(0.375f, e.hi, 0.5f), 0.f));
+}
 
 // The same rows for FP32 ensembles (the FP32 and tensor-core modes), in double-float (FP32
 // pair) arithmetic: this part issues FP32 at 64x its FP64 rate, and the FP64 version spends
@@ -235,8 +246,9 @@ __device__ __forceinline__ void innov_rows_df(
   // other lanes by shuffles: one FP64 evaluation per row instead of one per lane.
   for (int64_t i0 = i_begin + warp; i0 < i_end; i0 += 32 * nwarps) {
     const int64_t il = i0 + (int64_t)lane * nwarps;
-    df32 y_l, s_l, w_l;
+    df32 y_l, s_l, w_l, r_l;
     if (il < i_end) {
+      if (kr.senkf) r_l = df_from_double(r[il]);
       y_l = df_from_double(y[il]);
       if (emode == 2) s_l = df_from_double(sqrt(r[il]));
       const int kf = rowptr[il];
@@ -265,16 +277,35 @@ __device__ __forceinline__ void innov_rows_df(
       for (int o = 16; o > 0; o >>= 1)
         s = s + df32(__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o));
       const df32 zbar = s * inv_n;
-      if (kr.scale) {
+      if (kr.umax) {
         float rm = 0.f;
   #pragma unroll
         for (int q = 0; q < 4; ++q)
           if (2 * lane + (q & 1) + 64 * (q >> 1) < N) rm = fmaxf(rm, fabsf((z[q] - zbar).hi));
         rm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(rm)));
-        umax = fmaxf(umax, rm * kr.rsq[i].hi);
+        float wt;
+        if (kr.senkf) {
+          df32 q;
+  #pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (2 * lane + (e & 1) + 64 * (e >> 1) < N) {
+              const df32 hv = z[e] - zbar;
+              q = fma(hv, hv, q);
+            }
+  #pragma unroll
+          for (int o = 16; o > 0; o >>= 1)
+            q = q + df32(__shfl_xor_sync(0xffffffffu, q.hi, o), __shfl_xor_sync(0xffffffffu, q.lo, o));
+          const df32 rs = df_rsqrt(q + df32((float)(N - 1), 0.f) *
+                                           df32(__shfl_sync(0xffffffffu, r_l.hi, q32), __shfl_sync(0xffffffffu, r_l.lo, q32)));
+          if (lane == 0) kr.wsq[i - kr.row0] = rs;
+          wt = rs.hi;
+        } else {
+          wt = kr.rsq[i].hi;
+        }
+        umax = fmaxf(umax, rm * wt);
         // the exponent field of the power of two above rm (bounded away from both ends of the range)
         const int E = max(40, min(252, (int)(__float_as_uint(rm) >> 23)));
-        if (lane == 0) kr.scale[i] = __uint_as_float((uint32_t)(E + 1) << 23);
+        if (kr.scale && lane == 0) kr.scale[i - kr.row0] = __uint_as_float((uint32_t)(E + 1) << 23);
       }
   #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -282,13 +313,13 @@ __device__ __forceinline__ void innov_rows_df(
         if (jp >= N) continue;
         float nrm[2] = {0.f, 0.f};
         if (emode == 2) perturbation_pair_f32(i, jp, seed, counter, nrm[0], nrm[1]);
-        const int64_t e0 = i * N + jp;
+        const int64_t ein = i * N + jp, e0 = ein - kr.row0 * N;   // of the inputs, of the outputs
         df32 hv[2], dv[2];
   #pragma unroll
         for (int b = 0; b < 2; ++b) {
           df32 pert;
           if (jp + b < N) {
-            if (emode == 1) pert = df_from_double(E[e0 + b]);
+            if (emode == 1) pert = df_from_double(E[ein + b]);
             else if (emode == 2) pert = sr * df32(nrm[b], 0.f);
           }
           hv[b] = z[2 * h + b] - zbar;

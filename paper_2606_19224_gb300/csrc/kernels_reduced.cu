@@ -9,7 +9,8 @@
 //                          H touches, forms zbar, HA and Y~ for a tile of rows in shared
 //                          memory, and accumulates this CTA's partial HA^T R^{-1} [HA | Y~]
 //                          (the paper's "dominant cost ... formation of an N x N matrix",
-//                          Sec. 6.2.2); HA and D are never written to HBM
+//                          Sec. 6.2.2) in FP64; FP32 ensembles: gram_tc_kernel, the same products
+//                          on the tensor cores. HA and D stay on the chip
 //   reduced_sum_kernel     fixed-order sum of the CTA partials -> G, M (FP64)
 //   reduced_cg_kernel      one CTA per column of M; G staged in shared memory; FP64 CG
 //   update (kernels_fp.cu) X_a = X_f V (plain product mode)
@@ -23,9 +24,9 @@
 #include "common.cuh"
 #include "innov_device.cuh"
 #include "gram_stages.cuh"
+#include "krylov.cuh"
 
 #include <algorithm>
-#include <type_traits>
 
 namespace enkf {
 
@@ -44,34 +45,8 @@ template <> struct GramCfg<32> { static constexpr int KR = 32; };
 template <> struct GramCfg<64> { static constexpr int KR = 64; };
 template <> struct GramCfg<128> { static constexpr int KR = 32; };
 
-// A running product sum of the Gram pass: FP64 FMAs, or for double-float operands the
-// compensated pair of DFAcc (exact FP32 products, TwoSum, errors gathered in c), renormalised
-// every few terms. FP32 products of FP32-rounded anomalies would lose ~sqrt(m) in G's
-// cancelling off-diagonals; double-float keeps about 44 bits at 12 FP32 operations per term,
-// and FP32 issues at 64x the FP64 rate on this part.
-template <typename AT> struct GramAcc;
-template <> struct GramAcc<double> {
-  double v = 0.0;
-  __device__ __forceinline__ void add(double a, double b) { v = fma(a, b, v); }
-  __device__ __forceinline__ void renorm() {}
-  __device__ __forceinline__ double value() const { return v; }
-  __device__ __forceinline__ void set(double x) { v = x; }
-};
-template <> struct GramAcc<df32> {
-  DFAcc d;
-  __device__ __forceinline__ void add(const df32& a, const df32& b) { d.add(a, b); }
-  __device__ __forceinline__ void renorm() { d.renorm(); }
-  __device__ __forceinline__ double value() const { return (double)d.value(); }
-  __device__ __forceinline__ void set(double x) {
-    const df32 v(x);
-    d.s = v.hi;
-    d.c = v.lo;
-  }
-};
-
-// VT: type of X_f; AT: type of the staged tiles and the accumulators: FP64 for FP64
-// ensembles, double-float for FP32 ensembles (see GramAcc).
-template <typename VT, typename AT, int NT, bool SENKF = false>
+// FP64 ensembles. (FP32 ensembles: gram_tc_kernel below.)
+template <typename VT, int NT, bool SENKF = false>
 __global__ void __launch_bounds__(kThreads) reduced_gram_kernel(
     const VT* __restrict__ Xf, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
     const double* __restrict__ w, const double* __restrict__ y, const double* __restrict__ r,
@@ -83,16 +58,17 @@ __global__ void __launch_bounds__(kThreads) reduced_gram_kernel(
   constexpr int TPT = TILES >= kThreads ? TILES / kThreads : 1;   // tiles per thread
   constexpr int RG = TILES >= kThreads ? 1 : kThreads / TILES;    // row groups
   static_assert(TILES % kThreads == 0 || kThreads % TILES == 0, "mapping");
-  constexpr int TR = red_tr<AT, NT>();
+  constexpr int TR = red_tr<double, NT>();
   constexpr int QN = NT / 32;                 // members per lane in the gather (j = lane + 32 q)
   constexpr int QP = (NT + 63) / 64;          // perturbation pairs per lane (p = lane + 32 qp)
-  __shared__ __align__(16) AT sK[TR][NT];            // HA_i / r_i (sEnKF: HA_i / s_i)
-  __shared__ __align__(16) AT sJ[TR][JW];            // [HA_i | Y~_i] (sEnKF: D_i)
+  __shared__ __align__(16) double sK[TR][NT];            // HA_i / r_i (sEnKF: HA_i / s_i)
+  __shared__ __align__(16) double sJ[TR][JW];            // [HA_i | Y~_i] (sEnKF: D_i)
   __shared__ double sred[RG > 1 ? TILES * 16 : 1];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int g = t / (kThreads / RG);                 // row group of this thread
   const int kbase = blockIdx.y * KR;
-  GramAcc<AT> acc[TPT][4][4];   // zero-initialised
+  using AT = double;
+  double acc[TPT][4][4] = {};
 
   const double inv_n = 1.0 / (double)N;   // FP64 divisions run on the same pipe as the Gram's
                                            // FMAs: one per thread here, one per row below
@@ -129,7 +105,6 @@ __global__ void __launch_bounds__(kThreads) reduced_gram_kernel(
       const double yi = i < row1 ? y[i] : 0.0;
       const double sr = (emode == 2) ? sqrt(ri) : 0.0;
       // perturbation pair p (members 2p, 2p + 1) is drawn once, by lane p % 32 in slot p / 32
-      // (FP64 Box-Muller for FP64 ensembles, FP32 for FP32 ensembles, as in the innovations),
       // and handed to its two members' lanes with shuffles below
       double pr[QP][2];
 #pragma unroll
@@ -139,8 +114,7 @@ __global__ void __launch_bounds__(kThreads) reduced_gram_kernel(
         for (int qp = 0; qp < QP; ++qp) {
           const int jp = 2 * (lane + 32 * qp);
           if (jp < N) {
-            if constexpr (sizeof(VT) == 4) perturbation_pair_f32(i, jp, seed, counter, pr[qp][0], pr[qp][1]);
-            else perturbation_pair(i, jp, seed, counter, pr[qp][0], pr[qp][1]);
+            perturbation_pair(i, jp, seed, counter, pr[qp][0], pr[qp][1]);
           }
         }
       }
@@ -190,7 +164,6 @@ __global__ void __launch_bounds__(kThreads) reduced_gram_kernel(
     for (int q = 0; q < TPT; ++q) {
       const int u = (RG > 1) ? t % TILES : t + q * kThreads;
       const int tj = u % JG, tk = u / JG;
-      int terms = 0;
       for (int ii = g; ii < nrows; ii += RG) {
         AT a[4], b[4];
 #pragma unroll
@@ -200,18 +173,8 @@ __global__ void __launch_bounds__(kThreads) reduced_gram_kernel(
 #pragma unroll
         for (int x = 0; x < 4; ++x)
 #pragma unroll
-          for (int yy = 0; yy < 4; ++yy) acc[q][x][yy].add(a[x], b[yy]);
-        if ((++terms & 3) == 0) {
-#pragma unroll
-          for (int x = 0; x < 4; ++x)
-#pragma unroll
-            for (int yy = 0; yy < 4; ++yy) acc[q][x][yy].renorm();
-        }
+          for (int yy = 0; yy < 4; ++yy) acc[q][x][yy] = fma(a[x], b[yy], acc[q][x][yy]);
       }
-#pragma unroll
-      for (int x = 0; x < 4; ++x)
-#pragma unroll
-        for (int yy = 0; yy < 4; ++yy) acc[q][x][yy].renorm();
     }
   }
   // fold the row groups (fixed order) and write this CTA's partial rows (FP64)
@@ -223,14 +186,14 @@ __global__ void __launch_bounds__(kThreads) reduced_gram_kernel(
 #pragma unroll
         for (int x = 0; x < 4; ++x)
 #pragma unroll
-          for (int yy = 0; yy < 4; ++yy) sred[u * 16 + x * 4 + yy] = acc[0][x][yy].value();
+          for (int yy = 0; yy < 4; ++yy) sred[u * 16 + x * 4 + yy] = acc[0][x][yy];
       }
       __syncthreads();
       if (g == 0) {
 #pragma unroll
         for (int x = 0; x < 4; ++x)
 #pragma unroll
-          for (int yy = 0; yy < 4; ++yy) acc[0][x][yy].set(acc[0][x][yy].value() + sred[t * 16 + x * 4 + yy]);
+          for (int yy = 0; yy < 4; ++yy) acc[0][x][yy] += sred[t * 16 + x * 4 + yy];
       }
       __syncthreads();
     }
@@ -247,8 +210,114 @@ __global__ void __launch_bounds__(kThreads) reduced_gram_kernel(
       for (int yy = 0; yy < 4; ++yy) {
         const int k = kbase + tk * 4 + x, jj = tj * 4 + yy;
         const int half = jj / NT, j = jj % NT;
-        if (k < N && j < N) out[(int64_t)half * N * N + k * N + j] = acc[q][x][yy].value();
+        if (k < N && j < N) out[(int64_t)half * N * N + k * N + j] = acc[q][x][yy];
       }
+  }
+}
+
+// ------------------------------------------------------------------ FP32 ensembles: products on tensor cores
+// The same products from pass G of krylov.cuh (U^T U and U^T V with U = w HA, V = w D, w_i = 1/sqrt(r_i), or
+// 1/sqrt(s_i) for the sEnKF, whose W is U^T V; Reduced: Y~ = D + HA, so HA^T R^{-1} Y~ = F + K). A CTA forms HA
+// and D of up to kChunk of its rows with the innovations' double-float rows into a buffer of its own (it
+// stays in L2), then runs pass G over them. At m = 65,536, N = 64 the stage takes 0.16 ms, half of it the
+// innovations' rows; the products in double-float on the CUDA cores took 0.47 ms (Reduced) and 0.37 ms
+// (sEnKF), FP32-issue-bound at 12 operations per term.
+constexpr int kChunk = 512;
+
+struct GramTc {
+  const float* Xf;
+  const int32_t* rowptr;
+  const int32_t* col;
+  const double* w;
+  const double* y;
+  const double* r;
+  const double* E;
+  int emode;
+  uint64_t seed, counter;
+  int64_t m, rows_per;
+  int N;
+  bool senkf;
+  const df32* rsq;
+  df32* part;      // [grid][column groups][krylov_part(N)]
+  df32* scratch;   // [grid][2 chunk N + chunk]: HA, D and (sEnKF) the weights of a chunk (chunk % 8 == 0)
+  int64_t chunk;
+  int* status;
+};
+
+template <int NT>
+__global__ void __launch_bounds__(kKT, 1) gram_tc_kernel(GramTc g) {
+  using L = KLayout<NT>;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t mbar;
+  __shared__ uint32_t tmem_slot;
+  __shared__ unsigned umax;
+  KCta cta;
+  krylov_begin(cta, smem, &mbar, &tmem_slot, g.status);
+  const int N = g.N, t = threadIdx.x;
+  if (dynamic_smem_bytes() < (unsigned)L::bytes) {
+    if (t == 0) atomicOr(g.status, DS_SMEM);
+  } else {
+    const int ngr = (N + L::JC - 1) / L::JC;
+    const int64_t row0 = imin64(g.m, blockIdx.x * g.rows_per), row1 = imin64(g.m, row0 + g.rows_per);
+    df32* HA = g.scratch + (int64_t)blockIdx.x * (2 * g.chunk * N + g.chunk);
+    df32* D = HA + g.chunk * N;
+    df32* wsq = D + g.chunk * N;
+    KrylovParams p{};
+    p.N = N;
+    p.HAdf = HA;
+    p.Ddf = D;
+    p.umax = &umax;
+    int64_t c0 = row0;
+    do {   // at least once: a CTA without rows writes zeros
+      const int64_t c1 = imin64(row1, c0 + g.chunk);
+      if (t == 0) umax = 0u;
+      __syncthreads();
+      innov_rows_df<float>(g.Xf, g.rowptr, g.col, g.w, g.y, g.r, g.E, g.emode, g.seed, g.counter, g.m, N, nullptr, nullptr,
+                           nullptr, nullptr, nullptr, nullptr, 0, HA, D, c0, c1, t >> 5, kKT / 32, nullptr,
+                           InnovRows{nullptr, g.rsq, &umax, c0, g.senkf, wsq});
+      __syncthreads();
+      p.rsq = g.senkf ? wsq : g.rsq + c0;
+      for (int c = 0; c < ngr; ++c)
+        pass_gram<NT>(p, false, c, 0, c1 - c0, cta, g.part + ((int64_t)blockIdx.x * ngr + c) * krylov_part(N), c0 > row0);
+      c0 = c1;
+    } while (c0 < row1 && cta.ok);
+  }
+  krylov_end(cta);
+}
+
+// Fixed-order totals of the CTAs' partials, 32 consecutive entries (k, j) per CTA: G = I + K/(N-1) and
+// M = I + (F + K)/(N-1), or W = F.
+__global__ void __launch_bounds__(kThreads) gram_tc_sum_kernel(const df32* __restrict__ part, int grid, int N,
+                                                               double* __restrict__ Gm, double* __restrict__ Mm,
+                                                               double* __restrict__ W) {
+  constexpr int NW = kThreads / 32;
+  __shared__ double sk[NW][32], sf[NW][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
+  const int NJ = min(64, N), ngr = (N + 63) / 64, k = e / N, j = e % N, c = j / 64, jl = j % 64;
+  const int64_t PS = krylov_part(N);
+  df32 a, f;
+  if (e < N * N)
+#pragma unroll 4
+    for (int b = warp; b < grid; b += NW) {
+      const df32* src = part + ((int64_t)b * ngr + c) * PS + k * NJ + jl;
+      a = a + src[0];
+      f = f + src[(int64_t)N * NJ];
+    }
+  sk[warp][lane] = (double)a;
+  sf[warp][lane] = (double)f;
+  __syncthreads();
+  if (warp == 0 && e < N * N) {
+    double K = 0.0, F = 0.0;
+    for (int q = 0; q < NW; ++q) {
+      K += sk[q][lane];
+      F += sf[q][lane];
+    }
+    const double inv = 1.0 / (double)(N - 1), eye = k == j ? 1.0 : 0.0;
+    if (W) W[e] = F;
+    else {
+      Gm[e] = fma(K, inv, eye);
+      Mm[e] = fma(F + K, inv, eye);
+    }
   }
 }
 
@@ -412,26 +481,54 @@ __global__ void __launch_bounds__(kThreads) reduced_cg_kernel(
 }
 
 // ------------------------------------------------------------------ launchers
-template <typename VT, bool SENKF>
+template <bool SENKF>
 static cudaError_t gram_launch(enkf_handle_s* h, const void* Xf, const double* y, const double* E,
                                int emode, uint64_t seed, uint64_t counter, int grid) {
   const auto& c = h->cfg;
   auto& ws = h->ws;
   const int NT = c.N <= 32 ? 32 : (c.N <= 64 ? 64 : 128);
-  const VT* X = static_cast<const VT*>(Xf);
-  using AT = typename std::conditional<sizeof(VT) == 8, double, df32>::type;
+  const double* X = static_cast<const double*>(Xf);
   if (NT == 32)
-    reduced_gram_kernel<VT, AT, 32, SENKF><<<dim3(grid, 32 / GramCfg<32>::KR), kThreads, 0, h->stream>>>(X, ws.rowptr, ws.col, ws.w, y, ws.r, E, emode, seed, counter, c.m, c.N, ws.Tpart);
+    reduced_gram_kernel<double, 32, SENKF><<<dim3(grid, 32 / GramCfg<32>::KR), kThreads, 0, h->stream>>>(X, ws.rowptr, ws.col, ws.w, y, ws.r, E, emode, seed, counter, c.m, c.N, ws.Tpart);
   else if (NT == 64)
-    reduced_gram_kernel<VT, AT, 64, SENKF><<<dim3(grid, 64 / GramCfg<64>::KR), kThreads, 0, h->stream>>>(X, ws.rowptr, ws.col, ws.w, y, ws.r, E, emode, seed, counter, c.m, c.N, ws.Tpart);
+    reduced_gram_kernel<double, 64, SENKF><<<dim3(grid, 64 / GramCfg<64>::KR), kThreads, 0, h->stream>>>(X, ws.rowptr, ws.col, ws.w, y, ws.r, E, emode, seed, counter, c.m, c.N, ws.Tpart);
   else
-    reduced_gram_kernel<VT, AT, 128, SENKF><<<dim3(grid, 128 / GramCfg<128>::KR), kThreads, 0, h->stream>>>(X, ws.rowptr, ws.col, ws.w, y, ws.r, E, emode, seed, counter, c.m, c.N, ws.Tpart);
+    reduced_gram_kernel<double, 128, SENKF><<<dim3(grid, 128 / GramCfg<128>::KR), kThreads, 0, h->stream>>>(X, ws.rowptr, ws.col, ws.w, y, ws.r, E, emode, seed, counter, c.m, c.N, ws.Tpart);
   return cudaGetLastError();
 }
 
 int reduced_grid(const enkf_handle_s* h) {
-  const int64_t tiles = (h->cfg.m + 31) / 32;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)h->sms * 2));
+  const bool f64 = h->cfg.precision == ENKF_FP64;
+  const int64_t rows = f64 ? 32 : kKR;   // a tile
+  return (int)std::max<int64_t>(1, std::min<int64_t>((h->cfg.m + rows - 1) / rows, (int64_t)h->sms * (f64 ? 2 : 1)));
+}
+static int64_t gram_rows_per(const enkf_handle_s* h) { return (h->cfg.m + reduced_grid(h) - 1) / reduced_grid(h); }
+// (a multiple of 8: every CTA's buffers then begin on a 16-byte boundary, as the rows' stores need)
+static int64_t gram_chunk(const enkf_handle_s* h) { return std::min<int64_t>(kChunk, (gram_rows_per(h) + 7) / 8 * 8); }
+size_t gram_tc_part_bytes(const enkf_handle_s* h) {
+  return sizeof(df32) * (size_t)krylov_part(h->cfg.N) * ((h->cfg.N + 63) / 64) * reduced_grid(h);
+}
+size_t gram_tc_scratch_bytes(const enkf_handle_s* h) {
+  return sizeof(df32) * (size_t)reduced_grid(h) * gram_chunk(h) * (2 * h->cfg.N + 1);
+}
+
+template <int NT>
+static cudaError_t gram_tc_launch(const GramTc& g, int grid, cudaStream_t s) {
+  const cudaError_t e = cudaFuncSetAttribute(gram_tc_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, KLayout<NT>::bytes);
+  if (e != cudaSuccess) return e;
+  gram_tc_kernel<NT><<<grid, kKT, KLayout<NT>::bytes, s>>>(g);
+  return cudaGetLastError();
+}
+static cudaError_t launch_gram_tc(enkf_handle_s* h, const void* Xf, const double* y, const double* E, int emode,
+                                  uint64_t seed, uint64_t counter) {
+  const auto& c = h->cfg;
+  auto& ws = h->ws;
+  const GramTc g{static_cast<const float*>(Xf), ws.rowptr, ws.col, ws.w, y, ws.r, E, emode, seed, counter, c.m,
+                 gram_rows_per(h), c.N, c.variant == ENKF_SENKF, static_cast<const df32*>(ws.rsq),
+                 static_cast<df32*>(ws.kpart), static_cast<df32*>(ws.HAdf), gram_chunk(h), ws.status};
+  if (c.N <= 32) return gram_tc_launch<32>(g, reduced_grid(h), h->stream);
+  if (c.N <= 64) return gram_tc_launch<64>(g, reduced_grid(h), h->stream);
+  return gram_tc_launch<128>(g, reduced_grid(h), h->stream);
 }
 
 cudaError_t launch_gram_stage(enkf_handle_s* h, const void* Xf, const double* y, const double* E,
@@ -447,19 +544,22 @@ cudaError_t launch_gram_stage(enkf_handle_s* h, const void* Xf, const double* y,
     if (e == cudaSuccess) e = cudaMemsetAsync(ws.col_true, 0, sizeof(double) * c.N, h->stream);
   }
   if (e != cudaSuccess) return e;
-  const bool f64 = c.precision == ENKF_FP64;
-  if (senkf)
-    return f64 ? gram_launch<double, true>(h, Xf, y, E, emode, seed, counter, grid)
-               : gram_launch<float, true>(h, Xf, y, E, emode, seed, counter, grid);
-  return f64 ? gram_launch<double, false>(h, Xf, y, E, emode, seed, counter, grid)
-             : gram_launch<float, false>(h, Xf, y, E, emode, seed, counter, grid);
+  if (c.precision != ENKF_FP64) return launch_gram_tc(h, Xf, y, E, emode, seed, counter);
+  return senkf ? gram_launch<true>(h, Xf, y, E, emode, seed, counter, grid)
+               : gram_launch<false>(h, Xf, y, E, emode, seed, counter, grid);
 }
 
 cudaError_t launch_nxn_stage(enkf_handle_s* h) {
   const auto& c = h->cfg;
   auto& ws = h->ws;
   const int grid = reduced_grid(h);
-  if (c.variant == ENKF_SENKF) {
+  const bool f64 = c.precision == ENKF_FP64;
+  if (!f64) {
+    const bool senkf = c.variant == ENKF_SENKF;
+    gram_tc_sum_kernel<<<(c.N * c.N + 31) / 32, kThreads, 0, h->stream>>>(
+        static_cast<const df32*>(ws.kpart), grid, c.N, ws.Tred, ws.Wacc, senkf ? ws.W : nullptr);
+    if (senkf) return cudaGetLastError();
+  } else if (c.variant == ENKF_SENKF) {
     const int NN = c.N * c.N;
     senkf_sum_kernel<<<(NN + 31) / 32, kThreads, 0, h->stream>>>(ws.Tpart, grid, c.N, ws.W);
     return cudaGetLastError();
@@ -467,7 +567,7 @@ cudaError_t launch_nxn_stage(enkf_handle_s* h) {
   double* Gm = ws.Tred;            // N x N
   double* Mm = ws.Wacc;            // N x N
   const int NN2 = 2 * c.N * c.N;
-  reduced_sum_kernel<<<(NN2 + 31) / 32, kThreads, 0, h->stream>>>(ws.Tpart, grid, c.N, Gm, Mm);
+  if (f64) reduced_sum_kernel<<<(NN2 + 31) / 32, kThreads, 0, h->stream>>>(ws.Tpart, grid, c.N, Gm, Mm);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const size_t smem = sizeof(double) * ((size_t)c.N * (c.N + 1) + 5 * c.N + kThreads);

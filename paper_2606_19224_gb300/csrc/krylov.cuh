@@ -377,7 +377,8 @@ __device__ __forceinline__ void stage_columns(const df32* __restrict__ src, int 
 }
 
 // ------------------------------------------------------------------ pass G
-// The CTA's rows of U = R^{-1/2} HA and V = R^{-1/2} b (b = D, or the FP32 residual B), sliced per tile:
+// The CTA's rows of U = R^{-1/2} HA and V = R^{-1/2} b (b = D, or the FP32 residual B), sliced per tile
+// (add: onto what `out` holds):
 // U scaled by the power of two above its largest entry in the problem (the innovations record it),
 // each column of V by that of its largest entry in the tile; K = U^T U and F = U^T V accumulate over
 // the tiles in double-float registers. Column group c takes the columns [64 c, 64 c + JC) of K and F.
@@ -386,7 +387,7 @@ __device__ __forceinline__ void stage_columns(const df32* __restrict__ src, int 
 // the loads of the next tile are in flight behind the products.
 template <int NT>
 __device__ __noinline__ void pass_gram(const KrylovParams& p, bool from_b, int c, int64_t row0, int64_t row1,
-                                       KCta& cta, df32* __restrict__ out) {
+                                       KCta& cta, df32* __restrict__ out, bool add = false) {
   using L = KLayout<NT>;
   using UI = KItems<NT>;
   using VI = KItems<L::JC>;
@@ -551,13 +552,14 @@ __device__ __noinline__ void pass_gram(const KrylovParams& p, bool from_b, int c
   }
   // the CTA's partial: K[k][jl] at k NJ + jl, F[k][jl] behind it, then the column sums
   const int NJ = min(JC, N);
+  auto put = [&](int e, const df32& v) { out[e] = add ? out[e] + v : v; };
   if constexpr (NT == 128) {
     if (ln < N)
 #pragma unroll
       for (int q = 0; q < NC; ++q) {
         const int jl = sub * NC + q;
-        out[ln * NJ + jl] = acc[q].value();
-        out[N * NJ + ln * NJ + jl] = accF[q].value();
+        put(ln * NJ + jl, acc[q].value());
+        put(N * NJ + ln * NJ + jl, accF[q].value());
       }
   } else {
     // lanes [0, NT): K[k = lane][col]; lanes [NT, 2 NT): F^T[j = lane - NT][k = col]
@@ -565,8 +567,8 @@ __device__ __noinline__ void pass_gram(const KrylovParams& p, bool from_b, int c
     for (int q = 0; q < NC; ++q) {
       const int col = sub * NC + q;
       if (col < N) {
-        if (ln < N) out[ln * NJ + col] = acc[q].value();
-        else if (ln >= NT && ln - NT < N) out[N * NJ + col * NJ + (ln - NT)] = acc[q].value();
+        if (ln < N) put(ln * NJ + col, acc[q].value());
+        else if (ln >= NT && ln - NT < N) put(N * NJ + col * NJ + (ln - NT), acc[q].value());
       }
     }
   }
@@ -584,7 +586,7 @@ __device__ __noinline__ void pass_gram(const KrylovParams& p, bool from_b, int c
     const int which = t / JC, j = t % JC;
     double s = 0.0;
     for (int q = 0; q < 64; ++q) s += red[(which * 64 + q) * JC + j];
-    out[2 * N * NJ + which * 64 + j] = df32(s);
+    put(2 * N * NJ + which * 64 + j, df32(s));
   }
   __syncthreads();
 }
