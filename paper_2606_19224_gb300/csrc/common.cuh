@@ -228,7 +228,6 @@ cudaError_t launch_solve_mixed(enkf_handle_s* h);
 size_t mixed_image_bytes(const enkf_handle_s* h);   // tile images of HA (zeroed at create)
 // kernels_small.cu: one cluster of CTAs per column (0: not for this problem)
 int small_cluster(const enkf_config& c, int sms);
-cudaError_t plan_small(enkf_handle_s* h);
 cudaError_t launch_small(enkf_handle_s* h);
 // kernels_krylov.cu: CG preconditioned by R in the coordinates of its Krylov space
 bool krylov_config(const enkf_config& c);

@@ -116,7 +116,7 @@ cudaError_t plan_solve(enkf_handle_s* h) {
   h->launch.smem = smem;
   // a problem whose HA fits the shared memory of a few SMs is solved column by column
   h->small_c = small_cluster(h->cfg, h->sms);
-  return h->small_c ? plan_small(h) : cudaSuccess;
+  return cudaSuccess;
 }
 
 cudaError_t launch_innovations(enkf_handle_s* h, const void* Xf, const double* y, const double* E,

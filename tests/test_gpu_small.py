@@ -25,19 +25,24 @@ def _run(lib, p, prec, **cfg):
     return an, Xa.double().cpu().numpy(), an.stats()
 
 
-# (N, m, CTAs per column): one CTA and no row beyond it, odd sizes, two, four and eight CTAs with ragged blocks
-FP64 = [(2, 1, 1), (20, 20, 1), (33, 31, 1), (64, 150, 1), (128, 90, 1), (64, 301, 2), (37, 530, 4), (17, 1100, 8)]
+def _small(st, N):
+    # N clusters of one to eight CTAs (how many of a size are resident at once is the chip's)
+    return st["grid_blocks"] % N == 0 and 1 <= st["grid_blocks"] // N <= 8
+
+
+# one CTA per column and no row beyond it, odd sizes, up to eight CTAs with ragged blocks
+FP64 = [(2, 1), (20, 20), (33, 31), (64, 150), (128, 90), (64, 301), (37, 530), (17, 1100)]
 
 
 @pytest.mark.parametrize("pc", [0, 1])
-@pytest.mark.parametrize("N,m,C", FP64)
-def test_fp64_iterates_match_the_oracle(lib, N, m, C, pc):
+@pytest.mark.parametrize("N,m", FP64)
+def test_fp64_iterates_match_the_oracle(lib, N, m, pc):
     p = _problem(N, m, 31 * N + m, np.float64)
     if pc:
         p.r[:] = 0.8   # the oracle's CG is unpreconditioned: the same iterates when R is a multiple of I
     k = min(4, N)
     an, Xa, st = _run(lib, p, "fp64", fixed_iters=k, precondition=pc)
-    assert st["grid_blocks"] == N * C, st
+    assert _small(st, N), st
     E = oracle.obs_perturbations(6, 2, p.r, p.N)
     ref, info = oracle.cgd_enkf(p.Xf, p.rowptr, p.col, p.w, p.r, p.y, E, fixed_iters=k)
     _, D, Z, W = (t.cpu().numpy() for t in an.intermediates())
@@ -50,11 +55,11 @@ def test_fp64_iterates_match_the_oracle(lib, N, m, C, pc):
     assert oracle.rel_frobenius(X2, X3) <= 1e-8
 
 
-@pytest.mark.parametrize("N,m,C", [(2, 3, 1), (20, 200, 1), (128, 380, 1), (64, 900, 2), (37, 3001, 4), (18, 5003, 8)])
-def test_fp32_plain_analyses_match_the_exact_and_the_persistent_solve(lib, N, m, C):
+@pytest.mark.parametrize("N,m", [(2, 3), (20, 200), (31, 500), (128, 380), (64, 900), (37, 3001), (18, 5003)])
+def test_fp32_plain_analyses_match_the_exact_and_the_persistent_solve(lib, N, m):
     p = _problem(N, m, 17 * N + m, np.float32)
     an, Xa, st = _run(lib, p, "fp32", tol=1e-8)
-    assert st["grid_blocks"] == N * C and st["status"] == "ok" and st["true_relres_max"] <= 1e-8, st
+    assert _small(st, N) and st["status"] == "ok" and st["true_relres_max"] <= 1e-8, st
     E = oracle.obs_perturbations(6, 2, p.r, p.N)
     ref = oracle.enkf_exact(p.Xf.astype(np.float64), p.rowptr, p.col, p.w, p.r, p.y, E)
     assert oracle.rel_frobenius(Xa, ref) <= 1e-6
