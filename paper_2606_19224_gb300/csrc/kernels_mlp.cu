@@ -15,10 +15,10 @@
 // Parameter layout (FP32): per layer W [out][in] then b [out]; then mu_in [in], sd_in [in],
 // mu_out [out], sd_out [out].
 //
-// The dense layers are FP32 SIMT tiles (64 x 64 outputs per 256-thread CTA, K-steps of 16
-// staged in shared memory): the network is small (about 1.2 M weights) and its cost is a few
-// microseconds per analysis, far below the solve; the forward kernel also serves training
-// with a row gather and the input standardisation fused into its operand load.
+// The dense layers are FP32 tiles on the CUDA cores, split along K over thread-block clusters
+// (mlp_gemm_kernel).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 #include <string>
@@ -68,8 +68,15 @@ __device__ __forceinline__ float gelu_grad_f(float x) {
 
 // ------------------------------------------------------------------ tiled FP32 GEMM
 // C[M][N] = sum_k A(m, k) B(k, n) with A(m, k) = A[m * sam + k * sak] and
-// B(k, n) = B[k * sbk + n * sbn], and a fused epilogue.
-constexpr int GBM = 64, GBN = 64, GBK = 32;
+// B(k, n) = B[k * sbk + n * sbn], and a fused epilogue. One of sam, sak and one of sbk, sbn is 1.
+// 64 x 64 outputs per CTA of 256 threads, 4 x 4 per thread, operands staged 32 deep as [row][k] and read
+// four k at a time (12 shared-memory wavefronts against 16 FMA cycles per warp and four k); K is split over
+// a cluster of up to 8 CTAs, whose partial tiles are added in rank order through distributed shared memory:
+// the network's products have 8 to 136 tiles, which alone leave most SMs idle. Loads run along the
+// contiguous index of each operand. (32 x 32 tiles with 2 x 2 outputs per thread and loads along the
+// strided index took 15 to 30 us per product at batch 256, 1088 -> 512^3 -> 64; loss and gradient 345 us, now
+// 172.)
+constexpr int GT = 64, GBK = 32, GLD = GBK + 4;
 
 enum : int { EPI_HIDDEN = 0, EPI_OUT = 1, EPI_BWD = 2, EPI_STORE = 3 };
 
@@ -85,138 +92,201 @@ struct GemmArgs {
   float* C2;             // EPI_HIDDEN: GELU(C); EPI_OUT: raw output mu_out + sd_out * C
   const float* mu_out;
   const float* sd_out;
+  float* rowsum;         // EPI_STORE: sum_k A(m, k) (the bias gradient) or nullptr
+  int split;             // CTAs per cluster along K
 };
 
-// TM x TM outputs per thread, (16 TM) x (16 TM) per CTA: TM = 4 for large products, TM = 2
-// when the 64 x 64 grid would leave most SMs idle (the per-analysis inference, batch N).
-template <int EPI, int TM>
-__global__ void __launch_bounds__(256) mlp_gemm_kernel(const GemmArgs g) {
-  constexpr int BM = 16 * TM, BN = 16 * TM;
-  __shared__ float As[GBK][BM + 4];
-  __shared__ float Bs[GBK][BN + 4];
-  const int t = threadIdx.x, tx = t % 16, ty = t / 16;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  float acc[TM][TM] = {};
-  // the next k-step's operands are loaded into registers while the current one is computed
-  constexpr int LA = BM * GBK / 256, LB = GBK * BN / 256;
-  float ra[LA], rb[LB];
-  auto fetch = [&](int k0) {
+// rows [r0, r0 + 64) and k in [k0, k0 + 32) of an operand X(r, k) = X[r sr + k sk] as [row][k]
+struct GemmTile {
+  float v[8];
+  __device__ __forceinline__ void fetch(const float* X, int64_t sr, int64_t sk, int r0, int rows, int k0, int k1) {
+    const int t = threadIdx.x;
+    if (sk == 1) {   // along k: eight threads per row, four k each, rows t / 8 and t / 8 + 32
+      const bool vec = (sr & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
 #pragma unroll
-    for (int q = 0; q < LA; ++q) {
-      const int e = t + q * 256, mm = e / GBK, kk = e % GBK;
-      const int m = m0 + mm, k = k0 + kk;
-      ra[q] = (m < g.M && k < g.K) ? g.A[(int64_t)m * g.sam + (int64_t)k * g.sak] : 0.f;
-    }
+      for (int h = 0; h < 2; ++h) {
+        const int r = r0 + t / 8 + 32 * h, k = k0 + (t % 8) * 4;
+        const float* src = X + (int64_t)r * sr + k;
+        if (vec && r < rows && k + 4 <= k1) {
+          const float4 q = *reinterpret_cast<const float4*>(src);
+          v[4 * h] = q.x; v[4 * h + 1] = q.y; v[4 * h + 2] = q.z; v[4 * h + 3] = q.w;
+        } else {
 #pragma unroll
-    for (int q = 0; q < LB; ++q) {
-      const int e = t + q * 256, kk = e / BN, nn = e % BN;
-      const int k = k0 + kk, n = n0 + nn;
-      rb[q] = (k < g.K && n < g.N) ? g.B[(int64_t)k * g.sbk + (int64_t)n * g.sbn] : 0.f;
-    }
-  };
-  fetch(0);
-  for (int k0 = 0; k0 < g.K; k0 += GBK) {
+          for (int e = 0; e < 4; ++e) v[4 * h + e] = (r < rows && k + e < k1) ? src[e] : 0.f;
+        }
+      }
+    } else {         // along the rows: 64 consecutive threads per k, k t / 64 + 4 e
 #pragma unroll
-    for (int q = 0; q < LA; ++q) {
-      const int e = t + q * 256;
-      As[e % GBK][e / GBK] = ra[q];
-    }
-#pragma unroll
-    for (int q = 0; q < LB; ++q) {
-      const int e = t + q * 256;
-      Bs[e / BN][e % BN] = rb[q];
-    }
-    __syncthreads();
-    if (k0 + GBK < g.K) fetch(k0 + GBK);
-#pragma unroll
-    for (int kk = 0; kk < GBK; ++kk) {
-      float a[TM], b[TM];
-#pragma unroll
-      for (int x = 0; x < TM; ++x) a[x] = As[kk][ty * TM + x];
-#pragma unroll
-      for (int y = 0; y < TM; ++y) b[y] = Bs[kk][tx * TM + y];
-#pragma unroll
-      for (int x = 0; x < TM; ++x)
-#pragma unroll
-        for (int y = 0; y < TM; ++y) acc[x][y] = fmaf(a[x], b[y], acc[x][y]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int x = 0; x < TM; ++x) {
-    const int m = m0 + ty * TM + x;
-    if (m >= g.M) continue;
-#pragma unroll
-    for (int y = 0; y < TM; ++y) {
-      const int n = n0 + tx * TM + y;
-      if (n >= g.N) continue;
-      const int64_t e = (int64_t)m * g.N + n;
-      float v = acc[x][y];
-      if (EPI == EPI_HIDDEN) {
-        v += g.bias[n];
-        g.C[e] = v;
-        g.C2[e] = gelu_f(v);
-      } else if (EPI == EPI_OUT) {
-        v += g.bias[n];
-        g.C[e] = v;
-        if (g.C2) g.C2[e] = g.mu_out[n] + g.sd_out[n] * v;
-      } else if (EPI == EPI_BWD) {
-        g.C[e] = v * gelu_grad_f(g.zprev[e]);
-      } else {
-        g.C[e] = v;
+      for (int e = 0; e < 8; ++e) {
+        const int r = r0 + t % 64, k = k0 + t / 64 + 4 * e;
+        v[e] = (r < rows && k < k1) ? X[(int64_t)r * sr + (int64_t)k * sk] : 0.f;
       }
     }
   }
+  __device__ __forceinline__ void put(float* s, int64_t sk) const {
+    const int t = threadIdx.x;
+    if (sk == 1) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        *reinterpret_cast<float4*>(s + (t / 8 + 32 * h) * GLD + (t % 8) * 4) =
+            make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) s[(t % 64) * GLD + t / 64 + 4 * e] = v[e];
+    }
+  }
+};
+
+template <int EPI>
+__global__ void __launch_bounds__(256) mlp_gemm_kernel(const GemmArgs g) {
+  __shared__ __align__(16) float As[2][GT * GLD];
+  __shared__ __align__(16) float Bs[2][GT * GLD];
+  // this CTA's partial, column 64 the row sums of A: over the operands once they are used up
+  static_assert(sizeof(float) * GT * (GT + 1) <= sizeof(As), "the partial tile lies over As");
+  float (*tile)[GT + 1] = reinterpret_cast<float(*)[GT + 1]>(&As[0][0]);
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int S = g.split, rank = S > 1 ? (int)cluster.block_rank() : 0;
+  const int t = threadIdx.x, tx = t % 16, ty = t / 16;
+  const int m0 = blockIdx.y * GT, n0 = (blockIdx.x / S) * GT;
+  const int steps = (g.K + GBK - 1) / GBK, per = (steps + S - 1) / S;
+  const int kb = min(g.K, rank * per * GBK), ke = min(g.K, kb + per * GBK);
+  float acc[4][4] = {}, rs[4] = {};
+  const bool rows = EPI == EPI_STORE && g.rowsum != nullptr && n0 == 0 && tx == 0;
+  GemmTile ta, tb;
+  if (kb < ke) {
+    ta.fetch(g.A, g.sam, g.sak, m0, g.M, kb, ke);
+    tb.fetch(g.B, g.sbn, g.sbk, n0, g.N, kb, ke);
+  }
+  int buf = 0;
+  for (int k0 = kb; k0 < ke; k0 += GBK, buf ^= 1) {
+    ta.put(As[buf], g.sak);
+    tb.put(Bs[buf], g.sbk);
+    __syncthreads();   // (the other buffer's readers passed the barrier of the step before)
+    if (k0 + GBK < ke) {
+      ta.fetch(g.A, g.sam, g.sak, m0, g.M, k0 + GBK, ke);
+      tb.fetch(g.B, g.sbn, g.sbk, n0, g.N, k0 + GBK, ke);
+    }
+    // thread (ty, tx): rows ty + 16 x of A, columns tx + 16 y of B
+#pragma unroll
+    for (int kk = 0; kk < GBK; kk += 4) {
+      float4 a[4], b[4];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) a[x] = *reinterpret_cast<const float4*>(&As[buf][(ty + 16 * x) * GLD + kk]);
+#pragma unroll
+      for (int y = 0; y < 4; ++y) b[y] = *reinterpret_cast<const float4*>(&Bs[buf][(tx + 16 * y) * GLD + kk]);
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+          acc[x][y] = fmaf(a[x].x, b[y].x, acc[x][y]);
+          acc[x][y] = fmaf(a[x].y, b[y].y, acc[x][y]);
+          acc[x][y] = fmaf(a[x].z, b[y].z, acc[x][y]);
+          acc[x][y] = fmaf(a[x].w, b[y].w, acc[x][y]);
+        }
+      if (rows)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) rs[x] += (a[x].x + a[x].y) + (a[x].z + a[x].w);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+#pragma unroll
+    for (int y = 0; y < 4; ++y) tile[ty + 16 * x][tx + 16 * y] = acc[x][y];
+    if (tx == 0) tile[ty + 16 * x][GT] = rs[x];
+  }
+  if (S > 1) cluster.sync();
+  else __syncthreads();
+  // rank r finishes the rows [r 64/S, ...) of the tile
+  const int nrow = GT / S;
+  for (int e = t; e < nrow * GT; e += 256) {
+    const int r = rank * nrow + e / GT, c = e % GT, m = m0 + r, n = n0 + c;
+    float v = 0.f;
+    for (int q = 0; q < S; ++q) v += S > 1 ? *cluster.map_shared_rank(&tile[r][c], q) : tile[r][c];
+    if (m >= g.M || n >= g.N) continue;
+    const int64_t o = (int64_t)m * g.N + n;
+    if (EPI == EPI_HIDDEN) {
+      v += g.bias[n];
+      g.C[o] = v;
+      g.C2[o] = gelu_f(v);
+    } else if (EPI == EPI_OUT) {
+      v += g.bias[n];
+      g.C[o] = v;
+      if (g.C2) g.C2[o] = g.mu_out[n] + g.sd_out[n] * v;
+    } else if (EPI == EPI_BWD) {
+      g.C[o] = v * gelu_grad_f(g.zprev[o]);
+    } else {
+      g.C[o] = v;
+    }
+  }
+  if (EPI == EPI_STORE && g.rowsum != nullptr && n0 == 0 && t < nrow) {
+    const int r = rank * nrow + t;
+    float v = 0.f;
+    for (int q = 0; q < S; ++q) v += S > 1 ? *cluster.map_shared_rank(&tile[r][GT], q) : tile[r][GT];
+    if (m0 + r < g.M) g.rowsum[m0 + r] = v;
+  }
+  if (S > 1) cluster.sync();   // the tiles stay until every rank has read them
 }
 
 template <int EPI>
-static cudaError_t gemm(const GemmArgs& a, cudaStream_t s) {
-  const int64_t big = (int64_t)((a.N + GBN - 1) / GBN) * ((a.M + GBM - 1) / GBM);
-  if (big >= 128) {
-    dim3 grid((a.N + GBN - 1) / GBN, (a.M + GBM - 1) / GBM);
-    mlp_gemm_kernel<EPI, 4><<<grid, 256, 0, s>>>(a);
-  } else {
-    dim3 grid((a.N + 31) / 32, (a.M + 31) / 32);
-    mlp_gemm_kernel<EPI, 2><<<grid, 256, 0, s>>>(a);
-  }
-  return cudaGetLastError();
-}
-
-// Column sums of G [rows][cols] (the bias gradients), fixed order.
-__global__ void colsum_kernel(const float* __restrict__ G, int rows, int cols, float* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  float s = 0.f;
-  for (int r = 0; r < rows; ++r) s += G[(int64_t)r * cols + c];
-  out[c] = s;
+static cudaError_t gemm(GemmArgs a, cudaStream_t s) {
+  const int tn = (a.N + GT - 1) / GT, tm = (a.M + GT - 1) / GT, steps = (a.K + GBK - 1) / GBK;
+  // enough clusters to fill the chip once, and at least two steps along K per CTA
+  a.split = 1;
+  while (a.split < 8 && (int64_t)tn * tm * a.split * 2 <= 160 && steps >= 4 * a.split) a.split *= 2;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(tn * a.split, tm);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = a.split;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  void* args[] = {&a};
+  return cudaLaunchKernelExC(&cfg, (const void*)mlp_gemm_kernel<EPI>, args);
 }
 
 // Loss and output gradient: diff = y_std - (t - mu_out)/sd_out over B x out entries (rows of
-// T optionally gathered); G = 2 diff/(B out); loss = sum diff^2/(B out). One CTA, fixed order.
-__global__ void __launch_bounds__(256) mse_kernel(const float* __restrict__ Y, const float* __restrict__ T,
+// T optionally gathered); G = 2 diff/(B out); loss = sum diff^2/(B out). One cluster of 8 CTAs, fixed
+// order (a single CTA took 30 us for a batch of 256).
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(256) mse_kernel(const float* __restrict__ Y, const float* __restrict__ T,
                                                   const int32_t* __restrict__ rows, int B, int out,
                                                   const float* __restrict__ mu_out,
                                                   const float* __restrict__ sd_out, float* __restrict__ G,
                                                   float* __restrict__ loss) {
-  __shared__ double red[256];
+  __shared__ double red[8], part;
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
   const int t = threadIdx.x;
   const double inv = 1.0 / ((double)B * out);
+  const float g2 = (float)(2.0 * inv);
   double s = 0.0;
-  for (int64_t e = t; e < (int64_t)B * out; e += 256) {
+  for (int64_t e = (int64_t)blockIdx.x * 256 + t; e < (int64_t)B * out; e += 8 * 256) {
     const int b = (int)(e / out), o = (int)(e % out);
     const int64_t row = rows ? (int64_t)rows[b] : (int64_t)b;
     const float tt = (T[row * out + o] - mu_out[o]) / sd_out[o];
     const float d = Y[e] - tt;
-    G[e] = (float)(2.0 * inv) * d;
+    G[e] = g2 * d;
     s += (double)d * d;
   }
-  red[t] = s;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((t & 31) == 0) red[t / 32] = s;
   __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (t < w) red[t] += red[t + w];
-    __syncthreads();
+  if (t == 0) {
+    double v = 0.0;
+    for (int w = 0; w < 8; ++w) v += red[w];
+    part = v;
   }
-  if (t == 0 && loss) *loss = (float)(red[0] * inv);
+  cluster.sync();
+  if (blockIdx.x == 0 && t == 0 && loss) {
+    double v = 0.0;
+    for (int q = 0; q < 8; ++q) v += *cluster.map_shared_rank(&part, q);
+    *loss = (float)(v * inv);
+  }
+  cluster.sync();
 }
 
 __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
@@ -331,7 +401,7 @@ static cudaError_t mlp_loss_grad_impl(const MlpLayout& L, const float* P, const 
                                       cudaStream_t s) {
   cudaError_t e = mlp_forward_impl(L, P, X, rows, B, W, nullptr, s);
   if (e != cudaSuccess) return e;
-  mse_kernel<<<1, 256, 0, s>>>(W.Y, T, rows, B, L.out, P + L.mu_out, P + L.sd_out, W.G0, loss);
+  mse_kernel<<<8, 256, 0, s>>>(W.Y, T, rows, B, L.out, P + L.mu_out, P + L.sd_out, W.G0, loss);
   e = cudaGetLastError();
   float* g = W.G0;    // dL/dz of layer l, [B][fo]
   float* gn = W.G1;
@@ -349,10 +419,8 @@ static cudaError_t mlp_loss_grad_impl(const MlpLayout& L, const float* P, const 
     a.N = fi;
     a.K = B;
     a.C = grad + L.w_off[l];
+    a.rowsum = grad + L.b_off[l];   // db_l[o] = sum_b g[b][o]
     e = gemm<EPI_STORE>(a, s);
-    if (e != cudaSuccess) break;
-    colsum_kernel<<<(fo + 255) / 256, 256, 0, s>>>(g, B, fo, grad + L.b_off[l]);
-    e = cudaGetLastError();
     if (l > 0 && e == cudaSuccess) {
       // g_{l-1}[b][i] = (sum_o g[b][o] W_l[o][i]) GELU'(z_{l-1}[b][i])
       GemmArgs d{};
