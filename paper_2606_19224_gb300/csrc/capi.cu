@@ -222,6 +222,7 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
       {(void**)&ws.stage_y, sizeof(double) * c.m},
       {(void**)&ws.prof, sizeof(unsigned long long) * 8},
   };
+  if (gram && !gram_tc) allocs.push_back({&ws.HAdf, enkf::gram64_scratch_bytes(h)});
   if (gram_tc) {
     allocs.push_back({&ws.rdf, 8 * (size_t)c.m});
     allocs.push_back({&ws.rinv, 8 * (size_t)c.m});

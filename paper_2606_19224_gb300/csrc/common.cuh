@@ -239,10 +239,13 @@ cudaError_t launch_krylov(enkf_handle_s* h, int phase = 0, const float* w0 = nul
 cudaError_t launch_update(enkf_handle_s* h, const void* Xf, void* Xa);
 // kernels_update_tc.cu: X_a = X_f + A W on the tensor cores (FP32 ensembles)
 cudaError_t launch_update_tc(enkf_handle_s* h, const void* Xf, void* Xa);
+// kernels_update64.cu: X_a = X_f + A W, or X_f W (product), FP64 ensembles
+cudaError_t launch_update64(enkf_handle_s* h, const void* Xf, void* Xa, bool product);
 cudaError_t launch_update_product(enkf_handle_s* h, const void* Xf, void* Xa);
 // kernels_reduced.cu: Gram pass + N x N CG of CGD-EnKF-Reduced; V lands in ws.W,
 // G in ws.Tred, M in ws.Wacc; the CTA partials use ws.Tpart ([reduced_grid][2 N N]).
 int reduced_grid(const enkf_handle_s* h);
+size_t gram64_scratch_bytes(const enkf_handle_s* h);     // FP64 ensembles: a tile's rows per CTA in ws.HAdf
 size_t gram_tc_part_bytes(const enkf_handle_s* h);      // FP32 ensembles: ws.kpart and the chunks in ws.HAdf
 size_t gram_tc_scratch_bytes(const enkf_handle_s* h);
 cudaError_t launch_reduced(enkf_handle_s* h, const void* Xf, const double* y, const double* E,

@@ -104,7 +104,7 @@ __device__ __forceinline__ void innov_rows_f64(
     double* __restrict__ HA64, float* __restrict__ HA32, double* __restrict__ D,
     float* __restrict__ B32, __nv_bfloat16* __restrict__ HAb, __half* __restrict__ HAh,
     int split_lo, df32* __restrict__ HAdf, df32* __restrict__ Ddf, int64_t i_begin, int64_t i_end,
-    int64_t warp, int64_t nwarps) {
+    int64_t warp, int64_t nwarps, int64_t out0 = 0 /* outputs are written from row out0 on */) {
   // FP64 instructions are scarce on this part (2 per clock per SM): 1/N is applied as a
   // product and members 64..127 are skipped when N <= 64
   const int lane = threadIdx.x & 31;
@@ -135,13 +135,13 @@ __device__ __forceinline__ void innov_rows_f64(
       if (jp >= N) continue;
       double nrm[2] = {0.0, 0.0};
       if (emode == 2) perturbation_pair(i, jp, seed, counter, nrm[0], nrm[1]);
-      const int64_t e0 = i * N + jp;
+      const int64_t ein = i * N + jp, e0 = ein - out0 * N;   // of the inputs, of the outputs
       double hv[2], dv[2];
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
         double pert = 0.0;
         if (jp + b < N) {
-          if (emode == 1) pert = E[e0 + b];
+          if (emode == 1) pert = E[ein + b];
           else if (emode == 2) pert = sr * nrm[b];
         }
         hv[b] = z[2 * h + b] - zbar;

@@ -5,12 +5,11 @@
 //   M = I + P^T L^{-1} Y~  = I + HA^T R^{-1} Y~ / (N-1),  Y~ = (y - zbar) 1^T + E
 //   V = G^{-1} M by N independent CG recurrences (one per column of M), X_a = X_f V.
 //
-//   reduced_gram_kernel    one pass over the observation rows: gathers the rows of X_f that
-//                          H touches, forms zbar, HA and Y~ for a tile of rows in shared
-//                          memory, and accumulates this CTA's partial HA^T R^{-1} [HA | Y~]
-//                          (the paper's "dominant cost ... formation of an N x N matrix",
-//                          Sec. 6.2.2) in FP64; FP32 ensembles: gram_tc_kernel, the same products
-//                          on the tensor cores. HA and D stay on the chip
+//   gram64_kernel,         one pass over the observation rows: gathers the rows of X_f that
+//   gram_tc_kernel         H touches, forms HA and D for a tile of rows in a buffer that stays in L2,
+//   (FP64, FP32 ensembles) and accumulates this CTA's partial HA^T R^{-1} [HA | Y~] (the paper's
+//                          "dominant cost ... formation of an N x N matrix", Sec. 6.2.2) on the tensor
+//                          cores from exact integer slices
 //   reduced_sum_kernel     fixed-order sum of the CTA partials -> G, M (FP64)
 //   reduced_cg_kernel      one CTA per column of M; G staged in shared memory; FP64 CG
 //   update (kernels_fp.cu) X_a = X_f V (plain product mode)
@@ -25,194 +24,178 @@
 #include "innov_device.cuh"
 #include "gram_stages.cuh"
 #include "krylov.cuh"
+#include "slices64.cuh"
 
 #include <algorithm>
 
 namespace enkf {
 
-// observation rows staged per tile: keeps the static tiles (3 NT values per row) <= 40 KB
-template <typename VT, int NT> __host__ __device__ constexpr int red_tr() {
-  constexpr int t = 40960 / (3 * NT * (int)sizeof(VT));
-  return t >= 32 ? 32 : (t / 8) * 8;
-}
+// ------------------------------------------------------------------ FP64 ensembles
+// K = U^T U and F = U^T V with U = w HA, w_i = 1/sqrt(r_i) (sEnKF: 1/sqrt(s_i)) and V = w Y~ (sEnKF: w D), as
+// products of FP64 operands on the tensor cores (slices64.cuh). A CTA forms HA and D of a tile of up to 80
+// rows in a buffer of its own (it stays in L2), then cuts 64 columns at a time into digits, each column
+// scaled by the power of two above its largest entry in the tile: N <= 64, [U | V]^T U (M = 128: rows of
+// K, then of F^T); N > 64, [U_0 | U_1]^T times U_0, U_1, V_0 and V_1 in turn. At m = 10,000, N = 100 it takes
+// 171 us, most of them the FP64 logarithms and sines of the drawn perturbations; with the products on the FP64
+// unit it took 1.0 ms.
+struct Gram64 {
+  const double* Xf;
+  const int32_t* rowptr;
+  const int32_t* col;
+  const double* w;
+  const double* y;
+  const double* r;
+  const double* E;
+  int emode;
+  uint64_t seed, counter;
+  int64_t m, rows_per;
+  int N;
+  bool senkf;
+  double* part;      // [grid][2][N][N]: K and F (sEnKF: F in the first)
+  double* scratch;   // [grid][2][kDR][N]: HA and D of a tile
+  int* status;
+};
+struct Gram64Smem {
+  static constexpr int AP = kDR * 128 * 2, BR = kDg * 64 * 16;   // bytes per digit of A; per row group of B
+  static constexpr int off_b = kDg * AP, off_max = off_b + kDR / 8 * BR;
+  static constexpr int off_exp = off_max + kDR / 8 * 64 * 4, off_w = off_exp + 3 * 64 * 4, bytes = off_w + kDR * 8;
+  static_assert(bytes <= 226 * 1024, "shared memory");
+};
 
-// Gram pass. CTA (bx, ks) accumulates, over its block of observation rows, the rows
-// k in [ks*KR, (ks+1)*KR) of HA^T R^{-1} [HA | Y~] (an N x 2N product; sEnKF:
-// HA^T diag^{-1} D, N x N) with a 4x4 register tile per thread; gridDim.y = NT/KR splits k so
-// that a thread keeps at most 32 accumulators.
-template <int NT> struct GramCfg;
-template <> struct GramCfg<32> { static constexpr int KR = 32; };
-template <> struct GramCfg<64> { static constexpr int KR = 64; };
-template <> struct GramCfg<128> { static constexpr int KR = 32; };
-
-// FP64 ensembles. (FP32 ensembles: gram_tc_kernel below.)
-template <typename VT, int NT, bool SENKF = false>
-__global__ void __launch_bounds__(kThreads) reduced_gram_kernel(
-    const VT* __restrict__ Xf, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-    const double* __restrict__ w, const double* __restrict__ y, const double* __restrict__ r,
-    const double* __restrict__ E, int emode, uint64_t seed, uint64_t counter, int64_t m, int N,
-    double* __restrict__ part /* [gridDim.x][2][N][N]; sEnKF writes only [b][0] */) {
-  constexpr int KR = GramCfg<NT>::KR;
-  constexpr int JW = SENKF ? NT : 2 * NT;                          // columns of the right factor
-  constexpr int KG = KR / 4, JG = JW / 4, TILES = KG * JG;
-  constexpr int TPT = TILES >= kThreads ? TILES / kThreads : 1;   // tiles per thread
-  constexpr int RG = TILES >= kThreads ? 1 : kThreads / TILES;    // row groups
-  static_assert(TILES % kThreads == 0 || kThreads % TILES == 0, "mapping");
-  constexpr int TR = red_tr<double, NT>();
-  constexpr int QN = NT / 32;                 // members per lane in the gather (j = lane + 32 q)
-  constexpr int QP = (NT + 63) / 64;          // perturbation pairs per lane (p = lane + 32 qp)
-  __shared__ __align__(16) double sK[TR][NT];            // HA_i / r_i (sEnKF: HA_i / s_i)
-  __shared__ __align__(16) double sJ[TR][JW];            // [HA_i | Y~_i] (sEnKF: D_i)
-  __shared__ double sred[RG > 1 ? TILES * 16 : 1];
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int g = t / (kThreads / RG);                 // row group of this thread
-  const int kbase = blockIdx.y * KR;
-  using AT = double;
-  double acc[TPT][4][4] = {};
-
-  const double inv_n = 1.0 / (double)N;   // FP64 divisions run on the same pipe as the Gram's
-                                           // FMAs: one per thread here, one per row below
-  const int64_t rows_per = (m + gridDim.x - 1) / gridDim.x;
-  const int64_t row0 = min(m, (int64_t)blockIdx.x * rows_per);
-  const int64_t row1 = min(m, row0 + rows_per);
-  for (int64_t i0 = row0; i0 < row1; i0 += TR) {
-    __syncthreads();
-    // gather + anomalies + perturbed innovation-mean form: one warp per row of the tile
-    for (int ii = warp; ii < TR; ii += kThreads / 32) {
-      const int64_t i = i0 + ii;
-      double z[QN];
-#pragma unroll
-      for (int q = 0; q < QN; ++q) z[q] = 0.0;
-      if (i < row1) {
-        const int k0 = rowptr[i], k1 = rowptr[i + 1];
-        for (int k = k0; k < k1; ++k) {
-          const double wk = w[k];
-          const VT* xr = Xf + (int64_t)col[k] * N;
-#pragma unroll
-          for (int q = 0; q < QN; ++q) {
-            const int j = lane + 32 * q;
-            if (j < N) z[q] = fma(wk, (double)xr[j], z[q]);
-          }
-        }
-      }
-      double s = z[0];
-#pragma unroll
-      for (int q = 1; q < QN; ++q) s += z[q];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      const double zbar = s * inv_n;
-      const double ri = i < row1 ? r[i] : 1.0;
-      const double yi = i < row1 ? y[i] : 0.0;
-      const double sr = (emode == 2) ? sqrt(ri) : 0.0;
-      // perturbation pair p (members 2p, 2p + 1) is drawn once, by lane p % 32 in slot p / 32
-      // and handed to its two members' lanes with shuffles below
-      double pr[QP][2];
-#pragma unroll
-      for (int qp = 0; qp < QP; ++qp) pr[qp][0] = pr[qp][1] = 0.0;
-      if (emode == 2 && i < row1) {
-#pragma unroll
-        for (int qp = 0; qp < QP; ++qp) {
-          const int jp = 2 * (lane + 32 * qp);
-          if (jp < N) {
-            perturbation_pair(i, jp, seed, counter, pr[qp][0], pr[qp][1]);
-          }
-        }
-      }
-      double ha[QN], yt[QN];
-#pragma unroll
-      for (int q = 0; q < QN; ++q) {
-        const int j = lane + 32 * q;
-        // member j belongs to pair 16 q + (lane >> 1): lane 16 (q & 1) + (lane >> 1), slot q >> 1
-        const int src = 16 * (q & 1) + (lane >> 1);
-        const double n_even = __shfl_sync(0xffffffffu, pr[q >> 1][0], src);
-        const double n_odd = __shfl_sync(0xffffffffu, pr[q >> 1][1], src);
-        ha[q] = 0.0;
-        yt[q] = 0.0;
-        if (i < row1 && j < N) {
-          double pert = 0.0;
-          if (emode == 1) pert = E[i * N + j];
-          else if (emode == 2) pert = sr * ((lane & 1) ? n_odd : n_even);
-          ha[q] = z[q] - zbar;
-          yt[q] = (yi - zbar) + pert;
-        }
-      }
-      double wgt = ri;   // the row's weight divisor: r_i, or s_i = |HA_i|^2 + (N-1) r_i
-      if (SENKF) {
-        double hn = ha[0] * ha[0];
-#pragma unroll
-        for (int q = 1; q < QN; ++q) hn = fma(ha[q], ha[q], hn);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) hn += __shfl_xor_sync(0xffffffffu, hn, o);
-        wgt = hn + (double)(N - 1) * ri;
-      }
-      const double inv_w = 1.0 / wgt;
-#pragma unroll
-      for (int q = 0; q < QN; ++q) {
-        const int j = lane + 32 * q;   // < NT
-        sK[ii][j] = (AT)(ha[q] * inv_w);
-        if (SENKF) {
-          sJ[ii][j] = (AT)(yt[q] - ha[q]);
-        } else {
-          sJ[ii][j] = (AT)ha[q];
-          sJ[ii][NT + j] = (AT)yt[q];
-        }
-      }
-    }
-    __syncthreads();
-    const int nrows = (int)min((int64_t)TR, row1 - i0);
-#pragma unroll
-    for (int q = 0; q < TPT; ++q) {
-      const int u = (RG > 1) ? t % TILES : t + q * kThreads;
-      const int tj = u % JG, tk = u / JG;
-      for (int ii = g; ii < nrows; ii += RG) {
-        AT a[4], b[4];
-#pragma unroll
-        for (int x = 0; x < 4; ++x) a[x] = sK[ii][kbase + tk * 4 + x];
-#pragma unroll
-        for (int yy = 0; yy < 4; ++yy) b[yy] = sJ[ii][tj * 4 + yy];
-#pragma unroll
-        for (int x = 0; x < 4; ++x)
-#pragma unroll
-          for (int yy = 0; yy < 4; ++yy) acc[q][x][yy] = fma(a[x], b[yy], acc[q][x][yy]);
-      }
-    }
+__global__ void __launch_bounds__(kDT, 1) gram64_kernel(Gram64 g) {
+  using L = Gram64Smem;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t mbar;
+  __shared__ uint32_t tmem_slot;
+  KCta cta;
+  krylov_begin(cta, smem, &mbar, &tmem_slot, g.status);
+  const int N = g.N, t = threadIdx.x, lane = t & 31;
+  const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);
+  if (dynamic_smem_bytes() < (unsigned)L::bytes) {
+    if (t == 0) atomicOr(g.status, DS_SMEM);
+    krylov_end(cta);
+    return;
   }
-  // fold the row groups (fixed order) and write this CTA's partial rows (FP64)
-  if (RG > 1) {
+  int* s_max = reinterpret_cast<int*>(smem + L::off_max);      // [10][64] largest |x| (high words)
+  int* s_exp = reinterpret_cast<int*>(smem + L::off_exp);      // exponents of A's two column blocks and B's
+  double* s_w = reinterpret_cast<double*>(smem + L::off_w);
+  const bool wide = N > 64;
+  const int64_t row0 = imin64(g.m, blockIdx.x * g.rows_per), row1 = imin64(g.m, row0 + g.rows_per);
+  const int tiles = max(1, (int)((row1 - row0 + kDR - 1) / kDR)), per = (int)((row1 - row0 + tiles - 1) / tiles);
+  double* HA = g.scratch + (int64_t)blockIdx.x * 2 * kDR * N;
+  double* D = HA + kDR * N;
+  double* out = g.part + (int64_t)blockIdx.x * 2 * N * N;
+  const uint32_t base = smem_addr(smem), lead = warp == 0 ? elect_lane() : 0u;
+  // this thread's item: row r and columns [cc, cc + 8) of a block of 64
+  const int r = warp / 2 * 8 + (lane & 7), cc = warp % 2 * 32 + (lane >> 3) * 8;
+  for (int tile = 0; tile < tiles && cta.ok; ++tile) {   // at least one: a CTA without rows writes zeros
+    const int64_t c0 = imin64(row1, row0 + (int64_t)tile * per);
+    const int rows = (int)(imin64(row1, c0 + per) - c0), ks = (rows + 15) / 16;
+    innov_rows_f64<double>(g.Xf, g.rowptr, g.col, g.w, g.y, g.r, g.E, g.emode, g.seed, g.counter, g.m, N, HA, nullptr, D,
+                           nullptr, nullptr, nullptr, 0, nullptr, nullptr, c0, c0 + rows, warp, kDT / 32, c0);
     __syncthreads();
-    for (int gg = 1; gg < RG; ++gg) {
-      if (g == gg) {
-        const int u = t % TILES;
+    if (g.senkf) {
+      for (int i = warp; i < rows; i += kDT / 32) {
+        double q = 0.0;
+        for (int k = lane; k < N; k += 32) q = fma(HA[i * N + k], HA[i * N + k], q);
 #pragma unroll
-        for (int x = 0; x < 4; ++x)
-#pragma unroll
-          for (int yy = 0; yy < 4; ++yy) sred[u * 16 + x * 4 + yy] = acc[0][x][yy];
+        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        if (lane == 0) s_w[i] = 1.0 / sqrt(q + (double)(N - 1) * g.r[c0 + i]);
       }
+    } else if (t < rows) {
+      s_w[t] = 1.0 / sqrt(g.r[c0 + t]);
+    }
+    __syncthreads();
+    // columns [64 c, 64 c + 64) of U (v = false) or V into operand A's block `to_a` (if >= 0) and operand B
+    auto block = [&](bool v, int c, int to_a, bool to_b) {
+      double x[8];
+      int E[8];
+      const double wr = r < rows ? s_w[r] : 0.0;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int k = 64 * c + cc + e;
+        const bool in = r < rows && k < N;
+        double q = 0.0;
+        if (in) {
+          const double* at = HA + r * N + k;
+          q = !v ? at[0] : g.senkf ? at[kDR * N] : at[kDR * N] + at[0];
+        }
+        x[e] = q * wr;
+        E[e] = dg_abs_hi(x[e]);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) E[e] = max(E[e], __shfl_xor_sync(0xffffffffu, E[e], o));
+      }
+      if ((lane & 7) == 0)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s_max[warp / 2 * 64 + cc + e] = E[e];
+      tc_fence_before();
+      __syncthreads();   // (and the reads of the last product's sums and scales are done)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        int mx = 0;
+#pragma unroll
+        for (int b = 0; b < kDR / 8; ++b) mx = max(mx, s_max[b * 64 + cc + e]);
+        E[e] = dg_exp(mx);
+        if (r == 0) {
+          if (to_a >= 0) s_exp[to_a * 64 + cc + e] = E[e];
+          if (to_b) s_exp[128 + cc + e] = E[e];
+        }
+      }
+      Digits8 dg;
+      dg.make(x, E);
+      if (to_a >= 0) dg.store(smem + ((r >> 3) * 16 + to_a * 8 + (cc >> 3)) * 128 + (r & 7) * 16, L::AP);
+      if (to_b) dg.store(smem + L::off_b + (r >> 3) * L::BR + (cc >> 3) * 128 + (r & 7) * 16, 64 * 16);
+      fence_async_smem();
       __syncthreads();
-      if (g == 0) {
-#pragma unroll
-        for (int x = 0; x < 4; ++x)
-#pragma unroll
-          for (int yy = 0; yy < 4; ++yy) acc[0][x][yy] += sred[t * 16 + x * 4 + yy];
+    };
+    // A^T B, then put(lane row, column, value)
+    auto product = [&](auto put) {
+      if (warp == 0) {
+        tc_fence_after();
+        dg_issue<true, true, L::AP, 2 * 2048, 64 * 16, 2 * L::BR>(cta.tmem, umma_desc(base, 2048, 128),
+                                                                 umma_desc(base + L::off_b, L::BR, 128), max(ks, 1), false, cta.mbar, lead);
       }
-      __syncthreads();
+      k_wait(cta);
+      if (warp < 16) {
+        const int qd = warp & 3, ln = 32 * qd + lane, ea = s_exp[ln];
+#pragma unroll 1
+        for (int q0 = (warp >> 2) * 16; q0 < (warp >> 2) * 16 + 16; q0 += 4) {
+          float lv[kDl][4];
+          tmem_ld_levels<kDl, 4>(cta.tmem + ((uint32_t)(32 * qd) << 16) + q0, 64, lv);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) put(ln, q0 + q, dg_value(dg_join(lv, q), ea, s_exp[128 + q0 + q]));
+        }
+      }
+    };
+    auto add = [&](int64_t e, double v) { out[e] = tile > 0 ? out[e] + v : v; };
+    const int64_t fo = g.senkf ? 0 : (int64_t)N * N;
+    if (!wide) {
+      block(false, 0, 0, true);
+      block(true, 0, 1, false);
+      product([&](int ln, int c, double v) {
+        if (c >= N) return;
+        if (ln < 64) {
+          if (ln < N && !g.senkf) add(c * N + ln, v);   // K is symmetric
+        } else if (ln - 64 < N) {
+          add(fo + c * N + (ln - 64), v);               // F[c][ln - 64]
+        }
+      });
+    } else {
+      block(false, 0, 0, !g.senkf);
+      block(false, 1, 1, false);
+      for (int q = g.senkf ? 2 : 0; q < 4; ++q) {
+        if (q > 0) block(q >= 2, q & 1, -1, true);
+        product([&](int ln, int c, double v) {
+          const int j = 64 * (q & 1) + c;
+          if (ln >= N || j >= N) return;
+          if (q < 2) add(j * N + ln, v);
+          else add(fo + ln * N + j, v);
+        });
+      }
     }
+    __syncthreads();   // s_w and the buffer are rewritten
   }
-  if (RG > 1 && g != 0) return;
-  double* out = part + (int64_t)blockIdx.x * 2 * N * N;
-#pragma unroll
-  for (int q = 0; q < TPT; ++q) {
-    const int u = (RG > 1) ? t % TILES : t + q * kThreads;
-    const int tj = u % JG, tk = u / JG;
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-      for (int yy = 0; yy < 4; ++yy) {
-        const int k = kbase + tk * 4 + x, jj = tj * 4 + yy;
-        const int half = jj / NT, j = jj % NT;
-        if (k < N && j < N) out[(int64_t)half * N * N + k * N + j] = acc[q][x][yy];
-      }
-  }
+  krylov_end(cta);
 }
 
 // ------------------------------------------------------------------ FP32 ensembles: products on tensor cores
@@ -481,30 +464,15 @@ __global__ void __launch_bounds__(kThreads) reduced_cg_kernel(
 }
 
 // ------------------------------------------------------------------ launchers
-template <bool SENKF>
-static cudaError_t gram_launch(enkf_handle_s* h, const void* Xf, const double* y, const double* E,
-                               int emode, uint64_t seed, uint64_t counter, int grid) {
-  const auto& c = h->cfg;
-  auto& ws = h->ws;
-  const int NT = c.N <= 32 ? 32 : (c.N <= 64 ? 64 : 128);
-  const double* X = static_cast<const double*>(Xf);
-  if (NT == 32)
-    reduced_gram_kernel<double, 32, SENKF><<<dim3(grid, 32 / GramCfg<32>::KR), kThreads, 0, h->stream>>>(X, ws.rowptr, ws.col, ws.w, y, ws.r, E, emode, seed, counter, c.m, c.N, ws.Tpart);
-  else if (NT == 64)
-    reduced_gram_kernel<double, 64, SENKF><<<dim3(grid, 64 / GramCfg<64>::KR), kThreads, 0, h->stream>>>(X, ws.rowptr, ws.col, ws.w, y, ws.r, E, emode, seed, counter, c.m, c.N, ws.Tpart);
-  else
-    reduced_gram_kernel<double, 128, SENKF><<<dim3(grid, 128 / GramCfg<128>::KR), kThreads, 0, h->stream>>>(X, ws.rowptr, ws.col, ws.w, y, ws.r, E, emode, seed, counter, c.m, c.N, ws.Tpart);
-  return cudaGetLastError();
-}
-
 int reduced_grid(const enkf_handle_s* h) {
   const bool f64 = h->cfg.precision == ENKF_FP64;
   const int64_t rows = f64 ? 32 : kKR;   // a tile
-  return (int)std::max<int64_t>(1, std::min<int64_t>((h->cfg.m + rows - 1) / rows, (int64_t)h->sms * (f64 ? 2 : 1)));
+  return (int)std::max<int64_t>(1, std::min<int64_t>((h->cfg.m + rows - 1) / rows, h->sms));
 }
 static int64_t gram_rows_per(const enkf_handle_s* h) { return (h->cfg.m + reduced_grid(h) - 1) / reduced_grid(h); }
 // (a multiple of 8: every CTA's buffers then begin on a 16-byte boundary, as the rows' stores need)
 static int64_t gram_chunk(const enkf_handle_s* h) { return std::min<int64_t>(kChunk, (gram_rows_per(h) + 7) / 8 * 8); }
+size_t gram64_scratch_bytes(const enkf_handle_s* h) { return sizeof(double) * (size_t)reduced_grid(h) * 2 * kDR * h->cfg.N; }
 size_t gram_tc_part_bytes(const enkf_handle_s* h) {
   return sizeof(df32) * (size_t)krylov_part(h->cfg.N) * ((h->cfg.N + 63) / 64) * reduced_grid(h);
 }
@@ -531,12 +499,23 @@ static cudaError_t launch_gram_tc(enkf_handle_s* h, const void* Xf, const double
   return gram_tc_launch<128>(g, reduced_grid(h), h->stream);
 }
 
+static cudaError_t launch_gram64(enkf_handle_s* h, const void* Xf, const double* y, const double* E, int emode,
+                                 uint64_t seed, uint64_t counter) {
+  const auto& c = h->cfg;
+  auto& ws = h->ws;
+  const Gram64 g{static_cast<const double*>(Xf), ws.rowptr, ws.col, ws.w, y, ws.r, E, emode, seed, counter, c.m,
+                 gram_rows_per(h), c.N, c.variant == ENKF_SENKF, ws.Tpart, static_cast<double*>(ws.HAdf), ws.status};
+  const cudaError_t e = cudaFuncSetAttribute(gram64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Gram64Smem::bytes);
+  if (e != cudaSuccess) return e;
+  gram64_kernel<<<reduced_grid(h), kDT, Gram64Smem::bytes, h->stream>>>(g);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_gram_stage(enkf_handle_s* h, const void* Xf, const double* y, const double* E,
                               int emode, uint64_t seed, uint64_t counter) {
   const auto& c = h->cfg;
   auto& ws = h->ws;
   const bool senkf = c.variant == ENKF_SENKF;
-  const int grid = reduced_grid(h);
   cudaError_t e = cudaMemsetAsync(ws.status, 0, 4 * sizeof(int32_t), h->stream);
   if (senkf) {   // no solve: the per-column statistics read back as 0 iterations, residual 0
     if (e == cudaSuccess) e = cudaMemsetAsync(ws.col_iters, 0, sizeof(int32_t) * c.N, h->stream);
@@ -544,9 +523,8 @@ cudaError_t launch_gram_stage(enkf_handle_s* h, const void* Xf, const double* y,
     if (e == cudaSuccess) e = cudaMemsetAsync(ws.col_true, 0, sizeof(double) * c.N, h->stream);
   }
   if (e != cudaSuccess) return e;
-  if (c.precision != ENKF_FP64) return launch_gram_tc(h, Xf, y, E, emode, seed, counter);
-  return senkf ? gram_launch<true>(h, Xf, y, E, emode, seed, counter, grid)
-               : gram_launch<false>(h, Xf, y, E, emode, seed, counter, grid);
+  return c.precision == ENKF_FP64 ? launch_gram64(h, Xf, y, E, emode, seed, counter)
+                                  : launch_gram_tc(h, Xf, y, E, emode, seed, counter);
 }
 
 cudaError_t launch_nxn_stage(enkf_handle_s* h) {
