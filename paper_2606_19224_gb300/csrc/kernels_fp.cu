@@ -208,22 +208,20 @@ cudaError_t launch_solve(enkf_handle_s* h) {
                                      h->launch.smem, h->stream);
 }
 
-template <int MODE>
-static cudaError_t launch_update_mode(enkf_handle_s* h, const void* Xf, void* Xa) {
+cudaError_t launch_update(enkf_handle_s* h, const void* Xf, void* Xa) {
+  // the A W product on the tensor cores (kernels_update_tc.cu, kernels_update64.cu)
+  return h->cfg.precision != ENKF_FP64 ? launch_update_tc(h, Xf, Xa) : launch_update64(h, Xf, Xa, false);
+}
+
+// X_a = X_f V (Reduced)
+cudaError_t launch_update_product(enkf_handle_s* h, const void* Xf, void* Xa) {
   const auto& c = h->cfg;
+  if (c.precision == ENKF_FP64) return launch_update64(h, Xf, Xa, true);
   const int NT = h->launch.NT;
-  const bool fp64 = c.precision == ENKF_FP64;
   const int TRB = NT == 32 ? Tile<32>::TRB : (NT == 64 ? Tile<64>::TRB : Tile<128>::TRB);
   const int tiles = (int)std::min<int64_t>((c.n + TRB - 1) / TRB, (int64_t)h->sms * 8);
-  void* fn;
-  int smem;
-  if (fp64) {
-    fn = NT == 32 ? (void*)update_kernel<double, 32, MODE> : NT == 64 ? (void*)update_kernel<double, 64, MODE> : (void*)update_kernel<double, 128, MODE>;
-    smem = NT == 32 ? update_smem_bytes<double, 32>() : NT == 64 ? update_smem_bytes<double, 64>() : update_smem_bytes<double, 128>();
-  } else {
-    fn = NT == 32 ? (void*)update_kernel<float, 32, MODE> : NT == 64 ? (void*)update_kernel<float, 64, MODE> : (void*)update_kernel<float, 128, MODE>;
-    smem = NT == 32 ? update_smem_bytes<float, 32>() : NT == 64 ? update_smem_bytes<float, 64>() : update_smem_bytes<float, 128>();
-  }
+  void* fn = NT == 32 ? (void*)update_kernel<float, 32, 1> : NT == 64 ? (void*)update_kernel<float, 64, 1> : (void*)update_kernel<float, 128, 1>;
+  const int smem = NT == 32 ? update_smem_bytes<float, 32>() : NT == 64 ? update_smem_bytes<float, 64>() : update_smem_bytes<float, 128>();
   cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
   const double* W = h->ws.W;
@@ -231,16 +229,6 @@ static cudaError_t launch_update_mode(enkf_handle_s* h, const void* Xf, void* Xa
   int N = c.N;
   void* args[] = {const_cast<void**>(&Xf), &Xa, const_cast<double**>(&W), &n, &N};
   return cudaLaunchKernel(fn, dim3(tiles), dim3(kThreads), args, smem, h->stream);
-}
-
-cudaError_t launch_update(enkf_handle_s* h, const void* Xf, void* Xa) {
-  // FP32 ensembles: the A W product on the tensor cores (kernels_update_tc.cu); FP64 on CUDA cores
-  if (h->cfg.precision != ENKF_FP64) return launch_update_tc(h, Xf, Xa);
-  return launch_update_mode<0>(h, Xf, Xa);
-}
-
-cudaError_t launch_update_product(enkf_handle_s* h, const void* Xf, void* Xa) {
-  return launch_update_mode<1>(h, Xf, Xa);
 }
 
 cudaError_t launch_draw_perturbations(uint64_t seed, uint64_t counter, const double* r, int64_t m,
