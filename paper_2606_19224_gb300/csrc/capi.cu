@@ -175,9 +175,14 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
   h->nnz = nnz;
   h->tri = tri;
   h->krylov = enkf::krylov_config(c);
+  h->r_const = tri;   // (whitened: 1)
   if (!tri && c.m > 0) {
     double sl = 0.0;
-    for (int64_t i = 0; i < c.m; ++i) sl += std::log2(r_diag[i]);
+    h->r_const = true;
+    for (int64_t i = 0; i < c.m; ++i) {
+      sl += std::log2(r_diag[i]);
+      h->r_const = h->r_const && r_diag[i] == r_diag[0];
+    }
     const long k = std::lround(sl / (double)c.m);
     h->r_pow2 = std::ldexp(1.f, (int)std::max(-120L, std::min(120L, k)));
   }
@@ -241,7 +246,7 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
     allocs.push_back({&ws.ksmall, 8 * ((size_t)4 * c.N * c.N + 2 * c.N)});
   }
   if (!gram && !krylov) {
-    allocs.push_back({(void**)&ws.Sv, vs * mN});
+    if (!h->solve64) allocs.push_back({(void**)&ws.Sv, vs * mN});
     allocs.push_back({(void**)&ws.D, sizeof(double) * mN});
     allocs.push_back({(void**)&ws.Res, vs * mN});
     allocs.push_back({(void**)&ws.P, vs * mN});

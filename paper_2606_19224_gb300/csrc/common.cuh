@@ -209,6 +209,8 @@ struct enkf_handle_s {
   enkf::BatchState* batch = nullptr;   // non-NULL for a handle made by enkf_batch_create
   enkf::WarmState* warm = nullptr;     // learned warm start (enkf_set_warm_model / enkf_warm_features)
   bool krylov = false;                 // the solve runs in Krylov coordinates (kernels_krylov.cu)
+  bool r_const = false;                // all of R's diagonal is one number (known at create only)
+  bool solve64 = false;                // FP64 solve on the tensor cores (kernels_solve64.cu)
   int small_c = 0;                     // > 0: CTAs per column of the small-problem solve (kernels_small.cu)
   bool tri = false;                    // tridiagonal R: analyses run on the whitened problem
   float r_pow2 = 1.f;                  // power of two nearest the geometric mean of R's diagonal
@@ -227,8 +229,13 @@ cudaError_t plan_solve_mixed(enkf_handle_s* h);
 cudaError_t launch_solve_mixed(enkf_handle_s* h);
 size_t mixed_image_bytes(const enkf_handle_s* h);   // tile images of HA (zeroed at create)
 // kernels_small.cu: one cluster of CTAs per column (0: not for this problem)
-int small_cluster(const enkf_config& c, int sms);
+int small_cluster(const enkf_handle_s* h);
 cudaError_t launch_small(enkf_handle_s* h);
+// kernels_solve64.cu: FP64, N <= 64
+bool steady_fp64(const enkf_handle_s* h);   // see there
+bool solve64_config(const enkf_handle_s* h);
+cudaError_t plan_solve64(enkf_handle_s* h);
+cudaError_t launch_solve64(enkf_handle_s* h);
 // kernels_krylov.cu: CG preconditioned by R in the coordinates of its Krylov space
 bool krylov_config(const enkf_config& c);
 cudaError_t plan_krylov(enkf_handle_s* h);

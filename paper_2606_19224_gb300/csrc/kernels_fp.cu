@@ -78,20 +78,17 @@ __global__ void __launch_bounds__(kThreads) update_kernel(const VT* Xf, VT* Xa,
 // ------------------------------------------------------------------ host launchers
 static int pick_nt(int N) { return N <= 32 ? 32 : (N <= 64 ? 64 : 128); }
 
-template <typename VT>
-static void* solve_fn(int NT, bool pc) {
-  if (pc) {
-    if (NT == 32) return (void*)solve_kernel<VT, 32, true>;
-    if (NT == 64) return (void*)solve_kernel<VT, 64, true>;
-    return (void*)solve_kernel<VT, 128, true>;
-  }
-  if (NT == 32) return (void*)solve_kernel<VT, 32, false>;
-  if (NT == 64) return (void*)solve_kernel<VT, 64, false>;
-  return (void*)solve_kernel<VT, 128, false>;
+template <typename VT, int NT>
+static void* solve_fn_nt(bool pc) { return pc ? (void*)solve_kernel<VT, NT, true> : (void*)solve_kernel<VT, NT, false>; }
+static void* solve_fn(bool fp64, int NT, bool pc) {
+  if (fp64 && NT == 128) return solve_fn_nt<double, 128>(pc);
+  if (fp64)   // (preconditioned: kernels_solve64.cu)
+    return NT == 32 ? (void*)solve_kernel<double, 32, false> : (void*)solve_kernel<double, 64, false>;
+  return NT == 32 ? solve_fn_nt<float, 32>(pc) : NT == 64 ? solve_fn_nt<float, 64>(pc) : solve_fn_nt<float, 128>(pc);
 }
-template <typename VT>
-static size_t solve_smem(int NT) {
-  return NT == 32 ? solve_smem_bytes<VT, 32>() : (NT == 64 ? solve_smem_bytes<VT, 64>() : solve_smem_bytes<VT, 128>());
+static size_t solve_smem(bool fp64, int NT) {
+  if (fp64) return NT == 32 ? solve_smem_bytes<double, 32>() : (NT == 64 ? solve_smem_bytes<double, 64>() : solve_smem_bytes<double, 128>());
+  return NT == 32 ? solve_smem_bytes<float, 32>() : (NT == 64 ? solve_smem_bytes<float, 64>() : solve_smem_bytes<float, 128>());
 }
 
 cudaError_t plan_solve(enkf_handle_s* h) {
@@ -99,8 +96,12 @@ cudaError_t plan_solve(enkf_handle_s* h) {
   const int NT = pick_nt(N);
   const bool fp64 = h->cfg.precision == ENKF_FP64;
   const bool pc = h->cfg.precondition != 0;
-  void* fn = fp64 ? solve_fn<double>(NT, pc) : solve_fn<float>(NT, pc);
-  const size_t smem = fp64 ? solve_smem<double>(NT) : solve_smem<float>(NT);
+  // a problem whose HA fits the shared memory of a few SMs is solved column by column
+  h->small_c = small_cluster(h);
+  h->solve64 = solve64_config(h);
+  if (h->solve64) return plan_solve64(h);
+  void* fn = solve_fn(fp64, NT, pc);
+  const size_t smem = solve_smem(fp64, NT);
   cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   int occ = 0;
@@ -114,8 +115,6 @@ cudaError_t plan_solve(enkf_handle_s* h) {
   h->launch.G = G;
   h->launch.NT = NT;
   h->launch.smem = smem;
-  // a problem whose HA fits the shared memory of a few SMs is solved column by column
-  h->small_c = small_cluster(h->cfg, h->sms);
   return cudaSuccess;
 }
 
@@ -153,6 +152,7 @@ cudaError_t launch_convert_r(enkf_handle_s* h) {
 
 cudaError_t launch_solve(enkf_handle_s* h) {
   if (h->small_c) return launch_small(h);
+  if (h->solve64) return launch_solve64(h);
   const auto& c = h->cfg;
   auto& ws = h->ws;
   const bool fp64 = c.precision == ENKF_FP64;
@@ -202,7 +202,7 @@ cudaError_t launch_solve(enkf_handle_s* h) {
   err = cudaMemsetAsync(ws.status, 0, 4 * sizeof(int32_t), h->stream);
   if (err != cudaSuccess) return err;
   const bool pc = c.precondition != 0;
-  void* fn = fp64 ? solve_fn<double>(h->launch.NT, pc) : solve_fn<float>(h->launch.NT, pc);
+  void* fn = solve_fn(fp64, h->launch.NT, pc);
   void* args[] = {&p};
   return cudaLaunchCooperativeKernel(fn, dim3(h->launch.G), dim3(kThreads), args,
                                      h->launch.smem, h->stream);

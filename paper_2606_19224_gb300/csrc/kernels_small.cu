@@ -753,12 +753,14 @@ static void small_launch_config(const enkf_config& c, int C, cudaStream_t stream
 // lies in one part of the chip. 37 clusters of 4 ran as two waves, 1.92 ms against 0.98.)
 // (The limit on dynamic shared memory belongs to the kernel, not to the handle, so it is never set lower.)
 constexpr int kSmallSmem = 224 * 1024;
-int small_cluster(const enkf_config& c, int sms) {
+int small_cluster(const enkf_handle_s* h) {
+  const enkf_config& c = h->cfg;
   if (c.variant != ENKF_CGD || c.precision > ENKF_FP32 || c.warm_start || c.grid_blocks > 0) return 0;
   const bool fp64 = c.precision == ENKF_FP64;
+  if (fp64 && !steady_fp64(h)) return 0;
   void* fn = small_fn(fp64, c.precondition != 0);
   int best = 0;
-  for (int C = 1; C <= 8 && (int64_t)c.N * C <= sms; ++C) {
+  for (int C = 1; C <= 8 && (int64_t)c.N * C <= h->sms; ++C) {
     const int64_t rp = (c.m + C - 1) / C;
     if (rp > 65536 || small_smem(fp64, c.N, (int)rp, C) > kSmallSmem) continue;
     if (best != 0 && rp < 128) break;
