@@ -4,9 +4,6 @@
 // kernel (kernels_batch.cu).
 #pragma once
 
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
 #include "cg_device.cuh"
 
 namespace enkf {
@@ -100,11 +97,9 @@ template <typename VT>
 __device__ __forceinline__ void innov_rows_f64(
     const VT* __restrict__ Xf, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
     const double* __restrict__ w, const double* __restrict__ y, const double* __restrict__ r,
-    const double* __restrict__ E, int emode, uint64_t seed, uint64_t counter, int64_t m, int N,
-    double* __restrict__ HA64, float* __restrict__ HA32, double* __restrict__ D,
-    float* __restrict__ B32, __nv_bfloat16* __restrict__ HAb, __half* __restrict__ HAh,
-    int split_lo, df32* __restrict__ HAdf, df32* __restrict__ Ddf, int64_t i_begin, int64_t i_end,
-    int64_t warp, int64_t nwarps, int64_t out0 = 0 /* outputs are written from row out0 on */) {
+    const double* __restrict__ E, int emode, uint64_t seed, uint64_t counter, int N,
+    double* __restrict__ HA64, double* __restrict__ D, int64_t i_begin, int64_t i_end, int64_t warp, int64_t nwarps,
+    int64_t out0 = 0 /* outputs are written from row out0 on */) {
   // FP64 instructions are scarce on this part (2 per clock per SM): 1/N is applied as a
   // product and members 64..127 are skipped when N <= 64
   const int lane = threadIdx.x & 31;
@@ -150,46 +145,15 @@ __device__ __forceinline__ void innov_rows_f64(
       if ((N & 1) == 0) {
         // both members present and e0 even: one 8- or 16-byte store per array per lane, so a
         // warp writes contiguous row segments
-        if (HA64) *reinterpret_cast<double2*>(HA64 + e0) = make_double2(hv[0], hv[1]);
+        *reinterpret_cast<double2*>(HA64 + e0) = make_double2(hv[0], hv[1]);
         *reinterpret_cast<double2*>(D + e0) = make_double2(dv[0], dv[1]);
-        if (HA32) *reinterpret_cast<float2*>(HA32 + e0) = make_float2((float)hv[0], (float)hv[1]);
-        if (B32) *reinterpret_cast<float2*>(B32 + e0) = make_float2((float)dv[0], (float)dv[1]);
-        if (HAdf) {
-          const df32 a0(hv[0]), a1(hv[1]);
-          *reinterpret_cast<float4*>(HAdf + e0) = make_float4(a0.hi, a0.lo, a1.hi, a1.lo);
-        }
-        if (Ddf) {
-          const df32 d0(dv[0]), d1(dv[1]);
-          *reinterpret_cast<float4*>(Ddf + e0) = make_float4(d0.hi, d0.lo, d1.hi, d1.lo);
-        }
       } else {
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
           if (jp + b >= N) continue;
           const int64_t e = e0 + b;
-          if (HA64) HA64[e] = hv[b];
+          HA64[e] = hv[b];
           D[e] = dv[b];
-          if (HA32) HA32[e] = (float)hv[b];
-          if (B32) B32[e] = (float)dv[b];
-          if (HAdf) HAdf[e] = df32(hv[b]);
-          if (Ddf) Ddf[e] = df32(dv[b]);
-        }
-      }
-      // low-precision copies: hi part at [0, m N), lo part (ha - hi) at [m N, 2 m N) when split
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        if (jp + b >= N) continue;
-        const int64_t e = e0 + b;
-        const double ha = hv[b];
-        if (HAb) {
-          const __nv_bfloat16 hi = __double2bfloat16(ha);
-          HAb[e] = hi;
-          if (split_lo) HAb[m * N + e] = __double2bfloat16(ha - (double)__bfloat162float(hi));
-        }
-        if (HAh) {
-          const __half hi = __double2half(ha);
-          HAh[e] = hi;
-          if (split_lo) HAh[m * N + e] = __double2half(ha - (double)__half2float(hi));
         }
       }
     }
@@ -225,21 +189,46 @@ __device__ __forceinline__ df32 df_rsqrt(const df32& s) {
 // bits, the precision of the HAdf and Ddf arrays they fill), E = sqrt(r_i) times the FP32
 // normal as an exact double-float product; HA32 and B32 are the high parts, and only the
 // FP64 copy of D is widened per element.
-template <typename VT>
+//
+// A row takes the lanes of half a warp for N <= 64 (HALF) and of a whole one otherwise, four members each
+// (2 l, 2 l + 1 and the same 32 or 64 further on, so that each perturbation pair is drawn once). What bounds it is
+// latency: a row was a chain of four dependent loads, and the tree of its mean took as many
+// instructions for two members per lane as for four. The offsets, first columns and row values of 32 rows are read
+// ahead, lane q for row q of the warp, and each row's first gather is in flight behind the row before.
+template <typename VT, bool HALF>
 __device__ __forceinline__ void innov_rows_df(
     const VT* __restrict__ Xf, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
     const double* __restrict__ w, const double* __restrict__ y, const double* __restrict__ r,
-    const double* __restrict__ E, int emode, uint64_t seed, uint64_t counter, int64_t m, int N,
-    double* __restrict__ HA64, float* __restrict__ HA32, double* __restrict__ D,
-    float* __restrict__ B32, __nv_bfloat16* __restrict__ HAb, __half* __restrict__ HAh,
-    int split_lo, df32* __restrict__ HAdf, df32* __restrict__ Ddf, int64_t i_begin, int64_t i_end,
-    int64_t warp, int64_t nwarps, unsigned* hamax = nullptr, const InnovRows kr = InnovRows{}) {
+    const double* __restrict__ E, int emode, uint64_t seed, uint64_t counter, int N,
+    double* __restrict__ D, float* __restrict__ HA32, float* __restrict__ B32, df32* __restrict__ HAdf,
+    df32* __restrict__ Ddf, int64_t i_begin, int64_t i_end, int64_t warp, int64_t nwarps, unsigned* hamax,
+    const InnovRows kr) {
   static_assert(sizeof(VT) == 4, "double-float innovations take an FP32 ensemble");
-  const int lane = threadIdx.x & 31;
+  constexpr int GL = HALF ? 16 : 32, RW = 32 / GL;   // lanes per row, rows per warp
+  const int lane = threadIdx.x & 31, gl = lane % GL, sub = lane / GL;
+  const unsigned group = HALF ? 0xFFFFu << (16 * sub) : 0xffffffffu;
   float hmax = 0.f;   // largest |HA| of the warp's rows (hamax: atomic maximum of the float bits)
   float umax = 0.f;   // largest |HA| / sqrt(r) of the warp's rows
   const df32 inv_n(1.0 / (double)N);
-  const bool wide = N > 64;   // members 64..127 present (warp-uniform)
+  const bool even = (N & 1) == 0, vec = even && (reinterpret_cast<uintptr_t>(Xf) & 7) == 0;
+  bool in[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) in[q] = 2 * gl + (q & 1) + 2 * GL * (q >> 1) < N;
+  // the row's members of this lane
+  auto gather = [&](int c, float (&x)[4]) {
+    const VT* xr = Xf + (int64_t)c * N + 2 * gl;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (vec) {   // both members of a pair, at an 8-byte boundary
+        const float2 v = in[2 * h] ? *reinterpret_cast<const float2*>(xr + 2 * GL * h) : make_float2(0.f, 0.f);
+        x[2 * h] = v.x;
+        x[2 * h + 1] = v.y;
+      } else {
+        x[2 * h] = in[2 * h] ? (float)xr[2 * GL * h] : 0.f;
+        x[2 * h + 1] = in[2 * h + 1] ? (float)xr[2 * GL * h + 1] : 0.f;
+      }
+    }
+  };
   // The warp's rows are i0 + q nwarps, q = 0, 1, ...; the per-row values that come from FP64
   // inputs (y_i, sqrt(r_i) and the weight of the row's first operator entry as double-float
   // pairs) are formed for 32 rows at a time, lane q for row i0 + q nwarps, and handed to the
@@ -247,149 +236,130 @@ __device__ __forceinline__ void innov_rows_df(
   for (int64_t i0 = i_begin + warp; i0 < i_end; i0 += 32 * nwarps) {
     const int64_t il = i0 + (int64_t)lane * nwarps;
     df32 y_l, s_l, w_l, r_l;
+    int k_l = 0, n_l = 0, c_l = 0;   // first entry, entries after it (-1: none), its column
+    float q_l = 0.f;
     if (il < i_end) {
+      k_l = rowptr[il];
+      n_l = rowptr[il + 1] - k_l - 1;
+      if (kr.umax && !kr.senkf) q_l = kr.rsq[il].hi;
       if (kr.senkf) r_l = df_from_double(r[il]);
       y_l = df_from_double(y[il]);
       if (emode == 2) s_l = df_from_double(sqrt(r[il]));
-      const int kf = rowptr[il];
-      if (kf < rowptr[il + 1]) w_l = df_from_double(w[kf]);
-    }
-    for (int q32 = 0; q32 < 32; ++q32) {
-      const int64_t i = i0 + (int64_t)q32 * nwarps;
-      if (i >= i_end) break;   // warp-uniform
-      const df32 yd(__shfl_sync(0xffffffffu, y_l.hi, q32), __shfl_sync(0xffffffffu, y_l.lo, q32));
-      const df32 sr(__shfl_sync(0xffffffffu, s_l.hi, q32), __shfl_sync(0xffffffffu, s_l.lo, q32));
-      const df32 w0(__shfl_sync(0xffffffffu, w_l.hi, q32), __shfl_sync(0xffffffffu, w_l.lo, q32));
-      df32 z[4];
-      const int k0 = rowptr[i], k1 = rowptr[i + 1];
-      for (int k = k0; k < k1; ++k) {
-        const df32 wk = k == k0 ? w0 : df_from_double(w[k]);
-        const VT* xr = Xf + (int64_t)col[k] * N;
-  #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int j = 2 * lane + (q & 1) + 64 * (q >> 1);
-          if (j < N) z[q] = fma(wk, df32((float)xr[j], 0.f), z[q]);
-        }
+      if (n_l >= 0) {
+        c_l = col[k_l];
+        w_l = df_from_double(w[k_l]);
       }
-      df32 s = z[0] + z[1];
-      if (wide) s = s + (z[2] + z[3]);
-  #pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
+    }
+    float xn[4];
+    gather(__shfl_sync(0xffffffffu, c_l, sub), xn);   // (column 0 where there is no entry: weight 0)
+#pragma unroll 1
+    for (int q32 = 0; q32 < 32; q32 += RW) {
+      const int64_t i = i0 + (int64_t)(q32 + sub) * nwarps;
+      if (i0 + (int64_t)q32 * nwarps >= i_end) break;   // warp-uniform
+      const bool row = i < i_end;
+      const int src = q32 + sub;
+      const df32 yd(__shfl_sync(0xffffffffu, y_l.hi, src), __shfl_sync(0xffffffffu, y_l.lo, src));
+      const df32 sr(__shfl_sync(0xffffffffu, s_l.hi, src), __shfl_sync(0xffffffffu, s_l.lo, src));
+      const df32 w0(__shfl_sync(0xffffffffu, w_l.hi, src), __shfl_sync(0xffffffffu, w_l.lo, src));
+      const int more = __shfl_sync(0xffffffffu, n_l, src), k0 = __shfl_sync(0xffffffffu, k_l, src);
+      const float wq = __shfl_sync(0xffffffffu, q_l, src);
+      df32 z[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (more >= 0) z[q] = w0 * df32(xn[q], 0.f);
+      gather(__shfl_sync(0xffffffffu, c_l, min(src + RW, 31)), xn);
+      for (int k = 1; k <= more; ++k) {
+        const df32 wk = df_from_double(w[k0 + k]);
+        float x[4];
+        gather(col[k0 + k], x);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) z[q] = fma(wk, df32(x[q], 0.f), z[q]);
+      }
+      __syncwarp();
+      df32 s = (z[0] + z[1]) + (z[2] + z[3]);   // (zeros past N)
+#pragma unroll
+      for (int o = GL / 2; o > 0; o >>= 1)
         s = s + df32(__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o));
       const df32 zbar = s * inv_n;
+      df32 hv[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        hv[q] = z[q] - zbar;
+        if (in[q] && row) hmax = fmaxf(hmax, fabsf(hv[q].hi));
+      }
       if (kr.umax) {
         float rm = 0.f;
-  #pragma unroll
+#pragma unroll
         for (int q = 0; q < 4; ++q)
-          if (2 * lane + (q & 1) + 64 * (q >> 1) < N) rm = fmaxf(rm, fabsf((z[q] - zbar).hi));
-        rm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(rm)));
-        float wt;
+          if (in[q]) rm = fmaxf(rm, fabsf(hv[q].hi));
+        rm = __uint_as_float(__reduce_max_sync(group, __float_as_uint(rm)));
+        float wt = wq;
         if (kr.senkf) {
-          df32 q;
-  #pragma unroll
-          for (int e = 0; e < 4; ++e)
-            if (2 * lane + (e & 1) + 64 * (e >> 1) < N) {
-              const df32 hv = z[e] - zbar;
-              q = fma(hv, hv, q);
-            }
-  #pragma unroll
-          for (int o = 16; o > 0; o >>= 1)
-            q = q + df32(__shfl_xor_sync(0xffffffffu, q.hi, o), __shfl_xor_sync(0xffffffffu, q.lo, o));
-          const df32 rs = df_rsqrt(q + df32((float)(N - 1), 0.f) *
-                                           df32(__shfl_sync(0xffffffffu, r_l.hi, q32), __shfl_sync(0xffffffffu, r_l.lo, q32)));
-          if (lane == 0) kr.wsq[i - kr.row0] = rs;
+          df32 q2;
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (in[q]) q2 = fma(hv[q], hv[q], q2);
+#pragma unroll
+          for (int o = GL / 2; o > 0; o >>= 1)
+            q2 = q2 + df32(__shfl_xor_sync(0xffffffffu, q2.hi, o), __shfl_xor_sync(0xffffffffu, q2.lo, o));
+          const df32 rs = df_rsqrt(q2 + df32((float)(N - 1), 0.f) *
+                                            df32(__shfl_sync(0xffffffffu, r_l.hi, src), __shfl_sync(0xffffffffu, r_l.lo, src)));
+          if (row && gl == 0) kr.wsq[i - kr.row0] = rs;
           wt = rs.hi;
-        } else {
-          wt = kr.rsq[i].hi;
         }
-        umax = fmaxf(umax, rm * wt);
-        // the exponent field of the power of two above rm (bounded away from both ends of the range)
-        const int E = max(40, min(252, (int)(__float_as_uint(rm) >> 23)));
-        if (kr.scale && lane == 0) kr.scale[i - kr.row0] = __uint_as_float((uint32_t)(E + 1) << 23);
+        if (row) {
+          umax = fmaxf(umax, rm * wt);
+          // the exponent field of the power of two above rm (bounded away from both ends of the range)
+          const int Ex = max(40, min(252, (int)(__float_as_uint(rm) >> 23)));
+          if (kr.scale && gl == 0) kr.scale[i - kr.row0] = __uint_as_float((uint32_t)(Ex + 1) << 23);
+        }
       }
-  #pragma unroll
+#pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int jp = 2 * lane + 64 * h;   // even member of the pair
-        if (jp >= N) continue;
+        const int jp = 2 * gl + 2 * GL * h;   // even member of the pair
+        if (!in[2 * h] || !row) continue;
         float nrm[2] = {0.f, 0.f};
         if (emode == 2) perturbation_pair_f32(i, jp, seed, counter, nrm[0], nrm[1]);
         const int64_t ein = i * N + jp, e0 = ein - kr.row0 * N;   // of the inputs, of the outputs
-        df32 hv[2], dv[2];
-  #pragma unroll
+        df32 dv[2];
+#pragma unroll
         for (int b = 0; b < 2; ++b) {
           df32 pert;
-          if (jp + b < N) {
+          if (in[2 * h + b]) {
             if (emode == 1) pert = df_from_double(E[ein + b]);
             else if (emode == 2) pert = sr * df32(nrm[b], 0.f);
           }
-          hv[b] = z[2 * h + b] - zbar;
           dv[b] = (yd - z[2 * h + b]) + pert;
-          if (jp + b < N) hmax = fmaxf(hmax, fabsf(hv[b].hi));
         }
-        if ((N & 1) == 0) {
+        const df32* ha = hv + 2 * h;
+        if (even) {
           // both members present and e0 even: one 8- or 16-byte store per array per lane
           if (D) *reinterpret_cast<double2*>(D + e0) = make_double2(df_to_double(dv[0]), df_to_double(dv[1]));
-          if (HA32) *reinterpret_cast<float2*>(HA32 + e0) = make_float2(hv[0].hi, hv[1].hi);
+          if (HA32) *reinterpret_cast<float2*>(HA32 + e0) = make_float2(ha[0].hi, ha[1].hi);
           if (B32) *reinterpret_cast<float2*>(B32 + e0) = make_float2(dv[0].hi, dv[1].hi);
-          if (HAdf) *reinterpret_cast<float4*>(HAdf + e0) = make_float4(hv[0].hi, hv[0].lo, hv[1].hi, hv[1].lo);
+          if (HAdf) *reinterpret_cast<float4*>(HAdf + e0) = make_float4(ha[0].hi, ha[0].lo, ha[1].hi, ha[1].lo);
           if (Ddf) *reinterpret_cast<float4*>(Ddf + e0) = make_float4(dv[0].hi, dv[0].lo, dv[1].hi, dv[1].lo);
         } else {
-  #pragma unroll
+#pragma unroll
           for (int b = 0; b < 2; ++b) {
-            if (jp + b >= N) continue;
+            if (!in[2 * h + b]) continue;
             const int64_t e = e0 + b;
             if (D) D[e] = df_to_double(dv[b]);
-            if (HA32) HA32[e] = hv[b].hi;
+            if (HA32) HA32[e] = ha[b].hi;
             if (B32) B32[e] = dv[b].hi;
-            if (HAdf) HAdf[e] = hv[b];
+            if (HAdf) HAdf[e] = ha[b];
             if (Ddf) Ddf[e] = dv[b];
-          }
-        }
-        // optional copies (not requested by the current callers): FP64 HA and 16-bit images
-  #pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          if (jp + b >= N) continue;
-          const int64_t e = e0 + b;
-          if (HA64) HA64[e] = (double)hv[b];
-          if (HAb) {
-            const __nv_bfloat16 hi = __float2bfloat16(hv[b].hi);
-            HAb[e] = hi;
-            if (split_lo) HAb[m * N + e] = __float2bfloat16((hv[b] - df32(__bfloat162float(hi), 0.f)).hi);
-          }
-          if (HAh) {
-            const __half hi = __float2half(hv[b].hi);
-            HAh[e] = hi;
-            if (split_lo) HAh[m * N + e] = __float2half((hv[b] - df32(__half2float(hi), 0.f)).hi);
           }
         }
       }
     }
   }
-  if (kr.umax && lane == 0 && umax > 0.f) atomicMax(kr.umax, __float_as_uint(umax));
+  if (kr.umax && gl == 0 && umax > 0.f) atomicMax(kr.umax, __float_as_uint(umax));
   if (hamax) {
     // non-negative floats order as their bit patterns
     const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(hmax));
     if (lane == 0 && mb > 0u) atomicMax(hamax, mb);
   }
-}
-
-// Rows [i_begin, i_end) of the innovation step: FP64 arithmetic for FP64 ensembles,
-// double-float for FP32 ones.
-template <typename VT>
-__device__ __forceinline__ void innov_rows(
-    const VT* __restrict__ Xf, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-    const double* __restrict__ w, const double* __restrict__ y, const double* __restrict__ r,
-    const double* __restrict__ E, int emode, uint64_t seed, uint64_t counter, int64_t m, int N,
-    double* __restrict__ HA64, float* __restrict__ HA32, double* __restrict__ D,
-    float* __restrict__ B32, __nv_bfloat16* __restrict__ HAb, __half* __restrict__ HAh,
-    int split_lo, df32* __restrict__ HAdf, df32* __restrict__ Ddf, int64_t i_begin, int64_t i_end,
-    int64_t warp, int64_t nwarps, unsigned* hamax = nullptr, const InnovRows kr = InnovRows{}) {
-  if constexpr (sizeof(VT) == 4)
-    innov_rows_df<VT>(Xf, rowptr, col, w, y, r, E, emode, seed, counter, m, N, HA64, HA32, D, B32,
-                      HAb, HAh, split_lo, HAdf, Ddf, i_begin, i_end, warp, nwarps, hamax, kr);
-  else
-    innov_rows_f64<VT>(Xf, rowptr, col, w, y, r, E, emode, seed, counter, m, N, HA64, HA32, D, B32,
-                       HAb, HAh, split_lo, HAdf, Ddf, i_begin, i_end, warp, nwarps);
 }
 
 }  // namespace enkf

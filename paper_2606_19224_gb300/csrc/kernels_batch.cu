@@ -15,6 +15,7 @@
 // re-plans from the measured per-problem durations, and keeps the fastest plan; the choice
 // can be cached in the text file named by the ENKF_TUNE_CACHE variable.
 #include <algorithm>
+#include <type_traits>
 #include <array>
 #include <cmath>
 #include <cstdio>
@@ -125,11 +126,14 @@ __global__ void __launch_bounds__(kKT, 1) batch_kernel(
     // innovations over this CTA's share of the observation rows
     const int64_t rows_per = (sp.m + G - 1) / G;
     const int64_t r0 = imin64(sp.m, (int64_t)rank * rows_per), r1 = imin64(sp.m, r0 + rows_per);
-    innov_rows<float>(s_io.Xf, probs[pi].rowptr, probs[pi].col, probs[pi].w, s_io.y, probs[pi].r, nullptr,
-                      perturb ? 2 : 0, s_io.seed, s_io.counter, sp.m, sp.N, nullptr, nullptr, nullptr, nullptr,
-                      nullptr, nullptr, 0, const_cast<df32*>(sp.HAdf),
-                      const_cast<df32*>(sp.Ddf), r0, r1, warp, kKT / 32, nullptr,
-                      InnovRows{const_cast<float*>(sp.hs), sp.rsq, const_cast<unsigned*>(sp.umax)});
+    auto innovations = [&](auto half) {
+      innov_rows_df<float, decltype(half)::value>(
+          s_io.Xf, probs[pi].rowptr, probs[pi].col, probs[pi].w, s_io.y, probs[pi].r, nullptr, perturb ? 2 : 0, s_io.seed,
+          s_io.counter, sp.N, nullptr, nullptr, nullptr, const_cast<df32*>(sp.HAdf), const_cast<df32*>(sp.Ddf), r0, r1, warp,
+          kKT / 32, nullptr, InnovRows{const_cast<float*>(sp.hs), sp.rsq, const_cast<unsigned*>(sp.umax)});
+    };
+    if (sp.N <= 64) innovations(std::true_type{});
+    else innovations(std::false_type{});
     bool ok = bar.sync();
     if (ok) {
       if (NT == 32) batch_solve<32>(sp, G, rank, bar, cta);

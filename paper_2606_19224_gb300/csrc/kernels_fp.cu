@@ -35,18 +35,20 @@ __global__ void __launch_bounds__(kThreads, (NT == 128 || sizeof(VT) == 8 || asy
   solve_body<VT, NT, PC>(p, (int)gridDim.x, (int)blockIdx.x, bar, smem);
 }
 
-template <typename VT>
-__global__ void __launch_bounds__(kThreads) innov_kernel(
+template <typename VT, bool HALF>   // HALF: N <= 64 (FP32 ensembles)
+__global__ void __launch_bounds__(kThreads, 4) innov_kernel(
     const VT* __restrict__ Xf, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
     const double* __restrict__ w, const double* __restrict__ y, const double* __restrict__ r,
     const double* __restrict__ E, int emode, uint64_t seed, uint64_t counter, int64_t m, int N,
     double* __restrict__ HA64, float* __restrict__ HA32, double* __restrict__ D,
-    float* __restrict__ B32, __nv_bfloat16* __restrict__ HAb, __half* __restrict__ HAh,
-    int split_lo, df32* __restrict__ HAdf, df32* __restrict__ Ddf, unsigned* hamax, InnovRows kr) {
+    float* __restrict__ B32, df32* __restrict__ HAdf, df32* __restrict__ Ddf, unsigned* hamax, InnovRows kr) {
   const int64_t warp = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  innov_rows<VT>(Xf, rowptr, col, w, y, r, E, emode, seed, counter, m, N, HA64, HA32, D, B32, HAb,
-                 HAh, split_lo, HAdf, Ddf, 0, m, warp, nwarps, hamax, kr);
+  if constexpr (sizeof(VT) == 4)
+    innov_rows_df<VT, HALF>(Xf, rowptr, col, w, y, r, E, emode, seed, counter, N, D, HA32, B32, HAdf, Ddf, 0, m, warp, nwarps,
+                            hamax, kr);
+  else
+    innov_rows_f64<VT>(Xf, rowptr, col, w, y, r, E, emode, seed, counter, N, HA64, D, 0, m, warp, nwarps);
 }
 
 __global__ void draw_perturbations_kernel(uint64_t seed, uint64_t counter,
@@ -131,14 +133,14 @@ cudaError_t launch_innovations(enkf_handle_s* h, const void* Xf, const double* y
     if (e != cudaSuccess) return e;
   }
   if (fp64)
-    innov_kernel<double><<<blocks, kThreads, 0, h->stream>>>(
+    innov_kernel<double, false><<<blocks, kThreads, 0, h->stream>>>(
         static_cast<const double*>(Xf), ws.rowptr, ws.col, ws.w, y, ws.r, E, emode, seed, counter,
-        c.m, c.N, ws.HA64, nullptr, ws.D, nullptr, nullptr, nullptr, 0, nullptr, nullptr, nullptr, InnovRows{});
+        c.m, c.N, ws.HA64, nullptr, ws.D, nullptr, nullptr, nullptr, nullptr, InnovRows{});
   else
-    innov_kernel<float><<<blocks, kThreads, 0, h->stream>>>(
+    (c.N <= 64 ? innov_kernel<float, true> : innov_kernel<float, false>)<<<blocks, kThreads, 0, h->stream>>>(
         static_cast<const float*>(Xf), ws.rowptr, ws.col, ws.w, y, ws.r, E, emode, seed, counter,
-        c.m, c.N, ws.HA64, ws.HA32, ws.D, h->krylov ? nullptr : static_cast<float*>(ws.B),
-        nullptr, nullptr, 0, static_cast<df32*>(ws.HAdf), static_cast<df32*>(ws.Ddf), h->krylov ? nullptr : ws.hamax,
+        c.m, c.N, nullptr, ws.HA32, ws.D, h->krylov ? nullptr : static_cast<float*>(ws.B),
+        static_cast<df32*>(ws.HAdf), static_cast<df32*>(ws.Ddf), h->krylov ? nullptr : ws.hamax,
         InnovRows{ws.hs, static_cast<const df32*>(ws.rsq), h->krylov ? ws.hamax : nullptr});
   return cudaGetLastError();
 }

@@ -91,8 +91,8 @@ __global__ void __launch_bounds__(kDT, 1) gram64_kernel(Gram64 g) {
   for (int tile = 0; tile < tiles && cta.ok; ++tile) {   // at least one: a CTA without rows writes zeros
     const int64_t c0 = imin64(row1, row0 + (int64_t)tile * per);
     const int rows = (int)(imin64(row1, c0 + per) - c0), ks = (rows + 15) / 16;
-    innov_rows_f64<double>(g.Xf, g.rowptr, g.col, g.w, g.y, g.r, g.E, g.emode, g.seed, g.counter, g.m, N, HA, nullptr, D,
-                           nullptr, nullptr, nullptr, 0, nullptr, nullptr, c0, c0 + rows, warp, kDT / 32, c0);
+    innov_rows_f64<double>(g.Xf, g.rowptr, g.col, g.w, g.y, g.r, g.E, g.emode, g.seed, g.counter, N, HA, D, c0,
+                           c0 + rows, warp, kDT / 32, c0);
     __syncthreads();
     if (g.senkf) {
       for (int i = warp; i < rows; i += kDT / 32) {
@@ -255,9 +255,9 @@ __global__ void __launch_bounds__(kKT, 1) gram_tc_kernel(GramTc g) {
       const int64_t c1 = imin64(row1, c0 + g.chunk);
       if (t == 0) umax = 0u;
       __syncthreads();
-      innov_rows_df<float>(g.Xf, g.rowptr, g.col, g.w, g.y, g.r, g.E, g.emode, g.seed, g.counter, g.m, N, nullptr, nullptr,
-                           nullptr, nullptr, nullptr, nullptr, 0, HA, D, c0, c1, t >> 5, kKT / 32, nullptr,
-                           InnovRows{nullptr, g.rsq, &umax, c0, g.senkf, wsq});
+      innov_rows_df<float, (NT <= 64)>(g.Xf, g.rowptr, g.col, g.w, g.y, g.r, g.E, g.emode, g.seed, g.counter, N, nullptr, nullptr,
+                                       nullptr, HA, D, c0, c1, t >> 5, kKT / 32, nullptr,
+                                       InnovRows{nullptr, g.rsq, &umax, c0, g.senkf, wsq});
       __syncthreads();
       p.rsq = g.senkf ? wsq : g.rsq + c0;
       for (int c = 0; c < ngr; ++c)
