@@ -21,6 +21,10 @@
 
 namespace enkf {
 
+constexpr int kUT = 512;   // threads: four per row of a tile (with two per row and 256 threads the conversion of a
+                          // tile took three times as long as its bytes: 65 us at n = 262,144, N = 64 and 471 us at
+                          // n = 1,048,576, N = 128)
+
 template <int NT> struct UpdLayout {
   static constexpr int LDX = NT + 4;                       // staged X_f row stride (floats)
   static constexpr int XT = kTR * LDX * 4;                 // bytes per staged tile
@@ -31,8 +35,7 @@ template <int NT> struct UpdLayout {
   static constexpr int off_a = ((NBUF * XT + 1023) / 1024) * 1024;
   static constexpr int off_b = off_a + AIMG;
   static constexpr int off_rs = off_b + BIMG;              // per-row 2^-e scale [128]
-  static constexpr int off_mean = off_rs + 4 * kTR;        // per-row mean [128]
-  static constexpr int off_ws = off_mean + 4 * kTR;        // per-column 1/scale of W [NT]
+  static constexpr int off_ws = off_rs + 4 * kTR;          // per-column 1/scale of W [NT]
   static constexpr int bytes = off_ws + 4 * NT;
   static_assert(off_a % 1024 == 0 && off_b % 1024 == 0, "operand alignment");
 };
@@ -47,7 +50,7 @@ __device__ __forceinline__ float pow2_scale(float vmax) {
 }
 
 template <int NT>
-__global__ void __launch_bounds__(kThreads, 1) update_tc_kernel(const float* Xf, float* Xa,
+__global__ void __launch_bounds__(kUT, 1) update_tc_kernel(const float* Xf, float* Xa,
                                                                 const double* __restrict__ W, int64_t n,
                                                                 int N, int* status) {
   using L = UpdLayout<NT>;
@@ -57,13 +60,14 @@ __global__ void __launch_bounds__(kThreads, 1) update_tc_kernel(const float* Xf,
   constexpr int TMC = 2 * NT;   // D1 (hi*hi) at column 0, D2 (the cross terms) at column NT
   constexpr uint32_t idesc = umma_idesc(H16<__half>::fmt, NT);
   constexpr uint32_t sbo = (NT / 8) * 128;
-  constexpr int C4 = NT / 4, HALF = NT / 2, CH = HALF / 16;
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, qd = warp & 3, half = warp >> 2;
+  constexpr int C4 = NT / 4;
+  constexpr int EP = NT < 64 ? 2 : 4, CH = NT / EP / 16;   // epilogue: column parts, 16-column chunks of each
+  constexpr int PRE = kTR * C4 / kUT;                      // 16-byte pieces of a tile per thread
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, qd = warp & 3, part = warp >> 2;
   float* sX0 = reinterpret_cast<float*>(smem + L::off_x);
   __half* sA = reinterpret_cast<__half*>(smem + L::off_a);
   __half* sB = reinterpret_cast<__half*>(smem + L::off_b);
   float* s_rs = reinterpret_cast<float*>(smem + L::off_rs);
-  float* s_mean = reinterpret_cast<float*>(smem + L::off_mean);
   float* s_ws = reinterpret_cast<float*>(smem + L::off_ws);
   if (dynamic_smem_bytes() < (unsigned)L::bytes) {
     if (t == 0) atomicOr(status, DS_SMEM);
@@ -75,17 +79,28 @@ __global__ void __launch_bounds__(kThreads, 1) update_tc_kernel(const float* Xf,
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   // W: per-column power-of-two scale, then the hi/lo image (rows j, K-major over k)
-  if (t < NT) {
-    float mx = 0.f;
-    if (t < N)
-      for (int k = 0; k < N; ++k) mx = fmaxf(mx, fabsf((float)__ldcg(W + k * N + t)));
+  {
+    constexpr int WP = kUT / NT, WK = NT / WP;   // threads per column, entries of each
+    const int j = t % NT, w = t / NT;
+    float v[WK], mx = 0.f;
+#pragma unroll
+    for (int q = 0; q < WK; ++q) {
+      const int k = w + q * WP;
+      v[q] = (j < N && k < N) ? (float)__ldcg(W + k * N + j) : 0.f;
+      mx = fmaxf(mx, fabsf(v[q]));
+    }
+    sX0[w * NT + j] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < WP; ++q) mx = fmaxf(mx, sX0[q * NT + j]);
     const float sc = pow2_scale(mx);
-    s_ws[t] = 1.f / sc;                                   // exact (a power of two)
-    for (int k = 0; k < NT; ++k) {
-      const float v = (t < N && k < N) ? (float)__ldcg(W + k * N + t) * sc : 0.f;
-      const __half hi = __float2half_rn(v);
-      sB[core_idx(t, k, NT)] = hi;
-      sB[NT * NT + core_idx(t, k, NT)] = __float2half_rn((v - __half2float(hi)) * 2048.f);
+    if (w == 0) s_ws[j] = 1.f / sc;                       // exact (a power of two)
+#pragma unroll
+    for (int q = 0; q < WK; ++q) {
+      const float x = v[q] * sc;
+      const __half hi = __float2half_rn(x);
+      sB[core_idx(j, w + q * WP, NT)] = hi;
+      sB[NT * NT + core_idx(j, w + q * WP, NT)] = __float2half_rn((x - __half2float(hi)) * 2048.f);
     }
   }
   tc_fence_before();
@@ -96,7 +111,7 @@ __global__ void __launch_bounds__(kThreads, 1) update_tc_kernel(const float* Xf,
   const int64_t ntiles = (n + kTR - 1) / kTR;
   auto stage = [&](int64_t tile, float* sX) {
     const int64_t i0 = tile * kTR;
-    for (int c = t; c < kTR * C4; c += kThreads) {
+    for (int c = t; c < kTR * C4; c += kUT) {
       const int r = c / C4, c0 = (c % C4) * 4;
       const int64_t i = i0 + r;
       const bool ok = i < n && c0 < N;
@@ -121,10 +136,28 @@ __global__ void __launch_bounds__(kThreads, 1) update_tc_kernel(const float* Xf,
       if (tq < ntiles) stage(tq, xbuf(q));
       else cp_async_commit();
     }
+  // one buffer only: the next tile waits in registers
+  float4 pre[PRE];
+  auto fetch = [&](int64_t tile) {
+#pragma unroll
+    for (int q = 0; q < PRE; ++q) {
+      const int c = t + q * kUT, r = c / C4, c0 = (c % C4) * 4;
+      const int64_t i = tile * kTR + r;
+      pre[q] = (i < n && c0 < N) ? *reinterpret_cast<const float4*>(Xf + i * N + c0) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  if (L::NBUF == 1 && vec && blockIdx.x < ntiles) fetch(blockIdx.x);
   int64_t k = 0;
   for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++k) {
     float* sX = xbuf(k);
-    if (L::NBUF == 1) {
+    if (L::NBUF == 1 && vec) {
+#pragma unroll
+      for (int q = 0; q < PRE; ++q) {
+        const int c = t + q * kUT;
+        *reinterpret_cast<float4*>(sX + c / C4 * L::LDX + (c % C4) * 4) = pre[q];
+      }
+      if (tile + gridDim.x < ntiles) fetch(tile + gridDim.x);
+    } else if (L::NBUF == 1) {
       stage(tile, sX);
       cp_async_wait<0>();
     } else {
@@ -134,33 +167,48 @@ __global__ void __launch_bounds__(kThreads, 1) update_tc_kernel(const float* Xf,
       cp_async_wait<(L::NBUF > 1 ? L::NBUF - 1 : 0)>();
     }
     __syncthreads();
-    // row means and the largest anomaly of each row: two threads per row
+    // row means and the largest anomaly of each row: four threads per row, each with every fourth group of
+    // eight members in registers
     {
-      const int r = t >> 1, hf = t & 1;
-      float sum = 0.f;
-      for (int k = hf; k < N; k += 2) sum += sX[r * L::LDX + k];
+      constexpr int KC = NT / 32;
+      const int r = t >> 2, hf = t & 3;
+      float x[KC][8], sum = 0.f;
+#pragma unroll
+      for (int c = 0; c < KC; ++c) {
+        const float* src = sX + r * L::LDX + (4 * c + hf) * 8;
+        const float4 a = *reinterpret_cast<const float4*>(src), b = *reinterpret_cast<const float4*>(src + 4);
+        x[c][0] = a.x; x[c][1] = a.y; x[c][2] = a.z; x[c][3] = a.w;
+        x[c][4] = b.x; x[c][5] = b.y; x[c][6] = b.z; x[c][7] = b.w;
+        sum += ((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w));   // (zeros past N)
+      }
       sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+      sum += __shfl_xor_sync(0xffffffffu, sum, 2);
       const float mean = sum / (float)N;
       float mx = 0.f;
-      for (int k = hf; k < N; k += 2) mx = fmaxf(mx, fabsf(sX[r * L::LDX + k] - mean));
+#pragma unroll
+      for (int c = 0; c < KC; ++c)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          x[c][e] = (4 * c + hf) * 8 + e < N ? x[c][e] - mean : 0.f;
+          mx = fmaxf(mx, fabsf(x[c][e]));
+        }
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
       const float sc = pow2_scale(mx);
-      if (hf == 0) {
-        s_mean[r] = mean;
-        s_rs[r] = sc;
-      }
-      // the scaled anomalies as hi + lo FP16, 8 consecutive k (one 16-byte core row) at a time
-      for (int kc = hf; kc < NT / 8; kc += 2) {
+      if (hf == 0) s_rs[r] = sc;
+      // the scaled anomalies as hi + lo FP16, one 16-byte core row at a time
+#pragma unroll
+      for (int c = 0; c < KC; ++c) {
         __align__(16) __half hv[8], lv[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-          const int k = kc * 8 + e;
-          const float a = k < N ? (sX[r * L::LDX + k] - mean) * sc : 0.f;
+          const float a = x[c][e] * sc;
           hv[e] = __float2half_rn(a);
           lv[e] = __float2half_rn((a - __half2float(hv[e])) * 2048.f);
         }
-        *reinterpret_cast<uint4*>(sA + core_idx(r, kc * 8, NT)) = *reinterpret_cast<const uint4*>(hv);
-        *reinterpret_cast<uint4*>(sA + kTR * NT + core_idx(r, kc * 8, NT)) = *reinterpret_cast<const uint4*>(lv);
+        const int kc = (4 * c + hf) * 8;
+        *reinterpret_cast<uint4*>(sA + core_idx(r, kc, NT)) = *reinterpret_cast<const uint4*>(hv);
+        *reinterpret_cast<uint4*>(sA + kTR * NT + core_idx(r, kc, NT)) = *reinterpret_cast<const uint4*>(lv);
       }
     }
     fence_async_smem();
@@ -184,9 +232,10 @@ __global__ void __launch_bounds__(kThreads, 1) update_tc_kernel(const float* Xf,
     const int rt = 32 * qd + lane;
     const int64_t i = tile * kTR + rt;
     const float irs = 1.f / s_rs[rt];
+    if (part < EP)
 #pragma unroll
     for (int c = 0; c < CH; ++c) {
-      const int j0 = half * HALF + 16 * c;
+      const int j0 = (part * CH + c) * 16;
       float d[16], d2[16];
       tmem_ld16(tmem + ((uint32_t)(32 * qd) << 16) + j0, d);
       tmem_ld16(tmem + ((uint32_t)(32 * qd) << 16) + NT + j0, d2);
@@ -210,7 +259,7 @@ __global__ void __launch_bounds__(kThreads, 1) update_tc_kernel(const float* Xf,
     tc_fence_before();
     __syncthreads();
     // the finished tile out: consecutive threads on consecutive 16-byte pieces of a row
-    for (int c = t; c < kTR * C4; c += kThreads) {
+    for (int c = t; c < kTR * C4; c += kUT) {
       const int r = c / C4, c0 = (c % C4) * 4;
       const int64_t ig = tile * kTR + r;
       if (ig < n && c0 < N) {
@@ -235,7 +284,7 @@ static cudaError_t launch_one(const float* Xf, float* Xa, const double* W, int64
   if (e != cudaSuccess) return e;
   const int64_t tiles = (n + kTR - 1) / kTR;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)sms));
-  update_tc_kernel<NT><<<grid, kThreads, smem, s>>>(Xf, Xa, W, n, N, status);
+  update_tc_kernel<NT><<<grid, kUT, smem, s>>>(Xf, Xa, W, n, N, status);
   return cudaGetLastError();
 }
 
