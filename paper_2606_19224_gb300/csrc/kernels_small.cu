@@ -508,20 +508,25 @@ __global__ void __launch_bounds__(kST) small_cg_f32_kernel(SmallParams p) {
     }
     return sync();
   };
-  // (HA T)_i over the SUB lanes s of row i (every lane of the warp calls it)
-  auto row_dot = [&](int i, int s) {
-    float4 a = {0.f, 0.f, 0.f, 0.f};
-    if (i < nr) {
-      const float* h = sH + i * LD;
+  // (HA T)_i and (HA T)_k over the SUB lanes s of the rows i and k (every lane of the warp calls it): two rows
+  // share the reads of T
+  auto row_dots = [&](int i, int k, int s, float& u, float& v) {
+    float4 a = {0.f, 0.f, 0.f, 0.f}, b = a;
+    const float* h = sH + min(i, nr - 1) * LD;   // (nr > 0 where rows are walked)
+    const float* g = sH + min(k, nr - 1) * LD;
 #pragma unroll 4
-      for (int q = s; q < Q4; q += SUB) {
-        const float4 x = *reinterpret_cast<const float4*>(h + 4 * q), y = *reinterpret_cast<const float4*>(sT + 4 * q);
-        a.x = fmaf(x.x, y.x, a.x); a.y = fmaf(x.y, y.y, a.y); a.z = fmaf(x.z, y.z, a.z); a.w = fmaf(x.w, y.w, a.w);
-      }
+    for (int q = s; q < Q4; q += SUB) {
+      const float4 y = *reinterpret_cast<const float4*>(sT + 4 * q);
+      const float4 x = *reinterpret_cast<const float4*>(h + 4 * q), w = *reinterpret_cast<const float4*>(g + 4 * q);
+      a.x = fmaf(x.x, y.x, a.x); a.y = fmaf(x.y, y.y, a.y); a.z = fmaf(x.z, y.z, a.z); a.w = fmaf(x.w, y.w, a.w);
+      b.x = fmaf(w.x, y.x, b.x); b.y = fmaf(w.y, y.y, b.y); b.z = fmaf(w.z, y.z, b.z); b.w = fmaf(w.w, y.w, b.w);
     }
-    float u = (a.x + a.y) + (a.z + a.w);
-    for (int o = SUB / 2; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
-    return u;
+    u = (a.x + a.y) + (a.z + a.w);
+    v = (b.x + b.y) + (b.z + b.w);
+    for (int o = SUB / 2; o > 0; o >>= 1) {
+      u += __shfl_xor_sync(0xffffffffu, u, o);
+      v += __shfl_xor_sync(0xffffffffu, v, o);
+    }
   };
   // sum over the cluster's rows of f(i), in FP64
   auto sum64 = [&](auto f) {
@@ -620,24 +625,27 @@ __global__ void __launch_bounds__(kST) small_cg_f32_kernel(SmallParams p) {
       const float al = sc[0], be = sc[1], finv = (float)inv;
       // u = HA T, SUB lanes per row, the step on the row, and the sums of the next one
       float v0 = 0.f, v1 = 0.f, v2 = 0.f, v3 = 0.f;
-      for (int i0 = 0; i0 < nr; i0 += kST / SUB) {
-        const int i = i0 + t / SUB, s = t % SUB;
-        const float u = row_dot(i, s);
-        if (i < nr && s == 0) {
-          const float z = sb[i], ri = sr[i];
-          const float pn = it == 0 ? z : fmaf(be, sp[i], z);
-          const float q = fmaf(u, finv, ri * pn);
-          const float rn = fmaf(-al, q, sres[i]);
-          const float zn = PC ? rn * (1.f / ri) : rn, rz = ri * zn;
-          sp[i] = pn;
-          sx[i] = fmaf(al, pn, sx[i]);
-          sres[i] = rn;
-          sb[i] = zn;
-          v0 = fmaf(rn, zn, v0);
-          v1 = fmaf(rn, rn, v1);
-          v2 = fmaf(rz, zn, v2);
-          v3 = fmaf(rz, pn, v3);
-        }
+      auto step = [&](int i, float u) {
+        const float z = sb[i], ri = sr[i];
+        const float pn = it == 0 ? z : fmaf(be, sp[i], z);
+        const float q = fmaf(u, finv, ri * pn);
+        const float rn = fmaf(-al, q, sres[i]);
+        const float zn = PC ? rn * (1.f / ri) : rn, rz = ri * zn;
+        sp[i] = pn;
+        sx[i] = fmaf(al, pn, sx[i]);
+        sres[i] = rn;
+        sb[i] = zn;
+        v0 = fmaf(rn, zn, v0);
+        v1 = fmaf(rn, rn, v1);
+        v2 = fmaf(rz, zn, v2);
+        v3 = fmaf(rz, pn, v3);
+      };
+      for (int i0 = 0; i0 < nr; i0 += 2 * kST / SUB) {
+        const int i = i0 + t / SUB, k = i + kST / SUB, s = t % SUB;
+        float u, v;
+        row_dots(i, k, s, u, v);
+        if (i < nr && s == 0) step(i, u);
+        if (k < nr && s == 0) step(k, v);
       }
       warp_sums(v0, v1, v2, v3);
       __syncthreads();
