@@ -344,8 +344,13 @@ __global__ void __launch_bounds__(kThreads) senkf_sum_kernel(const double* __res
   sum_partials(part, nparts, 2 * (int64_t)N * N, N * N, [&](int e, double s) { W[e] = s; });
 }
 
-// One CTA per column j of M: CG for G v_j = m_j (FP64), G staged in shared memory.
-// V is [N][N] row-major (V[k][j]).
+// One CTA per column j of M: CG for G v_j = m_j (FP64), G staged in shared memory; V is [N][N] row-major
+// (V[k][j]). The step has one product and one round of sums: with g = G r, (p, G p) =
+// (r, g) - beta^2 (p, G p)_old and G p = g + beta (G p)_old. What bounds it is the FP64 unit (2 per clock
+// per SM; a warp's instruction holds its scheduler's unit for about 64 cycles): N^2 DFMAs are 2,048
+// cycles at N = 64, so the scalars run on one warp, the reciprocal for beta beside the product, and the sums of a
+// step share one shuffle tree per warp. 28 steps at N = 64 take 105 us; the two-reduction form, with every
+// warp folding every sum and dividing, took 128.
 __global__ void __launch_bounds__(kThreads) reduced_cg_kernel(
     const double* __restrict__ Gm, const double* __restrict__ Mm, int N, double tol, int max_iter,
     int fixed_iters, double* __restrict__ V, int* __restrict__ col_iters,
@@ -354,107 +359,120 @@ __global__ void __launch_bounds__(kThreads) reduced_cg_kernel(
   // G with row stride N + 1: lanes on consecutive rows k then read distinct banks
   const int ld = N + 1;
   double* sG = sm;                 // N x (N + 1)
-  double* sx = sG + N * ld;        // N
-  double* sr = sx + N;             // N
-  double* sp = sr + N;             // N
-  double* sq = sp + N;             // N
-  double* sb = sq + N;             // N (right-hand side)
-  double* spart = sb + N;          // [kThreads] partial row sums of the matvec
-  __shared__ double red[kThreads / 32];
+  double* su = sG + N * ld;        // N: the product's operand
+  double* spart = su + N;          // [kThreads] partial row sums of the product
+  __shared__ double red[2][4], sc[5];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int j = blockIdx.x;
+  // the product: thread t forms the partial sum of row k = t % NP over columns l = g, g + P, ...
+  // (g = t / NP, P = kThreads / NP groups); thread k adds the P partials of row k in order
+  const int NP = N <= 64 ? 64 : 128, P = kThreads / NP, NW = NP / 32;
   for (int e = t; e < N * N; e += kThreads) sG[(e / N) * ld + e % N] = Gm[e];
-  for (int k = t; k < N; k += kThreads) {
-    const double b = Mm[k * N + j];
-    sb[k] = b;
-    sx[k] = 0.0;
-    sr[k] = b;
-    sp[k] = b;
-  }
+  const bool own = t < N;          // thread k keeps row k of the vectors
+  const double b = own ? Mm[t * N + j] : 0.0;
+  double x = 0.0, r = b, p = 0.0, h = 0.0;
+  if (own) su[t] = b;
   __syncthreads();
-  // block-wide sum, the same fixed-order tree in every warp (FP64 instructions are scarce on
-  // this part, so the eight warp sums are folded by three shuffle steps, not a serial loop)
-  auto block_sum = [&](double v) -> double {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    double s = lane < kThreads / 32 ? red[lane] : 0.0;
-#pragma unroll
-    for (int o = kThreads / 64; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    return __shfl_sync(0xffffffffu, s, 0);
-  };
-  // G u: thread t forms the partial sum of row k = t % NP over columns l = g, g + P, ...
-  // (g = t / NP, P = kThreads / NP groups); row k's owner (thread k) adds the P partials in
-  // a fixed order. Ends with the partials written and synchronised.
-  const int NP = N <= 64 ? 64 : 128, P = kThreads / NP;
-  auto matvec_partials = [&](const double* u) {
+  auto product = [&]() -> double {
     const int k = t % NP, g = t / NP;
-    double acc = 0.0;
-    if (k < N)
-      for (int l = g; l < N; l += P) acc = fma(sG[k * ld + l], u[l], acc);
-    spart[t] = acc;
+    double a0 = 0.0, a1 = 0.0;
+    if (k < N) {
+      int l = g;
+      for (; l + P < N; l += 2 * P) {
+        a0 = fma(sG[k * ld + l], su[l], a0);
+        a1 = fma(sG[k * ld + l + P], su[l + P], a1);
+      }
+      if (l < N) a0 = fma(sG[k * ld + l], su[l], a0);
+    }
+    spart[t] = a0 + a1;
     __syncthreads();
-  };
-  auto row_of = [&](int k) -> double {
-    double s = spart[k];
-    for (int g = 1; g < P; ++g) s += spart[g * NP + k];
+    double s = 0.0;
+    if (own) {
+      s = spart[t];
+      for (int g2 = 1; g2 < P; ++g2) s += spart[g2 * NP + t];
+    }
     return s;
   };
-  double v = 0.0;
-  for (int k = t; k < N; k += kThreads) v = fma(sb[k], sb[k], v);
-  const double bn2 = block_sum(v);
-  // |r| <= tol |b| compared in squares, with tol shrunk by 4 ulps so that a stop always gives
-  // sqrt(rr / bn2) <= tol for the residual reported below
-  const double tol_s = tol * (1.0 - 4.0 * 2.220446049250313e-16);
-  const double stop2 = tol_s * tol_s * bn2;
-  double rr = bn2;
+  // totals of two values over the CTA's owners, into red (warp w's part in red[.][w])
+  auto fold = [&](double u, double v) {
+    if (warp < NW) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        u += __shfl_xor_sync(0xffffffffu, u, o);
+        v += __shfl_xor_sync(0xffffffffu, v, o);
+      }
+      if (lane == 0) {
+        red[0][warp] = u;
+        red[1][warp] = v;
+      }
+    }
+    __syncthreads();
+  };
+  auto folded = [&](int q) {
+    double s = red[q][0];
+    for (int w = 1; w < NW; ++w) s += red[q][w];
+    return s;
+  };
   const bool fixed = fixed_iters > 0;
   const int limit = fixed ? fixed_iters : max_iter;
+  double bn2 = 0.0, rr = 0.0, pq = 0.0, stop2 = 0.0;   // warp 0's
   int it = 0;
-  bool active = rr > 0.0;
-  for (; it < limit && active; ++it) {
-    // q = G p
-    matvec_partials(sp);
-    v = 0.0;
-    for (int k = t; k < N; k += kThreads) {
-      const double qk = row_of(k);
-      sq[k] = qk;
-      v = fma(sp[k], qk, v);
+  for (;;) {
+    // one thread divides for the next beta beside the product
+    if (it > 0 && t == kThreads - 1) sc[3] = 1.0 / sc[4];
+    const double g = product();
+    fold(r * r, r * g);
+    if (warp == 0) {
+      const double r2 = folded(0), rg = folded(1);
+      if (it == 0) {
+        // |r| <= tol |b| compared in squares, with tol shrunk by 4 ulps so that a stop always gives
+        // sqrt(rr / bn2) <= tol for the residual reported below
+        const double tol_s = tol * (1.0 - 4.0 * 2.220446049250313e-16);
+        bn2 = r2;
+        stop2 = tol_s * tol_s * bn2;
+      }
+      bool go = it < limit && (it == 0 || fixed ? r2 > 0.0 : r2 > stop2);
+      const double be = go && it > 0 ? r2 * sc[3] : 0.0;
+      double al = 0.0;
+      if (go) {
+        const double q = fma(-be * be, pq, rg);
+        if (!(q > 0.0) || !isfinite(q)) {
+          if (lane == 0) atomicOr(status, isfinite(q) ? DS_BREAKDOWN : DS_NONFINITE);
+          go = false;
+        } else {
+          pq = q;
+          al = r2 / q;
+        }
+      }
+      rr = r2;
+      if (lane == 0) {
+        sc[0] = al;
+        sc[1] = be;
+        sc[2] = go ? 1.0 : 0.0;
+        sc[4] = r2;
+      }
     }
-    const double pq = block_sum(v);
-    if (!(pq > 0.0) || !isfinite(pq)) {
-      if (t == 0) atomicOr(status, isfinite(pq) ? DS_BREAKDOWN : DS_NONFINITE);
-      break;
-    }
-    const double alpha = rr / pq;
-    v = 0.0;
-    for (int k = t; k < N; k += kThreads) {
-      sx[k] = fma(alpha, sp[k], sx[k]);
-      const double rn = fma(-alpha, sq[k], sr[k]);
-      sr[k] = rn;
-      v = fma(rn, rn, v);
-    }
-    const double rn2 = block_sum(v);
-    const double beta = rn2 / rr;
-    rr = rn2;
-    for (int k = t; k < N; k += kThreads) sp[k] = fma(beta, sp[k], sr[k]);
     __syncthreads();
-    if (fixed) active = rr > 0.0;
-    else active = rr > stop2;
+    if (sc[2] == 0.0) break;
+    const double al = sc[0], be = sc[1];
+    if (own) {
+      p = fma(be, p, r);
+      h = fma(be, h, g);
+      x = fma(al, p, x);
+      r = fma(-al, h, r);
+      su[t] = r;
+    }
+    ++it;
+    __syncthreads();
   }
   // true residual m_j - G v_j (FP64)
+  if (own) su[t] = x;
   __syncthreads();
-  matvec_partials(sx);
-  v = 0.0;
-  for (int k = t; k < N; k += kThreads) {
-    const double d = sb[k] - row_of(k);
-    v = fma(d, d, v);
-  }
-  const double tr2 = block_sum(v);
-  for (int k = t; k < N; k += kThreads) V[k * N + j] = sx[k];
+  const double d = b - product();
+  fold(own ? d * d : 0.0, 0.0);
+  if (own) V[t * N + j] = x;
   if (t == 0) {
+    const double tr2 = folded(0);
     col_iters[j] = it;
     const double rel = bn2 > 0.0 ? sqrt(rr / bn2) : 0.0;
     col_relres[j] = rel;
@@ -548,7 +566,7 @@ cudaError_t launch_nxn_stage(enkf_handle_s* h) {
   if (f64) reduced_sum_kernel<<<(NN2 + 31) / 32, kThreads, 0, h->stream>>>(ws.Tpart, grid, c.N, Gm, Mm);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const size_t smem = sizeof(double) * ((size_t)c.N * (c.N + 1) + 5 * c.N + kThreads);
+  const size_t smem = sizeof(double) * ((size_t)c.N * (c.N + 1) + c.N + kThreads);
   e = cudaFuncSetAttribute(reduced_cg_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   reduced_cg_kernel<<<c.N, kThreads, smem, h->stream>>>(Gm, Mm, c.N, c.tol, c.max_iter, c.fixed_iters,
