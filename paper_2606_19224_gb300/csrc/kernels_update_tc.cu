@@ -1,10 +1,10 @@
 // The ensemble update X_a = X_f + A W (Fig. 2, Algorithm 1: A = X_f - xbar 1^T, W = HA^T Z/(N-1))
 // on the 5th-generation tensor cores, for FP32 ensembles.
 //
-// Per 128-row tile of X_f: the rows are staged in shared memory (16-byte cp.async; for N <= 64
-// the next two tiles' copies are in flight behind the current one), each row's mean and largest anomaly are
-// formed, and the anomalies scaled by an exact power of two per row (so FP16 neither overflows
-// nor flushes) are split into hi + lo FP16 parts in the canonical K-major core-matrix layout,
+// Per 128-row tile of X_f: the rows are staged in shared memory (the next tile's are in flight in
+// registers meanwhile; two CTAs per SM for N <= 64, so that one converts while the other's stores drain),
+// each row's mean and largest anomaly are formed, and the anomalies scaled by an exact power of two per
+// row (so FP16 neither overflows nor flushes) are split into hi + lo FP16 parts in the canonical K-major core-matrix layout,
 // the lo part stored times 2^11 so that it stays in FP16's normal range. W is staged once per
 // CTA the same way (rows j, K-major over k, a power-of-two scale per column). D = A W runs as
 // three M = 128 x N = NT x K = NT MMAs per K block with FP32 accumulation in TMEM: hi*hi into
@@ -30,9 +30,8 @@ template <int NT> struct UpdLayout {
   static constexpr int XT = kTR * LDX * 4;                 // bytes per staged tile
   static constexpr int AIMG = 2 * kTR * NT * 2;            // A image: hi and lo parts
   static constexpr int BIMG = 2 * NT * NT * 2;             // W image: hi and lo parts
-  static constexpr int NBUF = NT <= 64 ? 3 : 1;            // staged tiles (NT = 128: one, smem)
   static constexpr int off_x = 0;
-  static constexpr int off_a = ((NBUF * XT + 1023) / 1024) * 1024;
+  static constexpr int off_a = ((XT + 1023) / 1024) * 1024;
   static constexpr int off_b = off_a + AIMG;
   static constexpr int off_rs = off_b + BIMG;              // per-row 2^-e scale [128]
   static constexpr int off_ws = off_rs + 4 * kTR;          // per-column 1/scale of W [NT]
@@ -50,9 +49,8 @@ __device__ __forceinline__ float pow2_scale(float vmax) {
 }
 
 template <int NT>
-__global__ void __launch_bounds__(kUT, 1) update_tc_kernel(const float* Xf, float* Xa,
-                                                                const double* __restrict__ W, int64_t n,
-                                                                int N, int* status) {
+__global__ void __launch_bounds__(kUT, NT <= 64 ? 2 : 1) update_tc_kernel(
+    const float* Xf, float* Xa, const double* __restrict__ W, int64_t n, int N, int* status) {
   using L = UpdLayout<NT>;
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t mbar;
@@ -64,7 +62,7 @@ __global__ void __launch_bounds__(kUT, 1) update_tc_kernel(const float* Xf, floa
   constexpr int EP = NT < 64 ? 2 : 4, CH = NT / EP / 16;   // epilogue: column parts, 16-column chunks of each
   constexpr int PRE = kTR * C4 / kUT;                      // 16-byte pieces of a tile per thread
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31, qd = warp & 3, part = warp >> 2;
-  float* sX0 = reinterpret_cast<float*>(smem + L::off_x);
+  float* sX = reinterpret_cast<float*>(smem + L::off_x);
   __half* sA = reinterpret_cast<__half*>(smem + L::off_a);
   __half* sB = reinterpret_cast<__half*>(smem + L::off_b);
   float* s_rs = reinterpret_cast<float*>(smem + L::off_rs);
@@ -89,10 +87,10 @@ __global__ void __launch_bounds__(kUT, 1) update_tc_kernel(const float* Xf, floa
       v[q] = (j < N && k < N) ? (float)__ldcg(W + k * N + j) : 0.f;
       mx = fmaxf(mx, fabsf(v[q]));
     }
-    sX0[w * NT + j] = mx;
+    sX[w * NT + j] = mx;
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < WP; ++q) mx = fmaxf(mx, sX0[q * NT + j]);
+    for (int q = 0; q < WP; ++q) mx = fmaxf(mx, sX[q * NT + j]);
     const float sc = pow2_scale(mx);
     if (w == 0) s_ws[j] = 1.f / sc;                       // exact (a power of two)
 #pragma unroll
@@ -109,63 +107,28 @@ __global__ void __launch_bounds__(kUT, 1) update_tc_kernel(const float* Xf, floa
   const uint32_t tmem = tmem_base;
   const bool vec = (N & 3) == 0;
   const int64_t ntiles = (n + kTR - 1) / kTR;
-  auto stage = [&](int64_t tile, float* sX) {
-    const int64_t i0 = tile * kTR;
-    for (int c = t; c < kTR * C4; c += kUT) {
-      const int r = c / C4, c0 = (c % C4) * 4;
-      const int64_t i = i0 + r;
-      const bool ok = i < n && c0 < N;
-      if (vec) {
-        cp_async16(sX + r * L::LDX + c0, ok ? Xf + i * N + c0 : Xf, ok);
-      } else {
-        float a[4] = {0.f, 0.f, 0.f, 0.f};
-        if (ok) ld4<float>(a, Xf + i * N, c0, N, false);
-        *reinterpret_cast<float4*>(sX + r * L::LDX + c0) = make_float4(a[0], a[1], a[2], a[3]);
-      }
-    }
-    cp_async_commit();
-  };
   uint32_t ph = 0;
   bool ok = true;
-  auto xbuf = [&](int64_t k) { return sX0 + (int)(k % L::NBUF) * (L::XT / 4); };
-  // NBUF - 1 tiles in flight ahead of the one being processed (one commit group per tile,
-  // empty past the end, so that "all but the newest NBUF - 1 groups" is always this tile)
-  if (L::NBUF > 1)
-    for (int q = 0; q < L::NBUF - 1; ++q) {
-      const int64_t tq = (int64_t)blockIdx.x + (int64_t)q * gridDim.x;
-      if (tq < ntiles) stage(tq, xbuf(q));
-      else cp_async_commit();
-    }
-  // one buffer only: the next tile waits in registers
+  // the next tile waits in registers
   float4 pre[PRE];
   auto fetch = [&](int64_t tile) {
 #pragma unroll
     for (int q = 0; q < PRE; ++q) {
       const int c = t + q * kUT, r = c / C4, c0 = (c % C4) * 4;
       const int64_t i = tile * kTR + r;
-      pre[q] = (i < n && c0 < N) ? *reinterpret_cast<const float4*>(Xf + i * N + c0) : make_float4(0.f, 0.f, 0.f, 0.f);
+      float a[4] = {0.f, 0.f, 0.f, 0.f};
+      if (i < n && c0 < N) ld4<float>(a, Xf + i * N, c0, N, vec);
+      pre[q] = make_float4(a[0], a[1], a[2], a[3]);
     }
   };
-  if (L::NBUF == 1 && vec && blockIdx.x < ntiles) fetch(blockIdx.x);
-  int64_t k = 0;
-  for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++k) {
-    float* sX = xbuf(k);
-    if (L::NBUF == 1 && vec) {
+  if (blockIdx.x < ntiles) fetch(blockIdx.x);
+  for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
 #pragma unroll
-      for (int q = 0; q < PRE; ++q) {
-        const int c = t + q * kUT;
-        *reinterpret_cast<float4*>(sX + c / C4 * L::LDX + (c % C4) * 4) = pre[q];
-      }
-      if (tile + gridDim.x < ntiles) fetch(tile + gridDim.x);
-    } else if (L::NBUF == 1) {
-      stage(tile, sX);
-      cp_async_wait<0>();
-    } else {
-      const int64_t nxt = tile + (int64_t)(L::NBUF - 1) * gridDim.x;
-      if (nxt < ntiles) stage(nxt, xbuf(k + L::NBUF - 1));   // the buffer of tile k - 1, consumed
-      else cp_async_commit();
-      cp_async_wait<(L::NBUF > 1 ? L::NBUF - 1 : 0)>();
+    for (int q = 0; q < PRE; ++q) {
+      const int c = t + q * kUT;
+      *reinterpret_cast<float4*>(sX + c / C4 * L::LDX + (c % C4) * 4) = pre[q];
     }
+    if (tile + gridDim.x < ntiles) fetch(tile + gridDim.x);
     __syncthreads();
     // row means and the largest anomaly of each row: four threads per row, each with every fourth group of
     // eight members in registers
@@ -270,7 +233,6 @@ __global__ void __launch_bounds__(kUT, 1) update_tc_kernel(const float* Xf, floa
     }
     __syncthreads();   // the staged tile, the A image and TMEM are rewritten by the next tile
   }
-  cp_async_wait<0>();
   tc_fence_before();
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMC));
@@ -283,7 +245,7 @@ static cudaError_t launch_one(const float* Xf, float* Xa, const double* W, int64
   cudaError_t e = cudaFuncSetAttribute(update_tc_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const int64_t tiles = (n + kTR - 1) / kTR;
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)sms));
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)sms * (NT <= 64 ? 2 : 1)));
   update_tc_kernel<NT><<<grid, kUT, smem, s>>>(Xf, Xa, W, n, N, status);
   return cudaGetLastError();
 }
