@@ -61,6 +61,11 @@ MIXED_WORKLOAD = "grf1024_N128_m262144"
 #                 + 2 m 8 (r_i, twice);  F = 4 m N^2 (HA^T p and HA (.))
 #   per refresh:  B = 2 m N s_HA + 3 m N s_v (HA twice, Z, D in, residual out)
 # s_HA = s_v = 8 (FP64), 4 (FP32); s_HA = 2 for BF16/FP16 HA with FP32 vectors.
+# Preconditioned by R, the FP32-ensemble modes carry CG in the coordinates of its Krylov space
+# (csrc/krylov.cuh): the steps touch N x N matrices only, and a refinement cycle is three passes over
+# the rows in double-float:
+#   per cycle:    B = 68 m N (pass G: HA, D; Z: HA, D in, Z out; R: HA, D, Z in, residual out)
+#                 F = 10 m N^2 (K, F = HA^T R^-1 D, HA w, HA^T Z, HA T)
 S_BYTES = {"fp64": (8, 8), "fp32": (4, 4), "fp16": (2, 4), "bf16": (2, 4)}
 
 
@@ -76,6 +81,14 @@ def B_REF(m, N, prec="fp32"):
 
 def F_ITER(m, N):
     return 4.0 * m * N * N
+
+
+def B_CYCLE(m, N):
+    return 68 * m * N
+
+
+def F_CYCLE(m, N):
+    return 10.0 * m * N * N
 
 
 def B_FUSED(m, N):
@@ -107,12 +120,16 @@ def _tensor_peak():
         return 1700.0
 
 
-def analysis_roofline(m, N, prec, iters, refreshes, solve_ms, kernel, traffic=None):
-    """Roofline of one solve launch on the byte and flop model above."""
+def analysis_roofline(m, N, prec, iters, refreshes, solve_ms, kernel, traffic=None, krylov=False):
+    """Roofline of one solve launch on the byte and flop models above (krylov: the passes of its
+    refinement cycles, whose products run on the tensor cores in every mode)."""
     bw, bw_src = _peaks()
-    pf, pf_src = _peak_flops(prec)
-    B = iters * B_ITER(m, N, prec) + refreshes * B_REF(m, N, prec)
-    F = iters * F_ITER(m, N)
+    pf, pf_src = _peak_flops("fp16" if krylov else prec)
+    if krylov:
+        B, F = refreshes * B_CYCLE(m, N), refreshes * F_CYCLE(m, N)
+    else:
+        B = iters * B_ITER(m, N, prec) + refreshes * B_REF(m, N, prec)
+        F = iters * F_ITER(m, N)
     t_b = B / (bw * 1e9)
     t_f = F / (pf * 1e12)
     t = solve_ms / 1e3
@@ -139,10 +156,10 @@ NCU_TRAFFIC = {"fp32": {"bytes": 0.765940e9, "src_sha": "e360a9e69a4aec5f"},
 # profiles/batch_kernel_batched256_grf_dram.md for the sources with this hash.
 NCU_TRAFFIC_BATCH = {"bytes": 1.436453e12, "problems": 256, "seed": 1, "src_sha": "869cf69968486ece"}
 _KERNEL_SOURCES = {
-    "fp32": ("kernels_fp.cu", "common.cuh", "cg_device.cuh", "solve_body.cuh"),
-    "fp16": ("kernels_tc.cu", "kernels_tc_fp16.cu", "tc_mixed.cuh", "common.cuh", "cg_device.cuh"),
-    "bf16": ("kernels_tc.cu", "kernels_tc_bf16.cu", "tc_mixed.cuh", "common.cuh", "cg_device.cuh"),
-    "batch": ("kernels_batch.cu", "solve_body.cuh", "innov_device.cuh", "common.cuh", "cg_device.cuh"),
+    "fp32": ("kernels_krylov.cu", "krylov.cuh", "tc_mixed.cuh", "common.cuh", "cg_device.cuh"),
+    "fp16": ("kernels_krylov.cu", "krylov.cuh", "tc_mixed.cuh", "common.cuh", "cg_device.cuh"),
+    "bf16": ("kernels_krylov.cu", "krylov.cuh", "tc_mixed.cuh", "common.cuh", "cg_device.cuh"),
+    "batch": ("kernels_batch.cu", "krylov.cuh", "solve_body.cuh", "innov_device.cuh", "common.cuh", "cg_device.cuh"),
 }
 
 
@@ -163,30 +180,17 @@ def _src_hash(precision="fp32"):
     return h.hexdigest()[:16]
 
 
-# FP32 instruction rate of a GB300 at its 2.07 GHz maximum clock: 152 SMs x 128 FP32 lanes,
-# one operation per lane and clock (tera-operations per second)
-FP32_OPS_PEAK_T = 152 * 128 * 2.07e9 / 1e12
-# FP32 operations per term of a double-float product sum (exact product by FMA with the
-# cross terms, TwoSum into the running sum, error gathered in the compensation word)
-DF_OPS_PER_TERM = 12
-
-
 def _gram_roofline(terms, ms, m, N, ens_bytes=4):
     """The Gram pass of the Reduced and sEnKF variants (`terms` products m N^2 or 2 m N^2 per
     launch, reading the observed rows of X_f plus the CSR operator, r and y). The roofline is
-    the slower of the products at the FP32 FMA peak and the bytes at HBM bandwidth; the
-    issue efficiency of the double-float implementation (12 FP32 operations per product
-    against the FP32 lanes x clock) is reported beside it, not as the roofline fraction."""
+    the slower of the products at the FP32 FMA peak and the bytes at HBM bandwidth (the products
+    run on the tensor cores from exact FP16 slices)."""
     bw, bw_src = _peaks()
     t = ms / 1e3
     B = ens_bytes * m * N + 32 * m
     t_f = 2.0 * terms / (FP32_TFLOPS * 1e12)
     t_b = B / (bw * 1e9)
-    ops = DF_OPS_PER_TERM * terms
-    issue = ops / t / 1e12
-    base = {"terms_per_launch": terms, "algorithmic_bytes_per_launch": B, "launch_ms": ms,
-            "issue_efficiency": {"achieved": issue, "peak": FP32_OPS_PEAK_T, "unit": "T FP32 op/s",
-                                 "frac": issue / FP32_OPS_PEAK_T, "ops_per_term": DF_OPS_PER_TERM}}
+    base = {"terms_per_launch": terms, "algorithmic_bytes_per_launch": B, "launch_ms": ms}
     if t_f >= t_b:
         base.update({"bound": "alu", "achieved": 2.0 * terms / t / 1e12, "peak": FP32_TFLOPS, "unit": "TFLOP/s",
                      "frac": t_f / t, "peak_source": "FP32 FMA, measured"})
@@ -453,13 +457,21 @@ def _err(out, ref):
 
 # how each step's sums over the CTAs are formed (enkf_config.reduce_order)
 DTYPE = {"fp32": "f32", "fp16": "f16", "bf16": "bf16"}
+# (preconditioned by R, the three modes share the Krylov-coordinate solve, its products on exact FP16 slices
+# in tcgen05 and its double-float residual)
 PRECISION_NAME = {"fp32": "fp32 CG + double-float residual refresh",
-                  "fp16": "FP16 hi/lo tensor-core contractions (tcgen05) + double-float refresh",
-                  "bf16": "BF16 hi/lo tensor-core contractions (tcgen05) + double-float refresh"}
+                  "fp16": "FP16 tensor-core contractions (tcgen05) + double-float refresh",
+                  "bf16": "BF16 tensor-core contractions (tcgen05) + double-float refresh"}
 REDUCE_NAME = {0: "fixed order (bitwise repeatable)",
                1: "atomic adds (N <= 64; last bits vary from run to run)"}
 KERNEL_NAME = {"fp64": "solve_kernel<double>", "fp32": "solve_kernel<float>",
                "fp16": "solve_mixed_kernel<half>", "bf16": "solve_mixed_kernel<bf16>"}
+
+
+def _solve_kernel(prec, pc):
+    if not pc:
+        return KERNEL_NAME[prec], False
+    return ("solve64_kernel", False) if prec == "fp64" else ("krylov_kernel", True)
 
 
 def _variant(enkf, p, prec, pc, timer, Xd, y, seed, steps, warmup, ref, reduce_order=0, traffic=None):
@@ -479,7 +491,7 @@ def _variant(enkf, p, prec, pc, timer, Xd, y, seed, steps, warmup, ref, reduce_o
     res["solver"] = "CG preconditioned by R" if pc else "plain CG"
     res["reduce_order"] = REDUCE_NAME[reduce_order]
     res["roofline"] = analysis_roofline(p.m, p.N, prec, res["iters"], res["refinements"] if prec != "fp64" else 1,
-                                        res["solve_ms"], KERNEL_NAME[prec], traffic)
+                                        res["solve_ms"], _solve_kernel(prec, pc)[0], traffic, _solve_kernel(prec, pc)[1])
     an.close()
     return res
 
@@ -572,12 +584,13 @@ def run_ours(args):
     solve_avg_ms = float(np.mean(solve_ms))
     traffic = _recorded_traffic(args.precision, args.precondition, args.reduce_order)
     roofline = analysis_roofline(m, N, args.precision, it_avg, ref_avg, solve_avg_ms,
-                                 KERNEL_NAME[args.precision] + ("<64, preconditioned>" if args.precondition else "<64>"),
-                                 traffic)
-    roofline["fused_pass_model"] = {
-        "bytes_per_launch": it_avg * B_FUSED(m, N) + ref_avg * 56 * m * N,
-        "note": "HA read once per step, x, r, p read and written (28 m N + 4 m) and a double-float refresh "
-                "of 56 m N bytes: what the fused implementation moves at minimum"}
+                                 _solve_kernel(args.precision, args.precondition)[0] + "<64>", traffic,
+                                 _solve_kernel(args.precision, args.precondition)[1])
+    if not args.precondition:
+        roofline["fused_pass_model"] = {
+            "bytes_per_launch": it_avg * B_FUSED(m, N) + ref_avg * 56 * m * N,
+            "note": "HA read once per step, x, r, p read and written (28 m N + 4 m) and a double-float refresh "
+                    "of 56 m N bytes: what the fused implementation moves at minimum"}
 
     prec_name = PRECISION_NAME[args.precision]
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
@@ -858,8 +871,8 @@ def _batch_run(args, enkf, dev, timer, probs, seed, steps, warmup, ws=1, barrier
     # roofline: algorithmic bytes of all problems of one launch over the launch time
     alg = 0.0
     for i, p in enumerate(probs):
-        alg += float(st["iters_max"][i]) * B_ITER(p.m, p.N) + float(st["refinements"][i]) * B_REF(p.m, p.N)
-        alg += 4 * p.n * p.N * 2 + 3 * 4 * p.m * p.N   # update (X_f in, X_a out); innovations (HA, D written, X_f rows read)
+        alg += float(st["refinements"][i]) * B_CYCLE(p.m, p.N)
+        alg += 4 * p.n * p.N * 2 + 20 * p.m * p.N   # update (X_f in, X_a out); innovations (HA, D written, X_f rows read)
     launch_ms = ms / steps
     peak, peak_src = _peaks()
     achieved = alg / (launch_ms / 1e3) / 1e9
