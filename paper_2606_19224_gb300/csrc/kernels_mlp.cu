@@ -75,7 +75,7 @@ __device__ __forceinline__ float gelu_grad_f(float x) {
 // the network's products have 8 to 136 tiles, which alone leave most SMs idle. Loads run along the
 // contiguous index of each operand. (32 x 32 tiles with 2 x 2 outputs per thread and loads along the
 // strided index took 15 to 30 us per product at batch 256, 1088 -> 512^3 -> 64; loss and gradient 345 us, now
-// 172.)
+// 164.)
 constexpr int GT = 64, GBK = 32, GLD = GBK + 4;
 
 enum : int { EPI_HIDDEN = 0, EPI_OUT = 1, EPI_BWD = 2, EPI_STORE = 3 };
@@ -231,9 +231,13 @@ __global__ void __launch_bounds__(256) mlp_gemm_kernel(const GemmArgs g) {
 template <int EPI>
 static cudaError_t gemm(GemmArgs a, cudaStream_t s) {
   const int tn = (a.N + GT - 1) / GT, tm = (a.M + GT - 1) / GT, steps = (a.K + GBK - 1) / GBK;
-  // enough clusters to fill the chip once, and at least two steps along K per CTA
+  // enough clusters to fill the chip once, and a step along K per CTA at least
   a.split = 1;
-  while (a.split < 8 && (int64_t)tn * tm * a.split * 2 <= 160 && steps >= 4 * a.split) a.split *= 2;
+  while (a.split < 8 && (int64_t)tn * tm * a.split * 2 <= 160 && steps >= 2 * a.split) a.split *= 2;
+  if (a.split == 1) {
+    mlp_gemm_kernel<EPI><<<dim3(tn, tm), 256, 0, s>>>(a);
+    return cudaGetLastError();
+  }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(tn * a.split, tm);
   cfg.blockDim = dim3(256);
