@@ -6,7 +6,7 @@
 //                  (Sec. 3.3, Eq. matvec_decomp); N independent recurrences share each
 //                  matvec; FP64 scalars; FP32 mode = FP32 inner solves + double-float residual
 //                  refresh (iterative refinement), all on the device in one launch
-//   update_kernel  X_a = X_f + A W, W = HA^T Z/(N-1), A = X_f - xbar 1^T  (Fig. 2, Alg. 1)
+//   update_kernel  X_a = X_f V of CGD-EnKF-Reduced, FP32 ensembles (Algorithm 2)
 //
 // Data layout: every [rows][N] array is row-major with the member index fastest. The
 // persistent grid splits the m observation rows into contiguous blocks, one per CTA (the
@@ -68,14 +68,12 @@ __global__ void convert_r_kernel(const double* __restrict__ r, float* __restrict
     r32[i] = (float)r[i];
 }
 
-template <typename VT, int NT, int MODE = 0>
-__global__ void __launch_bounds__(kThreads) update_kernel(const VT* Xf, VT* Xa,
-                                                          const double* __restrict__ W,
+template <int NT>
+__global__ void __launch_bounds__(kThreads) update_kernel(const float* Xf, float* Xa, const double* __restrict__ W,
                                                           int64_t n, int N) {
   extern __shared__ __align__(16) unsigned char smem[];
-  update_rows<VT, NT, MODE>(Xf, Xa, W, n, N, blockIdx.x, gridDim.x, smem);
+  update_rows<float, NT, 1>(Xf, Xa, W, n, N, blockIdx.x, gridDim.x, smem);
 }
-
 
 // ------------------------------------------------------------------ host launchers
 static int pick_nt(int N) { return N <= 32 ? 32 : (N <= 64 ? 64 : 128); }
@@ -222,7 +220,7 @@ cudaError_t launch_update_product(enkf_handle_s* h, const void* Xf, void* Xa) {
   const int NT = h->launch.NT;
   const int TRB = NT == 32 ? Tile<32>::TRB : (NT == 64 ? Tile<64>::TRB : Tile<128>::TRB);
   const int tiles = (int)std::min<int64_t>((c.n + TRB - 1) / TRB, (int64_t)h->sms * 8);
-  void* fn = NT == 32 ? (void*)update_kernel<float, 32, 1> : NT == 64 ? (void*)update_kernel<float, 64, 1> : (void*)update_kernel<float, 128, 1>;
+  void* fn = NT == 32 ? (void*)update_kernel<32> : NT == 64 ? (void*)update_kernel<64> : (void*)update_kernel<128>;
   const int smem = NT == 32 ? update_smem_bytes<float, 32>() : NT == 64 ? update_smem_bytes<float, 64>() : update_smem_bytes<float, 128>();
   cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;

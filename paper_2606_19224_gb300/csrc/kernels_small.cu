@@ -767,11 +767,10 @@ int small_cluster(const enkf_handle_s* h) {
   const bool fp64 = c.precision == ENKF_FP64;
   if (fp64 && !steady_fp64(h)) return 0;
   void* fn = small_fn(fp64, c.precondition != 0);
-  int best = 0;
-  for (int C = 1; C <= 8 && (int64_t)c.N * C <= h->sms; ++C) {
-    const int64_t rp = (c.m + C - 1) / C;
-    if (rp > 65536 || small_smem(fp64, c.N, (int)rp, C) > kSmallSmem) continue;
-    if (best != 0 && rp < 128) break;
+  auto fits = [&](int C) { return (c.m + C - 1) / C <= 65536 && small_smem(fp64, c.N, (int)((c.m + C - 1) / C), C) <= kSmallSmem; };
+  // from the largest down (a query of the driver only for a size that would be taken)
+  for (int C = std::min(8, h->sms / c.N); C >= 1 && fits(C); --C) {
+    if (C > 1 && (c.m + C - 1) / C < 128 && fits(C - 1)) continue;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[1];
     small_launch_config(c, C, nullptr, cfg, at);
@@ -781,9 +780,9 @@ int small_cluster(const enkf_handle_s* h) {
       cudaGetLastError();
       continue;
     }
-    if (resident >= c.N) best = C;
+    if (resident >= c.N) return C;
   }
-  return best;
+  return 0;
 }
 
 cudaError_t launch_small(enkf_handle_s* h) {
