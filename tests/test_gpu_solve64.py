@@ -84,3 +84,22 @@ def test_varying_r(lib):
     exact = oracle.enkf_exact(p.Xf, p.rowptr, p.col, p.w, p.r, p.y, E)
     assert st["status"] == "ok"
     assert oracle.rel_frobenius(Xa, exact) <= 1e-8
+
+
+@pytest.mark.parametrize("N,m,pc,varying", [(64, 1500, 1, True), (40, 900, 0, False), (24, 700, 0, True), (20, 90, 1, True)])
+def test_the_allocation_free_entry_point_takes_the_same_route(lib, N, m, pc, varying):
+    # the same analysis through a handle and on the fixed array; without preconditioning the latter does not
+    # know whether R is constant and keeps the m-vector solve, whose result agrees to the tolerance
+    p = _problem(N, m, 3 * N + m)
+    if not varying:
+        p.r[:] = 0.9
+    _, Xa, st = _run(lib, p, tol=1e-11, precondition=pc)
+    cfg = lib.default_config(p.n, p.m, p.N, precision="fp64", tol=1e-11, precondition=pc)
+    dev = (torch.from_numpy(p.rowptr).cuda(), torch.from_numpy(p.col).cuda(), torch.from_numpy(p.w).cuda(), torch.from_numpy(p.r).cuda())
+    X2, st2 = lib.analyze_noalloc(cfg, *dev, torch.from_numpy(np.ascontiguousarray(p.Xf)).cuda(), torch.from_numpy(p.y).cuda(), seed=6, counter=2)
+    assert st["status"] == "ok" and st2["status"] == "ok"
+    X2 = X2.cpu().numpy()
+    if pc or varying:
+        assert np.array_equal(Xa, X2)
+    else:
+        assert oracle.rel_frobenius(X2, Xa) <= 1e-9
