@@ -75,7 +75,7 @@ __device__ __forceinline__ float gelu_grad_f(float x) {
 // the network's products have 8 to 136 tiles, which alone leave most SMs idle. Loads run along the
 // contiguous index of each operand. (32 x 32 tiles with 2 x 2 outputs per thread and loads along the
 // strided index took 15 to 30 us per product at batch 256, 1088 -> 512^3 -> 64; loss and gradient 345 us, now
-// 164.)
+// 158.)
 constexpr int GT = 64, GBK = 32, GLD = GBK + 4;
 
 enum : int { EPI_HIDDEN = 0, EPI_OUT = 1, EPI_BWD = 2, EPI_STORE = 3 };
@@ -231,9 +231,9 @@ __global__ void __launch_bounds__(256) mlp_gemm_kernel(const GemmArgs g) {
 template <int EPI>
 static cudaError_t gemm(GemmArgs a, cudaStream_t s) {
   const int tn = (a.N + GT - 1) / GT, tm = (a.M + GT - 1) / GT, steps = (a.K + GBK - 1) / GBK;
-  // enough clusters to fill the chip once, and a step along K per CTA at least
+  // up to two CTAs per SM, and a step along K per CTA at least
   a.split = 1;
-  while (a.split < 8 && (int64_t)tn * tm * a.split * 2 <= 160 && steps >= 2 * a.split) a.split *= 2;
+  while (a.split < 8 && (int64_t)tn * tm * a.split * 2 <= 304 && steps >= 2 * a.split) a.split *= 2;
   if (a.split == 1) {
     mlp_gemm_kernel<EPI><<<dim3(tn, tm), 256, 0, s>>>(a);
     return cudaGetLastError();
@@ -255,20 +255,23 @@ static cudaError_t gemm(GemmArgs a, cudaStream_t s) {
 
 // Loss and output gradient: diff = y_std - (t - mu_out)/sd_out over B x out entries (rows of
 // T optionally gathered); G = 2 diff/(B out); loss = sum diff^2/(B out). One cluster of 8 CTAs, fixed
-// order (a single CTA took 30 us for a batch of 256).
-__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(256) mse_kernel(const float* __restrict__ Y, const float* __restrict__ T,
+// order (a single CTA took 30 us for a batch of 256, 8 x 256 threads 15: the entries' loads are latency).
+constexpr int kMT = 1024;
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(kMT) mse_kernel(const float* __restrict__ Y, const float* __restrict__ T,
                                                   const int32_t* __restrict__ rows, int B, int out,
                                                   const float* __restrict__ mu_out,
                                                   const float* __restrict__ sd_out, float* __restrict__ G,
                                                   float* __restrict__ loss) {
-  __shared__ double red[8], part;
+  __shared__ double red[kMT / 32], part;
   cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
   const int t = threadIdx.x;
   const double inv = 1.0 / ((double)B * out);
   const float g2 = (float)(2.0 * inv);
   double s = 0.0;
-  for (int64_t e = (int64_t)blockIdx.x * 256 + t; e < (int64_t)B * out; e += 8 * 256) {
-    const int b = (int)(e / out), o = (int)(e % out);
+  const int64_t total = (int64_t)B * out;
+  const bool small = total < (1ll << 31);   // 32-bit divisions
+  for (int64_t e = (int64_t)blockIdx.x * kMT + t; e < total; e += 8 * kMT) {
+    const int b = small ? (int)e / out : (int)(e / out), o = (int)(e - (int64_t)b * out);
     const int64_t row = rows ? (int64_t)rows[b] : (int64_t)b;
     const float tt = (T[row * out + o] - mu_out[o]) / sd_out[o];
     const float d = Y[e] - tt;
@@ -281,7 +284,7 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(256) mse_kernel(cons
   __syncthreads();
   if (t == 0) {
     double v = 0.0;
-    for (int w = 0; w < 8; ++w) v += red[w];
+    for (int w = 0; w < kMT / 32; ++w) v += red[w];
     part = v;
   }
   cluster.sync();
@@ -405,7 +408,7 @@ static cudaError_t mlp_loss_grad_impl(const MlpLayout& L, const float* P, const 
                                       cudaStream_t s) {
   cudaError_t e = mlp_forward_impl(L, P, X, rows, B, W, nullptr, s);
   if (e != cudaSuccess) return e;
-  mse_kernel<<<8, 256, 0, s>>>(W.Y, T, rows, B, L.out, P + L.mu_out, P + L.sd_out, W.G0, loss);
+  mse_kernel<<<8, kMT, 0, s>>>(W.Y, T, rows, B, L.out, P + L.mu_out, P + L.sd_out, W.G0, loss);
   e = cudaGetLastError();
   float* g = W.G0;    // dL/dz of layer l, [B][fo]
   float* gn = W.G1;
