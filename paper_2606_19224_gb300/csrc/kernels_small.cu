@@ -190,7 +190,9 @@ __global__ void __launch_bounds__(kST64) small_cg_f64_kernel(SmallParams p) {
       if (lane == 0) sc[8 + warp] = a;
     }
   };
-  __syncthreads();
+  // every CTA of the cluster has started (a peer's shared memory may not be stored into before) and HA is staged
+  if (C > 1) cluster.sync();
+  else __syncthreads();
   // ||d_j||^2
   if (warp == 0) {
     double a = 0.0;
@@ -541,6 +543,7 @@ __global__ void __launch_bounds__(kST) small_cg_f32_kernel(SmallParams p) {
     }
     return total64(sync(), NP);
   };
+  if (C > 1) cluster.sync();   // every CTA has started: a peer's shared memory may not be stored into before
   const double dn2 = sum64([&](int i) {
     const double d = p.D[(row0 + i) * N + j];
     return d * d;
