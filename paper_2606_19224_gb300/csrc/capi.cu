@@ -243,7 +243,7 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
     allocs.push_back({(void**)&ws.hs, sizeof(float) * c.m});
     allocs.push_back({(void**)&ws.hamax, sizeof(unsigned) * 4});
     allocs.push_back({&ws.kpart, enkf::krylov_part_bytes(h)});
-    allocs.push_back({&ws.ksmall, 8 * ((size_t)4 * c.N * c.N + 2 * c.N)});
+    allocs.push_back({&ws.ksmall, 8 * ((size_t)4 * c.N * c.N + 3 * c.N)});
   }
   if (!gram && !krylov) {
     if (!h->solve64) allocs.push_back({(void**)&ws.Sv, vs * mN});

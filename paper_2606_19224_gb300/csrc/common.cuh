@@ -159,7 +159,7 @@ struct Workspace {
   void* rsq = nullptr;
   float* hs = nullptr;          // [m] a power of two above each row's largest |HA|
   void* kpart = nullptr;        // [G][2 N JC + 128] double-float partial products
-  void* ksmall = nullptr;       // four N x N matrices, two N-vectors (double-float)
+  void* ksmall = nullptr;       // four N x N matrices, three N-vectors (double-float)
   // tridiagonal R (kernels_whiten.cu): the caller's H, the whitening scan's coefficients and
   // buffers; rowptr / col / w / r above then hold H' = I and r' = 1 of the whitened problem
   int32_t* Hrowptr = nullptr;   // [m+1]

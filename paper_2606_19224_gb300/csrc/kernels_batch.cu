@@ -51,9 +51,9 @@ struct BatchIO {
 };
 
 // Double-float entries a CTA contributes to its team's buffers: two partials (a CTA alone takes both
-// column groups), two rows of column sums, four N x N matrices and two N-vectors.
+// column groups), two rows of column sums, four N x N matrices and three N-vectors.
 __host__ __device__ constexpr int64_t team_stride(int64_t part_max, int n_max) {
-  return 2 * part_max + 256 + 4 * (int64_t)n_max * n_max + 2 * n_max;
+  return 2 * part_max + 256 + 4 * (int64_t)n_max * n_max + 3 * n_max;
 }
 
 // The per-problem phases as separate (not inlined) device functions, so that each gets the
@@ -112,6 +112,7 @@ __global__ void __launch_bounds__(kKT, 1) batch_kernel(
       s_sp.wred = small + 2 * NN;
       s_sp.Tred = small + 3 * NN;
       s_sp.sums = small + 4 * NN;
+      s_sp.hold = reinterpret_cast<int*>(s_sp.sums + 2 * s_sp.N);
       s_io = io[pi];
       s_n = probs[pi].n;
       s_nt = probs[pi].NT;

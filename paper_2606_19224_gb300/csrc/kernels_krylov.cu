@@ -98,13 +98,14 @@ cudaError_t launch_krylov(enkf_handle_s* h, int phase, const float* w0, const do
   p.umax = ws.hamax;
   df32* q = static_cast<df32*>(ws.kpart);
   p.part = q;
-  q = static_cast<df32*>(ws.ksmall);   // four N x N matrices and two N-vectors
+  q = static_cast<df32*>(ws.ksmall);   // four N x N matrices and three N-vectors
   const int NN = c.N * c.N;
   p.Kred = q;
   p.Fred = q + NN;
   p.wred = q + 2 * NN;
   p.Tred = q + 3 * NN;
   p.sums = q + 4 * NN;
+  p.hold = reinterpret_cast<int*>(q + 4 * NN + 2 * c.N);
   p.rrpart = ws.rrpart;
   p.W = ws.W;
   p.tol = c.tol;

@@ -64,6 +64,7 @@ struct KrylovParams {
   df32* wred;           // [N][N] row j holds w_j
   df32* Tred;           // [N][N] T^T
   df32* sums;           // [2][N] ||d_j||^2 and (b_j, R^{-1} b_j)
+  int* hold;            // [N] columns whose recurrences of this cycle gained nothing
   double* rrpart;       // [2][G][NT]
   double* W;            // [N][N]
   double tol;
@@ -675,6 +676,9 @@ __device__ __forceinline__ df32 df_shfl_xor(const df32& v, int o) {
 // N = 64 and 5.3 at N = 128. A step is one product (each thread keeps its block of K in
 // registers, shared by the CTA's columns) and one round of sums: with kr = K rho, (p, S p)
 // is (rho, kr) + (kr, kr) - beta^2 (p, S p)_old.
+// The recurrences start from R^{-1} b, whose residual is larger than b by up to the largest eigenvalue of K, and
+// where they end early (the step limit, or rounding at a large K) it may still be: a column whose
+// (r, R^{-1} r) is not below (b, R^{-1} b) is held for this cycle (w = 0, Z as it was).
 template <int NT>
 struct KMat {
   static constexpr int TPR = kKT / NT, KPT = NT / TPR;   // threads per row, entries per thread
@@ -689,6 +693,7 @@ struct KColumns {
   const int* bad;
   const float* w0;       // learned start or nullptr
   int* iters;            // [N] steps so far (global)
+  int* hold;             // [N] (global)
   bool first;            // first cycle: iters is not read
   int max_iter;
   int* status;
@@ -704,13 +709,12 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
   const bool mine = warp < nc;
   const int j = j0 + warp * step;
   df32 rho[EPL], f[EPL], h[EPL], w[EPL], rr, pq;
-  float stop = 0.f;
+  float stop = 0.f, top = 0.f, last = 0.f;   // (r, R^{-1} r)/(N-1): tolerance, of b, of the last step
   int it = 0, limit = 0, used = 0, act = 0;
   bool start = false;
   if (mine) {
     used = C.first ? 0 : *(volatile int*)&C.iters[j];
     limit = C.done[j] ? 0 : max(0, C.max_iter - used);
-    stop = (float)(C.itol[j] * C.itol[j] * C.bb[j] * (double)inv_nm1.hi);   // of rho^T K rho
     start = C.w0 && !C.bad[j] && !C.done[j];
     act = 1;
 #pragma unroll
@@ -718,7 +722,7 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
       const int k = lane + 32 * e;
       rho[e] = k < N ? ld_df(C.F + (int64_t)j * N + k) * inv_nm1 : df32(0.f, 0.f);
       if (start && k < N) w[e] = df32(C.w0[(int64_t)k * N + j], 0.f);
-      s_rho[warp * NT + k] = start ? w[e] : rho[e];
+      if (C.w0) s_rho[warp * NT + k] = w[e];
     }
   }
   if (t < 16) s_act[t] = t < nc;
@@ -753,12 +757,16 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
   if (C.w0) {   // rho = g - (I + K) w0 (the same for every column; without a start w = 0)
     __syncthreads();
     product();
-    if (mine)
+    if (start)
 #pragma unroll
-      for (int e = 0; e < EPL; ++e) {
-        if (start) rho[e] = rho[e] - (w[e] + row(lane + 32 * e));
-        s_rho[warp * NT + lane + 32 * e] = rho[e];
-      }
+      for (int e = 0; e < EPL; ++e) rho[e] = rho[e] - (w[e] + row(lane + 32 * e));
+  }
+  if (mine) {
+    const double t2 = C.bb[j] * (double)inv_nm1.hi;
+    top = (float)t2;
+    stop = (float)(C.itol[j] * C.itol[j] * t2);
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) s_rho[warp * NT + lane + 32 * e] = rho[e];
   }
   while (__syncthreads_or(act)) {
     product();
@@ -777,6 +785,7 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
       }
       // a non-finite value ends the column (the true residual reports it); so does a (p, S p) that
       // is not positive: rounding has used up this cycle
+      last = d1.hi;
       if (!isfinite(d1.hi)) {
         if (lane == 0) atomicOr(C.status, DS_NONFINITE);
         act = 0;
@@ -806,10 +815,15 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
     }
   }
   if (mine) {
+    const bool gain = last <= top;   // (false for NaN)
 #pragma unroll
     for (int e = 0; e < EPL; ++e)
-      if (lane + 32 * e < N) C.w[(int64_t)j * N + lane + 32 * e] = w[e];
-    if (lane == 0) C.iters[j] = used + it;
+      if (lane + 32 * e < N)
+        C.w[(int64_t)j * N + lane + 32 * e] = gain ? w[e] : df32(0.f, 0.f);
+    if (lane == 0) {
+      C.iters[j] = used + it;
+      C.hold[j] = gain ? 0 : 1;
+    }
   }
   __syncthreads();
 }
@@ -825,7 +839,7 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
 // NT <= 64: the next tile is loaded and sliced behind the products of the current one.
 template <int NT, bool RESID>
 __device__ __noinline__ void pass_rows(const KrylovParams& p, bool from_b, int c, int64_t row0, int64_t row1,
-                                       KCta& cta, const int* s_done, df32* __restrict__ out, double* rr_out) {
+                                       KCta& cta, const int* s_hold, df32* __restrict__ out, double* rr_out) {
   using L = KLayout<NT>;
   using HI = KItems<NT>;
   constexpr int JC = L::JC, NB = L::NB;
@@ -846,8 +860,8 @@ __device__ __noinline__ void pass_rows(const KrylovParams& p, bool from_b, int c
   const int ln = 32 * qd + lane, jl = ln % JC, j = 64 * c + jl;
   const int copy = ln / JC;                       // NT = 128: lanes 64.. hold no column
   const bool mine = copy < CP && sub < NSUB, live = mine && j < N;
-  // a column that is done keeps its Z: its right-hand side is zero in the cycles of the others
-  const bool frozen = !RESID && from_b && live && s_done[j];
+  // a column that is done or held keeps its Z: its right-hand side and w are zero
+  const bool frozen = !RESID && live && s_hold[j];
   const int rg = mine ? copy * NSUB + sub : 0, r0 = rg * RPT;   // this thread's rows of the tile
   const uint32_t lead = warp == 0 ? elect_lane() : 0u;
   const uint32_t aT = smem_addr(cta.smem + L::off_t), aH = smem_addr(cta.smem + L::off_h), aV = smem_addr(sV);
@@ -919,10 +933,10 @@ __device__ __noinline__ void pass_rows(const KrylovParams& p, bool from_b, int c
         const bool in = live && i < row1;
         const int64_t e = in ? i * N + j : 0;
         df32 dv(0.f, 0.f), zv(0.f, 0.f);
-        if (!RESID && from_b) dv.hi = frozen ? 0.f : p.B[e];
+        if (!RESID && from_b) dv.hi = p.B[e];
         else dv = p.Ddf[e];
         if (RESID || from_b) zv = p.Zdf[e];
-        d[q] = in ? dv : df32(0.f, 0.f);
+        d[q] = in && !frozen ? dv : df32(0.f, 0.f);
         z[(RESID ? 0 : q0) + q] = in ? zv : df32(0.f, 0.f);
       }
     };
@@ -1060,7 +1074,7 @@ __device__ void krylov_body(const KrylovParams& p, const int G, const int b, Gri
   double* s_tmp = s_itol + NT;
   double* s_bb = s_tmp + NT;
   int* s_done = reinterpret_cast<int*>(s_bb + NT);
-  int* s_bad = s_done + NT;
+  int* s_bad = s_done + NT;     // rejected learned starts, then the columns held in this cycle
   double* scratch = reinterpret_cast<double*>(cta.smem + L::off_scr);
   const int N = p.N, t = threadIdx.x, NJ = min(JC, N);
   if (dynamic_smem_bytes() < (unsigned)L::bytes) {
@@ -1172,19 +1186,21 @@ __device__ void krylov_body(const KrylovParams& p, const int G, const int b, Gri
         }
       }
       const KColumns C{p.Fred, p.wred, s_bb, s_itol, s_done, s_bad, from_b ? nullptr : p.w0,
-                       p.col_iters, !from_b, p.max_iter, p.status};
+                       p.col_iters, p.hold, !from_b, p.max_iter, p.status};
       for (int j = b; j < N; j += 16 * G)
         krylov_cg<NT>(M, N, df32(inv_nm1), j, G, min(16, (N - j + G - 1) / G), C, cta.smem);
     }
     tick(PH_PASS);
     if (!(ok = bar.sync())) break;
     tick(PH_BAR1);
+    if (t < NT) s_bad[t] = t < N && (__ldcg(p.hold + t) || (from_b && s_done[t])) ? 1 : 0;
+    __syncthreads();
     // ---- pass Z and the reduction of T (W = T/(N-1))
     for (int c = c0; c < c1; ++c)
       if (has_rows) {
         stage_columns<NT, L::TROWS, JC>(p.wred, 64 * c, N, cta.smem + L::off_t, reinterpret_cast<float*>(cta.smem + L::off_col));
         __syncthreads();
-        pass_rows<NT, false>(p, from_b, c, row0, row1, cta, s_done, part_of(rb, c), nullptr);
+        pass_rows<NT, false>(p, from_b, c, row0, row1, cta, s_bad, part_of(rb, c), nullptr);
       }
     tick(PH_REFRESH);
     if (!(ok = bar.sync() && cta.ok)) break;
@@ -1207,7 +1223,7 @@ __device__ void krylov_body(const KrylovParams& p, const int G, const int b, Gri
       if (has_rows) {
         stage_columns<NT, L::TROWS, JC>(p.Tred, 64 * c, N, cta.smem + L::off_t, reinterpret_cast<float*>(cta.smem + L::off_col));
         __syncthreads();
-        pass_rows<NT, true>(p, from_b, c, row0, row1, cta, s_done, nullptr, s_tmp);
+        pass_rows<NT, true>(p, from_b, c, row0, row1, cta, s_bad, nullptr, s_tmp);
       }
     if (!(ok = column_totals() && cta.ok)) break;
     ++cycles;
@@ -1219,8 +1235,8 @@ __device__ void krylov_body(const KrylovParams& p, const int G, const int b, Gri
       const double tr = !fin ? (double)NAN : (s_dn2[t] > 0.0 ? sqrt(s_tmp[t] / s_dn2[t]) : 0.0);
       s_true[t] = tr;
       const int used = *(volatile int*)&p.col_iters[t];
-      // done: converged, non-finite, stalled (no halving over a cycle) or out of steps
-      if (!fin || tr <= p.tol || (cycles >= 2 && tr > 0.5 * s_prev[t]) || used >= p.max_iter) s_done[t] = 1;
+      // done: converged, non-finite, held, stalled (no halving over a cycle) or out of steps
+      if (!fin || tr <= p.tol || s_bad[t] || (cycles >= 2 && tr > 0.5 * s_prev[t]) || used >= p.max_iter) s_done[t] = 1;
       s_prev[t] = tr;
       s_itol[t] = fmin(0.5, fmax(tr > 0.0 ? 0.02 * p.tol / tr : 0.5, 1e-14));
     }
