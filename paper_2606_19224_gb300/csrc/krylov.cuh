@@ -676,15 +676,19 @@ __device__ __forceinline__ df32 df_shfl_xor(const df32& v, int o) {
 // N = 64 and 5.3 at N = 128. A step is one product (each thread keeps its block of K in
 // registers, shared by the CTA's columns) and one round of sums: with kr = K rho, (p, S p)
 // is (rho, kr) + (kr, kr) - beta^2 (p, S p)_old.
-// The recurrences start from R^{-1} b, whose residual is larger than b by up to the largest eigenvalue of K, and
-// where they end early (the step limit, or rounding at a large K) it may still be: a column whose
-// (r, R^{-1} r) is not below (b, R^{-1} b) is held for this cycle (w = 0, Z as it was).
+// These sums go from |K g|^2 down to the tolerance, more than FP32's exponents hold once the variances of
+// R lie some 10^8 below those of HA; the vectors of a column are therefore carried times a power of two
+// that puts |K rho|^2 of the start just below the top of the range. The recurrences start from
+// R^{-1} b, whose residual is larger than b by up to the largest eigenvalue of K, and where they end early (the
+// step limit, or rounding at such an R) it may still be: a column whose (r, R^{-1} r) is not below
+// (b, R^{-1} b) is held for this cycle (w = 0, Z as it was).
 template <int NT>
 struct KMat {
   static constexpr int TPR = kKT / NT, KPT = NT / TPR;   // threads per row, entries per thread
   df32 k[KPT];
 };
 struct KColumns {
+  const df32* K;         // [N][N]
   const df32* F;         // [N][N]
   df32* w;               // [N][N]
   const double* bb;      // shared: (b_j, R^{-1} b_j), tolerance, done and rejected starts per column
@@ -710,6 +714,7 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
   const int j = j0 + warp * step;
   df32 rho[EPL], f[EPL], h[EPL], w[EPL], rr, pq;
   float stop = 0.f, top = 0.f, last = 0.f;   // (r, R^{-1} r)/(N-1): tolerance, of b, of the last step
+  float kmax = 0.f, unscale = 1.f;
   int it = 0, limit = 0, used = 0, act = 0;
   bool start = false;
   if (mine) {
@@ -721,6 +726,7 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
     for (int e = 0; e < EPL; ++e) {
       const int k = lane + 32 * e;
       rho[e] = k < N ? ld_df(C.F + (int64_t)j * N + k) * inv_nm1 : df32(0.f, 0.f);
+      if (k < N) kmax = fmaxf(kmax, fabsf(ld_df(C.K + k * N + k).hi));   // (K is positive semidefinite)
       if (start && k < N) w[e] = df32(C.w0[(int64_t)k * N + j], 0.f);
       if (C.w0) s_rho[warp * NT + k] = w[e];
     }
@@ -762,11 +768,24 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
       for (int e = 0; e < EPL; ++e) rho[e] = rho[e] - (w[e] + row(lane + 32 * e));
   }
   if (mine) {
-    const double t2 = C.bb[j] * (double)inv_nm1.hi;
+    // rho and w times 2^-ex: N^2 max|K| max|rho| to about 2^60
+    float rmax = 0.f;
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) rmax = fmaxf(rmax, fmaxf(fabsf(rho[e].hi), fabsf(w[e].hi)));
+    const unsigned kb = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(kmax, 1.f)));
+    const unsigned rb = __reduce_max_sync(0xffffffffu, __float_as_uint(rmax));
+    const int ex = max(-100, min(100, (int)(kb >> 23) - 127 + (int)(rb >> 23) - 127 + 2 * (31 - __clz(N)) + 2 - 60));
+    const float sc = __uint_as_float((uint32_t)(127 - ex) << 23);
+    unscale = __uint_as_float((uint32_t)(127 + ex) << 23);
+    const double t2 = C.bb[j] * (double)inv_nm1.hi * __hiloint2double((1023 - 2 * ex) << 20, 0);
     top = (float)t2;
     stop = (float)(C.itol[j] * C.itol[j] * t2);
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) s_rho[warp * NT + lane + 32 * e] = rho[e];
+    for (int e = 0; e < EPL; ++e) {
+      rho[e] = df32(rho[e].hi * sc, rho[e].lo * sc);
+      w[e] = df32(w[e].hi * sc, w[e].lo * sc);
+      s_rho[warp * NT + lane + 32 * e] = rho[e];
+    }
   }
   while (__syncthreads_or(act)) {
     product();
@@ -819,7 +838,7 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
 #pragma unroll
     for (int e = 0; e < EPL; ++e)
       if (lane + 32 * e < N)
-        C.w[(int64_t)j * N + lane + 32 * e] = gain ? w[e] : df32(0.f, 0.f);
+        C.w[(int64_t)j * N + lane + 32 * e] = gain ? df32(w[e].hi * unscale, w[e].lo * unscale) : df32(0.f, 0.f);
     if (lane == 0) {
       C.iters[j] = used + it;
       C.hold[j] = gain ? 0 : 1;
@@ -1185,7 +1204,7 @@ __device__ void krylov_body(const KrylovParams& p, const int G, const int b, Gri
           M.k[q] = ld_df(p.Kred + k * N + r);
         }
       }
-      const KColumns C{p.Fred, p.wred, s_bb, s_itol, s_done, s_bad, from_b ? nullptr : p.w0,
+      const KColumns C{p.Kred, p.Fred, p.wred, s_bb, s_itol, s_done, s_bad, from_b ? nullptr : p.w0,
                        p.col_iters, p.hold, !from_b, p.max_iter, p.status};
       for (int j = b; j < N; j += 16 * G)
         krylov_cg<NT>(M, N, df32(inv_nm1), j, G, min(16, (N - j + G - 1) / G), C, cta.smem);

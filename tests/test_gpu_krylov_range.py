@@ -1,8 +1,14 @@
-"""The preconditioned solve in Krylov coordinates (csrc/krylov.cuh) where its N x N recurrences end early: a
-step limit, and inputs that are not numbers."""
+"""The preconditioned solve in Krylov coordinates (csrc/krylov.cuh) where its N x N recurrences are hard:
+variances of R far below the ensemble's, a step limit, and inputs
+that are not numbers.
+
+Bar of the analyses: Z, HA and the sums hold about 47 bits and the residual of a rounded Z is up to
+lambda = the largest eigenvalue of HA^T R^-1 HA/(N-1) times its rounding, so the increment X_a - X_f is off by
+at most 1e-6 (the FP32 path's bar) + 2^-46 lambda of its size, converged or not."""
 import numpy as np
 import pytest
 
+import oracle
 import synth
 
 pytestmark = pytest.mark.gpu
@@ -20,6 +26,26 @@ def _run(lib, p, prec="fp32", **cfg):
     st = an.stats()
     an.close()
     return Xa, st
+
+
+def _check(lib, p, prec):
+    X = p.Xf.astype(np.float64)
+    HA = oracle.ensemble_stats(X, p.rowptr, p.col, p.w)[4]
+    lam = np.linalg.eigvalsh(HA.T @ (HA / p.r[:, None]) / (p.N - 1)).max()
+    ref = oracle.enkf_exact(X, p.rowptr, p.col, p.w, p.r, p.y, oracle.obs_perturbations(6, 2, p.r, p.N), m_dense=0)
+    Xa, st = _run(lib, p, prec)
+    assert st["status"] in ("ok", "not_converged"), st
+    err = np.linalg.norm(Xa - ref) / np.linalg.norm(ref - X)
+    assert err <= 1e-6 + 2.0 ** -46 * lam, (err, lam, st)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp16"])
+@pytest.mark.parametrize("N,m", [(20, 4000), (64, 1024), (100, 2000)])
+@pytest.mark.parametrize("decades", [4, 8])
+def test_observations_far_more_accurate_than_the_ensemble(lib, N, m, decades, prec):
+    p = _problem(N, m, 3)
+    p.r = p.r * 10.0 ** -decades
+    _check(lib, p, prec)
 
 
 @pytest.mark.parametrize("N,m", [(20, 300), (64, 2000), (100, 2000)])
