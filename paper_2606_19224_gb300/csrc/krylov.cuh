@@ -674,8 +674,11 @@ __device__ __forceinline__ df32 df_shfl_xor(const df32& v, int o) {
 // FP64 unit for about 64 cycles, and the first form of this loop, with the vectors and scalars of
 // a step in FP64 (some 60 such instructions in one warp's serial chain), took 2.9 us per step at
 // N = 64 and 5.3 at N = 128. A step is one product (each thread keeps its block of K in
-// registers, shared by the CTA's columns) and one round of sums: with kr = K rho, (p, S p)
-// is (rho, kr) + (kr, kr) - beta^2 (p, S p)_old.
+// registers, shared by the CTA's columns) and one round of sums: with kr = K rho and h = K f of the step
+// before, (p, S p) is (rho + kr, kr) + 2 beta (rho + kr, h) + beta^2 (p, S p)_old. (The middle sum is
+// -beta (p, S p)_old while directions are conjugate. Without it a member 10^4 times the others, one eigenvalue
+// of K far above the rest, took 796 steps of the first cycle to a residual of 9.1 ||d||; it takes 146 to 0.083
+// and the second cycle ends at 1.8e-6. At m = 65,536, N = 64 a solve takes 29 steps either way.)
 // These sums go from |K g|^2 down to the tolerance, more than FP32's exponents hold once the variances of
 // R lie some 10^8 below those of HA; the vectors of a column are therefore carried times a power of two
 // that puts |K rho|^2 of the start just below the top of the range. The recurrences start from
@@ -790,17 +793,19 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
   while (__syncthreads_or(act)) {
     product();
     if (act) {
-      df32 kr[EPL], d1, d2;
+      df32 kr[EPL], d1, d2, d3;   // (rho, kr), (kr, kr), (rho + kr, h)
 #pragma unroll
       for (int e = 0; e < EPL; ++e) {
         kr[e] = row(lane + 32 * e);
         d1 = fma(rho[e], kr[e], d1);
         d2 = fma(kr[e], kr[e], d2);
+        d3 = fma(rho[e] + kr[e], h[e], d3);   // (h = 0 before the first step)
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         d1 = d1 + df_shfl_xor(d1, o);
         d2 = d2 + df_shfl_xor(d2, o);
+        d3 = d3 + df_shfl_xor(d3, o);
       }
       // a non-finite value ends the column (the true residual reports it); so does a (p, S p) that
       // is not positive: rounding has used up this cycle
@@ -813,7 +818,7 @@ __device__ __forceinline__ void krylov_cg(const KMat<NT>& M, int N, const df32 i
       } else {
         df32 beta;
         if (it > 0) beta = df_div(d1, rr);
-        pq = (d1 + d2) - (it > 0 ? beta * beta * pq : df32(0.f, 0.f));
+        pq = fma(beta, fma(beta, pq, d3 + d3), d1 + d2);
         rr = d1;
         if (!(pq.hi > 0.f) || !isfinite(pq.hi)) {
           act = 0;

@@ -1,5 +1,5 @@
 """The preconditioned solve in Krylov coordinates (csrc/krylov.cuh) where its N x N recurrences are hard:
-variances of R far below the ensemble's, a step limit, and inputs
+variances of R far below the ensemble's, a member far larger than the others, a step limit, and inputs
 that are not numbers.
 
 Bar of the analyses: Z, HA and the sums hold about 47 bits and the residual of a rounded Z is up to
@@ -46,6 +46,13 @@ def test_observations_far_more_accurate_than_the_ensemble(lib, N, m, decades, pr
     p = _problem(N, m, 3)
     p.r = p.r * 10.0 ** -decades
     _check(lib, p, prec)
+
+
+@pytest.mark.parametrize("factor", [1e2, 1e4])
+def test_a_member_far_larger_than_the_others(lib, factor):
+    p = _problem(64, 1024, 6)
+    p.Xf[:, 5] *= np.float32(factor)
+    _check(lib, p, "fp32")
 
 
 @pytest.mark.parametrize("N,m", [(20, 300), (64, 2000), (100, 2000)])
