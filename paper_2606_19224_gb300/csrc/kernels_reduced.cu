@@ -431,7 +431,12 @@ __global__ void __launch_bounds__(kThreads) reduced_cg_kernel(
         bn2 = r2;
         stop2 = tol_s * tol_s * bn2;
       }
+      // a NaN or an infinity in G or in m_j ends the column at once (and fails every comparison below)
       bool go = it < limit && (it == 0 || fixed ? r2 > 0.0 : r2 > stop2);
+      if (!isfinite(r2)) {
+        if (lane == 0) atomicOr(status, DS_NONFINITE);
+        go = false;
+      }
       const double be = go && it > 0 ? r2 * sc[3] : 0.0;
       double al = 0.0;
       if (go) {
@@ -474,9 +479,10 @@ __global__ void __launch_bounds__(kThreads) reduced_cg_kernel(
   if (t == 0) {
     const double tr2 = folded(0);
     col_iters[j] = it;
-    const double rel = bn2 > 0.0 ? sqrt(rr / bn2) : 0.0;
+    const bool fin = isfinite(bn2) && isfinite(rr);
+    const double rel = !fin ? (double)NAN : bn2 > 0.0 ? sqrt(rr / bn2) : 0.0;
     col_relres[j] = rel;
-    col_true[j] = bn2 > 0.0 ? sqrt(tr2 / bn2) : 0.0;
+    col_true[j] = !fin ? (double)NAN : bn2 > 0.0 ? sqrt(tr2 / bn2) : 0.0;
     if (!fixed && !(rel <= tol)) atomicOr(status, DS_NOT_CONVERGED);
   }
 }
