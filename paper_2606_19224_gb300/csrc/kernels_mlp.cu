@@ -811,13 +811,12 @@ cudaError_t warm_set_model(enkf_handle_s* h, const enkf_mlp_shape* shape, const 
   w.work = nullptr;
   e = cudaMalloc((void**)&w.work, sizeof(float) * mlp_work_floats(L, N));
   if (e != cudaSuccess) { err = "allocation"; return e; }
-  const int smem = (int)(sizeof(float) * (size_t)(2 * N + 16) * (N + 1));   // up to 140 KB at N = 128
+  // limits for the largest N: they belong to the kernels, and a handle of fewer members must not lower them
+  constexpr int smem = (int)(sizeof(float) * (2 * 128 + 16) * (128 + 1)), rsm = (int)(sizeof(float) * (128 + 16) * (128 + 1));
   e = cudaFuncSetAttribute(warm_decode_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(warm_decode_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(warm_decode_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  const int rsm = (int)(sizeof(float) * (size_t)(N + 16) * (N + 1));   // up to 74 KB
-  if (e == cudaSuccess && rsm > 48 * 1024)
-    e = cudaFuncSetAttribute(warm_resid_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, rsm);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(warm_resid_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, rsm);
   if (e != cudaSuccess) { err = "decoder shared memory"; return e; }
   w.L = L;
   w.params = params;

@@ -572,8 +572,10 @@ cudaError_t launch_nxn_stage(enkf_handle_s* h) {
   if (f64) reduced_sum_kernel<<<(NN2 + 31) / 32, kThreads, 0, h->stream>>>(ws.Tpart, grid, c.N, Gm, Mm);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const size_t smem = sizeof(double) * ((size_t)c.N * (c.N + 1) + c.N + kThreads);
-  e = cudaFuncSetAttribute(reduced_cg_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (the limit belongs to the kernel: set for the largest N, also between another thread's limit and launch)
+  auto bytes = [](size_t N) { return sizeof(double) * (N * (N + 1) + N + kThreads); };
+  const size_t smem = bytes(c.N);
+  e = cudaFuncSetAttribute(reduced_cg_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(128));
   if (e != cudaSuccess) return e;
   reduced_cg_kernel<<<c.N, kThreads, smem, h->stream>>>(Gm, Mm, c.N, c.tol, c.max_iter, c.fixed_iters,
                                                        ws.W, ws.col_iters, ws.col_relres, ws.col_true,
