@@ -296,34 +296,47 @@ static enkf_status create_impl(const enkf_config* cfg, const int32_t* h_rowptr, 
       return cuda_fail(nullptr, e, "enkf_create: cudaMalloc");
     }
   }
+  // on the handle's stream, whose kernels read them: a copy from pageable memory on the legacy stream may still be
+  // in flight when it returns, and nothing orders a non-blocking stream behind it (the sources live until
+  // the synchronisation below)
+  e = cudaSuccess;
+  auto put = [&](void* dst, const void* src, size_t bytes) {
+    if (e == cudaSuccess && bytes > 0) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, h->stream);
+  };
+  auto zero = [&](void* dst, size_t bytes) {
+    if (e == cudaSuccess) e = cudaMemsetAsync(dst, 0, bytes, h->stream);
+  };
+  std::vector<int32_t> idx;
+  std::vector<double> ones;
   if (!tri) {
-    e = cudaMemcpy(ws.rowptr, h_rowptr, sizeof(int32_t) * (c.m + 1), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && nnz > 0) e = cudaMemcpy(ws.col, h_col, sizeof(int32_t) * nnz, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && nnz > 0) e = cudaMemcpy(ws.w, h_w, sizeof(double) * nnz, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(ws.r, r_diag, sizeof(double) * c.m, cudaMemcpyHostToDevice);
+    put(ws.rowptr, h_rowptr, sizeof(int32_t) * (c.m + 1));
+    put(ws.col, h_col, sizeof(int32_t) * nnz);
+    put(ws.w, h_w, sizeof(double) * nnz);
+    put(ws.r, r_diag, sizeof(double) * c.m);
   } else {
     // the whitened problem: H' = I, r' = 1; the caller's H for the whitening pass
-    std::vector<int32_t> idx(c.m + 1);
+    idx.resize(c.m + 1);
     for (int64_t i = 0; i <= c.m; ++i) idx[i] = (int32_t)i;
-    const std::vector<double> ones(c.m, 1.0);
-    e = cudaMemcpy(ws.rowptr, idx.data(), sizeof(int32_t) * (c.m + 1), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(ws.col, idx.data(), sizeof(int32_t) * c.m, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(ws.w, ones.data(), sizeof(double) * c.m, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(ws.r, ones.data(), sizeof(double) * c.m, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(ws.Hrowptr, h_rowptr, sizeof(int32_t) * (c.m + 1), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && hnnz > 0) e = cudaMemcpy(ws.Hcol, h_col, sizeof(int32_t) * hnnz, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && hnnz > 0) e = cudaMemcpy(ws.Hw, h_w, sizeof(double) * hnnz, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(ws.wa, wa.data(), sizeof(double) * c.m, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(ws.wb, wb.data(), sizeof(double) * c.m, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(ws.wcp, wcp.data(), sizeof(double) * c.m, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(ws.wmu, wmu.data(), sizeof(double) * nblk, cudaMemcpyHostToDevice);
+    ones.assign(c.m, 1.0);
+    put(ws.rowptr, idx.data(), sizeof(int32_t) * (c.m + 1));
+    put(ws.col, idx.data(), sizeof(int32_t) * c.m);
+    put(ws.w, ones.data(), sizeof(double) * c.m);
+    put(ws.r, ones.data(), sizeof(double) * c.m);
+    put(ws.Hrowptr, h_rowptr, sizeof(int32_t) * (c.m + 1));
+    put(ws.Hcol, h_col, sizeof(int32_t) * hnnz);
+    put(ws.Hw, h_w, sizeof(double) * hnnz);
+    put(ws.wa, wa.data(), sizeof(double) * c.m);
+    put(ws.wb, wb.data(), sizeof(double) * c.m);
+    put(ws.wcp, wcp.data(), sizeof(double) * c.m);
+    put(ws.wmu, wmu.data(), sizeof(double) * nblk);
   }
-  if (e == cudaSuccess) e = cudaMemset(ws.status, 0, sizeof(int32_t) * 4);
-  if (e == cudaSuccess && ws.HA16) e = cudaMemset(ws.HA16, 0, enkf::mixed_image_bytes(h));
-  if (e == cudaSuccess) e = cudaMemset(ws.bar, 0, sizeof(unsigned) * 4);
+  zero(ws.status, sizeof(int32_t) * 4);
+  if (ws.HA16) zero(ws.HA16, enkf::mixed_image_bytes(h));
+  zero(ws.bar, sizeof(unsigned) * 4);
   if (e == cudaSuccess) e = enkf::launch_convert_r(h);
   if (e == cudaSuccess && (krylov || gram_tc)) e = enkf::launch_krylov_rows(h);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  const cudaError_t es = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess) e = es;
   if (e != cudaSuccess) {
     free_workspace(ws);
     delete h;

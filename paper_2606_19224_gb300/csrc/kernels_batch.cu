@@ -409,12 +409,12 @@ static cudaError_t apply_plan(BatchState& B, const BatchPlan& P, cudaStream_t s)
   for (const auto* v : {&P.cta_team, &P.cta_rank, &P.team_size, &P.team_first, &P.order})
     flat.insert(flat.end(), v->begin(), v->end());
   drop_graph(B);
-  cudaError_t e = cudaStreamSynchronize(s);   // no replay of the old plan is still reading
+  // in stream order: behind the replays that read the old plan, ahead of those that read this one
+  cudaError_t e = cudaMemcpyAsync(B.d_plan, flat.data(), flat.size() * sizeof(int), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
-    e = cudaMemcpy(B.d_plan, flat.data(), flat.size() * sizeof(int), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess)
-    e = cudaMemcpy(B.d_probs, B.probs.data(), B.probs.size() * sizeof(BatchProblem), cudaMemcpyHostToDevice);
-  return e;
+    e = cudaMemcpyAsync(B.d_probs, B.probs.data(), B.probs.size() * sizeof(BatchProblem), cudaMemcpyHostToDevice, s);
+  const cudaError_t es = cudaStreamSynchronize(s);   // (flat, and the callers' arrays of the uploads before)
+  return e == cudaSuccess ? es : e;
 }
 
 static cudaError_t enqueue_batch(BatchState& B, cudaStream_t s) {
@@ -539,7 +539,7 @@ cudaError_t batch_build(enkf_handle_s* h, int count, const enkf_config* cfgs,
   if (e == cudaSuccess) e = cudaMalloc((void**)&B.d_status, sizeof(int) * 4 * count);
   if (e == cudaSuccess) e = cudaMalloc((void**)&B.d_bar, sizeof(unsigned) * (4 * (size_t)count + 4));
   if (e == cudaSuccess) e = cudaMalloc((void**)&B.d_time, sizeof(unsigned long long) * 2 * count);
-  if (e == cudaSuccess) e = cudaMemset(B.d_time, 0, sizeof(unsigned long long) * 2 * count);
+  if (e == cudaSuccess) e = cudaMemsetAsync(B.d_time, 0, sizeof(unsigned long long) * 2 * count, h->stream);
   if (e == cudaSuccess)
     e = cudaMalloc((void**)&B.d_team, sizeof(df32) * (size_t)team_stride(krylov_part(nmax), nmax) * B.max_grid);
   if (e != cudaSuccess) { err = "enkf_batch_create: device allocation"; return e; }
@@ -579,16 +579,25 @@ cudaError_t batch_build(enkf_handle_s* h, int count, const enkf_config* cfgs,
     bp.col = static_cast<const int32_t*>(ptr[9]);
     bp.w = static_cast<const double*>(ptr[10]);
     const int64_t nnz = rowptr[i][c.m];
-    e = cudaMemcpy(ptr[8], rowptr[i], 4 * ((size_t)c.m + 1), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && nnz > 0) e = cudaMemcpy(ptr[9], col[i], 4 * (size_t)nnz, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && nnz > 0) e = cudaMemcpy(ptr[10], w[i], 8 * (size_t)nnz, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(ptr[4], r[i], 8 * (size_t)c.m, cudaMemcpyHostToDevice);
+    // on the handle's stream, whose kernels read them: a copy from pageable memory on the legacy stream may
+    // still be in flight when it returns, and nothing orders a non-blocking stream behind it
+    auto put = [&](void* dst, const void* src, size_t bytes) {
+      if (e == cudaSuccess && bytes > 0) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, h->stream);
+    };
+    put(ptr[8], rowptr[i], 4 * ((size_t)c.m + 1));
+    put(ptr[9], col[i], 4 * (size_t)nnz);
+    put(ptr[10], w[i], 8 * (size_t)nnz);
+    put(ptr[4], r[i], 8 * (size_t)c.m);
     if (e == cudaSuccess)
       e = launch_krylov_rows(bp.r, c.m, static_cast<df32*>(ptr[5]), static_cast<df32*>(ptr[6]),
                              static_cast<df32*>(ptr[7]), h->stream);
     B.probs.push_back(bp);
   }
-  if (e != cudaSuccess) { err = "enkf_batch_create: upload of the observation operators"; return e; }
+  if (e != cudaSuccess) {
+    cudaStreamSynchronize(h->stream);   // the copies that were begun read the caller's arrays
+    err = "enkf_batch_create: upload of the observation operators";
+    return e;
+  }
   // a tuning result for this batch: "key alpha [rows f_0 .. f_3] [cost_0 .. cost_{count-1}]"
   // (row-block floors per N class, measured one-CTA costs); the last one wins
   double alpha = 1.0;
@@ -836,7 +845,7 @@ cudaError_t batch_set_phase_timing(enkf_handle_s* h, bool on) {
   if (on && !B.d_phase) {
     const size_t bytes = sizeof(unsigned long long) * PH_COUNT * (size_t)B.count;
     e = cudaMalloc((void**)&B.d_phase, bytes);
-    if (e == cudaSuccess) e = cudaMemset(B.d_phase, 0, bytes);
+    if (e == cudaSuccess) e = cudaMemsetAsync(B.d_phase, 0, bytes, h->stream);
     if (e != cudaSuccess) return e;
   }
   for (int i = 0; i < B.count; ++i) B.probs[i].sp.prof = on ? B.d_phase + (size_t)PH_COUNT * i : nullptr;
