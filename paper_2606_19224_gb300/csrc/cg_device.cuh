@@ -191,6 +191,11 @@ __device__ __forceinline__ void ld4(CT (&d)[4], const CT* p, int j0, int N, bool
 #pragma unroll
   for (int y = 0; y < 4; ++y) d[y] = (j0 + y < N) ? p[j0 + y] : CT(0);
 }
+// Whether the rows of N entries behind two pointers of a caller take 16-byte accesses
+template <typename CT>
+__device__ __forceinline__ bool rows_vec(const CT* a, const CT* b, int N) {
+  return (N & 3) == 0 && ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0;
+}
 template <typename CT>
 __device__ __forceinline__ void st4(CT* p, int j0, int N, bool vec, const CT (&s)[4]) {
   if (vec) { store_vec4<CT>(p + j0, s); return; }

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kUT, NT <= 64 ? 2 : 1) update_tc_kernel(
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base;
-  const bool vec = (N & 3) == 0;
+  const bool vec = rows_vec(Xf, Xa, N);
   const int64_t ntiles = (n + kTR - 1) / kTR;
   uint32_t ph = 0;
   bool ok = true;

@@ -506,13 +506,13 @@ __device__ __forceinline__ void update_rows(const VT* Xf, VT* Xa, const double* 
   VT* sXb[2] = {sW + NT * LD, sW + NT * LD + TRB * LD};   // X_f row tiles, double-buffered
   VT* smean = sW + NT * LD + 2 * TRB * LD;
   const int t = threadIdx.x, tj = t % NJ, ti = t / NJ, j0 = tj * 4, r0 = ti * 4;
-  const bool vec = (N & 3) == 0;
+  const bool vec = rows_vec(Xf, Xa, N);
   for (int e = t; e < NT * LD; e += TH) {
     const int k = e / LD, j = e % LD;
     sW[e] = (k < N && j < N) ? (VT)__ldcg(W + k * N + j) : VT(0);   // W may be written by this launch
   }
   // the tile of rows [i0, i0 + TRB) into dst: 16-byte cp.async pieces (zero-filled past n and
-  // N) when rows are 16-byte aligned (N % 4 == 0), else plain loads
+  // N) when X_f's and X_a's rows are 16-byte aligned, else plain loads
   auto load_tile = [&](int64_t i0, VT* dst) {
 #pragma unroll
     for (int c = t; c < TRB * C4; c += TH) {
