@@ -129,9 +129,13 @@ typedef struct enkf_config {
                              the recurrences in the coordinates of their Krylov space:
                              z = R^-1 (d - HA w) with an N-vector w per column, started at
                              w = 0 (z = R^-1 d). The products with HA that remain run on the
-                             tensor cores with operands of five FP16 slices (48 bits, exact
-                             FP32 sums), the N x N recurrences in FP32 pairs, and the
-                             result is certified by the true residual as in every mode    */
+                             tensor cores with operands of five FP16 slices (48 bits below
+                             the largest entry of a row or column, exact FP32 sums), the
+                             N x N recurrences in FP32 pairs, and the result is certified by
+                             the true residual as in every mode. A column whose recurrences
+                             end (max_iter, rounding) before (r, R^-1 r) is below that of
+                             their right-hand side keeps the z it had (0 at first).
+                             enkf_analyze_noalloc keeps the recurrences on m-vectors      */
   int32_t lowprec_terms;  /* BF16/FP16 modes: 3 (or 0, the default) splits every operand
                              into hi + lo parts and forms hi*hi + hi*lo + lo*hi (about 16
                              significant bits); 1 uses single BF16/FP16 operands, whose
@@ -142,7 +146,9 @@ typedef struct enkf_config {
                              1 every finite start is kept. Either way a non-finite start
                              starts from zero and the result is certified by the same
                              double-float true residual <= tol                          */
-  int32_t reduce_order;   /* 0 (default): every step's column sums and Gram are summed over
+  int32_t reduce_order;   /* Solves on m-vectors (solves in Krylov coordinates, see
+                             precondition, sum in a fixed order whatever is given here).
+                             0 (default): every step's column sums and Gram are summed over
                              the CTAs in a fixed order (bitwise repeatable results, two
                              grid barriers per step); 1: ENKF_CGD in the FP32, BF16 and
                              FP16 modes with N <= 64 adds them into the total by

@@ -8,8 +8,12 @@
 // working memory in one file-scope device array of fixed size (kScratchBytes, below),
 // which every GPU that loads the library holds until the process exits.
 //
-// The analysis is the same as enkf_create + enkf_analyze + enkf_get_stats (same kernels,
-// same launch plan), with the observation operator and R passed as device pointers.
+// The analysis is that of enkf_create + enkf_analyze + enkf_get_stats, with the observation
+// operator and R passed as device pointers, and with the same kernels but for two solves, whose
+// results agree to tol only: FP32 with precondition = 1 keeps the recurrences on m-vectors (or one
+// cluster per column), where a handle carries them in Krylov coordinates with tables formed from R at
+// creation; and FP64 with precondition = 0 keeps the persistent m-vector solve, since R lies on the
+// device and whether it is constant is not known here (a handle takes the routes of steady_fp64).
 #include <cstring>
 #include <mutex>
 
