@@ -11,17 +11,17 @@ N = 64 members, m = 65,536 randomly placed observations, r ~ U[0.5, 1.5], CG tol
 
 Prints one JSON line (rank 0). `value` is analyses/s summed over ranks (each rank runs its
 own independent analyses: weak scaling, no collective on the data path). The timed headline
-is CG preconditioned by R with both HA contractions of every step on the tensor cores
-(tcgen05, FP16 hi/lo operands, FP32 accumulation), FP32 vectors, FP64 scalars, each step's
-sums over the CTAs formed by atomic adds (`--reduce-order 0`: in a fixed order, bitwise
-repeatable) and a double-float residual refresh (meets 1e-6 relative Frobenius error against
-the FP64 oracle; `--precision fp32` times the FP32 CUDA-core solve instead). On one GPU the
-same run then
-measures, after the timed region, every other configuration of the method as keys of the
-same line:
+is CG preconditioned by R in the coordinates of its Krylov space: FP32 ensemble, every product
+with HA on the tensor cores (tcgen05) from operands of five exact FP16 slices (48 bits, exact
+FP32 sums), double-float recurrences and a double-float true residual, sums over the CTAs in a
+fixed order (bitwise repeatable; meets 1e-6 relative Frobenius error against the FP64 oracle).
+The FP16, BF16 and FP32 modes share this solve; `--precondition 0` times plain CG on m-vectors,
+where `--precision` and `--reduce-order` choose the kernel. On one GPU the same run then
+measures, after the timed region, every other configuration of the method. The line holds one
+figure of each (`sections`); the whole of them goes to stderr as one more JSON line, and to the
+file named by `--details`:
   c1_variants      the 512x512 workload in plain FP64 CG (the comparison point), FP64 CG
-                   preconditioned by R, plain FP32 CG, and the other preconditioned solves
-                   (FP32 on the CUDA cores, BF16 / FP16 on the tensor cores)
+                   preconditioned by R, plain FP32 CG, and the other preconditioned modes
   reduced_variant, senkf_comparator   the two one-pass variants on the same ensemble
   c2_mixed         1024x1024 GRF, N = 128, m = 262,144: BF16 / FP16 / FP32 / FP64
   c3_batch         256 uneven analyses in one persistent launch (tuned plan, CUDA graph)
@@ -455,15 +455,76 @@ def _err(out, ref):
             "max_abs_err_over_max_abs": float(np.max(np.abs(X - ref)) / np.max(np.abs(ref)))}
 
 
-# how each step's sums over the CTAs are formed (enkf_config.reduce_order)
-DTYPE = {"fp32": "f32", "fp16": "f16", "bf16": "bf16"}
-# (preconditioned by R, the three modes share the Krylov-coordinate solve, its products on exact FP16 slices
-# in tcgen05 and its double-float residual)
+DTYPE = {"fp64": "f64", "fp32": "f32", "fp16": "f16", "bf16": "bf16"}
 PRECISION_NAME = {"fp32": "fp32 CG + double-float residual refresh",
                   "fp16": "FP16 tensor-core contractions (tcgen05) + double-float refresh",
                   "bf16": "BF16 tensor-core contractions (tcgen05) + double-float refresh"}
+# how the sums over the CTAs are formed (enkf_config.reduce_order)
 REDUCE_NAME = {0: "fixed order (bitwise repeatable)",
                1: "atomic adds (N <= 64; last bits vary from run to run)"}
+
+
+def _labels(prec, pc, reduce_order):
+    """(dtype, precision, order of the sums) of a solve. Preconditioned by R, the modes of FP32 ensembles share
+    the solve in Krylov coordinates: products from exact FP16 slices, everything else in FP32 pairs, sums in
+    a fixed order whatever reduce_order says."""
+    if pc and prec != "fp64":
+        return ("f32", f"{prec} mode: products on tcgen05 from exact FP16 slices (48 bits), double-float recurrences and "
+                       "residual", REDUCE_NAME[0])
+    return DTYPE[prec], PRECISION_NAME.get(prec, "fp64 CG"), REDUCE_NAME[reduce_order if prec != "fp64" else 0]
+
+
+def _launches(prec, pc):
+    """Kernels of this library per analysis: innovations, (tile images of HA,) solve, update."""
+    return 4 if prec in ("fp16", "bf16") and not pc else 3
+
+
+# What the line on stdout holds; everything else (5 of its 20 KB are prose) goes to stderr and --details.
+_LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+              "vs_baseline", "dtype", "data", "config", "roofline", "e2e", "gpu_launches", "clocks", "error",
+              "speedup_vs_fp64_plain_cg", "speedup_vs_fp64_pcg")
+
+
+def _section_figures(line):
+    """One figure of every section that was measured: ms per analysis or launch, or a rate."""
+    out = {}
+    for group in ("c1_variants", "c2_mixed"):
+        for k, v in line.get(group, {}).items():
+            if isinstance(v, dict) and "ms_per_step" in v:
+                out[f"{group[:2]}_{k}_ms"] = round(v["ms_per_step"], 4)
+    for k in ("reduced_variant", "senkf_comparator"):
+        if k in line:
+            out[k + "_ms"] = round(line[k]["ms_per_step"], 4)
+    for sec, key in (("c3_batch", "ms_per_launch"), ("c4_warm_start", "loss_last"), ("c0_l96", "cycles_per_s")):
+        if key in line.get(sec, {}):
+            out[f"{sec}_{key}"] = round(line[sec][key], 5)
+    for p, row in line.get("e2b_table5", {}).items():
+        if isinstance(row, dict) and "enkf_reduced_ms" in row:
+            out[f"e2b_{p}_ms"] = round(row["enkf_reduced_ms"], 4)
+    return out
+
+
+def _emit(line, details=None):
+    """The line on stdout, short enough for a reader that keeps the last few KB, and all of it on stderr (and in the
+    file `details`) when there is more."""
+    head = {k: line[k] for k in _LINE_KEYS if k in line}
+    head["e2e"] = {k: v for k, v in line["e2e"].items() if k != "note"} if "e2e" in line else None
+    if head["e2e"] is None:
+        del head["e2e"]
+    if "cpu_baseline" in line:
+        head["cpu_baseline"] = {k: v for k, v in line["cpu_baseline"].items() if k != "sample"}
+    figures = _section_figures(line)
+    if figures:
+        head["sections"] = figures
+    text = json.dumps(line)
+    if details:
+        with open(details, "w") as f:
+            f.write(text + "\n")
+    if set(line) - set(head):
+        print(text, file=sys.stderr, flush=True)
+    print(json.dumps(head), flush=True)
+
+
 KERNEL_NAME = {"fp64": "solve_kernel<double>", "fp32": "solve_kernel<float>",
                "fp16": "solve_mixed_kernel<half>", "bf16": "solve_mixed_kernel<bf16>"}
 
@@ -489,7 +550,7 @@ def _variant(enkf, p, prec, pc, timer, Xd, y, seed, steps, warmup, ref, reduce_o
     res["value"] = 1e3 / res["ms_per_step"]
     res["unit"] = UNIT
     res["solver"] = "CG preconditioned by R" if pc else "plain CG"
-    res["reduce_order"] = REDUCE_NAME[reduce_order]
+    res["reduce_order"] = _labels(prec, pc, reduce_order)[2]
     res["roofline"] = analysis_roofline(p.m, p.N, prec, res["iters"], res["refinements"] if prec != "fp64" else 1,
                                         res["solve_ms"], _solve_kernel(prec, pc)[0], traffic, _solve_kernel(prec, pc)[1])
     an.close()
@@ -592,23 +653,22 @@ def run_ours(args):
             "note": "HA read once per step, x, r, p read and written (28 m N + 4 m) and a double-float refresh "
                     "of 56 m N bytes: what the fused implementation moves at minimum"}
 
-    prec_name = PRECISION_NAME[args.precision]
+    dtype, prec_name, order = _labels(args.precision, args.precondition, args.reduce_order)
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None,
-            "dtype": DTYPE[args.precision],
+            "dtype": dtype,
             "data": "synthetic (seeded 512x512 GRF ensemble, random point observations)",
             "config": {"workload": WORKLOAD, "n": n, "m": m, "N": N, "tol": 1e-8, "precision": prec_name,
                        "solver": "CG preconditioned by R" if args.precondition else "plain CG",
-                       "reduce_order": REDUCE_NAME[args.reduce_order],
+                       "reduce_order": order,
                        "l2": "flushed between steps", "status": last_status["status"]},
             "roofline": roofline, "e2e": e2e,
-            # innovations, (tile images of HA for the tensor-core path,) solve, update
-            "gpu_launches": (3 if args.precision == "fp32" else 4) * args.steps,
+            "gpu_launches": _launches(args.precision, args.precondition) * args.steps,
             "clocks": clk}
     if ws > 1 or args.headline_only:
         if rank == 0:
-            print(json.dumps(line), flush=True)
+            _emit(line, args.details)
         return
 
     # ---- everything below: one GPU, after the timed region
@@ -630,11 +690,6 @@ def run_ours(args):
     c1["fp64_plain_cg"] = _variant(enkf, p, "fp64", 0, timer, X64, y, seed, args.fp64_steps, 1, ref)
     c1["fp64_pcg"] = _variant(enkf, p, "fp64", 1, timer, X64, y, seed, args.fp64_steps, 1, ref)
     c1["fp32_plain_cg"] = _variant(enkf, p, "fp32", 0, timer, Xf, y, seed, args.fp64_steps, 1, ref)
-    # the headline's precision with the other reduction order, then the other precisions with
-    # the headline's order
-    other = 1 - args.reduce_order
-    c1[args.precision + "_pcg_" + ("atomic" if other else "fixed_order")] = _variant(
-        enkf, p, args.precision, 1, timer, Xf, y, seed, max(3, args.steps // 4), 2, ref, reduce_order=other)
     for prec in ("fp32", "fp16", "bf16"):
         if prec != args.precision:
             c1[prec + "_pcg"] = _variant(enkf, p, prec, 1, timer, Xf, y, seed, max(3, args.steps // 4), 2, ref,
@@ -708,7 +763,7 @@ def run_ours(args):
         line["cpu_plain_fp64_cg"] = cpu_cg_baseline(p, seed, int(round(c1["fp64_plain_cg"]["iters"])))
         t_sec["cpu"] = time.time() - t0
     line["section_wall_s"] = t_sec
-    print(json.dumps(line), flush=True)
+    _emit(line, args.details)
 
 
 def _torch_cg_context(enkf, p, X64, y, seed, N, dev, stream):
@@ -1094,7 +1149,7 @@ def run_batched(args):
                        "generation_s": gen_s},
             "roofline": sec.pop("roofline"), "e2e": sec.pop("e2e"), "gpu_launches": args.steps,
             "clocks": clk, "batch": sec}
-    print(json.dumps(line), flush=True)
+    _emit(line, args.details)
 
 
 def run_mixed(args):
@@ -1121,13 +1176,13 @@ def run_mixed(args):
         return
     line = {"metric": METRIC, "value": _job_rate(1, ms / 1e3, ws), "unit": UNIT, "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
-            "vs_baseline": None, "dtype": DTYPE[key[:4]],
+            "vs_baseline": None, "dtype": _labels(key[:4], 1, 0)[0],
             "data": "synthetic (seeded 1024x1024 GRF ensemble, random point observations)",
             "config": {"workload": MIXED_WORKLOAD, "n": res["n"], "m": res["m"], "N": res["N"], "tol": 1e-8,
-                       "precision": PRECISION_NAME[key[:4]], "l2": "flushed between steps"},
-            "roofline": res[key]["roofline"], "variants": res, "gpu_launches": 4 * args.steps,
+                       "precision": _labels(key[:4], 1, 0)[1], "l2": "flushed between steps"},
+            "roofline": res[key]["roofline"], "variants": res, "gpu_launches": _launches(key[:4], 1) * args.steps,
             "clocks": clk}
-    print(json.dumps(line), flush=True)
+    _emit(line, args.details)
 
 
 def main():
@@ -1148,10 +1203,11 @@ def main():
     ap.add_argument("--warm-train-seeds", type=int, default=40,
                     help="ensembles (x 8 observation draws) the learned warm start trains on in the default run")
     ap.add_argument("--reduce-order", type=int, default=1, choices=[0, 1],
-                    help="1 sums each CG step over the CTAs by atomic adds (one grid barrier per step; "
-                         "N <= 64), 0 in a fixed order (bitwise repeatable)")
+                    help="plain CG: 1 sums each step over the CTAs by atomic adds (one grid barrier per step; "
+                         "N <= 64), 0 in a fixed order (bitwise repeatable); preconditioned CG ignores it")
     ap.add_argument("--precision", default="fp16", choices=["fp32", "fp16", "bf16"],
-                    help="inner-solve precision of the timed path (default workload)")
+                    help="mode of the timed path (default workload); preconditioned, the three share one solve")
+    ap.add_argument("--details", default="", help="file that takes the whole of the results as one JSON line")
     ap.add_argument("--batch-count", type=int, default=256,
                     help="problems of the batched workload (256 is the benchmark; fewer for profiling)")
     ap.add_argument("--workload", default=WORKLOAD, choices=[WORKLOAD, BATCH_WORKLOAD, MIXED_WORKLOAD])
