@@ -3,8 +3,10 @@
 // Algorithm 1 (innovations, CG solve of S Z = D with the matrix-free product of the
 // matvec decomposition, X_a = X_f + A HA^T Z / (N - 1)), in the FP32-with-refresh mode.
 //
-// Planning (host): a problem is costed at m N^2 (N + 8) + 2 n N^2 (about N preconditioned
-// steps of 4 m N^2 flops each, plus the update). The planner minimises the estimated
+// Planning (host): a problem is costed at m N^2 (N + 8) + 2 n N^2, a model of about N
+// preconditioned steps on m-vectors of 4 m N^2 flops each, plus the update. (The solve in Krylov
+// coordinates costs three passes over 64-row tiles per cycle, nearly alike for N up to 64 and twice that
+// above, so the model gives large N too many CTAs; the tuner's measured costs replace it.) The planner minimises the estimated
 // makespan: problems costlier than the target get a team of CTAs of their own, the rest wait
 // in a queue, longest first (make_plan). Every team works through its problem; for each it
 // runs the innovations over its rows, the persistent CG solve with a bounded barrier over the
@@ -221,6 +223,7 @@ struct BatchState {
 
 static int nt_of(int N) { return N <= 32 ? 32 : (N <= 64 ? 64 : 128); }
 
+// (a model of the steps on m-vectors: see the head of this file)
 static double problem_cost(const enkf_config& c) {
   const double m = (double)c.m, N = c.N, n = (double)c.n;
   return m * N * N * (N + 8.0) + 2.0 * n * N * N;

@@ -12,8 +12,8 @@
 // [(r, z) | (r, r) | sum r_i z^2 | sum r_i z p]. FP64 mode: scalars in FP64, X is the solution, with a true
 // residual after the solve. FP32 mode: scalars and sums in double-float, inner solves from zero refined by the
 // double-float residual (HA's low parts read from global memory), as in the persistent solve.
-// Measured (analysis, persistent solve before): m = N = 20 in FP64 650 -> 131 us, m = 3,001, N = 37 in
-// FP32 without preconditioning 2,610 -> 712 us.
+// Measured (analysis, persistent solve before): m = N = 20 in FP64 685 -> 116 us, m = 3,001, N = 37 in
+// FP32 without preconditioning 2,550 -> 672 us.
 #include <cooperative_groups.h>
 
 #include <algorithm>

@@ -7,9 +7,12 @@
 // memory: with K <= 128 terms and at most seven digit pairs per level i + j = g, a level's sum is at most
 // 7 x 128 x 2^14 < 2^24 whatever the operands. The levels 0 to 7 (34 digit products) are kept: what is left out
 // is below 5 x 2^-64 of a full-scale term, an entry is cut at 2^-56 of its row's or column's largest and a sum
-// at 2^-56 of a full-scale term, so that a sum is as good as one in FP64, whose terms and partial sums are
-// rounded at 2^-53. (With the levels 0 to 6 and sums cut downwards at 2^-53 the analysis at m = 10,000,
-// N = 100 lost a digit: 3.8e-14 against 2.3e-15.) A sum leaves tensor memory as integers, and becomes an FP64
+// at 2^-56 of a full-scale term, so that a product is as good as one in FP64 in norm: an FP64 sum's terms and
+// partial sums are rounded at 2^-53 of themselves. Entry by entry it is not: entries below an eighth of their
+// row's or column's largest hold fewer than 53 bits, and a sum of such entries only (a member much smaller
+// than the others, in the products whose scales run across members) loses those bits. (With the levels 0 to 6
+// and sums cut downwards at 2^-53 the analysis at m = 10,000, N = 100 lost a digit: 3.8e-14 against 2.3e-15;
+// with these it is 1.9e-15 off.) A sum leaves tensor memory as integers, and becomes an FP64
 // number with integer operations only: conversions and scalings on the FP64 unit would take longer
 // than the products.
 //
