@@ -431,12 +431,9 @@ __global__ void __launch_bounds__(kThreads) reduced_cg_kernel(
         bn2 = r2;
         stop2 = tol_s * tol_s * bn2;
       }
-      // a NaN or an infinity in G or in m_j ends the column at once (and fails every comparison below)
       bool go = it < limit && (it == 0 || fixed ? r2 > 0.0 : r2 > stop2);
-      if (!isfinite(r2)) {
-        if (lane == 0) atomicOr(status, DS_NONFINITE);
-        go = false;
-      }
+      // (a NaN in G or m_j fails the comparisons at step 0; an infinity makes q below non-finite)
+      if (!go && !isfinite(r2) && lane == 0) atomicOr(status, DS_NONFINITE);
       const double be = go && it > 0 ? r2 * sc[3] : 0.0;
       double al = 0.0;
       if (go) {
