@@ -122,9 +122,13 @@ def _tensor_peak():
 
 def analysis_roofline(m, N, prec, iters, refreshes, solve_ms, kernel, traffic=None, krylov=False):
     """Roofline of one solve launch on the byte and flop models above (krylov: the passes of its
-    refinement cycles, whose products run on the tensor cores in every mode)."""
+    refinement cycles, whose products run on the tensor cores in every mode; solve64_kernel: FP64
+    products of 34 FP16 products each)."""
     bw, bw_src = _peaks()
     pf, pf_src = _peak_flops("fp16" if krylov else prec)
+    digits = kernel == "solve64_kernel"
+    if digits:
+        pf, pf_src = _tensor_peak() / 34.0, "dense BF16/FP16 tensor, measured sustained, 34 digit products per FP64 product"
     if krylov:
         B, F = refreshes * B_CYCLE(m, N), refreshes * F_CYCLE(m, N)
     else:
@@ -140,18 +144,17 @@ def analysis_roofline(m, N, prec, iters, refreshes, solve_ms, kernel, traffic=No
                 "launch_ms": solve_ms, "cg_iterations": iters, "refreshes": refreshes,
                 "compute_bound_frac": t_f / t}
     unit = "TFLOP/s"
-    return {"bound": "tensor" if prec in ("fp16", "bf16") else "alu", "achieved": F / t / 1e12, "peak": pf,
+    return {"bound": "tensor" if prec in ("fp16", "bf16") or digits else "alu", "achieved": F / t / 1e12, "peak": pf,
             "unit": unit, "frac": t_f / t, "traffic": traffic, "kernel": kernel, "peak_source": pf_src,
             "algorithmic_bytes_per_launch": B, "algorithmic_flops_per_launch": F, "launch_ms": solve_ms,
             "cg_iterations": iters, "refreshes": refreshes, "hbm_frac": t_b / t}
 
-# DRAM bytes (read + write) of one solve launch on this workload per precision, from the ncu
-# captures summarised under profiles/ (FP32: solve_kernel_fp32_hs_grf512_N64_m65536.md; FP16:
-# solve_mixed_kernel_fp16_grf512_N64_m65536.md; both with atomic step sums, the default), with
-# the hash of the kernel sources each capture measured; reported as null once those sources
+# DRAM bytes (read + write) of one preconditioned solve launch on this workload, from the ncu
+# capture summarised in profiles/krylov_and_digit_kernels.md (the modes share the kernel), with
+# the hash of the kernel sources the capture measured; reported as null once those sources
 # have changed.
-NCU_TRAFFIC = {"fp32": {"bytes": 0.765940e9, "src_sha": "e360a9e69a4aec5f"},
-               "fp16": {"bytes": 0.800592e9, "src_sha": "ceff5266981415e8"}}
+NCU_TRAFFIC = {"fp32": {"bytes": 0.279462e9, "src_sha": "485bc9be846a45cd"},
+               "fp16": {"bytes": 0.279462e9, "src_sha": "485bc9be846a45cd"}}
 # DRAM bytes of one batch_kernel launch on the 256-problem batch (seed 1), recorded in
 # profiles/batch_kernel_batched256_grf_dram.md for the sources with this hash.
 NCU_TRAFFIC_BATCH = {"bytes": 1.436453e12, "problems": 256, "seed": 1, "src_sha": "869cf69968486ece"}
@@ -165,7 +168,7 @@ _KERNEL_SOURCES = {
 
 def _recorded_traffic(precision, precondition, reduce_order):
     """The captured DRAM bytes of one solve launch on the 512^2 workload, if the capture's
-    configuration (CG preconditioned by R, atomic step sums) and kernel sources are these."""
+    configuration (CG preconditioned by R, the default reduce_order) and kernel sources are these."""
     tr = NCU_TRAFFIC.get(precision)
     if tr is None or precondition != 1 or reduce_order != 1 or tr["src_sha"] != _src_hash(precision):
         return None
@@ -529,8 +532,8 @@ KERNEL_NAME = {"fp64": "solve_kernel<double>", "fp32": "solve_kernel<float>",
                "fp16": "solve_mixed_kernel<half>", "bf16": "solve_mixed_kernel<bf16>"}
 
 
-def _solve_kernel(prec, pc):
-    if not pc:
+def _solve_kernel(prec, pc, N):
+    if not pc or (prec == "fp64" and N > 64):
         return KERNEL_NAME[prec], False
     return ("solve64_kernel", False) if prec == "fp64" else ("krylov_kernel", True)
 
@@ -552,7 +555,8 @@ def _variant(enkf, p, prec, pc, timer, Xd, y, seed, steps, warmup, ref, reduce_o
     res["solver"] = "CG preconditioned by R" if pc else "plain CG"
     res["reduce_order"] = _labels(prec, pc, reduce_order)[2]
     res["roofline"] = analysis_roofline(p.m, p.N, prec, res["iters"], res["refinements"] if prec != "fp64" else 1,
-                                        res["solve_ms"], _solve_kernel(prec, pc)[0], traffic, _solve_kernel(prec, pc)[1])
+                                        res["solve_ms"], _solve_kernel(prec, pc, p.N)[0], traffic,
+                                        _solve_kernel(prec, pc, p.N)[1])
     an.close()
     return res
 
@@ -645,8 +649,8 @@ def run_ours(args):
     solve_avg_ms = float(np.mean(solve_ms))
     traffic = _recorded_traffic(args.precision, args.precondition, args.reduce_order)
     roofline = analysis_roofline(m, N, args.precision, it_avg, ref_avg, solve_avg_ms,
-                                 _solve_kernel(args.precision, args.precondition)[0] + "<64>", traffic,
-                                 _solve_kernel(args.precision, args.precondition)[1])
+                                 _solve_kernel(args.precision, args.precondition, N)[0] + "<64>", traffic,
+                                 _solve_kernel(args.precision, args.precondition, N)[1])
     if not args.precondition:
         roofline["fused_pass_model"] = {
             "bytes_per_launch": it_avg * B_FUSED(m, N) + ref_avg * 56 * m * N,
@@ -736,14 +740,14 @@ def run_ours(args):
         "phases_ms": dict(zip(("gram", "nxn_cg", "update"), reduced_ph)),
         "cg_iterations": reduced_st["iters_max"], "status": reduced_st["status"], **err_reduced,
         "roofline_gram": _gram_roofline(2.0 * m * N * N, reduced_ph[0], m, N),
-        "method": "Algorithm 2 with CG on I + P^T P (N x N), FP32 ensemble, double-float Gram"}
+        "method": "Algorithm 2 with CG on I + P^T P (N x N), FP32 ensemble, Gram products from exact FP16 slices"}
     line["senkf_comparator"] = {
         "ms_per_step": senkf_ms, "value": 1e3 / senkf_ms, "unit": UNIT,
         "phases_ms": dict(zip(("gram", "sum", "update"), senkf_ph)),
         "rel_frobenius_vs_exact_enkf": err_senkf, "rel_frobenius_vs_oracle_senkf": err_senkf_oracle,
         "roofline_gram": _gram_roofline(1.0 * m * N * N, senkf_ph[0], m, N),
-        "method": "Algorithm 3 (diagonal inverse of S, no solve), FP32 ensemble, double-float Gram; "
-                  "an approximation of the EnKF analysis"}
+        "method": "Algorithm 3 (diagonal inverse of S, no solve), FP32 ensemble, Gram products from exact FP16 "
+                  "slices; an approximation of the EnKF analysis"}
     line["torch_fp64_cg_context"] = _torch_cg_context(enkf, p, X64, y, seed, N, dev, stream)
     t_sec["c1"] = time.time() - t0
 

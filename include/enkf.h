@@ -225,7 +225,9 @@ enkf_status enkf_create_tridiag(const enkf_config* cfg, const int32_t* h_rowptr,
    Box-Muller give the normal, E_ij = sqrt(r_i) * normal; ENKF_FP64 evaluates Box-Muller in
    FP64, the FP32 and tensor-core modes (every variant) in FP32 from the same uniforms,
    within about 1e-7 of the FP64 normal). d_Xa: device [n][N], same dtype
-   as d_Xf; d_Xa == d_Xf (in-place) is allowed, partial overlap is not. Never allocates. */
+   as d_Xf; d_Xa == d_Xf (in-place) is allowed, partial overlap is not. Both need the
+   alignment of their elements only (16-byte boundaries and N % 4 == 0 take the wider
+   accesses of the update). Never allocates. */
 enkf_status enkf_analyze(enkf_handle h, const void* d_Xf, const double* d_y, uint64_t seed,
                          uint64_t counter, void* d_Xa);
 
