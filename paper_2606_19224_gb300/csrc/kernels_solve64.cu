@@ -488,7 +488,9 @@ __global__ void __launch_bounds__(kQT, 1) solve64_kernel(Solve64Params p) {
 
 // Whether FP64 CG ends before rounding decides where it goes. Preconditioned by R, or with R a multiple of the
 // identity, it sees at most N + 1 distinct eigenvalues and takes some 25 steps to 1e-8 (m = 16,384, N = 64): two
-// evaluation orders then agree to 1e-13. Without, a varying R spreads the spectrum: 90 steps, the recurrences
+// evaluation orders then agree to 1e-13. (With few rows per member it takes more, 38 at m = 438, N = 66, and
+// half a unit in HA's last place moves the analysis by up to 1e-8 here too, at the same distance from the exact
+// one: results of this route and of the persistent solve agree to tol there, 4e-9.) Without, a varying R spreads the spectrum: 90 steps, the recurrences
 // lose their orthogonality, and inputs that differ in the last bit give analyses that differ by as much as
 // the tolerance leaves, 2.5e-8. Such an analysis keeps the persistent solve of solve_body.cuh and with it its results.
 bool steady_fp64(const enkf_handle_s* h) { return h->cfg.precondition != 0 || h->r_const; }

@@ -1,8 +1,8 @@
 """What rounding alone does to plain FP64 CG with a varying R, and to CG preconditioned by R: the same solve with
 every entry of HA moved by half a unit in its last place. Plain CG takes some 90 steps here, its recurrences lose
 their orthogonality, and where they stop (||r|| <= 1e-8 ||d||) depends on the last bits: the analyses
-differ by up to what that tolerance leaves, whichever form evaluates them. Preconditioned CG ends before
-rounding matters. (The GPU library keeps one evaluation order for the former and chooses freely for the latter.)"""
+differ by up to what that tolerance leaves, whichever form evaluates them. Preconditioned CG, with some tens of
+rows per member, ends before rounding matters. (The GPU library keeps one evaluation order for the former and chooses freely for the latter.)"""
 import numpy as np
 
 import synth
